@@ -1,12 +1,14 @@
-"""ctypes binding over libnpas.so: argument marshalling only, every step runs in the CUDA kernels.
+"""Binding over libnpas.so: argument marshalling only, every step runs in the CUDA kernels.
 
 The function names mirror the C ABI (include/npas.h).  Tensors are torch CUDA tensors used purely
-as device buffers; calls are enqueued on torch's current stream.  There is no CPU fallback: when
-the shared library is missing or a call fails, an exception is raised.
+as device buffers; calls are enqueued on torch's current stream.  The compute calls go through a
+CPython extension (csrc/host_ext.cpp), the rest through ctypes.  There is no CPU fallback: when
+a shared library is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -15,9 +17,11 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libnpas.so")
+HOST_PATH = os.path.join(_HERE, "_npas_host.so")
 WORKSPACE_BYTES = 256
 F32, BF16 = 0, 1
 _lib = None
+_host = None                     # the extension module, from the first load() on
 
 
 class NpasError(RuntimeError):
@@ -55,10 +59,11 @@ EXPORTS = ["npas_status_string", "npas_abi_version", "npas_mask_bp_from_dense", 
 
 def load() -> ctypes.CDLL:
     """Load the CUDA library; raises if it has not been built (there is no other code path)."""
-    global _lib
+    global _lib, _host
     if _lib is None:
-        if not os.path.exists(LIB_PATH):
-            raise FileNotFoundError(f"{LIB_PATH} is missing: build it with paper_2012_00596_b200/build.py")
+        for path in (LIB_PATH, HOST_PATH):
+            if not os.path.exists(path):
+                raise FileNotFoundError(f"{path} is missing: build it with paper_2012_00596_b200/build.py")
         lib = ctypes.CDLL(LIB_PATH)
         for name in EXPORTS:
             getattr(lib, name)
@@ -70,8 +75,15 @@ def load() -> ctypes.CDLL:
             if name == "npas_launch_count":
                 continue
             getattr(lib, name).restype = ctypes.c_int
-        _lib = lib
+        spec = importlib.util.spec_from_file_location("_npas_host", HOST_PATH)
+        host = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(host)
+        _host, _lib = host, lib
     return _lib
+
+
+def _refused(code: int, what: str):
+    raise NpasError(code, what)
 
 
 def status_string(code: int) -> str:
@@ -285,42 +297,18 @@ def blob_check(blob) -> None:
 def conv2d_bp(x: torch.Tensor, blob: BpBlob, bias=None, residual=None, *, stride=1, pad=1, relu=False,
               out_dtype=None, out=None, ws=None, path=0, variant=0) -> torch.Tensor:
     """npas_conv2d_bp on NHWC x; returns NHWC y (allocated here unless ``out`` is given)."""
-    lib = load()
-    assert x.is_cuda and x.is_contiguous() and x.dim() == 4
-    N, H, W, C = x.shape
-    d = blob.desc
-    P = (H + 2 * pad - d.R) // stride + 1
-    Q = (W + 2 * pad - d.S) // stride + 1
-    ydt = x.dtype if out_dtype is None else out_dtype
-    if out is None:
-        out = torch.empty((N, P, Q, d.K), dtype=ydt, device=x.device)
-    if ws is None:
-        ws = workspace(x.device)
-    cd = ConvDesc(N, H, W, C, d.K, d.R, d.S, stride, pad, _dt(x), _dt(out), int(bool(relu)),
-                  int(bias is not None), int(residual is not None), path, variant)
-    _check(lib.npas_conv2d_bp(ctypes.byref(cd), ctypes.byref(d), _p(x), _p(blob.data), _p(bias), _p(residual),
-                              _p(out), _p(ws), ctypes.c_size_t(ws.numel()), _stream()), "npas_conv2d_bp")
-    return out
+    if _host is None:
+        load()
+    y = _host.conv2d_bp(x, blob.data, blob.desc, bias, residual, stride, pad, relu, out_dtype, out, ws, path, variant)
+    return y if type(y) is not int else _refused(y, "npas_conv2d_bp")
 
 
 def linear_bb(x: torch.Tensor, blob: BbBlob, bias=None, residual=None, *, relu=False, out_dtype=None, out=None,
               ws=None, path=0, variant=0) -> torch.Tensor:
-    lib = load()
-    assert x.is_cuda and x.is_contiguous() and x.dim() == 2
-    M, I = x.shape
-    d = blob.desc
-    ydt = x.dtype if out_dtype is None else out_dtype
-    if out is None:
-        out = torch.empty((M, d.O), dtype=ydt, device=x.device)
-    if ws is None:
-        ws = workspace(x.device)
-    if residual is not None:
-        assert residual.is_cuda and residual.is_contiguous() and residual.shape == out.shape and residual.dtype == out.dtype
-    ld = LinearDesc(M, I, d.O, _dt(x), _dt(out), int(bool(relu)), int(bias is not None), int(residual is not None), path,
-                    variant)
-    _check(lib.npas_linear_bb(ctypes.byref(ld), ctypes.byref(d), _p(x), _p(blob.data), _p(bias), _p(residual), _p(out),
-                              _p(ws), ctypes.c_size_t(ws.numel()), _stream()), "npas_linear_bb")
-    return out
+    if _host is None:
+        load()
+    y = _host.linear_bb(x, blob.data, blob.desc, bias, residual, relu, out_dtype, out, ws, path, variant)
+    return y if type(y) is not int else _refused(y, "npas_linear_bb")
 
 
 def subsample2d(x: torch.Tensor, stride: int) -> torch.Tensor:
@@ -356,22 +344,11 @@ def conv2d_bp_maxpool(x: torch.Tensor, blob: BpBlob, bias=None, *, stride=1, pad
                       ws=None, path=0) -> torch.Tensor:
     """npas_conv2d_bp_maxpool: convolution + bias + ReLU + max-pool fused in one kernel; returns the pooled
     NHWC tensor.  Raises NpasError(8) where no kernel has the fused epilogue (run the two calls then)."""
-    lib = load()
-    assert x.is_cuda and x.is_contiguous() and x.dim() == 4
-    N, H, W, C = x.shape
-    d = blob.desc
-    P = (H + 2 * pad - d.R) // stride + 1
-    Q = (W + 2 * pad - d.S) // stride + 1
+    if _host is None:
+        load()
     pr, ps, pp = pool
-    PP, PQ = (P + 2 * pp - pr) // ps + 1, (Q + 2 * pp - pr) // ps + 1
-    if out is None:
-        out = torch.empty((N, PP, PQ, d.K), dtype=x.dtype, device=x.device)
-    if ws is None:
-        ws = workspace(x.device)
-    cd = ConvDesc(N, H, W, C, d.K, d.R, d.S, stride, pad, _dt(x), _dt(out), int(bool(relu)), int(bias is not None), 0, path, 0)
-    _check(lib.npas_conv2d_bp_maxpool(ctypes.byref(cd), ctypes.byref(d), pr, ps, pp, _p(x), _p(blob.data), _p(bias), _p(out),
-                                      _p(ws), ctypes.c_size_t(ws.numel()), _stream()), "npas_conv2d_bp_maxpool")
-    return out
+    y = _host.conv2d_bp_maxpool(x, blob.data, blob.desc, bias, stride, pad, relu, pr, ps, pp, out, ws, path)
+    return y if type(y) is not int else _refused(y, "npas_conv2d_bp_maxpool")
 
 
 def conv2d_bp_static_ws(x: torch.Tensor, blob: BpBlob, bias=None, residual=None, *, stride=1, pad=1, relu=False,

@@ -1,0 +1,267 @@
+// The compute calls of the Python binding, in native code: argument checks, descriptors, the output tensor, the
+// current stream and the library call, without a Python-level step in between.
+//
+// A call through ctypes spent 14 us of host time (descriptor objects, pointer wrappers, stream lookup, and torch's
+// own Python entry for the output tensor), more than most layers take on the GPU.  This file is an ordinary CPython
+// extension that links against libnpas.so; binding.py keeps the public functions, with their arguments, defaults
+// and errors, and hands their arguments over positionally.  A compute function returns the output tensor, or the
+// npas_status as an int when the library refused the call (binding.py raises).
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <ATen/cuda/EmptyTensor.h>
+#include <ATen/ops/zeros.h>
+#include <c10/cuda/CUDAGuard.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Dtype.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <atomic>
+#include <mutex>
+
+#include "npas.h"
+
+namespace {
+
+bool fail_assert(const char *what)
+{
+    PyErr_SetString(PyExc_AssertionError, what);
+    return false;
+}
+
+// A tensor argument (None allowed where `optional`); the reference stays borrowed from the argument.
+bool tensor_arg(PyObject *o, const at::Tensor *&t, bool optional, const char *name)
+{
+    t = nullptr;
+    if (optional && o == Py_None) return true;
+    if (!THPVariable_Check(o)) { PyErr_Format(PyExc_TypeError, "%s must be a torch.Tensor", name); return false; }
+    t = &THPVariable_Unpack(o);
+    return true;
+}
+
+bool int_arg(PyObject *o, int32_t &v)
+{
+    const long l = PyLong_AsLong(o);
+    if (l == -1 && PyErr_Occurred()) return false;
+    v = (int32_t)l;
+    return true;
+}
+
+bool dtype_of(at::ScalarType t, int32_t &code)
+{
+    if (t == at::kFloat) { code = NPAS_F32; return true; }
+    if (t == at::kBFloat16) { code = NPAS_BF16; return true; }
+    PyErr_Format(PyExc_TypeError, "unsupported dtype %s", c10::toString(t));
+    return false;
+}
+
+bool dtype_arg(PyObject *o, at::ScalarType otherwise, at::ScalarType &t)
+{
+    if (o == Py_None) { t = otherwise; return true; }
+    if (!THPDtype_Check(o)) { PyErr_SetString(PyExc_TypeError, "out_dtype must be a torch.dtype"); return false; }
+    t = reinterpret_cast<THPDtype *>(o)->scalar_type;
+    return true;
+}
+
+// The descriptor structures are ctypes objects that the caller may have changed: read through the buffer protocol.
+template <typename D>
+bool desc_arg(PyObject *o, D &d)
+{
+    Py_buffer view;
+    if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) return false;
+    const bool ok = view.len == (Py_ssize_t)sizeof(D);
+    if (ok) memcpy(&d, view.buf, sizeof(D));
+    PyBuffer_Release(&view);
+    if (!ok) PyErr_SetString(PyExc_TypeError, "descriptor of the wrong type");
+    return ok;
+}
+
+void *ptr(const at::Tensor *t) { return t ? t->data_ptr() : nullptr; }
+
+at::Tensor new_tensor(at::IntArrayRef size, at::ScalarType t, const at::Device &dev)
+{
+    return at::Tensor(at::detail::empty_cuda(size, t, dev, std::nullopt));
+}
+
+// Status words for calls that bring no workspace: nobody can read them afterwards, so all such calls on a device share
+// one buffer, kept for the life of the process (a zeroed allocation per call cost a launch).  A call inside a stream
+// capture that finds none yet gets one of its own.
+bool shared_workspace(const at::Device &dev, at::Tensor &own, void *&p)
+{
+    constexpr int kMaxDevices = 64;
+    static std::atomic<void *> kept[kMaxDevices];
+    static std::mutex mu;
+    const int i = dev.index();
+    if (i >= 0 && i < kMaxDevices && (p = kept[i].load(std::memory_order_acquire)) != nullptr) return true;
+    const auto opt = at::TensorOptions().dtype(at::kByte).device(dev);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(c10::cuda::getCurrentCUDAStream().stream(), &cap);
+    if (cap != cudaStreamCaptureStatusNone || i < 0 || i >= kMaxDevices) {
+        own = at::zeros({NPAS_WORKSPACE_BYTES}, opt);
+        p = own.data_ptr();
+        return true;
+    }
+    std::lock_guard<std::mutex> lock(mu);
+    if ((p = kept[i].load(std::memory_order_acquire)) == nullptr) {
+        auto *t = new at::Tensor(at::zeros({NPAS_WORKSPACE_BYTES}, opt));      // (never freed: it lives as long as the process)
+        cudaStreamSynchronize(c10::cuda::getCurrentCUDAStream().stream());     // other streams may use it from here on
+        p = t->data_ptr();
+        kept[i].store(p, std::memory_order_release);
+    }
+    return true;
+}
+
+bool workspace_arg(const at::Tensor *ws, const at::Tensor &x, at::Tensor &own, void *&p, size_t &bytes)
+{
+    if (ws) { p = ws->data_ptr(); bytes = (size_t)ws->numel(); return true; }
+    bytes = NPAS_WORKSPACE_BYTES;
+    return shared_workspace(x.device(), own, p);
+}
+
+PyObject *result(npas_status s, PyObject *out_given, at::Tensor &&made)
+{
+    if (s != NPAS_OK) return PyLong_FromLong((long)s);
+    if (out_given) { Py_INCREF(out_given); return out_given; }
+    return THPVariable_Wrap(std::move(made));
+}
+
+template <typename F>
+PyObject *guarded(F f)
+{
+    try {
+        return f();
+    } catch (const std::exception &e) {
+        if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
+        return nullptr;
+    }
+}
+
+// conv2d_bp(x, blob, desc, bias, residual, stride, pad, relu, out_dtype, out, ws, path, variant)
+PyObject *conv2d_bp(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        const at::Tensor *x, *blob, *bias, *res, *out, *ws;
+        npas_bp_desc bp;
+        npas_conv_desc d = {};
+        at::ScalarType ot;
+        if (n != 13) { PyErr_SetString(PyExc_TypeError, "conv2d_bp takes 13 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], x, false, "x") || !tensor_arg(a[1], blob, false, "blob.data") || !desc_arg(a[2], bp) ||
+            !tensor_arg(a[3], bias, true, "bias") || !tensor_arg(a[4], res, true, "residual") || !int_arg(a[5], d.stride) ||
+            !int_arg(a[6], d.pad) || !tensor_arg(a[9], out, true, "out") || !tensor_arg(a[10], ws, true, "ws") ||
+            !int_arg(a[11], d.path) || !int_arg(a[12], d.variant))
+            return nullptr;
+        const int relu = PyObject_IsTrue(a[7]);
+        if (relu < 0) return nullptr;
+        if (!(x->is_cuda() && x->is_contiguous() && x->dim() == 4)) { fail_assert("x must be a contiguous 4-D CUDA tensor"); return nullptr; }
+        if (!dtype_arg(a[8], x->scalar_type(), ot)) return nullptr;
+        if (d.stride == 0) { PyErr_SetString(PyExc_ZeroDivisionError, "stride is zero"); return nullptr; }
+        d.N = (int32_t)x->size(0); d.H = (int32_t)x->size(1); d.W = (int32_t)x->size(2); d.C = (int32_t)x->size(3);
+        d.K = bp.K; d.R = bp.R; d.S = bp.S;
+        d.relu = relu; d.has_bias = bias != nullptr; d.has_residual = res != nullptr;
+        auto positions = [&](int64_t in, int64_t taps) {      // floor division, as the shape of the output tensor
+            const int64_t v = in + 2 * (int64_t)d.pad - taps, q = v / d.stride;
+            return q - ((v % d.stride != 0) && ((v < 0) != (d.stride < 0)) ? 1 : 0) + 1;
+        };
+        at::Tensor made, own;
+        if (!out) made = new_tensor({x->size(0), positions(x->size(1), bp.R), positions(x->size(2), bp.S), bp.K}, ot, x->device());
+        if (!dtype_of(x->scalar_type(), d.x_dtype) || !dtype_of(out ? out->scalar_type() : ot, d.y_dtype)) return nullptr;
+        void *w = nullptr, *y = out ? out->data_ptr() : made.data_ptr();
+        size_t wb = 0;
+        if (!workspace_arg(ws, *x, own, w, wb)) return nullptr;
+        void *st = c10::cuda::getCurrentCUDAStream().stream();
+        npas_status s;
+        Py_BEGIN_ALLOW_THREADS
+        s = npas_conv2d_bp(&d, &bp, x->data_ptr(), blob->data_ptr(), static_cast<const float *>(ptr(bias)), ptr(res), y, w, wb, st);
+        Py_END_ALLOW_THREADS
+        return result(s, out ? a[9] : nullptr, std::move(made));
+    });
+}
+
+// conv2d_bp_maxpool(x, blob, desc, bias, stride, pad, relu, pool_r, pool_stride, pool_pad, out, ws, path)
+PyObject *conv2d_bp_maxpool(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        const at::Tensor *x, *blob, *bias, *out, *ws;
+        npas_bp_desc bp;
+        npas_conv_desc d = {};
+        int32_t pr, ps, pp;
+        if (n != 13) { PyErr_SetString(PyExc_TypeError, "conv2d_bp_maxpool takes 13 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], x, false, "x") || !tensor_arg(a[1], blob, false, "blob.data") || !desc_arg(a[2], bp) ||
+            !tensor_arg(a[3], bias, true, "bias") || !int_arg(a[4], d.stride) || !int_arg(a[5], d.pad) || !int_arg(a[7], pr) ||
+            !int_arg(a[8], ps) || !int_arg(a[9], pp) || !tensor_arg(a[10], out, true, "out") || !tensor_arg(a[11], ws, true, "ws") ||
+            !int_arg(a[12], d.path))
+            return nullptr;
+        const int relu = PyObject_IsTrue(a[6]);
+        if (relu < 0) return nullptr;
+        if (!(x->is_cuda() && x->is_contiguous() && x->dim() == 4)) { fail_assert("x must be a contiguous 4-D CUDA tensor"); return nullptr; }
+        if (d.stride == 0 || ps == 0) { PyErr_SetString(PyExc_ZeroDivisionError, "stride is zero"); return nullptr; }
+        d.N = (int32_t)x->size(0); d.H = (int32_t)x->size(1); d.W = (int32_t)x->size(2); d.C = (int32_t)x->size(3);
+        d.K = bp.K; d.R = bp.R; d.S = bp.S;
+        d.relu = relu; d.has_bias = bias != nullptr;
+        auto floor_div = [](int64_t v, int64_t q) { return v / q - ((v % q != 0) && ((v < 0) != (q < 0)) ? 1 : 0); };
+        const int64_t P = floor_div(x->size(1) + 2 * d.pad - bp.R, d.stride) + 1, Q = floor_div(x->size(2) + 2 * d.pad - bp.S, d.stride) + 1;
+        at::Tensor made, own;
+        if (!out) made = new_tensor({x->size(0), floor_div(P + 2 * pp - pr, ps) + 1, floor_div(Q + 2 * pp - pr, ps) + 1, bp.K}, x->scalar_type(), x->device());
+        if (!dtype_of(x->scalar_type(), d.x_dtype) || !dtype_of(out ? out->scalar_type() : x->scalar_type(), d.y_dtype)) return nullptr;
+        void *w = nullptr, *y = out ? out->data_ptr() : made.data_ptr();
+        size_t wb = 0;
+        if (!workspace_arg(ws, *x, own, w, wb)) return nullptr;
+        void *st = c10::cuda::getCurrentCUDAStream().stream();
+        npas_status s;
+        Py_BEGIN_ALLOW_THREADS
+        s = npas_conv2d_bp_maxpool(&d, &bp, pr, ps, pp, x->data_ptr(), blob->data_ptr(), static_cast<const float *>(ptr(bias)), y, w, wb, st);
+        Py_END_ALLOW_THREADS
+        return result(s, out ? a[10] : nullptr, std::move(made));
+    });
+}
+
+// linear_bb(x, blob, desc, bias, residual, relu, out_dtype, out, ws, path, variant)
+PyObject *linear_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        const at::Tensor *x, *blob, *bias, *res, *out, *ws;
+        npas_bb_desc bb;
+        npas_linear_desc d = {};
+        at::ScalarType ot;
+        if (n != 11) { PyErr_SetString(PyExc_TypeError, "linear_bb takes 11 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], x, false, "x") || !tensor_arg(a[1], blob, false, "blob.data") || !desc_arg(a[2], bb) ||
+            !tensor_arg(a[3], bias, true, "bias") || !tensor_arg(a[4], res, true, "residual") || !tensor_arg(a[7], out, true, "out") ||
+            !tensor_arg(a[8], ws, true, "ws") || !int_arg(a[9], d.path) || !int_arg(a[10], d.variant))
+            return nullptr;
+        const int relu = PyObject_IsTrue(a[5]);
+        if (relu < 0) return nullptr;
+        if (!(x->is_cuda() && x->is_contiguous() && x->dim() == 2)) { fail_assert("x must be a contiguous 2-D CUDA tensor"); return nullptr; }
+        if (!dtype_arg(a[6], x->scalar_type(), ot)) return nullptr;
+        at::Tensor made, own;
+        if (!out) made = new_tensor({x->size(0), bb.O}, ot, x->device());
+        const at::Tensor &y = out ? *out : made;
+        if (res && !(res->is_cuda() && res->is_contiguous() && res->sizes() == y.sizes() && res->scalar_type() == y.scalar_type())) {
+            fail_assert("residual must be a contiguous CUDA tensor of the output's shape and dtype");
+            return nullptr;
+        }
+        d.M = (int32_t)x->size(0); d.I = (int32_t)x->size(1); d.O = bb.O;
+        if (!dtype_of(x->scalar_type(), d.x_dtype) || !dtype_of(y.scalar_type(), d.y_dtype)) return nullptr;
+        d.relu = relu; d.has_bias = bias != nullptr; d.has_residual = res != nullptr;
+        void *w = nullptr, *yp = y.data_ptr();
+        size_t wb = 0;
+        if (!workspace_arg(ws, *x, own, w, wb)) return nullptr;
+        void *st = c10::cuda::getCurrentCUDAStream().stream();
+        npas_status s;
+        Py_BEGIN_ALLOW_THREADS
+        s = npas_linear_bb(&d, &bb, x->data_ptr(), blob->data_ptr(), static_cast<const float *>(ptr(bias)), ptr(res), yp, w, wb, st);
+        Py_END_ALLOW_THREADS
+        return result(s, out ? a[7] : nullptr, std::move(made));
+    });
+}
+
+PyMethodDef kMethods[] = {
+    {"conv2d_bp", (PyCFunction)(void (*)(void))conv2d_bp, METH_FASTCALL, nullptr},
+    {"conv2d_bp_maxpool", (PyCFunction)(void (*)(void))conv2d_bp_maxpool, METH_FASTCALL, nullptr},
+    {"linear_bb", (PyCFunction)(void (*)(void))linear_bb, METH_FASTCALL, nullptr},
+    {nullptr, nullptr, 0, nullptr}};
+
+PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_npas_host", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__npas_host() { return PyModule_Create(&kModule); }
