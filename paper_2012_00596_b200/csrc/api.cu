@@ -132,19 +132,28 @@ static int conv_kernel_for(const npas_conv_desc &d, const npas_bp_desc &bp)
     return d.path == 2 ? 0 : 1;
 }
 
+// Path 5 has two forms: the persistent kernel, and for few output tiles the one that splits the input over a cluster
+// (asked for by the upper half of `variant`, or chosen when no kernel was asked for).
+static bool linear_split_k(const npas_linear_desc &d, const npas_bb_desc &bb)
+{
+    if (d.variant >> 16) return linear_sk_supported(d, bb);
+    return (d.path == 0 || d.path == 2) && linear_sk_preferred(d, bb);
+}
+
 // 1 CUDA cores, 3 gathered X (kept columns only), 5 masked dense image by TMA, 6 the same on CTA pairs.
 static int linear_kernel_for(const npas_linear_desc &d, const npas_bb_desc &bb)
 {
     switch (d.path) {
         case 1: return 1;
         case 3: return linear_tc_supported(d, bb) ? 3 : 0;
-        case 5: return linear_dn_supported(d, bb) ? 5 : 0;
+        case 5: return (d.variant >> 16 ? linear_sk_supported(d, bb) : linear_dn_supported(d, bb)) ? 5 : 0;
         case 6: return linear_d2_supported(d, bb) ? 6 : 0;
         case 0: case 2: break;
         default: return 0;
     }
     // automatic: both operands by TMA (on CTA pairs where measured faster: few rows, 256 or more input
     // features), then the gather kernel, then CUDA cores
+    if (linear_sk_preferred(d, bb)) return 5;
     if (d.I >= 256 && d.M <= 16384 && linear_d2_supported(d, bb)) return 6;
     if (linear_dn_supported(d, bb)) return 5;
     if (linear_tc_supported(d, bb)) return 3;
@@ -267,7 +276,9 @@ npas_status npas_linear_bb(const npas_linear_desc *d, const npas_bb_desc *bb, co
     switch (linear_kernel_for(*d, *bb)) {
         case 1: return linear_simt_launch(*d, *bb, x, blob, b, r, y, st);
         case 3: return linear_tc_launch(*d, *bb, x, blob, b, r, y, w, st);
-        case 5: return linear_dn_launch(*d, *bb, x, blob, b, r, y, w, st);
+        case 5:
+            if (linear_split_k(*d, *bb)) return linear_sk_launch(*d, *bb, x, blob, b, r, y, w, st);
+            return linear_dn_launch(*d, *bb, x, blob, b, r, y, w, st);
         case 6: return linear_d2_launch(*d, *bb, x, blob, b, r, y, w, st);
     }
     return NPAS_ERR_UNSUPPORTED;
@@ -352,7 +363,10 @@ npas_status npas_tune_linear_bb(const npas_linear_desc *d, const npas_bb_desc *b
     Timer t;
     if (!t.ok) return NPAS_ERR_CUDA;
     struct Cand { int path, variant; };
-    const Cand cands[] = {{6, 256}, {6, 128}, {5, 256}, {5, 128}, {5, 64}, {5, 32}, {5, 16}, {3, 0}, {1, 0}};
+    // (column tiles of the two persistent kernels; column tile and CTAs per tile of the split-input form)
+    const Cand cands[] = {{6, 256}, {6, 128}, {5, 256}, {5, 128}, {5, 64}, {5, 32}, {5, 16}, {5, 32 | (1 << 16)}, {5, 32 | (2 << 16)},
+                          {5, 32 | (4 << 16)}, {5, 64 | (1 << 16)}, {5, 64 | (2 << 16)}, {5, 64 | (4 << 16)}, {5, 64 | (8 << 16)},
+                          {5, 128 | (4 << 16)}, {3, 0}, {1, 0}};
     float best = -1.f;
     bool tensor_core_found = false;
     for (const Cand &c : cands) {

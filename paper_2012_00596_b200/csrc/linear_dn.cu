@@ -87,7 +87,7 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    float *bias_s = reinterpret_cast<float *>(smem + p.off_bias);      // [O]
+    float *bias_s = reinterpret_cast<float *>(smem + p.off_bias);      // [nNT * BN]
     LinDnBars *bars = reinterpret_cast<LinDnBars *>(smem + p.off_bar);
     volatile uint32_t *abort_flag = &bars->abort_flag;
 
@@ -113,7 +113,7 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     pdl_wait();                        // nothing above touches global memory
     // the biases: staged by the epilogue warps, which meet again before the first use
     if (warp >= kFirstEpiWarp && warp < kResWarp) {
-        for (int i = tid - kFirstEpiWarp * 32; i < p.O; i += kEpiWarps * 32) bias_s[i] = bias ? bias[i] : 0.f;
+        for (int i = tid - kFirstEpiWarp * 32; i < p.nNT * p.BN; i += kEpiWarps * 32) bias_s[i] = (bias && i < p.O) ? bias[i] : 0.f;
         epi_sync();
     }
     const uint32_t tmem_base = bars->tmem_base;
@@ -289,7 +289,8 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 
             // one chunk: + bias (+ residual), ReLU, one rounding, 32 (bf16) or 64 (fp32) bytes per thread
             auto finish = [&](const uint32_t (&r)[16], int c0) {
-                if (!valid) return;
+                const int left = p.O - nt * p.BN - c0;          // (O is a multiple of eight; the last tile may be cut short)
+                if (!valid || left <= 0) return;
                 float v[16];
                 const float4 *b4 = reinterpret_cast<const float4 *>(bs + c0);
 #pragma unroll
@@ -303,6 +304,7 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         const uint4 *rp = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0 + c0);
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
+                            if (8 * h >= left) break;
                             const uint4 u = rp[h];
                             const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
@@ -315,6 +317,7 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         const float4 *rp = reinterpret_cast<const float4 *>(static_cast<const float *>(res) + o0 + c0);
 #pragma unroll
                         for (int h = 0; h < 4; ++h) {
+                            if (4 * h >= left) break;
                             const float4 u = rp[h];
                             v[4 * h] += u.x; v[4 * h + 1] += u.y; v[4 * h + 2] += u.z; v[4 * h + 3] += u.w;
                         }
@@ -327,11 +330,12 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 if (p.y_bf16) {
                     uint4 *yp = reinterpret_cast<uint4 *>(static_cast<uint16_t *>(y) + o0 + c0);
                     yp[0] = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
-                    yp[1] = make_uint4(pack2(v[8], v[9]), pack2(v[10], v[11]), pack2(v[12], v[13]), pack2(v[14], v[15]));
+                    if (left > 8) yp[1] = make_uint4(pack2(v[8], v[9]), pack2(v[10], v[11]), pack2(v[12], v[13]), pack2(v[14], v[15]));
                 } else {
                     float4 *yp = reinterpret_cast<float4 *>(static_cast<float *>(y) + o0 + c0);
 #pragma unroll
-                    for (int h = 0; h < 4; ++h) yp[h] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+                    for (int h = 0; h < 4; ++h)
+                        if (4 * h < left) yp[h] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
                 }
             };
 
@@ -375,12 +379,12 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinDnParams &p)
 {
     if (d.x_dtype != NPAS_BF16 || bb.w_packed != NPAS_BF16) return false;
-    if (d.I % 64 || d.O % 16 || d.O > 16384) return false;
+    if (d.I % 8 || d.O % 8 || d.O > 16384) return false;      // rows of X, W and Y start on 16-byte boundaries
     p.M = d.M; p.I = d.I; p.O = d.O;
-    p.nK = d.I / 64;
+    p.nK = (d.I + 63) / 64;                                    // columns past the end read as zeros
     p.nMT = (d.M + kRows - 1) / kRows;
     p.relu = d.relu; p.y_bf16 = d.y_dtype == NPAS_BF16;
-    const uint32_t fixed = (uint32_t)d.O * 4 + 128 + (uint32_t)sizeof(LinDnBars) + 1024 + 256;
+    const uint32_t fixed = ((uint32_t)d.O + 256u) * 4 + 128 + (uint32_t)sizeof(LinDnBars) + 1024 + 256;
     // Column tile BN: the widest divisor of O that leaves room for enough stages (three once the K loop has
     // three or more steps), else the widest with two (measured: narrower tiles never won, the kernel is
     // bound by what the SMs take in from L2, and wide tiles take in the least per MAC).  Epilogue slots
@@ -392,7 +396,9 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinDnParams &p)
     p.BN = 0;
     for (int pass = 0; pass < 2 && !p.BN; ++pass)
         for (int bn = 256; bn >= 16; bn /= 2) {
-            if (d.O % bn || (want_bn && bn != want_bn)) continue;
+            if (want_bn && bn != want_bn) continue;
+            // (an output width that 16 does not divide: tiles of 128, the last one cut short by the tensor map and the store)
+            if (d.O % 16 ? (!want_bn && bn != 128) : (d.O % bn != 0)) continue;
             const int ns = (p.y_bf16 && bn % 64 == 0 && (d.has_residual || d.O >= d.I)) ? (d.has_residual ? kMaxSlots : 3) : 0;
             const uint32_t stage = round_up(kXBytes + (uint32_t)bn * 128u, 1024);   // multiples of 1024: swizzled tiles stay aligned
             const uint32_t need = fixed + (uint32_t)ns * kSlotBytes;
@@ -403,13 +409,13 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinDnParams &p)
             break;
         }
     if (p.BN == 0) return false;
-    p.nNT = d.O / p.BN;
+    p.nNT = (d.O + p.BN - 1) / p.BN;
     const long long tiles = (long long)p.nMT * p.nNT;
     if (tiles > 0x7FFFFFFF) return false;
     p.n_tiles = (int)tiles;
     p.off_slots = (uint32_t)p.S * p.stage_bytes;
     p.off_bias = p.off_slots + (uint32_t)p.NS * kSlotBytes;
-    p.off_bar = round_up(p.off_bias + (uint32_t)d.O * 4, 128);
+    p.off_bar = round_up(p.off_bias + (uint32_t)(p.nNT * p.BN) * 4, 128);
     p.smem_bytes = p.off_bar + sizeof(LinDnBars) + 1024;
     if (p.smem_bytes > kSmemLimit) return false;
     p.tmem_cols = 32;
