@@ -6,7 +6,7 @@ import torch
 import oracle
 import paper_2012_00596_b200 as npas
 from paper_2012_00596_b200 import inputs
-from util import TOL_BF16, dev, floored_rel_err, host
+from util import TOL_BF16, TOL_F32, dev, floored_rel_err, host
 
 pytestmark = pytest.mark.gpu
 
@@ -52,3 +52,18 @@ def test_split_that_does_not_fit_one_wave_is_declined():
     with pytest.raises(npas.NpasError) as e:
         npas.linear_bb(dev(c.x, "bf16"), blob, path=5, variant=64 | (8 << 16))
     assert e.value.code == 8
+
+
+@pytest.mark.parametrize("M,I,O,Bo,Bi,kr,kc", [(1, 64, 64, 64, 64, 64, 64), (33, 1088, 48, 16, 64, 11, 37), (31, 520, 24, 8, 8, 5, 3),
+                                               (65, 30, 21, 7, 5, 7, 5), (40, 1280, 100, 50, 64, 49, 1)])
+def test_float64_kernel_edges(M, I, O, Bo, Bi, kr, kc):
+    """fp32 layers: row tiles of 32 with remainders, inputs of more than one phase of columns, kept counts that neither the
+    matrix step (8 rows x 4 columns) nor the group of warps divides, rows that are not 16-byte aligned."""
+    c = inputs.linear_case(M=M, I=I, O=O, Bo=Bo, Bi=Bi, keep_rows=lambda a, b: max(0, kr - (a + b) % 2), keep_cols=kc, dtype="f32", w_sigma=0.3,
+                           seed=903)
+    blob = npas.pack_bb(dev(c.w), c.row_keep, c.col_keep, Bo, Bi)
+    res = torch.randn(M, O, generator=torch.Generator().manual_seed(3))
+    y = npas.linear_bb(dev(c.x), blob, dev(c.bias), res.cuda(), relu=True)
+    ref = oracle.linear_bb(c.x, c.w, c.row_keep, c.col_keep, Bo=Bo, Bi=Bi, bias=c.bias, relu=True, residual=res.to(torch.float64).numpy())
+    assert floored_rel_err(host(y), ref) < TOL_F32
+    assert torch.equal(y, npas.linear_bb(dev(c.x), blob, dev(c.bias), res.cuda(), relu=True))
