@@ -18,6 +18,7 @@
 
 #include <atomic>
 #include <mutex>
+#include <vector>
 
 #include "npas.h"
 
@@ -254,10 +255,153 @@ PyObject *linear_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
     });
 }
 
+// ---- a whole stack of layers --------------------------------------------------------------------------------------
+// One call for the forward pass of a chain of layers: what Python did between the layers (shapes, keys, liveness, two
+// allocations) took longer than the layers of a small batch.  The activations lie in one buffer, placed by first fit over
+// the layers' lifetimes; only the result is a tensor of its own.
+
+struct Span { int64_t lo, hi; };
+
+// First-fit placement of buffers with known lifetimes in [0, size): `busy` is kept sorted.
+class Arena {
+public:
+    int64_t take(int64_t bytes)
+    {
+        bytes = (bytes + 255) & ~int64_t(255);
+        int64_t at = 0;
+        size_t i = 0;
+        for (; i < busy_.size() && busy_[i].lo - at < bytes; ++i) at = busy_[i].hi;
+        busy_.insert(busy_.begin() + (long)i, Span{at, at + bytes});
+        if (at + bytes > size_) size_ = at + bytes;
+        return at;
+    }
+    void give(int64_t at)
+    {
+        for (size_t i = 0; i < busy_.size(); ++i)
+            if (busy_[i].lo == at) { busy_.erase(busy_.begin() + (long)i); return; }
+    }
+    int64_t size() const { return size_; }
+
+private:
+    std::vector<Span> busy_;
+    int64_t size_ = 0;
+};
+
+// One row of the topology: kind 0 first layer (followed by the max-pool), 1 convolution, 2 GEMM over the pixels.
+struct LayerRow { int32_t kind, stride, pad, relu, cout, src, res, reserved; };
+
+// stack_forward(x, rows, blobs, biases, ws, routes): rows = bytes of LayerRow; routes = None, or [path, variant] pairs as
+// a flat list.  src / res: index of a layer, -1 the network's input, -2 the pooled tensor, -3 (res only) none.
+PyObject *stack_forward(PyObject *, PyObject *const *a, Py_ssize_t nargs)
+{
+    return guarded([&]() -> PyObject * {
+        const at::Tensor *x, *ws;
+        if (nargs != 6) { PyErr_SetString(PyExc_TypeError, "stack_forward takes 6 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], x, false, "x") || !tensor_arg(a[4], ws, false, "ws")) return nullptr;
+        if (!PyBytes_Check(a[1]) || !PyList_Check(a[2]) || !PyList_Check(a[3])) { PyErr_SetString(PyExc_TypeError, "stack_forward: rows, blobs, biases"); return nullptr; }
+        const int L = (int)(PyBytes_GET_SIZE(a[1]) / (Py_ssize_t)sizeof(LayerRow));
+        const LayerRow *rows = reinterpret_cast<const LayerRow *>(PyBytes_AS_STRING(a[1]));
+        if (L < 1 || PyList_GET_SIZE(a[2]) != L || PyList_GET_SIZE(a[3]) != L) { fail_assert("stack_forward: one blob and one bias per layer"); return nullptr; }
+        if (!(x->is_cuda() && x->is_contiguous() && x->dim() == 4 && x->scalar_type() == at::kBFloat16)) { fail_assert("x must be a contiguous 4-D bf16 CUDA tensor"); return nullptr; }
+        struct Step {
+            npas_conv_desc cd; npas_linear_desc ld; npas_bp_desc bp; npas_bb_desc bb;
+            const void *blob; const float *bias;
+            int64_t h, w, p, q, out, sub;          // input and output height / width, buffer of the output, of the subsampled input (-1: none)
+            int64_t in_at, res_at;                  // -1: the network's input / none
+        };
+        std::vector<Step> steps((size_t)L);
+        struct Shape { int64_t h, w, c, at; };
+        std::vector<Shape> made((size_t)L);
+        std::vector<int> last((size_t)L, -1);
+        int pooled_last = -1;
+        for (int i = 0; i < L; ++i)
+            for (int s : {rows[i].src, rows[i].res}) {
+                if (s >= i || s < -3) { fail_assert("stack_forward: a layer reads a later one"); return nullptr; }
+                if (s >= 0) last[(size_t)s] = i;
+                if (s == -2) pooled_last = i;
+            }
+        Shape pooled{0, 0, 0, -1};
+        Arena arena;
+        const int64_t N = x->size(0);
+        for (int i = 0; i < L; ++i) {
+            const LayerRow &r = rows[i];
+            Step &st = steps[(size_t)i];
+            PyObject *bo = PyList_GET_ITEM(a[2], i);
+            PyObject *data = PyObject_GetAttrString(bo, "data");
+            if (!data) return nullptr;
+            Py_DECREF(data);                        // (the blob object keeps it)
+            PyObject *desc = PyObject_GetAttrString(bo, "desc");
+            if (!desc) return nullptr;
+            Py_DECREF(desc);
+            const at::Tensor *blob, *bias;
+            if (!tensor_arg(data, blob, false, "blob.data") || !tensor_arg(PyList_GET_ITEM(a[3], i), bias, false, "bias")) return nullptr;
+            st.blob = blob->data_ptr(); st.bias = static_cast<const float *>(bias->data_ptr());
+            int32_t path = 0, variant = 0;
+            if (a[5] != Py_None && (!int_arg(PyList_GetItem(a[5], 2 * i), path) || !int_arg(PyList_GetItem(a[5], 2 * i + 1), variant))) return nullptr;
+            const Shape in = r.src == -1 ? Shape{x->size(1), x->size(2), x->size(3), -1} : r.src == -2 ? pooled : made[(size_t)r.src];
+            st.h = in.h; st.w = in.w; st.in_at = in.at; st.sub = -1;
+            st.res_at = r.res == -2 ? pooled.at : r.res >= 0 ? made[(size_t)r.res].at : -1;
+            const bool has_res = r.res == -2 || r.res >= 0;
+            if (r.kind == 2) {
+                if (!desc_arg(desc, st.bb)) return nullptr;
+                st.p = (in.h - 1) / r.stride + 1; st.q = (in.w - 1) / r.stride + 1;
+                if (r.stride != 1) st.sub = arena.take(N * st.p * st.q * in.c * 2);
+                st.ld = npas_linear_desc{(int32_t)(N * st.p * st.q), (int32_t)in.c, r.cout, NPAS_BF16, NPAS_BF16, r.relu, 1, has_res, path, variant};
+            } else {
+                if (!desc_arg(desc, st.bp)) return nullptr;
+                st.p = (in.h + 2 * r.pad - st.bp.R) / r.stride + 1; st.q = (in.w + 2 * r.pad - st.bp.S) / r.stride + 1;
+                st.cd = npas_conv_desc{(int32_t)N, (int32_t)in.h, (int32_t)in.w, (int32_t)in.c, r.cout, st.bp.R, st.bp.S, r.stride, r.pad,
+                                       NPAS_BF16, NPAS_BF16, r.relu, 1, has_res, path, variant};
+                if (r.kind == 0) { st.p = (st.p + 2 - 3) / 2 + 1; st.q = (st.q + 2 - 3) / 2 + 1; }      // the pooled tensor
+            }
+            st.out = i == L - 1 ? -1 : arena.take(N * st.p * st.q * r.cout * 2);
+            made[(size_t)i] = Shape{st.p, st.q, r.cout, st.out};
+            if (r.kind == 0) pooled = made[(size_t)i];
+            if (st.sub >= 0) arena.give(st.sub);
+            // buffers that no later layer reads (the pooled tensor has one of its own name)
+            for (int j = 0; j <= i; ++j)
+                if (made[(size_t)j].at >= 0 && j != L - 1 && rows[j].kind != 0 && last[(size_t)j] <= i && (last[(size_t)j] == i || j == i)) { arena.give(made[(size_t)j].at); }
+            if (pooled.at >= 0 && pooled_last == i) arena.give(pooled.at);
+        }
+        const Step &end = steps[(size_t)L - 1];
+        at::Tensor y = new_tensor({N, end.p, end.q, rows[L - 1].cout}, at::kBFloat16, x->device());
+        at::Tensor buf = new_tensor({arena.size()}, at::kByte, x->device());
+        uint8_t *base = static_cast<uint8_t *>(buf.data_ptr());
+        void *xin = x->data_ptr(), *yout = y.data_ptr(), *w = ws->data_ptr(), *stream = c10::cuda::getCurrentCUDAStream().stream();
+        const size_t wb = (size_t)ws->numel();
+        npas_status s = NPAS_OK;
+        int at_layer = 0;
+        Py_BEGIN_ALLOW_THREADS
+        for (int i = 0; i < L && s == NPAS_OK; ++i) {
+            const LayerRow &r = rows[i];
+            const Step &st = steps[(size_t)i];
+            const void *in = st.in_at < 0 ? xin : base + st.in_at, *res = st.res_at < 0 ? nullptr : base + st.res_at;
+            void *out = st.out < 0 ? yout : base + st.out;
+            at_layer = i;
+            if (r.kind == 2) {
+                if (st.sub >= 0) {
+                    s = npas_subsample2d((int32_t)N, (int32_t)st.h, (int32_t)st.w, st.ld.I, r.stride, 2, in, base + st.sub, stream);
+                    if (s != NPAS_OK) break;
+                    in = base + st.sub;
+                }
+                s = npas_linear_bb(&st.ld, &st.bb, in, st.blob, st.bias, res, out, w, wb, stream);
+            } else if (r.kind == 0) {
+                s = npas_conv2d_bp_maxpool(&st.cd, &st.bp, 3, 2, 1, in, st.blob, st.bias, out, w, wb, stream);
+            } else {
+                s = npas_conv2d_bp(&st.cd, &st.bp, in, st.blob, st.bias, res, out, w, wb, stream);
+            }
+        }
+        Py_END_ALLOW_THREADS
+        if (s != NPAS_OK) return Py_BuildValue("(ii)", (int)s, at_layer);
+        return THPVariable_Wrap(std::move(y));
+    });
+}
+
 PyMethodDef kMethods[] = {
     {"conv2d_bp", (PyCFunction)(void (*)(void))conv2d_bp, METH_FASTCALL, nullptr},
     {"conv2d_bp_maxpool", (PyCFunction)(void (*)(void))conv2d_bp_maxpool, METH_FASTCALL, nullptr},
     {"linear_bb", (PyCFunction)(void (*)(void))linear_bb, METH_FASTCALL, nullptr},
+    {"stack_forward", (PyCFunction)(void (*)(void))stack_forward, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_npas_host", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};

@@ -7,6 +7,8 @@ weights and sequences the library calls; all arithmetic runs in the CUDA kernels
 """
 from __future__ import annotations
 
+import struct
+
 import torch
 
 from . import binding as npas
@@ -30,6 +32,10 @@ class Resnet50Stack:
         self.fuse_pool = True          # stem + max-pool as one fused call (False: the two separate kernels)
         self.plans = npas.PlanCache()  # measured (kernel, tile shape) per layer; empty = the library's own choice
         self._tuning = 0               # > 0: repetitions per candidate while tune() walks the stack
+        # the topology as the native forward reads it: kind, stride, pad, ReLU, filters, input, shortcut (-3: none)
+        kinds = {"stem": (0, 3), "conv3": (1, 1), "pw": (2, 0)}
+        self._rows = b"".join(struct.pack("8i", kinds[l.kind][0], l.stride, kinds[l.kind][1], int(l.relu), l.Cout, l.src,
+                                          l.res if l.res != -1 else -3, 0) for l in layers)
 
     def tune(self, x: torch.Tensor, reps: int = 20) -> "npas.PlanCache":
         """One pass over the stack on input x in which every layer asks the library's tuner (it times each kernel
@@ -70,9 +76,37 @@ class Resnet50Stack:
         return npas.conv2d_bp(x, self.blobs[i], self.biases[i], res, stride=lay.stride, pad=pad, relu=lay.relu,
                               out=out, ws=self.ws, path=pth, variant=var)
 
+    def _routes(self, x: torch.Tensor):
+        """Measured (kernel, tile shape) of every layer as a flat list, or None without measurements."""
+        if not self.plans.plans:
+            return None
+        shapes, routes = {-1: tuple(x.shape)}, []
+        for i, lay in enumerate(self.layers):
+            n, h, w, c = shapes[lay.src]
+            has_res = lay.res != -1
+            if lay.kind == "pw":
+                h, w = (h - 1) // lay.stride + 1, (w - 1) // lay.stride + 1
+                key = npas.PlanCache.linear_key(n * h * w, self.blobs[i], lay.relu, True, has_res)
+            else:
+                pad, R = (3, 7) if lay.kind == "stem" else (1, 3)
+                key = npas.PlanCache.conv_key((n, h, w, c), self.blobs[i], lay.stride, pad, lay.relu, True, has_res)
+                h, w = (h + 2 * pad - R) // lay.stride + 1, (w + 2 * pad - R) // lay.stride + 1
+            shapes[i] = (n, h, w, lay.Cout)
+            if lay.kind == "stem":
+                shapes[-2] = (n, (h - 1) // 2 + 1, (w - 1) // 2 + 1, lay.Cout)
+                routes += [0, 0]                       # (the fused first layer chooses its own kernel)
+            else:
+                routes += self.plans.get(key) or (0, 0)
+        return routes
+
     def forward(self, x: torch.Tensor, keep: bool = False):
         """x [N,H,W,3] bf16 -> [N,H/32,W/32,2048].  With ``keep`` also returns, per layer, the tuple
         (input, shortcut or None, output) the layer actually saw, for layer-by-layer checks."""
+        if not keep and not self._tuning and self.fuse_pool:
+            npas.load()
+            y = npas._host.stack_forward(x, self._rows, self.blobs, self.biases, self.ws, self._routes(x))
+            return y if type(y) is not tuple else npas._refused(y[0], f"layer {self.layers[y[1]].name}")
+        last_use = {s: j for j, l in enumerate(self.layers) for s in (l.src, l.res)}
         outs: dict[int, torch.Tensor] = {}
         seen = []
         for i, lay in enumerate(self.layers):
@@ -96,11 +130,7 @@ class Resnet50Stack:
                 outs[-2] = npas.maxpool2d(y, 3, 2, 1)
             # drop tensors no later layer reads
             if not keep:
-                last_use = {}
-                for j in range(i + 1, len(self.layers)):
-                    for s in (self.layers[j].src, self.layers[j].res):
-                        last_use[s] = j
-                for k in [k for k in outs if k not in last_use and k != i]:
+                for k in [k for k in outs if last_use.get(k, -1) <= i and k != i]:
                     del outs[k]
         npas_out = outs[len(self.layers) - 1]
         return (npas_out, seen, outs.get(-2)) if keep else npas_out
