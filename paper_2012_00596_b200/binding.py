@@ -107,12 +107,16 @@ def _stream():
     return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
-def _dt(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
+def _dt_code(dtype: torch.dtype) -> int:
+    if dtype == torch.float32:
         return F32
-    if t.dtype == torch.bfloat16:
+    if dtype == torch.bfloat16:
         return BF16
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    raise TypeError(f"unsupported dtype {dtype}")
+
+
+def _dt(t: torch.Tensor) -> int:
+    return _dt_code(t.dtype)
 
 
 def _torch_dt(code: int):
@@ -124,6 +128,15 @@ def _mask_to_device(mask, device) -> torch.Tensor:
     if isinstance(mask, torch.Tensor):
         return mask.to(device=device, dtype=torch.int64).contiguous()
     return torch.from_numpy(np.ascontiguousarray(mask, dtype=np.uint64).view(np.int64)).to(device)
+
+
+def _mask_words(mask, device) -> torch.Tensor:
+    """Mask words as the packers take them: an int64 tensor on ``device``, or on the CPU."""
+    if isinstance(mask, torch.Tensor):
+        if mask.dtype == torch.int64 and mask.device == device and mask.is_contiguous():
+            return mask
+        mask = mask_to_numpy(mask)
+    return torch.from_numpy(np.ascontiguousarray(mask, dtype=np.uint64).view(np.int64))
 
 
 def mask_to_numpy(mask: torch.Tensor) -> np.ndarray:
@@ -151,24 +164,15 @@ def workspace(device="cuda") -> torch.Tensor:
 
 def pack_bp(w: torch.Tensor, tap_mask, Mb: int, Nb: int, packed_dtype=None) -> BpBlob:
     """npas_pack_bp: dense KRSC weights + per-block tap bitsets -> blob (on w's device)."""
-    lib = load()
+    if _host is None:
+        load()
     assert w.is_cuda and w.is_contiguous() and w.dim() == 4
     K, R, S, C = w.shape
     w_in = _dt(w)
-    w_packed = w_in if packed_dtype is None else (_dt(torch.empty(0, dtype=packed_dtype)))
-    host = np.ascontiguousarray(mask_to_numpy(tap_mask) if isinstance(tap_mask, torch.Tensor) else tap_mask,
-                                dtype=np.uint64)
-    live = (1 << (R * S)) - 1
-    max_taps = max((bin(int(v) & live).count("1") for v in host.ravel()), default=0)
-    d = BpDesc(K, C, R, S, Mb, Nb, w_in, w_packed, max(1, max_taps))
-    size = ctypes.c_size_t(0)
-    _check(lib.npas_pack_bp_size(ctypes.byref(d), host.ctypes.data_as(ctypes.c_void_p), ctypes.byref(size)),
-           "npas_pack_bp_size")
-    dev_mask = _mask_to_device(host, w.device)
-    blob = torch.empty(size.value, dtype=torch.uint8, device=w.device)
-    _check(lib.npas_pack_bp(ctypes.byref(d), _p(w), _p(dev_mask), _p(blob), ctypes.c_size_t(size.value),
-                            _stream()), "npas_pack_bp")
-    return BpBlob(blob, d)
+    w_packed = w_in if packed_dtype is None else _dt_code(packed_dtype)
+    code, blob, max_taps = _host.pack_bp(w, _mask_words(tap_mask, w.device), Mb, Nb, w_in, w_packed)
+    _check(code, "npas_pack_bp")
+    return BpBlob(blob, BpDesc(K, C, R, S, Mb, Nb, w_in, w_packed, max_taps))
 
 
 def unpack_bp(blob: BpBlob):
@@ -183,36 +187,22 @@ def unpack_bp(blob: BpBlob):
 
 
 def pack_bb(w: torch.Tensor, row_keep, col_keep, Bo: int, Bi: int, packed_dtype=None) -> BbBlob:
-    lib = load()
+    if _host is None:
+        load()
     assert w.is_cuda and w.is_contiguous() and w.dim() == 2
     O, I = w.shape
     w_in = _dt(w)
-    w_packed = w_in if packed_dtype is None else (_dt(torch.empty(0, dtype=packed_dtype)))
-    rk = np.ascontiguousarray(mask_to_numpy(row_keep) if isinstance(row_keep, torch.Tensor) else row_keep, dtype=np.uint64)
-    ck = np.ascontiguousarray(mask_to_numpy(col_keep) if isinstance(col_keep, torch.Tensor) else col_keep, dtype=np.uint64)
-    live = (1 << Bi) - 1
-    max_cols = max((bin(int(v) & live).count("1") for v in ck.ravel()), default=0)
-    d = BbDesc(O, I, Bo, Bi, w_in, w_packed, max(1, max_cols))
-    size = ctypes.c_size_t(0)
-    _check(lib.npas_pack_bb_size(ctypes.byref(d), rk.ctypes.data_as(ctypes.c_void_p),
-                                 ck.ctypes.data_as(ctypes.c_void_p), ctypes.byref(size)), "npas_pack_bb_size")
-    drk, dck = _mask_to_device(rk, w.device), _mask_to_device(ck, w.device)
-    blob = torch.empty(size.value, dtype=torch.uint8, device=w.device)
-    _check(lib.npas_pack_bb(ctypes.byref(d), _p(w), _p(drk), _p(dck), _p(blob), ctypes.c_size_t(size.value),
-                            _stream()), "npas_pack_bb")
-    return BbBlob(blob, d)
+    w_packed = w_in if packed_dtype is None else _dt_code(packed_dtype)
+    code, blob, max_cols = _host.pack_bb(w, _mask_words(row_keep, w.device), _mask_words(col_keep, w.device), Bo, Bi, w_in, w_packed)
+    _check(code, "npas_pack_bb")
+    return BbBlob(blob, BbDesc(O, I, Bo, Bi, w_in, w_packed, max_cols))
 
 
 def unpack_bb(blob: BbBlob):
-    lib = load()
-    d = blob.desc
-    dev = blob.data.device
-    w = torch.empty((d.O, d.I), dtype=_torch_dt(d.w_packed), device=dev)
-    rk = torch.empty((d.O // d.Bo, d.I // d.Bi), dtype=torch.int64, device=dev)
-    ck = torch.empty_like(rk)
-    _check(lib.npas_unpack_bb(ctypes.byref(d), _p(blob.data), ctypes.c_size_t(blob.data.numel()), _p(w), _p(rk),
-                              _p(ck), _stream()), "npas_unpack_bb")
-    return w, rk, ck
+    if _host is None:
+        load()
+    r = _host.unpack_bb(blob.data, blob.desc)
+    return r if type(r) is not int else _refused(r, "npas_unpack_bb")
 
 
 def prune_bp_magnitude(w: torch.Tensor, Mb: int, Nb: int, keep_taps: int) -> torch.Tensor:
@@ -229,33 +219,22 @@ def prune_bp_magnitude(w: torch.Tensor, Mb: int, Nb: int, keep_taps: int) -> tor
 def prune_bp_magnitude_global(w: torch.Tensor, Mb: int, Nb: int, *, rate: float = None, n_keep: int = None) -> torch.Tensor:
     """npas_prune_bp_magnitude_global: keep the ``n_keep`` highest-scoring (block, tap) groups of the whole
     layer (``rate``: n_keep = round(groups / rate), e.g. 2.5 or 7); tap bitsets as an int64 device tensor."""
-    lib = load()
+    if _host is None:
+        load()
     assert w.is_cuda and w.is_contiguous() and w.dim() == 4 and (rate is None) != (n_keep is None)
     K, R, S, C = w.shape
-    d = BpDesc(K, C, R, S, Mb, Nb, _dt(w), _dt(w), 0)
-    groups = (K // Mb) * (C // Nb) * R * S
     if n_keep is None:
-        n_keep = int(np.floor(groups / float(rate) + 0.5))
-    size = ctypes.c_size_t(0)
-    _check(lib.npas_prune_bp_global_workspace(ctypes.byref(d), ctypes.byref(size)), "npas_prune_bp_global_workspace")
-    ws = torch.empty(size.value, dtype=torch.uint8, device=w.device)
-    tm = torch.empty((K // Mb, C // Nb), dtype=torch.int64, device=w.device)
-    _check(lib.npas_prune_bp_magnitude_global(ctypes.byref(d), _p(w), ctypes.c_int64(int(n_keep)), _p(tm), _p(ws),
-                                              ctypes.c_size_t(size.value), _stream()), "npas_prune_bp_magnitude_global")
-    return tm
+        n_keep = int(np.floor((K // Mb) * (C // Nb) * R * S / float(rate) + 0.5))
+    r = _host.prune_bp_global(w, Mb, Nb, _dt(w), int(n_keep))
+    return r if type(r) is not int else _refused(r, "npas_prune_bp_magnitude_global")
 
 
 def prune_bb_magnitude(w: torch.Tensor, Bo: int, Bi: int, keep_rows: int, keep_cols: int):
     """npas_prune_bb_magnitude: dense [O,I] weights -> (row bitsets, column bitsets), int64 tensors on the device."""
-    lib = load()
-    assert w.is_cuda and w.is_contiguous() and w.dim() == 2
-    O, I = w.shape
-    d = BbDesc(O, I, Bo, Bi, _dt(w), _dt(w), 0)
-    rk = torch.empty((O // Bo, I // Bi), dtype=torch.int64, device=w.device)
-    ck = torch.empty_like(rk)
-    _check(lib.npas_prune_bb_magnitude(ctypes.byref(d), _p(w), int(keep_rows), int(keep_cols), _p(rk), _p(ck), _stream()),
-           "npas_prune_bb_magnitude")
-    return rk, ck
+    if _host is None:
+        load()
+    r = _host.prune_bb(w, Bo, Bi, _dt(w), int(keep_rows), int(keep_cols))
+    return r if type(r) is not int else _refused(r, "npas_prune_bb_magnitude")
 
 
 def mask_bp_from_dense(dense_mask: torch.Tensor, Mb: int, Nb: int) -> torch.Tensor:

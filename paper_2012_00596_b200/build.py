@@ -30,7 +30,7 @@ def _build_host() -> None:
     from torch.utils import cpp_extension
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-DNDEBUG",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", os.path.join(ROOT, "include"),
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
            "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include")]
     for d in cpp_extension.include_paths():
         cmd += ["-isystem", d]

@@ -10,6 +10,7 @@
 #include <Python.h>
 
 #include <ATen/cuda/EmptyTensor.h>
+#include <ATen/ops/empty.h>
 #include <ATen/ops/zeros.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
@@ -21,6 +22,7 @@
 #include <vector>
 
 #include "npas.h"
+#include "pack_api.h"
 
 namespace {
 
@@ -255,6 +257,218 @@ PyObject *linear_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
     });
 }
 
+// ---- packing and pruning ------------------------------------------------------------------------------------------
+
+// The sums a blob's size follows from.  Kept bits per mask word below `live`.
+struct MaskSums { uint64_t total; uint32_t most; };
+__attribute__((target_clones("popcnt", "default"))) MaskSums count_bits(const uint64_t *m, size_t n, uint64_t live)
+{
+    MaskSums s{0, 0};
+    for (size_t i = 0; i < n; ++i) {
+        const uint32_t c = (uint32_t)__builtin_popcountll(m[i] & live);
+        s.total += c;
+        s.most = c > s.most ? c : s.most;
+    }
+    return s;
+}
+// stored values of a block-based layer (rows x columns of every block, rounded up to eight) and its fullest column set
+__attribute__((target_clones("popcnt", "default"))) MaskSums count_values(const uint64_t *r, const uint64_t *c, size_t n, uint64_t rlive, uint64_t clive)
+{
+    MaskSums s{0, 0};
+    for (size_t i = 0; i < n; ++i) {
+        const uint32_t nc = (uint32_t)__builtin_popcountll(c[i] & clive);
+        s.total += ((uint64_t)__builtin_popcountll(r[i] & rlive) * nc + 7) / 8 * 8;
+        s.most = nc > s.most ? nc : s.most;
+    }
+    return s;
+}
+uint64_t low_bits(int n) { return n >= 64 ? ~0ull : (1ull << n) - 1; }
+
+// Mask words on both sides: a CUDA tensor is copied to pinned memory (the caller synchronises), a CPU tensor to the GPU.
+struct Mask { at::Tensor dev, host; };
+bool both_sides(const at::Tensor &m, int64_t n, const at::Device &dev, cudaStream_t st, Mask &out)
+{
+    if (m.scalar_type() != at::kLong || !m.is_contiguous() || m.numel() < n) return fail_assert("mask words: contiguous int64, one per block");
+    cudaError_t e;
+    if (m.is_cuda()) {
+        out.dev = m;
+        out.host = at::empty({n}, at::TensorOptions().dtype(at::kLong).pinned_memory(true));
+        e = cudaMemcpyAsync(out.host.data_ptr(), m.data_ptr(), (size_t)n * 8, cudaMemcpyDeviceToHost, st);
+    } else {
+        out.host = m;
+        out.dev = new_tensor({n}, at::kLong, dev);
+        e = cudaMemcpyAsync(out.dev.data_ptr(), m.data_ptr(), (size_t)n * 8, cudaMemcpyHostToDevice, st);
+    }
+    if (e != cudaSuccess) { PyErr_SetString(PyExc_RuntimeError, cudaGetErrorString(e)); return false; }
+    return true;
+}
+bool wait_for(cudaStream_t st)
+{
+    cudaError_t e;
+    Py_BEGIN_ALLOW_THREADS
+    e = cudaStreamSynchronize(st);
+    Py_END_ALLOW_THREADS
+    if (e != cudaSuccess) PyErr_SetString(PyExc_RuntimeError, cudaGetErrorString(e));
+    return e == cudaSuccess;
+}
+PyObject *packed(npas_status s, at::Tensor &&blob, uint32_t most)
+{
+    PyObject *t = s == NPAS_OK ? THPVariable_Wrap(std::move(blob)) : (Py_INCREF(Py_None), Py_None);
+    return t ? Py_BuildValue("(iNI)", (int)s, t, most) : nullptr;
+}
+
+// pack_bp(w, mask, Mb, Nb, w_in, w_packed) -> (status, blob, fullest block's taps)
+PyObject *pack_bp(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        const at::Tensor *w, *m;
+        npas_bp_desc d = {};
+        if (n != 6) { PyErr_SetString(PyExc_TypeError, "pack_bp takes 6 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], w, false, "w") || !tensor_arg(a[1], m, false, "mask") || !int_arg(a[2], d.Mb) || !int_arg(a[3], d.Nb) ||
+            !int_arg(a[4], d.w_in) || !int_arg(a[5], d.w_packed))
+            return nullptr;
+        if (!(w->is_cuda() && w->is_contiguous() && w->dim() == 4)) { fail_assert("w must be a contiguous 4-D CUDA tensor"); return nullptr; }
+        d.K = (int32_t)w->size(0); d.R = (int32_t)w->size(1); d.S = (int32_t)w->size(2); d.C = (int32_t)w->size(3);
+        size_t bytes = 0;
+        npas_status s = npas_internal_bp_size(&d, 0, &bytes);
+        if (s != NPAS_OK) return packed(s, at::Tensor(), 0);
+        const cudaStream_t st = c10::cuda::getCurrentCUDAStream().stream();
+        const int64_t blocks = (int64_t)(d.K / d.Mb) * (d.C / d.Nb);
+        Mask mask;
+        if (!both_sides(*m, blocks, w->device(), st, mask) || (m->is_cuda() && !wait_for(st))) return nullptr;
+        const MaskSums sums = count_bits(static_cast<const uint64_t *>(mask.host.data_ptr()), (size_t)blocks, low_bits(d.R * d.S));
+        d.max_taps = sums.most ? (int32_t)sums.most : 1;
+        s = npas_internal_bp_size(&d, sums.total, &bytes);
+        if (s != NPAS_OK) return packed(s, at::Tensor(), 0);
+        at::Tensor blob = new_tensor({(int64_t)bytes}, at::kByte, w->device());
+        Py_BEGIN_ALLOW_THREADS
+        s = npas_internal_pack_bp(&d, w->data_ptr(), static_cast<const uint64_t *>(mask.dev.data_ptr()), blob.data_ptr(), bytes, st);
+        Py_END_ALLOW_THREADS
+        return packed(s, std::move(blob), (uint32_t)d.max_taps);
+    });
+}
+
+// pack_bb(w, rows, cols, Bo, Bi, w_in, w_packed) -> (status, blob, fullest block's columns)
+PyObject *pack_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        const at::Tensor *w, *mr, *mc;
+        npas_bb_desc d = {};
+        if (n != 7) { PyErr_SetString(PyExc_TypeError, "pack_bb takes 7 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], w, false, "w") || !tensor_arg(a[1], mr, false, "row_keep") || !tensor_arg(a[2], mc, false, "col_keep") ||
+            !int_arg(a[3], d.Bo) || !int_arg(a[4], d.Bi) || !int_arg(a[5], d.w_in) || !int_arg(a[6], d.w_packed))
+            return nullptr;
+        if (!(w->is_cuda() && w->is_contiguous() && w->dim() == 2)) { fail_assert("w must be a contiguous 2-D CUDA tensor"); return nullptr; }
+        d.O = (int32_t)w->size(0); d.I = (int32_t)w->size(1);
+        size_t bytes = 0;
+        npas_status s = npas_internal_bb_size(&d, 0, 0, &bytes);
+        if (s != NPAS_OK) return packed(s, at::Tensor(), 0);
+        const cudaStream_t st = c10::cuda::getCurrentCUDAStream().stream();
+        const int64_t blocks = (int64_t)(d.O / d.Bo) * (d.I / d.Bi);
+        Mask rows, cols;
+        const uint64_t *hr, *hc;
+        if (mr->is_cuda() && mc->is_cuda() && mr->numel() == blocks && mc->numel() == blocks &&
+            static_cast<const int64_t *>(mc->data_ptr()) == static_cast<const int64_t *>(mr->data_ptr()) + blocks && mr->scalar_type() == at::kLong &&
+            mc->scalar_type() == at::kLong && mr->is_contiguous() && mc->is_contiguous()) {
+            rows.dev = *mr; cols.dev = *mc;
+            rows.host = at::empty({2 * blocks}, at::TensorOptions().dtype(at::kLong).pinned_memory(true));
+            if (cudaMemcpyAsync(rows.host.data_ptr(), mr->data_ptr(), (size_t)blocks * 16, cudaMemcpyDeviceToHost, st) != cudaSuccess) {
+                PyErr_SetString(PyExc_RuntimeError, "copy of the masks failed");
+                return nullptr;
+            }
+            hr = static_cast<const uint64_t *>(rows.host.data_ptr()); hc = hr + blocks;
+        } else {
+            if (!both_sides(*mr, blocks, w->device(), st, rows) || !both_sides(*mc, blocks, w->device(), st, cols)) return nullptr;
+            hr = static_cast<const uint64_t *>(rows.host.data_ptr()); hc = static_cast<const uint64_t *>(cols.host.data_ptr());
+        }
+        if ((mr->is_cuda() || mc->is_cuda()) && !wait_for(st)) return nullptr;
+        const MaskSums sums = count_values(hr, hc, (size_t)blocks, low_bits(d.Bo), low_bits(d.Bi));
+        d.max_cols = sums.most ? (int32_t)sums.most : 1;
+        s = npas_internal_bb_size(&d, sums.total, sums.most, &bytes);
+        if (s != NPAS_OK) return packed(s, at::Tensor(), 0);
+        at::Tensor blob = new_tensor({(int64_t)bytes}, at::kByte, w->device());
+        Py_BEGIN_ALLOW_THREADS
+        s = npas_internal_pack_bb(&d, w->data_ptr(), static_cast<const uint64_t *>(rows.dev.data_ptr()),
+                                  static_cast<const uint64_t *>(cols.dev.data_ptr()), blob.data_ptr(), bytes, st);
+        Py_END_ALLOW_THREADS
+        return packed(s, std::move(blob), (uint32_t)d.max_cols);
+    });
+}
+
+// prune_bp_global(w, Mb, Nb, w_in, n_keep) -> masks, or the status
+PyObject *prune_bp_global(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        const at::Tensor *w;
+        npas_bp_desc d = {};
+        if (n != 5) { PyErr_SetString(PyExc_TypeError, "prune_bp_global takes 5 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], w, false, "w") || !int_arg(a[1], d.Mb) || !int_arg(a[2], d.Nb) || !int_arg(a[3], d.w_in)) return nullptr;
+        const long long n_keep = PyLong_AsLongLong(a[4]);
+        if (n_keep == -1 && PyErr_Occurred()) return nullptr;
+        if (!(w->is_cuda() && w->is_contiguous() && w->dim() == 4)) { fail_assert("w must be a contiguous 4-D CUDA tensor"); return nullptr; }
+        d.K = (int32_t)w->size(0); d.R = (int32_t)w->size(1); d.S = (int32_t)w->size(2); d.C = (int32_t)w->size(3);
+        d.w_packed = d.w_in;
+        size_t bytes = 0;
+        npas_status s = npas_prune_bp_global_workspace(&d, &bytes);
+        if (s != NPAS_OK) return PyLong_FromLong((long)s);
+        at::Tensor ws = new_tensor({(int64_t)bytes}, at::kByte, w->device()), tm = new_tensor({d.K / d.Mb, d.C / d.Nb}, at::kLong, w->device());
+        void *st = c10::cuda::getCurrentCUDAStream().stream();
+        Py_BEGIN_ALLOW_THREADS
+        s = npas_prune_bp_magnitude_global(&d, w->data_ptr(), n_keep, static_cast<uint64_t *>(tm.data_ptr()), ws.data_ptr(), bytes, st);
+        Py_END_ALLOW_THREADS
+        return result(s, nullptr, std::move(tm));
+    });
+}
+
+// prune_bb(w, Bo, Bi, w_in, keep_rows, keep_cols) -> (rows, columns), or the status
+PyObject *prune_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        const at::Tensor *w;
+        npas_bb_desc d = {};
+        int32_t kr, kc;
+        if (n != 6) { PyErr_SetString(PyExc_TypeError, "prune_bb takes 6 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], w, false, "w") || !int_arg(a[1], d.Bo) || !int_arg(a[2], d.Bi) || !int_arg(a[3], d.w_in) || !int_arg(a[4], kr) || !int_arg(a[5], kc))
+            return nullptr;
+        if (!(w->is_cuda() && w->is_contiguous() && w->dim() == 2)) { fail_assert("w must be a contiguous 2-D CUDA tensor"); return nullptr; }
+        d.O = (int32_t)w->size(0); d.I = (int32_t)w->size(1);
+        d.w_packed = d.w_in;
+        if (d.Bo == 0 || d.Bi == 0) { PyErr_SetString(PyExc_ZeroDivisionError, "block size is zero"); return nullptr; }
+        // one buffer for both (the packer then fetches them with one copy)
+        const at::Tensor both = new_tensor({2, d.O / d.Bo, d.I / d.Bi}, at::kLong, w->device());
+        at::Tensor rk = both[0], ck = both[1];
+        void *st = c10::cuda::getCurrentCUDAStream().stream();
+        npas_status s;
+        Py_BEGIN_ALLOW_THREADS
+        s = npas_prune_bb_magnitude(&d, w->data_ptr(), kr, kc, static_cast<uint64_t *>(rk.data_ptr()), static_cast<uint64_t *>(ck.data_ptr()), st);
+        Py_END_ALLOW_THREADS
+        if (s != NPAS_OK) return PyLong_FromLong((long)s);
+        return Py_BuildValue("(NN)", THPVariable_Wrap(std::move(rk)), THPVariable_Wrap(std::move(ck)));
+    });
+}
+
+// unpack_bb(blob, desc) -> (weights, rows, columns), or the status
+PyObject *unpack_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        const at::Tensor *blob;
+        npas_bb_desc d;
+        if (n != 2) { PyErr_SetString(PyExc_TypeError, "unpack_bb takes 2 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], blob, false, "blob.data") || !desc_arg(a[1], d)) return nullptr;
+        if (d.Bo == 0 || d.Bi == 0) { PyErr_SetString(PyExc_ZeroDivisionError, "block size is zero"); return nullptr; }
+        const at::Device dev = blob->device();
+        at::Tensor w = new_tensor({d.O, d.I}, d.w_packed == NPAS_F32 ? at::kFloat : at::kBFloat16, dev);
+        at::Tensor rk = new_tensor({d.O / d.Bo, d.I / d.Bi}, at::kLong, dev), ck = new_tensor({d.O / d.Bo, d.I / d.Bi}, at::kLong, dev);
+        void *st = c10::cuda::getCurrentCUDAStream().stream();
+        npas_status s;
+        Py_BEGIN_ALLOW_THREADS
+        s = npas_unpack_bb(&d, blob->data_ptr(), (size_t)blob->numel(), w.data_ptr(), static_cast<uint64_t *>(rk.data_ptr()), static_cast<uint64_t *>(ck.data_ptr()), st);
+        Py_END_ALLOW_THREADS
+        if (s != NPAS_OK) return PyLong_FromLong((long)s);
+        return Py_BuildValue("(NNN)", THPVariable_Wrap(std::move(w)), THPVariable_Wrap(std::move(rk)), THPVariable_Wrap(std::move(ck)));
+    });
+}
+
 // ---- a whole stack of layers --------------------------------------------------------------------------------------
 // One call for the forward pass of a chain of layers: what Python did between the layers (shapes, keys, liveness, two
 // allocations) took longer than the layers of a small batch.  The activations lie in one buffer, placed by first fit over
@@ -401,6 +615,11 @@ PyMethodDef kMethods[] = {
     {"conv2d_bp", (PyCFunction)(void (*)(void))conv2d_bp, METH_FASTCALL, nullptr},
     {"conv2d_bp_maxpool", (PyCFunction)(void (*)(void))conv2d_bp_maxpool, METH_FASTCALL, nullptr},
     {"linear_bb", (PyCFunction)(void (*)(void))linear_bb, METH_FASTCALL, nullptr},
+    {"pack_bp", (PyCFunction)(void (*)(void))pack_bp, METH_FASTCALL, nullptr},
+    {"pack_bb", (PyCFunction)(void (*)(void))pack_bb, METH_FASTCALL, nullptr},
+    {"prune_bp_global", (PyCFunction)(void (*)(void))prune_bp_global, METH_FASTCALL, nullptr},
+    {"prune_bb", (PyCFunction)(void (*)(void))prune_bb, METH_FASTCALL, nullptr},
+    {"unpack_bb", (PyCFunction)(void (*)(void))unpack_bb, METH_FASTCALL, nullptr},
     {"stack_forward", (PyCFunction)(void (*)(void))stack_forward, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 

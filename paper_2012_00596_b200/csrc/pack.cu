@@ -1,47 +1,82 @@
 // Packers and mask helpers: dense weights + block masks <-> the blobs described in npas.h.
-// These run once per layer (offline with respect to inference), so they are plain, coalesced
-// CUDA-core kernels; all index output is integer work and all value output is a bit copy or a
-// single round-to-nearest-even conversion.
+// These run once per layer (offline with respect to inference; in a search, once per candidate layer).  All index output
+// is integer work and all value output is a bit copy or a single round-to-nearest-even conversion.  A blob is written
+// once, section by section, zeros included: one CTA scans the masks (header, offsets, and the few bytes between the
+// sections), then a grid writes the sections 16 bytes per thread.  (Clearing the blob first and placing two-byte values
+// one by one took twice the bytes and partial writes: 512x3x3x512 with 16x8 blocks 14 us of placing after 10 of scanning.)
 #include "common.cuh"
+#include "pack_api.h"
+#include "tc_common.cuh"
 
 namespace npas {
 
 // ------------------------------------------------------------------------------------------------
-// Exclusive prefix sum of `count(i)` for i < n into out[0..n] by ONE block (n is a few thousand
-// at most: one entry per weight block).  Every thread scans a contiguous chunk.
+// Exclusive prefix sum of `count(i)` for i < n into out[0..n] by ONE block of 1024 threads, four consecutive items per
+// thread and step.
 template <typename F>
-__device__ void block_exclusive_scan(uint32_t n, F count, uint32_t *out, uint32_t *smem /*blockDim+1*/)
+__device__ void block_exclusive_scan(uint32_t n, F count, uint32_t *out, uint32_t *smem /* 33 words */)
 {
-    const uint32_t T = blockDim.x, t = threadIdx.x;
-    const uint32_t chunk = (n + T - 1) / T;
-    const uint32_t lo = min(n, t * chunk), hi = min(n, lo + chunk);
-    uint32_t sum = 0;
-    for (uint32_t i = lo; i < hi; ++i) sum += count(i);
-    smem[t] = sum;
-    __syncthreads();
-    if (t == 0) {
-        uint32_t run = 0;
-        for (uint32_t i = 0; i < T; ++i) { uint32_t v = smem[i]; smem[i] = run; run += v; }
-        smem[T] = run;
+    const uint32_t t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    uint32_t carry = 0;
+    for (uint32_t base = 0; base < n; base += 4096) {
+        const uint32_t i0 = base + 4 * t;
+        uint32_t c[4], sum = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { c[j] = i0 + j < n ? count(i0 + j) : 0u; sum += c[j]; }
+        uint32_t up = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) { const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, up, d); if (lane >= (uint32_t)d) up += v; }
+        if (lane == 31) smem[wid] = up;
+        __syncthreads();
+        if (wid == 0) {
+            uint32_t w = smem[lane];
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) { const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, w, d); if (lane >= (uint32_t)d) w += v; }
+            smem[lane] = w;
+        }
+        __syncthreads();
+        uint32_t run = carry + up - sum + (wid ? smem[wid - 1] : 0u);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { if (i0 + j < n) out[i0 + j] = run; run += c[j]; }
+        carry += smem[31];
+        __syncthreads();
     }
+    if (t == 0) out[n] = carry;
     __syncthreads();
-    uint32_t run = smem[t];
-    for (uint32_t i = lo; i < hi; ++i) { out[i] = run; run += count(i); }
-    if (t == 0) out[n] = smem[T];
-    __syncthreads();
+}
+
+// zeros in [lo, hi) of the blob (offsets are even)
+__device__ void zero_gap(uint8_t *blob, uint32_t lo, uint32_t hi)
+{
+    for (uint32_t o = lo + 2 * threadIdx.x; o < hi; o += 2 * blockDim.x) *reinterpret_cast<uint16_t *>(blob + o) = 0;
+}
+
+__device__ __forceinline__ uint64_t live_bits(int n) { return n == 64 ? ~0ull : ((1ull << n) - 1); }
+
+template <typename TIn, typename TOut> __device__ __forceinline__ TOut convert(TIn v)
+{
+    if constexpr (sizeof(TIn) == sizeof(TOut)) return v;
+    else return f32_bits_to_bf16(v);
 }
 
 // ---- block-punched ---------------------------------------------------------------------------
 
-__global__ void bp_scan_kernel(npas_bp_desc d, const uint64_t *__restrict__ tap_mask, uint8_t *blob,
-                               uint32_t blob_bytes)
+__global__ void __launch_bounds__(1024)
+bp_scan_kernel(npas_bp_desc d, const uint64_t *__restrict__ tap_mask, uint8_t *blob, uint32_t blob_bytes)
 {
-    __shared__ uint32_t sm[1025];
+    constexpr uint32_t kCounts = 32768;
+    __shared__ uint32_t sm[33];
+    __shared__ uint8_t cnt_s[kCounts];                   // kept taps per block (for the second scan)
+    tc::pdl_trigger();                                   // the section writers may fetch weights and masks meanwhile
     const uint32_t nFB = d.K / d.Mb, nCB = d.C / d.Nb, nBlk = nFB * nCB;
-    const uint64_t live = d.R * d.S == 64 ? ~0ull : ((1ull << (d.R * d.S)) - 1);
+    const uint64_t live = live_bits(d.R * d.S);
     uint32_t *hdr = reinterpret_cast<uint32_t *>(blob);
     uint32_t *blk_off = reinterpret_cast<uint32_t *>(blob + 128);
-    block_exclusive_scan(nBlk, [&](uint32_t i) { return (uint32_t)__popcll(tap_mask[i] & live); }, blk_off, sm);
+    if (threadIdx.x < 32) hdr[threadIdx.x] = 0;
+    block_exclusive_scan(nBlk, [&](uint32_t i) {
+        const uint32_t c = (uint32_t)__popcll(tap_mask[i] & live);
+        if (i < kCounts) cnt_s[i] = (uint8_t)c;
+        return c; }, blk_off, sm);
     const uint32_t nPairs = blk_off[nBlk];
     const BpLayout L = bp_layout(d, nPairs);
     if (L.total > blob_bytes) {
@@ -60,6 +95,22 @@ __global__ void bp_scan_kernel(npas_bp_desc d, const uint64_t *__restrict__ tap_
         hdr[BP_OFF_BLK] = 128; hdr[BP_OFF_PAIRS] = L.off_pairs; hdr[BP_OFF_VALUES] = L.off_values;
         hdr[BP_TOTAL] = L.total; hdr[BP_G] = L.G;
     }
+    // what lies between the sections, and behind the last one
+    const uint32_t values_end = L.off_values + nPairs * d.Mb * d.Nb * L.es;
+    zero_gap(blob, L.off_blk + 4 * (nBlk + 1), L.off_pairs);
+    zero_gap(blob, L.off_pairs + 4 * nPairs, L.off_values);
+    zero_gap(blob, values_end, L.off_image ? L.off_image : L.total);
+    if (L.off_image) {
+        const uint32_t tapu_end = L.off_tapu + (uint32_t)(d.K / L.GI) * (d.C / 16) * 4u;
+        zero_gap(blob, L.off_image + (uint32_t)d.K * d.R * d.S * d.C * 2u, L.off_tapu);
+        zero_gap(blob, tapu_end, L.off_kt ? L.off_ktoff : L.total);
+    }
+    if (L.off_kt) {
+        zero_gap(blob, L.off_ktoff + 4 * ((uint32_t)(d.C / 16) * L.nGrp + 1), L.off_kt);
+        zero_gap(blob, L.off_kt + L.nKt * d.Mb * 32u, L.total);
+    }
+    zero_gap(blob, L.total, blob_bytes & ~1u);
+    if (threadIdx.x == 0 && (blob_bytes & 1u)) blob[blob_bytes - 1] = 0;
     if (L.off_kt) {
         // tiles per (16-channel chunk, group of GS filter blocks), chunk major
         const uint32_t nCh = d.C / 16, cpb = d.Nb / 16;
@@ -67,12 +118,16 @@ __global__ void bp_scan_kernel(npas_bp_desc d, const uint64_t *__restrict__ tap_
         block_exclusive_scan(nCh * L.nGrp, [&](uint32_t i) {
             const uint32_t ch = i / L.nGrp, g = i % L.nGrp, cb = ch / cpb;
             uint32_t n = 0;
-            for (uint32_t fb = g * L.GS; fb < (g + 1) * L.GS; ++fb) n += (uint32_t)__popcll(tap_mask[fb * nCB + cb] & live);
+            for (uint32_t fb = g * L.GS; fb < (g + 1) * L.GS; ++fb) {
+                const uint32_t b = fb * nCB + cb;
+                n += b < kCounts ? cnt_s[b] : (uint32_t)__popcll(tap_mask[b] & live);
+            }
             return n; }, kt_off, sm);
     }
 }
 
-// One CTA per block (fb, cb): writes the block's pair words and gathers its kept weights.
+// Blobs without derived sections (fp32, or C % 16 != 0): one CTA per block (fb, cb) writes the block's pair words and
+// gathers its kept weights in the order of the destination.
 template <typename TIn, typename TOut>
 __global__ void bp_gather_kernel(npas_bp_desc d, const TIn *__restrict__ w, const uint64_t *__restrict__ tap_mask,
                                  uint8_t *blob)
@@ -80,65 +135,135 @@ __global__ void bp_gather_kernel(npas_bp_desc d, const TIn *__restrict__ w, cons
     const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
     if (hdr[BP_MAGIC] != kMagicBP) return;
     const uint32_t nCB = d.C / d.Nb, b = blockIdx.x, fb = b / nCB, cb = b % nCB;
-    auto nFB_of = [](const npas_bp_desc &q) { return (uint32_t)(q.K / q.Mb); };
     const uint32_t *blk_off = reinterpret_cast<const uint32_t *>(blob + 128);
     uint32_t *pairs = reinterpret_cast<uint32_t *>(blob + hdr[BP_OFF_PAIRS]);
     TOut *vals = reinterpret_cast<TOut *>(blob + hdr[BP_OFF_VALUES]);
     const uint32_t G = hdr[BP_G], Mb = d.Mb, Nb = d.Nb;
-    const uint64_t live = d.R * d.S == 64 ? ~0ull : ((1ull << (d.R * d.S)) - 1);
-    uint64_t bits = tap_mask[b] & live;
-    uint32_t j = blk_off[b];
-    // operand image (bf16 blobs with C % 16 == 0): element (k, tap, c) at
-    // ((((k / GI) * nCh + c / 16) * RS + tap) * 2 + (c % 16) / 8) * GI + k % GI) * 8 + c % 8, zeros elsewhere;
-    // and the union of kept taps per (filter group, 16-channel chunk)
-    const uint32_t off_image = hdr[BP_OFF_IMAGE], GI = hdr[BP_GI], nCh = d.C / 16, RS = d.R * d.S;
-    TOut *image = reinterpret_cast<TOut *>(blob + off_image);
-    if (off_image && threadIdx.x == 0 && bits) {
-        uint32_t *tapu = reinterpret_cast<uint32_t *>(blob + hdr[BP_OFF_TAPU]);
-        const uint32_t lo32 = RS > 32 ? 0xFFFFFFFFu : (uint32_t)bits;
-        for (uint32_t gi = fb * Mb / GI; gi <= ((fb + 1) * Mb - 1) / GI; ++gi)
-            for (uint32_t ch = cb * Nb / 16; ch <= ((cb + 1) * Nb - 1) / 16; ++ch) atomicOr(&tapu[gi * nCh + ch], lo32);
-    }
-    // tile section: where this block's tile of (chunk, tap) goes inside its (chunk, group) run
-    const uint32_t off_kt = hdr[BP_OFF_KT], GS = hdr[BP_GS];
-    const uint32_t nGrp = GS ? nFB_of(d) / GS : 0u, grp = GS ? fb / GS : 0u, cpb = Nb / 16;
-    const uint32_t *kt_off = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_KTOFF]);
-    TOut *kt = reinterpret_cast<TOut *>(blob + off_kt);
-    while (bits) {
+    uint64_t bits = tap_mask[b] & live_bits(d.R * d.S);
+    for (uint32_t j = blk_off[b]; bits; ++j, bits &= bits - 1) {
         const uint32_t tap = __ffsll((long long)bits) - 1;
-        bits &= bits - 1;
         if (threadIdx.x == 0) pairs[j] = cb | (tap << 16);
-        uint32_t kt_idx = 0;
-        if (off_kt) {
-            // tiles of lower taps of the whole group, then the lower blocks of the group that keep this tap
-            for (uint32_t f2 = grp * GS; f2 < (grp + 1) * GS; ++f2) {
-                const uint64_t m2 = tap_mask[f2 * nCB + cb] & live;
-                kt_idx += (uint32_t)__popcll(m2 & ((1ull << tap) - 1ull)) + (f2 < fb ? (uint32_t)((m2 >> tap) & 1ull) : 0u);
-            }
-        }
         for (uint32_t e = threadIdx.x; e < Mb * Nb; e += blockDim.x) {
-            // e enumerates the destination order [c/G][f][c%G] so that stores are contiguous
             const uint32_t cg = e / (Mb * G), f = (e / G) % Mb, cl = e % G, c = cg * G + cl;
-            const TIn v = w[((size_t)(fb * Mb + f) * (d.R * d.S) + tap) * d.C + cb * Nb + c];
-            TOut o;
-            if constexpr (sizeof(TIn) == sizeof(TOut)) o = v;
-            else o = f32_bits_to_bf16(v);
-            vals[(size_t)j * Mb * Nb + e] = o;
-            if (off_image) {
-                const uint32_t k = fb * Mb + f, cc = cb * Nb + c;
-                image[((((size_t)(k / GI) * nCh + cc / 16) * RS + tap) * 2 + (cc % 16) / 8) * GI * 8 + (k % GI) * 8 + cc % 8] = o;
-            }
-            if (off_kt) {
-                // tile = [Mb/8 filter octets][2 channel octets][8 filters][8 channels]
-                const uint32_t ch = cb * cpb + c / 16, c16 = c % 16;
-                const size_t tile = (size_t)kt_off[ch * nGrp + grp] + kt_idx;
-                kt[tile * Mb * 16 + (((f / 8) * 2 + c16 / 8) * 8 + f % 8) * 8 + c16 % 8] = o;
-            }
+            vals[(size_t)j * Mb * Nb + e] = convert<TIn, TOut>(w[((size_t)(fb * Mb + f) * (d.R * d.S) + tap) * d.C + cb * Nb + c]);
         }
-        ++j;
     }
 }
 
+// SUB consecutive weights as bf16 bits, packed two to a word (SUB = 1: in the low half)
+template <int SUB> struct Packed { uint32_t w[SUB >= 2 ? SUB / 2 : 1]; };
+template <int SUB> __device__ __forceinline__ Packed<SUB> load_packed(const uint16_t *p)
+{
+    Packed<SUB> r;
+    if constexpr (SUB == 8) { const uint4 u = __ldg(reinterpret_cast<const uint4 *>(p)); r.w[0] = u.x; r.w[1] = u.y; r.w[2] = u.z; r.w[3] = u.w; }
+    else if constexpr (SUB == 4) { const uint2 u = __ldg(reinterpret_cast<const uint2 *>(p)); r.w[0] = u.x; r.w[1] = u.y; }
+    else r.w[0] = __ldg(p);
+    return r;
+}
+template <int SUB> __device__ __forceinline__ Packed<SUB> load_packed(const uint32_t *p)
+{
+    Packed<SUB> r;
+    if constexpr (SUB == 1) r.w[0] = f32_bits_to_bf16(__ldg(p));
+    else {
+#pragma unroll
+        for (int h = 0; h < SUB / 4; ++h) {
+            const uint4 u = __ldg(reinterpret_cast<const uint4 *>(p) + h);
+            r.w[2 * h] = (uint32_t)f32_bits_to_bf16(u.x) | ((uint32_t)f32_bits_to_bf16(u.y) << 16);
+            r.w[2 * h + 1] = (uint32_t)f32_bits_to_bf16(u.z) | ((uint32_t)f32_bits_to_bf16(u.w) << 16);
+        }
+    }
+    return r;
+}
+template <int SUB> __device__ __forceinline__ void store_packed(uint16_t *p, const Packed<SUB> &r)
+{
+    if constexpr (SUB == 8) *reinterpret_cast<uint4 *>(p) = make_uint4(r.w[0], r.w[1], r.w[2], r.w[3]);
+    else if constexpr (SUB == 4) *reinterpret_cast<uint2 *>(p) = make_uint2(r.w[0], r.w[1]);
+    else *p = (uint16_t)r.w[0];
+}
+
+// Blobs with the derived sections.  A thread owns one 16-byte unit of the operand image (filter, tap, eight channels), in
+// the image's order, so that image stores are whole lines; what it keeps also goes, SUB channels at a time, to the packed
+// values and to the tile section.  SUB = 8 when a block's channels are whole octets (then a unit lies in one block), else
+// 4 or 1.  The CTAs behind the last unit write the tap unions, a warp per (filter group, 16-channel chunk).
+template <typename TIn, int SUB>
+__global__ void __launch_bounds__(256)
+bp_expand_kernel(npas_bp_desc d, BpLayout L, const TIn *__restrict__ w, const uint64_t *__restrict__ tap_mask, uint8_t *blob, uint32_t unit_ctas)
+{
+    const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
+    const uint32_t RS = d.R * d.S, nCh = d.C / 16, Mb = d.Mb, Nb = d.Nb, nCB = L.nCB, GI = L.GI, lane = threadIdx.x & 31;
+    const uint64_t live = live_bits((int)RS);
+    if (blockIdx.x >= unit_ctas) {
+        const uint32_t item = (blockIdx.x - unit_ctas) * 8 + (threadIdx.x >> 5);
+        if (item >= (d.K / GI) * nCh) return;
+        const uint32_t gi = item / nCh, ch = item - gi * nCh;
+        const uint32_t fb_lo = gi * GI / Mb, n_fb = ((gi + 1) * GI - 1) / Mb - fb_lo + 1, cb_lo = ch * 16 / Nb, n_cb = (ch * 16 + 15) / Nb - cb_lo + 1;
+        uint32_t u = 0;
+        for (uint32_t i = lane; i < n_fb * n_cb; i += 32) {
+            const uint64_t m = tap_mask[(size_t)(fb_lo + i / n_cb) * nCB + cb_lo + i % n_cb] & live;
+            if (m) u |= RS > 32 ? 0xFFFFFFFFu : (uint32_t)m;
+        }
+        u = __reduce_or_sync(0xFFFFFFFFu, u);
+        tc::pdl_wait();
+        if (lane == 0 && hdr[BP_MAGIC] == kMagicBP) reinterpret_cast<uint32_t *>(blob + hdr[BP_OFF_TAPU])[item] = u;
+        return;
+    }
+    const uint32_t u = blockIdx.x * 256u + threadIdx.x, units = (uint32_t)d.K * RS * (d.C / 8);
+    const uint32_t gsh = 31 - __clz(GI), kl = u & (GI - 1), v = u >> gsh, oct = v & 1, x = v >> 1;
+    const uint32_t y = x / RS, tap = x - y * RS, gi = y / nCh, ch = y - gi * nCh;
+    const uint32_t k = gi * GI + kl, c0 = ch * 16 + oct * 8, fb = k / Mb, f = k - fb * Mb;
+    const bool in = u < units;
+    // masks and weights first: they do not depend on the scan, which may still be running
+    uint64_t bits[8 / SUB];
+    Packed<SUB> r[8 / SUB];
+    bool kept8 = false;
+#pragma unroll
+    for (int h = 0; h < 8 / SUB; ++h) bits[h] = in ? tap_mask[(size_t)fb * nCB + (c0 + h * SUB) / Nb] & live : 0ull;
+#pragma unroll
+    for (int h = 0; h < 8 / SUB; ++h)
+        if ((bits[h] >> tap) & 1ull) {
+            kept8 = true;
+            r[h] = load_packed<SUB>(w + ((size_t)k * RS + tap) * d.C + c0 + h * SUB);
+        }
+    tc::pdl_wait();
+    if (hdr[BP_MAGIC] != kMagicBP) return;
+    const uint32_t *blk_off = reinterpret_cast<const uint32_t *>(blob + 128);
+    uint32_t *pairs = reinterpret_cast<uint32_t *>(blob + hdr[BP_OFF_PAIRS]);
+    uint16_t *vals = reinterpret_cast<uint16_t *>(blob + hdr[BP_OFF_VALUES]);
+    const uint32_t G = L.G;
+    Packed<8> img;
+    img.w[0] = img.w[1] = img.w[2] = img.w[3] = 0;
+#pragma unroll
+    for (int h = 0; h < 8 / SUB; ++h) {
+        if (!((bits[h] >> tap) & 1ull)) continue;
+        const uint32_t c = c0 + h * SUB, cb = c / Nb, cc = c - cb * Nb;
+        if constexpr (SUB == 1) img.w[h >> 1] |= r[h].w[0] << (16 * (h & 1));
+        else {
+#pragma unroll
+            for (int j = 0; j < SUB / 2; ++j) img.w[h * (SUB / 2) + j] = r[h].w[j];
+        }
+        const uint32_t j = blk_off[(size_t)fb * nCB + cb] + (uint32_t)__popcll(bits[h] & ((1ull << tap) - 1ull));
+        if (f == 0 && cc == 0) pairs[j] = cb | (tap << 16);
+        store_packed<SUB>(vals + ((size_t)(j * (Nb / G) + cc / G) * Mb + f) * G + cc % G, r[h]);
+    }
+    if (in) store_packed<8>(reinterpret_cast<uint16_t *>(blob + hdr[BP_OFF_IMAGE]) + (size_t)u * 8, img);
+    if constexpr (SUB == 8) {
+        // the tile of (chunk, tap, filter block): behind the tiles of lower taps of the whole group and those of the
+        // group's lower blocks that keep this tap.  (A warp holds filters of one group and one tap: with tiles, GI is at
+        // least 16, and two octets of 16 filters are a warp.)
+        const uint32_t off_kt = hdr[BP_OFF_KT];
+        if (off_kt && __any_sync(0xFFFFFFFFu, in)) {
+            const uint32_t GS = L.GS, grp = fb / GS, cb = c0 / Nb;
+            const uint64_t m2 = in && lane < GS ? tap_mask[(size_t)(grp * GS + lane) * nCB + cb] & live : 0ull;
+            const uint32_t below = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)__popcll(m2 & ((1ull << tap) - 1ull)));
+            const uint32_t keep = __ballot_sync(0xFFFFFFFFu, (m2 >> tap) & 1ull);
+            if (kept8) {
+                const uint32_t *kt_off = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_KTOFF]);
+                const size_t tile = (size_t)kt_off[ch * L.nGrp + grp] + below + __popc(keep & ((1u << (fb - grp * GS)) - 1u));
+                store_packed<8>(reinterpret_cast<uint16_t *>(blob + off_kt) + tile * Mb * 16 + (((f / 8) * 2 + oct) * 8 + f % 8) * 8, img);
+            }
+        }
+    }
+}
 template <typename T>
 __global__ void bp_scatter_kernel(npas_bp_desc d, const uint8_t *__restrict__ blob, T *w_out, uint64_t *tap_mask_out)
 {
@@ -185,29 +310,34 @@ __global__ void bp_mask_from_dense_kernel(npas_bp_desc d, const uint8_t *__restr
 
 // ---- block-based -----------------------------------------------------------------------------
 
-__global__ void bb_scan_kernel(npas_bb_desc d, const uint64_t *__restrict__ row_keep,
-                               const uint64_t *__restrict__ col_keep, uint8_t *blob, uint32_t blob_bytes,
-                               BbLayout L)
+__global__ void __launch_bounds__(1024)
+bb_scan_kernel(npas_bb_desc d, const uint64_t *__restrict__ row_keep,
+               const uint64_t *__restrict__ col_keep, uint8_t *blob, uint32_t blob_bytes, BbLayout L)
 {
-    __shared__ uint32_t sm[1025];
-    const uint64_t rlive = d.Bo == 64 ? ~0ull : ((1ull << d.Bo) - 1), clive = d.Bi == 64 ? ~0ull : ((1ull << d.Bi) - 1);
+    __shared__ uint32_t sm[33];
+    tc::pdl_trigger();                                     // the section writers may fetch weights and masks meanwhile
+    const uint64_t rlive = live_bits(d.Bo), clive = live_bits(d.Bi);
     uint32_t *hdr = reinterpret_cast<uint32_t *>(blob);
     uint32_t *voff = reinterpret_cast<uint32_t *>(blob + L.off_voff);
+    if (threadIdx.x < 32) hdr[threadIdx.x] = 0;
+    uint32_t mx = 0;                                       // largest kept-column count
     block_exclusive_scan(L.nBlk, [&](uint32_t i) {
-        return round_up((uint32_t)(__popcll(row_keep[i] & rlive) * __popcll(col_keep[i] & clive)), 8u); }, voff, sm);
-    // Kp = largest kept-column count, rounded up to 16 (at least 16)
-    uint32_t mx = 0;
-    for (uint32_t i = threadIdx.x; i < L.nBlk; i += blockDim.x) mx = max(mx, (uint32_t)__popcll(col_keep[i] & clive));
+        const uint32_t nc = (uint32_t)__popcll(col_keep[i] & clive);
+        mx = max(mx, nc);
+        return round_up((uint32_t)__popcll(row_keep[i] & rlive) * nc, 8u); }, voff, sm);
+    // Kp = that, rounded up to 16 (at least 16)
     mx = __reduce_max_sync(0xFFFFFFFFu, mx);
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = mx;
     __syncthreads();
+    for (uint32_t i = 0; i < 32; ++i) mx = max(mx, sm[i]);
+    const uint32_t Kp = max(16u, round_up(mx, 16u)), nVals = voff[L.nBlk];
+    const uint32_t off_tiles = L.off_values + round_up(nVals * L.es, 128), tiles_end = off_tiles + L.nBlk * Kp * d.Bo * L.es;
+    const uint32_t total = round_up(tiles_end, 128);
+    if (total > blob_bytes) {                              // magic and offsets stay 0: nothing is written
+        if (threadIdx.x == 0) hdr[BB_TOTAL] = total;
+        return;
+    }
     if (threadIdx.x == 0) {
-        for (uint32_t i = 0; i < blockDim.x / 32; ++i) mx = max(mx, sm[i]);
-        const uint32_t Kp = max(16u, round_up(mx, 16u));
-        const uint32_t nVals = voff[L.nBlk];
-        const uint32_t off_tiles = L.off_values + round_up(nVals * L.es, 128);
-        const uint32_t total = off_tiles + round_up(L.nBlk * Kp * d.Bo * L.es, 128);
-        if (total > blob_bytes) { hdr[BB_TOTAL] = total; return; }     // magic and offsets stay 0: nothing is written
         hdr[BB_MAGIC] = kMagicBB;
         hdr[BB_KP] = Kp; hdr[BB_OFF_TILES] = off_tiles; hdr[BB_OFF_DENSE] = L.off_dense;
         hdr[BB_VERSION] = kVersionBB; hdr[BB_DTYPE] = d.w_packed;
@@ -216,66 +346,135 @@ __global__ void bb_scan_kernel(npas_bb_desc d, const uint64_t *__restrict__ row_
         hdr[BB_OFF_CNT] = L.off_cnt; hdr[BB_OFF_ROWS] = L.off_rows; hdr[BB_OFF_COLS] = L.off_cols;
         hdr[BB_OFF_VOFF] = L.off_voff; hdr[BB_OFF_VALUES] = L.off_values; hdr[BB_TOTAL] = total;
     }
+    // what lies between the sections (the lists are bytes, so single bytes here), and behind the last one
+    const uint32_t gaps[7][2] = {{L.off_cnt + 2 * L.nBlk, L.off_rows}, {L.off_rows + d.Bo * L.nBlk, L.off_cols},
+                                 {L.off_cols + d.Bi * L.nBlk, L.off_voff}, {L.off_voff + 4 * (L.nBlk + 1), L.off_dense},
+                                 {L.off_dense + (uint32_t)d.O * d.I * L.es, L.off_values}, {L.off_values + nVals * L.es, off_tiles},
+                                 {tiles_end, blob_bytes}};
+    for (int g = 0; g < 7; ++g)
+        for (uint32_t o = gaps[g][0] + threadIdx.x; o < gaps[g][1]; o += blockDim.x) blob[o] = 0;
 }
 
-// One CTA per block: index lists (ascending) and the kept-rows x kept-cols values.
+// One CTA per block: the block's weights are staged once, then its part of every section is written whole, zeros
+// included, in the section's own order (consecutive threads, consecutive elements).
 template <typename TIn, typename TOut>
-__global__ void bb_gather_kernel(npas_bb_desc d, const TIn *__restrict__ w, const uint64_t *__restrict__ row_keep,
-                                 const uint64_t *__restrict__ col_keep, uint8_t *blob, BbLayout L)
+__global__ void __launch_bounds__(256)
+bb_gather_kernel(npas_bb_desc d, const TIn *__restrict__ w, const uint64_t *__restrict__ row_keep,
+                 const uint64_t *__restrict__ col_keep, uint8_t *blob, BbLayout L)
 {
+    constexpr uint32_t kP = 64 + 4 / sizeof(TOut);        // rows of the staged block on different banks
+    __shared__ TOut blk_s[64 * kP];
     __shared__ uint8_t rows[64], cols[64];
     const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
-    if (hdr[BB_MAGIC] != kMagicBB) return;
-    const uint32_t b = blockIdx.x, bo = b / L.nBi, bi = b % L.nBi, t = threadIdx.x;
-    const uint64_t rlive = d.Bo == 64 ? ~0ull : ((1ull << d.Bo) - 1), clive = d.Bi == 64 ? ~0ull : ((1ull << d.Bi) - 1);
-    const uint64_t rk = row_keep[b] & rlive, ck = col_keep[b] & clive;
+    const uint32_t b = blockIdx.x, bo = b / L.nBi, bi = b % L.nBi, t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const uint32_t Bo = d.Bo, Bi = d.Bi;
+    const uint64_t rk = row_keep[b] & live_bits(d.Bo), ck = col_keep[b] & live_bits(d.Bi);
     const uint32_t nr = __popcll(rk), nc = __popcll(ck);
     if (t < 64) {
         // rank of bit t among the set bits = its slot in the ascending list
         const uint64_t below = t == 0 ? 0ull : (~0ull >> (64 - t));
-        if (t < (uint32_t)d.Bo && (rk >> t) & 1) rows[__popcll(rk & below)] = (uint8_t)t;
-        if (t < (uint32_t)d.Bi && (ck >> t) & 1) cols[__popcll(ck & below)] = (uint8_t)t;
+        if (t < Bo && (rk >> t) & 1) rows[__popcll(rk & below)] = (uint8_t)t;
+        if (t < Bi && (ck >> t) & 1) cols[__popcll(ck & below)] = (uint8_t)t;
     }
+    const TIn *src = w + (size_t)bo * Bo * d.I + (size_t)bi * Bi;
+    TOut *dense = reinterpret_cast<TOut *>(blob + L.off_dense) + (size_t)bo * Bo * d.I + (size_t)bi * Bi;
+    TIn v[8][2];                                           // (all loads in flight together)
+#pragma unroll
+    for (uint32_t i = 0; i < 8; ++i)
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h) {
+            const uint32_t r = wid + 8 * i, c = lane + 32 * h;
+            v[i][h] = r < Bo && c < Bi ? __ldg(src + (size_t)r * d.I + c) : (TIn)0;
+        }
+#pragma unroll
+    for (uint32_t i = 0; i < 8; ++i)
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h) {
+            const uint32_t r = wid + 8 * i, c = lane + 32 * h;
+            blk_s[r * kP + c] = ((rk >> r) & (ck >> c) & 1ull) ? convert<TIn, TOut>(v[i][h]) : (TOut)0;
+        }
+    tc::pdl_wait();
     __syncthreads();
-    if (t < (uint32_t)d.Bo) blob[L.off_rows + b * d.Bo + t] = t < nr ? rows[t] : 0xFF;
-    if (t < (uint32_t)d.Bi) blob[L.off_cols + b * d.Bi + t] = t < nc ? cols[t] : 0xFF;
+    if (hdr[BB_MAGIC] != kMagicBB) return;
+    const uint32_t Kp = hdr[BB_KP];
+#pragma unroll 8
+    for (uint32_t r = wid; r < Bo; r += 8)
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h) {
+            const uint32_t c = lane + 32 * h;
+            if (c < Bi) dense[(size_t)r * d.I + c] = blk_s[r * kP + c];
+        }
+    if (t < Bo) blob[L.off_rows + b * Bo + t] = t < nr ? rows[t] : 0xFF;
+    if (t < Bi) blob[L.off_cols + b * Bi + t] = t < nc ? cols[t] : 0xFF;
     if (t == 0) { blob[L.off_cnt + 2 * b] = (uint8_t)nr; blob[L.off_cnt + 2 * b + 1] = (uint8_t)nc; }
+    // values [kept row][kept column], then zeros up to a multiple of eight elements
     const uint32_t v0 = reinterpret_cast<const uint32_t *>(blob + L.off_voff)[b];
     TOut *vals = reinterpret_cast<TOut *>(blob + L.off_values) + v0;
-    for (uint32_t e = t; e < nr * nc; e += blockDim.x) {
-        const TIn v = w[(size_t)(bo * d.Bo + rows[e / nc]) * d.I + bi * d.Bi + cols[e % nc]];
-        TOut o;
-        if constexpr (sizeof(TIn) == sizeof(TOut)) o = v;
-        else o = f32_bits_to_bf16(v);
-        vals[e] = o;
-        // the same weight in the block's [Kp/8][Bo][8] operand image (the blob was zeroed beforehand)
-        const uint32_t Kp = hdr[BB_KP], r = rows[e / nc], c = e % nc;
-        TOut *tile = reinterpret_cast<TOut *>(blob + hdr[BB_OFF_TILES]) + (size_t)b * Kp * d.Bo;
-        tile[((size_t)(c >> 3) * d.Bo + r) * 8 + (c & 7)] = o;
-        // and in the masked dense [O][I] image
-        reinterpret_cast<TOut *>(blob + L.off_dense)[(size_t)(bo * d.Bo + r) * d.I + bi * d.Bi + cols[c]] = o;
+#pragma unroll 4
+    for (uint32_t r = wid; r < nr; r += 8)
+        for (uint32_t c = lane; c < nc; c += 32) vals[r * nc + c] = blk_s[rows[r] * kP + cols[c]];
+    const uint32_t nv = nr * nc;
+    if (t < 8 && nv + t < round_up(nv, 8)) vals[nv + t] = 0;
+    // the operand image [Kp/8][Bo][8]: kept columns compacted, kept rows in place, zeros elsewhere
+    TOut *tile = reinterpret_cast<TOut *>(blob + hdr[BB_OFF_TILES]) + (size_t)b * Kp * Bo;
+    // (a thread per (octet of columns, row): eight elements)
+    for (uint32_t e = t; e < Kp / 8 * Bo; e += 256) {
+        const uint32_t q = e / Bo, r = e - q * Bo;
+        TOut o[8];
+        const bool row_on = (rk >> r) & 1ull;
+#pragma unroll
+        for (uint32_t j = 0; j < 8; ++j) o[j] = (row_on && q * 8 + j < nc) ? blk_s[r * kP + cols[q * 8 + j]] : (TOut)0;
+        TOut *dst = tile + (size_t)e * 8;
+        if constexpr (sizeof(TOut) == 2)
+            *reinterpret_cast<uint4 *>(dst) = make_uint4(o[0] | ((uint32_t)o[1] << 16), o[2] | ((uint32_t)o[3] << 16),
+                                                         o[4] | ((uint32_t)o[5] << 16), o[6] | ((uint32_t)o[7] << 16));
+        else {
+            reinterpret_cast<uint4 *>(dst)[0] = make_uint4(o[0], o[1], o[2], o[3]);
+            reinterpret_cast<uint4 *>(dst)[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        }
     }
 }
 
+// One CTA per block: the dense block is put together in shared memory and written whole, zeros included.
 template <typename T>
-__global__ void bb_scatter_kernel(npas_bb_desc d, const uint8_t *__restrict__ blob, T *w_out, uint64_t *rk_out,
-                                  uint64_t *ck_out, BbLayout L)
+__global__ void __launch_bounds__(256)
+bb_scatter_kernel(npas_bb_desc d, const uint8_t *__restrict__ blob, T *w_out, uint64_t *rk_out,
+                  uint64_t *ck_out, BbLayout L)
 {
-    const uint32_t b = blockIdx.x, bo = b / L.nBi, bi = b % L.nBi, t = threadIdx.x;
-    const uint32_t nr = blob[L.off_cnt + 2 * b], nc = blob[L.off_cnt + 2 * b + 1];
-    const uint8_t *rows = blob + L.off_rows + b * d.Bo, *cols = blob + L.off_cols + b * d.Bi;
-    if (t == 0) {
-        uint64_t rk = 0, ck = 0;
-        for (uint32_t i = 0; i < nr; ++i) rk |= 1ull << rows[i];
-        for (uint32_t i = 0; i < nc; ++i) ck |= 1ull << cols[i];
-        if (rk_out) rk_out[b] = rk;
-        if (ck_out) ck_out[b] = ck;
-    }
-    if (!w_out) return;
+    constexpr uint32_t kP = 64 + 4 / sizeof(T);
+    __shared__ T blk_s[64 * kP];
+    __shared__ uint8_t rows[64], cols[64];
+    const uint32_t b = blockIdx.x, bo = b / L.nBi, bi = b % L.nBi, t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const uint32_t Bo = d.Bo, Bi = d.Bi, nr = min((uint32_t)blob[L.off_cnt + 2 * b], Bo), nc = min((uint32_t)blob[L.off_cnt + 2 * b + 1], Bi);
+    if (t < Bo) rows[t] = t < nr ? blob[L.off_rows + b * Bo + t] & 63 : 0;
+    if (t < Bi) cols[t] = t < nc ? blob[L.off_cols + b * Bi + t] & 63 : 0;
     const uint32_t v0 = reinterpret_cast<const uint32_t *>(blob + L.off_voff)[b];
     const T *vals = reinterpret_cast<const T *>(blob + L.off_values) + v0;
-    for (uint32_t e = t; e < nr * nc; e += blockDim.x)
-        w_out[(size_t)(bo * d.Bo + rows[e / nc]) * d.I + bi * d.Bi + cols[e % nc]] = vals[e];
+    if (w_out)
+        for (uint32_t e = t; e < Bo * kP; e += 256) blk_s[e] = 0;
+    __syncthreads();
+    if (wid == 0) {
+        // the lists as bit sets
+        uint64_t rk = 0, ck = 0;
+        for (uint32_t i = lane; i < nr; i += 32) rk |= 1ull << rows[i];
+        for (uint32_t i = lane; i < nc; i += 32) ck |= 1ull << cols[i];
+        const uint32_t r0 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)rk), r1 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)(rk >> 32));
+        const uint32_t c0 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)ck), c1 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)(ck >> 32));
+        if (lane == 0 && rk_out) rk_out[b] = (uint64_t)r0 | ((uint64_t)r1 << 32);
+        if (lane == 0 && ck_out) ck_out[b] = (uint64_t)c0 | ((uint64_t)c1 << 32);
+    }
+    if (!w_out) return;
+#pragma unroll 8
+    for (uint32_t r = wid; r < nr; r += 8) {
+        const bool c1 = lane < nc, c2 = lane + 32 < nc;
+        const T v1 = c1 ? vals[r * nc + lane] : (T)0, v2 = c2 ? vals[r * nc + lane + 32] : (T)0;
+        if (c1) blk_s[rows[r] * kP + cols[lane]] = v1;
+        if (c2) blk_s[rows[r] * kP + cols[lane + 32]] = v2;
+    }
+    __syncthreads();
+    T *out = w_out + (size_t)bo * Bo * d.I + (size_t)bi * Bi;
+    for (uint32_t r = wid; r < Bo; r += 8)
+        for (uint32_t c = lane; c < Bi; c += 32) out[(size_t)r * d.I + c] = blk_s[r * kP + c];
 }
 
 __global__ void bb_mask_from_dense_kernel(npas_bb_desc d, const uint8_t *__restrict__ m, uint64_t *row_keep,
@@ -316,6 +515,15 @@ using namespace npas;
 // ================================================================================================
 extern "C" {
 
+npas_status npas_internal_bp_size(const npas_bp_desc *d, uint64_t n_pairs, size_t *blob_bytes)
+{
+    npas_status s = check_bp_desc(d);
+    if (s != NPAS_OK) return s;
+    if (n_pairs * d->Mb * d->Nb * 4 > 0x7FFFFFFFull) return NPAS_ERR_SHAPE;
+    *blob_bytes = bp_layout(*d, (uint32_t)n_pairs).total;
+    return NPAS_OK;
+}
+
 npas_status npas_pack_bp_size(const npas_bp_desc *d, const uint64_t *tap_mask_host, size_t *blob_bytes)
 {
     npas_status s = check_bp_desc(d);
@@ -324,33 +532,54 @@ npas_status npas_pack_bp_size(const npas_bp_desc *d, const uint64_t *tap_mask_ho
     const uint64_t live = d->R * d->S == 64 ? ~0ull : ((1ull << (d->R * d->S)) - 1);
     uint64_t n = 0;
     for (int i = 0; i < (d->K / d->Mb) * (d->C / d->Nb); ++i) n += __builtin_popcountll(tap_mask_host[i] & live);
-    if (n * d->Mb * d->Nb * 4 > 0x7FFFFFFFull) return NPAS_ERR_SHAPE;
-    *blob_bytes = bp_layout(*d, (uint32_t)n).total;
-    return NPAS_OK;
+    return npas_internal_bp_size(d, n, blob_bytes);
 }
 
-npas_status npas_pack_bp(const npas_bp_desc *d, const void *w, const uint64_t *tap_mask, void *blob,
-                         size_t blob_bytes, void *stream)
+npas_status npas_internal_pack_bp(const npas_bp_desc *d, const void *w, const uint64_t *tap_mask, void *blob,
+                                  size_t blob_bytes, void *stream)
 {
     npas_status s = check_bp_desc(d);
     if (s != NPAS_OK) return s;
     if (!w || !tap_mask || !blob) return NPAS_ERR_NULL;
     if (!aligned16(w) || !aligned16(blob) || (reinterpret_cast<uintptr_t>(tap_mask) & 7)) return NPAS_ERR_ALIGNMENT;
-    if (blob_bytes < bp_layout(*d, 0).total || blob_bytes > 0xFFFFFFFFull) return NPAS_ERR_BUFFER_TOO_SMALL;
+    const BpLayout L = bp_layout(*d, 0);
+    if (blob_bytes < L.total || blob_bytes > 0xFFFFFFFFull) return NPAS_ERR_BUFFER_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(blob, 0, blob_bytes, st) != cudaSuccess) return NPAS_ERR_CUDA;
     const uint32_t nBlk = (d->K / d->Mb) * (d->C / d->Nb);
     uint8_t *b8 = static_cast<uint8_t *>(blob);
     bp_scan_kernel<<<1, 1024, 0, st>>>(*d, tap_mask, b8, (uint32_t)blob_bytes);
-    if (d->w_in == NPAS_F32 && d->w_packed == NPAS_F32)
-        bp_gather_kernel<uint32_t, uint32_t><<<nBlk, 128, 0, st>>>(*d, static_cast<const uint32_t *>(w), tap_mask, b8);
+    const uint32_t *w32 = static_cast<const uint32_t *>(w);
+    const uint16_t *w16 = static_cast<const uint16_t *>(w);
+    if (L.off_image) {
+        const uint32_t units = (uint32_t)d->K * d->R * d->S * (d->C / 8), unit_ctas = (units + 255) / 256;
+        const uint32_t items = (uint32_t)(d->K / L.GI) * (d->C / 16), grid = unit_ctas + (items + 7) / 8;
+        cudaError_t e = cudaSuccess;
+        auto go = [&](auto kernel, auto *wp) { e = tc::launch_pdl(kernel, dim3(grid), dim3(256), 0, st, *d, L, wp, tap_mask, b8, unit_ctas); };
+        if (d->w_in == NPAS_F32) {
+            if (d->Nb % 8 == 0) go(bp_expand_kernel<uint32_t, 8>, w32);
+            else if (d->Nb % 4 == 0) go(bp_expand_kernel<uint32_t, 4>, w32);
+            else go(bp_expand_kernel<uint32_t, 1>, w32);
+        } else {
+            if (d->Nb % 8 == 0) go(bp_expand_kernel<uint16_t, 8>, w16);
+            else if (d->Nb % 4 == 0) go(bp_expand_kernel<uint16_t, 4>, w16);
+            else go(bp_expand_kernel<uint16_t, 1>, w16);
+        }
+        if (e != cudaSuccess) return NPAS_ERR_CUDA;
+    } else if (d->w_packed == NPAS_F32)
+        bp_gather_kernel<uint32_t, uint32_t><<<nBlk, 128, 0, st>>>(*d, w32, tap_mask, b8);
     else if (d->w_in == NPAS_F32)
-        bp_gather_kernel<uint32_t, uint16_t><<<nBlk, 128, 0, st>>>(*d, static_cast<const uint32_t *>(w), tap_mask, b8);
+        bp_gather_kernel<uint32_t, uint16_t><<<nBlk, 128, 0, st>>>(*d, w32, tap_mask, b8);
     else
-        bp_gather_kernel<uint16_t, uint16_t><<<nBlk, 128, 0, st>>>(*d, static_cast<const uint16_t *>(w), tap_mask, b8);
+        bp_gather_kernel<uint16_t, uint16_t><<<nBlk, 128, 0, st>>>(*d, w16, tap_mask, b8);
     count_launch(2);
-    if (launch_status() != NPAS_OK) return NPAS_ERR_CUDA;
-    return packed_fits(blob, BP_MAGIC, kMagicBP, st);
+    return launch_status();
+}
+
+npas_status npas_pack_bp(const npas_bp_desc *d, const void *w, const uint64_t *tap_mask, void *blob,
+                         size_t blob_bytes, void *stream)
+{
+    npas_status s = npas_internal_pack_bp(d, w, tap_mask, blob, blob_bytes, stream);
+    return s == NPAS_OK ? packed_fits(blob, BP_MAGIC, kMagicBP, static_cast<cudaStream_t>(stream)) : s;
 }
 
 npas_status npas_unpack_bp(const npas_bp_desc *d, const void *blob, size_t blob_bytes, void *w_out,
@@ -390,28 +619,37 @@ npas_status npas_mask_bp_from_dense(const npas_bp_desc *d, const uint8_t *m, uin
     return v ? NPAS_ERR_MASK_STRUCTURE : NPAS_OK;
 }
 
+npas_status npas_internal_bb_size(const npas_bb_desc *d, uint64_t n_vals, uint32_t max_cols, size_t *blob_bytes)
+{
+    npas_status s = check_bb_desc(d);
+    if (s != NPAS_OK) return s;
+    const BbLayout L = bb_layout(*d);
+    const uint32_t Kp = round_up(max_cols, 16u) < 16u ? 16u : round_up(max_cols, 16u);
+    const uint64_t tiles = (uint64_t)L.nBlk * Kp * d->Bo * L.es;
+    if (n_vals * 4 > 0x3FFFFFFFull || tiles > 0x3FFFFFFFull) return NPAS_ERR_SHAPE;
+    *blob_bytes = (size_t)L.off_values + round_up((uint32_t)n_vals * L.es, 128) + round_up((uint32_t)tiles, 128);
+    return NPAS_OK;
+}
+
 npas_status npas_pack_bb_size(const npas_bb_desc *d, const uint64_t *rk, const uint64_t *ck, size_t *blob_bytes)
 {
     npas_status s = check_bb_desc(d);
     if (s != NPAS_OK) return s;
     if (!rk || !ck || !blob_bytes) return NPAS_ERR_NULL;
-    const BbLayout L = bb_layout(*d);
     const uint64_t rlive = d->Bo == 64 ? ~0ull : ((1ull << d->Bo) - 1), clive = d->Bi == 64 ? ~0ull : ((1ull << d->Bi) - 1);
+    const uint32_t nBlk = (uint32_t)(d->O / d->Bo) * (uint32_t)(d->I / d->Bi);
     uint64_t n = 0;
     uint32_t mx = 0;
-    for (uint32_t i = 0; i < L.nBlk; ++i) {
-        n += round_up((uint32_t)(__builtin_popcountll(rk[i] & rlive) * __builtin_popcountll(ck[i] & clive)), 8u);
-        mx = mx > (uint32_t)__builtin_popcountll(ck[i] & clive) ? mx : (uint32_t)__builtin_popcountll(ck[i] & clive);
+    for (uint32_t i = 0; i < nBlk; ++i) {
+        const uint32_t nc = (uint32_t)__builtin_popcountll(ck[i] & clive);
+        n += round_up((uint32_t)__builtin_popcountll(rk[i] & rlive) * nc, 8u);
+        mx = mx > nc ? mx : nc;
     }
-    const uint32_t Kp = round_up(mx, 16u) < 16u ? 16u : round_up(mx, 16u);
-    const uint64_t tiles = (uint64_t)L.nBlk * Kp * d->Bo * L.es;
-    if (n * 4 > 0x3FFFFFFFull || tiles > 0x3FFFFFFFull) return NPAS_ERR_SHAPE;
-    *blob_bytes = (size_t)L.off_values + round_up((uint32_t)n * L.es, 128) + round_up((uint32_t)tiles, 128);
-    return NPAS_OK;
+    return npas_internal_bb_size(d, n, mx, blob_bytes);
 }
 
-npas_status npas_pack_bb(const npas_bb_desc *d, const void *w, const uint64_t *rk, const uint64_t *ck,
-                         void *blob, size_t blob_bytes, void *stream)
+npas_status npas_internal_pack_bb(const npas_bb_desc *d, const void *w, const uint64_t *rk, const uint64_t *ck,
+                                  void *blob, size_t blob_bytes, void *stream)
 {
     npas_status s = check_bb_desc(d);
     if (s != NPAS_OK) return s;
@@ -420,18 +658,22 @@ npas_status npas_pack_bb(const npas_bb_desc *d, const void *w, const uint64_t *r
     const BbLayout L = bb_layout(*d);
     if (blob_bytes < L.off_values || blob_bytes > 0xFFFFFFFFull) return NPAS_ERR_BUFFER_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(blob, 0, blob_bytes, st) != cudaSuccess) return NPAS_ERR_CUDA;
     uint8_t *b8 = static_cast<uint8_t *>(blob);
     bb_scan_kernel<<<1, 1024, 0, st>>>(*d, rk, ck, b8, (uint32_t)blob_bytes, L);
-    if (d->w_in == NPAS_F32 && d->w_packed == NPAS_F32)
-        bb_gather_kernel<uint32_t, uint32_t><<<L.nBlk, 128, 0, st>>>(*d, static_cast<const uint32_t *>(w), rk, ck, b8, L);
-    else if (d->w_in == NPAS_F32)
-        bb_gather_kernel<uint32_t, uint16_t><<<L.nBlk, 128, 0, st>>>(*d, static_cast<const uint32_t *>(w), rk, ck, b8, L);
-    else
-        bb_gather_kernel<uint16_t, uint16_t><<<L.nBlk, 128, 0, st>>>(*d, static_cast<const uint16_t *>(w), rk, ck, b8, L);
+    auto go = [&](auto kernel, auto *wp) { return tc::launch_pdl(kernel, dim3(L.nBlk), dim3(256), 0, st, *d, wp, rk, ck, b8, L); };
+    const uint32_t *w32 = static_cast<const uint32_t *>(w);
+    const cudaError_t e = d->w_packed == NPAS_F32 ? go(bb_gather_kernel<uint32_t, uint32_t>, w32)
+                          : d->w_in == NPAS_F32 ? go(bb_gather_kernel<uint32_t, uint16_t>, w32)
+                                                : go(bb_gather_kernel<uint16_t, uint16_t>, static_cast<const uint16_t *>(w));
     count_launch(2);
-    if (launch_status() != NPAS_OK) return NPAS_ERR_CUDA;
-    return packed_fits(blob, BB_MAGIC, kMagicBB, st);
+    return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;
+}
+
+npas_status npas_pack_bb(const npas_bb_desc *d, const void *w, const uint64_t *rk, const uint64_t *ck,
+                         void *blob, size_t blob_bytes, void *stream)
+{
+    npas_status s = npas_internal_pack_bb(d, w, rk, ck, blob, blob_bytes, stream);
+    return s == NPAS_OK ? packed_fits(blob, BB_MAGIC, kMagicBB, static_cast<cudaStream_t>(stream)) : s;
 }
 
 npas_status npas_unpack_bb(const npas_bb_desc *d, const void *blob, size_t blob_bytes, void *w_out,
@@ -444,12 +686,11 @@ npas_status npas_unpack_bb(const npas_bb_desc *d, const void *blob, size_t blob_
     const BbLayout L = bb_layout(*d);
     if (blob_bytes < L.off_values) return NPAS_ERR_BUFFER_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (w_out && cudaMemsetAsync(w_out, 0, (size_t)d->O * d->I * L.es, st) != cudaSuccess) return NPAS_ERR_CUDA;
     const uint8_t *b8 = static_cast<const uint8_t *>(blob);
     if (d->w_packed == NPAS_F32)
-        bb_scatter_kernel<uint32_t><<<L.nBlk, 128, 0, st>>>(*d, b8, static_cast<uint32_t *>(w_out), rk_out, ck_out, L);
+        bb_scatter_kernel<uint32_t><<<L.nBlk, 256, 0, st>>>(*d, b8, static_cast<uint32_t *>(w_out), rk_out, ck_out, L);
     else
-        bb_scatter_kernel<uint16_t><<<L.nBlk, 128, 0, st>>>(*d, b8, static_cast<uint16_t *>(w_out), rk_out, ck_out, L);
+        bb_scatter_kernel<uint16_t><<<L.nBlk, 256, 0, st>>>(*d, b8, static_cast<uint16_t *>(w_out), rk_out, ck_out, L);
     count_launch();
     return launch_status();
 }
