@@ -138,7 +138,10 @@ typedef struct {
     int32_t path;
     int32_t variant; /* 0 = the kernel's own planner chooses its tile shape; path 7: NT + (MT << 16), NT =
                         64 (only when 128 does not divide K), 128 or 256 filters per item, MT = 1 or 2 position tiles per CTA (a combination the
-                        geometry does not allow gives NPAS_ERR_UNSUPPORTED); other paths ignore it.
+                        geometry does not allow gives NPAS_ERR_UNSUPPORTED); path 6: NT + (KC << 16) +
+                        (KT << 24) asks for the form for few output tiles, in which a cluster of KC * KT <= 8
+                        CTAs shares 128 positions x NT filters (16 to 128) and splits the channels into KC and
+                        the taps into KT ranges; other paths ignore it.
                         npas_tune_conv2d_bp measures the candidates and returns the best (path, variant). */
 } npas_conv_desc;
 

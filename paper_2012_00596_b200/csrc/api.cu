@@ -110,13 +110,23 @@ npas_status npas_linear_bb_workspace(const npas_linear_desc *d, const npas_bb_de
 // Kernel ids (the values `path` takes to force one): 1 CUDA cores, 3 tcgen05 with both operands in
 // shared memory, 5 three-channel first layer, 6 dense operand image, 7 the same on CTA pairs, 8 kept
 // pairs only.  Returns 0 when the requested path does not take the geometry.
+// Path 6 has two forms: the persistent kernel, and for few output tiles the one that splits channels and taps over a
+// cluster (asked for by `variant`, or chosen when no kernel was asked for; where the pair kernel has half a wave of its
+// stride-1 items, that one stays the choice).
+static bool conv_split(const npas_conv_desc &d, const npas_bp_desc &bp)
+{
+    if (d.path == 6) return d.variant != 0;
+    if ((d.path != 0 && d.path != 2) || (d.stride == 1 && conv_d2_preferred(d, bp))) return false;
+    return conv_sk_preferred(d, bp);
+}
+
 static int conv_kernel_for(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     switch (d.path) {
         case 1: return 1;
         case 3: return conv_tc_supported(d, bp) ? 3 : 0;
         case 5: return conv_stem_supported(d, bp) ? 5 : 0;
-        case 6: return conv_dn_supported(d, bp) ? 6 : 0;
+        case 6: return (d.variant ? conv_sk_supported(d, bp) : conv_dn_supported(d, bp)) ? 6 : 0;
         case 7: return conv_d2_supported(d, bp) ? 7 : 0;
         case 8: return conv_kr_supported(d, bp) ? 8 : 0;
         case 0: case 2: break;
@@ -126,6 +136,7 @@ static int conv_kernel_for(const npas_conv_desc &d, const npas_bp_desc &bp)
     // blocks of 16 channels or more); else the dense-image kernels; else shared-memory operands; else CUDA cores
     if (conv_stem_supported(d, bp)) return 5;
     if (conv_kr_preferred(d, bp)) return 8;
+    if (conv_split(d, bp)) return 6;
     if (conv_d2_preferred(d, bp)) return 7;
     if (conv_dn_supported(d, bp)) return 6;
     if (conv_tc_supported(d, bp)) return 3;
@@ -226,7 +237,9 @@ npas_status npas_conv2d_bp(const npas_conv_desc *d, const npas_bp_desc *bp, cons
         case 1: return conv_simt_launch(*d, *bp, x, blob, b, r, y, st);
         case 3: return conv_tc_launch(*d, *bp, x, blob, b, r, y, w, st);
         case 5: return conv_stem_launch(*d, *bp, x, blob, b, y, w, st);
-        case 6: return conv_dn_launch(*d, *bp, x, blob, b, r, y, w, st);
+        case 6:
+            if (conv_split(*d, *bp)) return conv_sk_launch(*d, *bp, x, blob, b, r, y, w, st);
+            return conv_dn_launch(*d, *bp, x, blob, b, r, y, w, st);
         case 7: return conv_d2_launch(*d, *bp, x, blob, b, r, y, w, st);
         case 8: return conv_kr_launch(*d, *bp, x, blob, b, r, y, w, st);
     }
@@ -330,9 +343,12 @@ npas_status npas_tune_conv2d_bp(const npas_conv_desc *d, const npas_bp_desc *bp,
     Timer t;
     if (!t.ok) return NPAS_ERR_CUDA;
     struct Cand { int path, variant; };
-    // (every item shape of the pair kernel: filters per item 64, 128 or 256, position tiles per CTA 1 or 2)
+    // (every item shape of the pair kernel: filters per item 64, 128 or 256, position tiles per CTA 1 or 2; filters and
+    // channel ranges of the split form of path 6)
     const Cand cands[] = {{5, 0}, {8, 0}, {7, 64 | (1 << 16)}, {7, 64 | (2 << 16)}, {7, 128 | (1 << 16)}, {7, 128 | (2 << 16)},
-                          {7, 256 | (1 << 16)}, {7, 256 | (2 << 16)}, {6, 0}, {3, 0}, {1, 0}};
+                          {7, 256 | (1 << 16)}, {7, 256 | (2 << 16)}, {6, 0}, {6, 32 | (1 << 16) | (1 << 24)},
+                          {6, 32 | (2 << 16) | (1 << 24)}, {6, 32 | (4 << 16) | (1 << 24)}, {6, 64 | (1 << 16) | (1 << 24)}, {6, 64 | (2 << 16) | (1 << 24)},
+                          {6, 64 | (4 << 16) | (1 << 24)}, {6, 64 | (8 << 16) | (1 << 24)}, {3, 0}, {1, 0}};
     float best = -1.f;
     bool tensor_core_found = false;
     for (const Cand &c : cands) {

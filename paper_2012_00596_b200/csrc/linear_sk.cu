@@ -109,7 +109,8 @@ linear_bb_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     } else if (warp == 1) {
         if (elect_one()) {
             const uint32_t idesc = idesc_bf16_f32(128, p.BN);
-            const uint32_t base16 = (smem_u32(smem) >> 4) | kDescLboOne, stage16 = p.stage_bytes >> 4;
+            // (18 address bits: in the CTAs of a cluster a shared-memory address carries the CTA's rank above them)
+            const uint32_t base16 = ((smem_u32(smem) & 0x3FFFFu) >> 4) | kDescLboOne, stage16 = p.stage_bytes >> 4;
             uint32_t s = 0, ph = 0, a_lo = base16;
             bool go = true;
             for (int k = 0; k < k_n; ++k) {
