@@ -583,12 +583,17 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
     return true;
 }
 
+bool planned(const npas_conv_desc &d, const npas_bp_desc &b, ConvD2Params &p)
+{
+    return cached_plan(d, b, 0, p, [&](ConvD2Params &q) { return plan(d, b, q, pairs_available()); });
+}
+
 }  // namespace
 
 bool conv_d2_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvD2Params p;
-    return plan(d, bp, p, pairs_available());
+    return planned(d, bp, p);
 }
 
 // Whether the pair kernel is the better of the two dense-image kernels for this call (measured): always
@@ -600,7 +605,7 @@ bool conv_d2_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvD2Params p;
     const int pairs = pairs_available();
-    if (pairs < 1 || !plan(d, bp, p, pairs)) return false;
+    if (pairs < 1 || !planned(d, bp, p)) return false;
     if (p.nph == 4) return true;
     return (long long)p.n_tiles * ((d.K + 127) / 128) >= 64;
 }
@@ -611,7 +616,7 @@ npas_status conv_d2_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
 {
     ConvD2Params p;
     const int pairs = pairs_available();
-    if (pairs < 1 || !plan(d, bp, p, pairs)) return NPAS_ERR_UNSUPPORTED;
+    if (pairs < 1 || !planned(d, bp, p)) return NPAS_ERR_UNSUPPORTED;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return NPAS_ERR_CUDA;
     // X[N][H][W][C] bf16 as (C, W, H, N): a box of 64 channels x Wp columns x slab rows lands in shared

@@ -420,12 +420,17 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvDnParams &p, int 
     return true;
 }
 
+bool planned(const npas_conv_desc &d, const npas_bp_desc &b, ConvDnParams &p)
+{
+    return cached_plan(d, b, 0, p, [&](ConvDnParams &q) { return plan(d, b, q, sm_count()); });
+}
+
 }  // namespace
 
 bool conv_dn_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvDnParams p;
-    return plan(d, bp, p, sm_count());
+    return planned(d, bp, p);
 }
 
 npas_status conv_dn_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
@@ -434,7 +439,7 @@ npas_status conv_dn_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
 {
     ConvDnParams p;
     const int sms = sm_count();
-    if (!plan(d, bp, p, sms)) return NPAS_ERR_UNSUPPORTED;
+    if (!planned(d, bp, p)) return NPAS_ERR_UNSUPPORTED;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return NPAS_ERR_CUDA;
     // X[N][H][W][C] bf16 seen as (8 channels, W, H, C/8, N): a box lands in shared memory as

@@ -660,13 +660,23 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvKrParams &p, dim3
     return true;
 }
 
+struct PlannedKr { ConvKrParams p; dim3 grid; };
+
+bool planned(const npas_conv_desc &d, const npas_bp_desc &bp, ConvKrParams &p, dim3 &grid)
+{
+    PlannedKr k;
+    if (!cached_plan(d, bp, 0, k, [&](PlannedKr &q) { return plan(d, bp, q.p, q.grid); })) return false;
+    p = k.p; grid = k.grid;
+    return true;
+}
+
 }  // namespace
 
 bool conv_kr_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvKrParams p;
     dim3 grid;
-    return plan(d, bp, p, grid);
+    return planned(d, bp, p, grid);
 }
 
 // Where this kernel was measured faster than the dense-image kernels (64x28x28x512 -> 512 with random
@@ -676,7 +686,7 @@ bool conv_kr_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvKrParams p;
     dim3 grid;
-    if (bp.max_taps <= 0 || !plan(d, bp, p, grid)) return false;
+    if (bp.max_taps <= 0 || !planned(d, bp, p, grid)) return false;
     if (p.n_tiles * p.nGrp < sm_count()) return false;
     return bp.Mb >= 32 ? 9 * bp.max_taps <= 4 * p.RS : 3 * bp.max_taps <= p.RS;
 }
@@ -687,7 +697,7 @@ npas_status conv_kr_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
 {
     ConvKrParams p;
     dim3 grid;
-    if (!plan(d, bp, p, grid)) return NPAS_ERR_UNSUPPORTED;
+    if (!planned(d, bp, p, grid)) return NPAS_ERR_UNSUPPORTED;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return NPAS_ERR_CUDA;
     // X[N][H][W][C] bf16 seen as (8 channels, W, H, C/8, N): a box lands in shared memory as

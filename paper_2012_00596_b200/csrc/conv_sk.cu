@@ -406,12 +406,17 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvSkParams &p, int 
     return found;
 }
 
+bool planned(const npas_conv_desc &d, const npas_bp_desc &bp, ConvSkParams &p, bool one_wave)
+{
+    return cached_plan(d, bp, one_wave, p, [&](ConvSkParams &q) { return plan(d, bp, q, sm_count(), one_wave); });
+}
+
 }  // namespace
 
 bool conv_sk_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvSkParams p;
-    return plan(d, bp, p, sm_count(), false);
+    return planned(d, bp, p, false);
 }
 
 // Measured against the persistent kernels (this one, then the better of the two): 14x14x256 -> 256 one image 4.8 against
@@ -426,8 +431,8 @@ bool conv_sk_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
     const int sms = sm_count();
     if (d.variant) return false;
     const bool phases = d.stride == 2 && d.R == 3 && d.S == 3 && d.pad == 1;
-    if (phases && (d.C % 64 || d.K % 64)) return plan(d, bp, p, sms, false);
-    if (!plan(d, bp, p, sms, true)) return false;
+    if (phases && (d.C % 64 || d.K % 64)) return planned(d, bp, p, false);
+    if (!planned(d, bp, p, true)) return false;
     return phases ? p.nBlk > 1 : p.n_tiles * 2 <= sms;
 }
 
@@ -435,8 +440,7 @@ npas_status conv_sk_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
                            const void *res, void *y, uint32_t *ws, cudaStream_t st)
 {
     ConvSkParams p;
-    const int sms = sm_count();
-    if (!plan(d, bp, p, sms, !d.variant) && !plan(d, bp, p, sms, false)) return NPAS_ERR_UNSUPPORTED;
+    if (!planned(d, bp, p, !d.variant) && !planned(d, bp, p, false)) return NPAS_ERR_UNSUPPORTED;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return NPAS_ERR_CUDA;
     // X[N][H][W][C] as (C, W, H, N): a box of CB channels x Wp columns x slab rows (every other pixel for a parity class)

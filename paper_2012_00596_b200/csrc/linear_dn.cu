@@ -436,12 +436,17 @@ bool encode_2d(CUtensorMap *map, const void *base, uint64_t inner, uint64_t oute
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool planned(const npas_linear_desc &d, const npas_bb_desc &b, LinDnParams &p)
+{
+    return cached_plan(d, b, 0, p, [&](LinDnParams &q) { return plan(d, b, q); });
+}
+
 }  // namespace
 
 bool linear_dn_supported(const npas_linear_desc &d, const npas_bb_desc &bb)
 {
     LinDnParams p;
-    return plan(d, bb, p);
+    return planned(d, bb, p);
 }
 
 npas_status linear_dn_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
@@ -449,7 +454,7 @@ npas_status linear_dn_launch(const npas_linear_desc &d, const npas_bb_desc &bb, 
                              cudaStream_t st)
 {
     LinDnParams p;
-    if (!plan(d, bb, p)) return NPAS_ERR_UNSUPPORTED;
+    if (!planned(d, bb, p)) return NPAS_ERR_UNSUPPORTED;
     const BbLayout L = bb_layout(bb);
     // X[M][I] and the masked weights [O][I]: boxes of 64 columns land as 128-byte rows, 16-byte
     // pieces XOR-ed with the row number; rows past the end read as zeros

@@ -273,12 +273,17 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinSkParams &p, int
     return found;
 }
 
+bool planned(const npas_linear_desc &d, const npas_bb_desc &bb, LinSkParams &p, bool automatic)
+{
+    return cached_plan(d, bb, automatic, p, [&](LinSkParams &q) { return plan(d, bb, q, sm_count(), automatic); });
+}
+
 }  // namespace
 
 bool linear_sk_supported(const npas_linear_desc &d, const npas_bb_desc &bb)
 {
     LinSkParams p;
-    return plan(d, bb, p, sm_count(), false);
+    return planned(d, bb, p, false);
 }
 
 // Where the persistent kernels leave most SMs idle: fewer tiles of 128 x 128 than a quarter of the SMs.  Measured (this
@@ -294,14 +299,14 @@ bool linear_sk_preferred(const npas_linear_desc &d, const npas_bb_desc &bb)
     if (nMT * ((d.O + 127) / 128) * 4 >= sms) return false;
     if (d.I <= 256 && nMT > 1 && nMT * ((d.O + 31) / 32) * 5 < sms) return false;
     LinSkParams p;
-    return plan(d, bb, p, sms, true);
+    return planned(d, bb, p, true);
 }
 
 npas_status linear_sk_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x, const void *blob, const float *bias,
                              const void *res, void *y, uint32_t *ws, cudaStream_t st)
 {
     LinSkParams p;
-    if (!plan(d, bb, p, sm_count(), true)) return NPAS_ERR_UNSUPPORTED;
+    if (!planned(d, bb, p, true)) return NPAS_ERR_UNSUPPORTED;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return NPAS_ERR_CUDA;
     const BbLayout L = bb_layout(bb);
