@@ -178,6 +178,9 @@ bool conv_stem_pool_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 npas_status conv_stem_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                              const void *blob, const float *bias, void *y, uint32_t *ws, cudaStream_t st,
                              bool pool = false);
+bool conv_stem_rows_supported(const npas_conv_desc &d, const npas_bp_desc &bp, bool pool);
+npas_status conv_stem_rows_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x, const void *blob,
+                                  const float *bias, void *y, uint32_t *ws, cudaStream_t st, bool pool);
 bool conv_dn_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 npas_status conv_dn_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,

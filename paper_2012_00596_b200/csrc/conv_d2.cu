@@ -145,7 +145,9 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     tc_fence_before_sync();
     cluster_sync_all();                 // barriers of both CTAs exist before anything arrives on them
     tc_fence_after_sync();
-    pdl_wait();                         // nothing above touches global memory
+    // Nothing above touches global memory.  The weight producer does not wait: it reads the blob only, which no kernel that
+    // lets its successor start early writes, so the first ring of weights is on its way while the kernel before this one ends.
+    if (warp != 2) pdl_wait();
     const uint32_t tmem_base = bars->tmem_base;
     // the two producers start at once; the other warps first stage the biases and the tap unions
     if (warp != 0 && warp != 2) {

@@ -114,7 +114,19 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     tc_fence_before_sync();
     cluster_sync_all();                 // barriers of both CTAs exist before anything arrives on them
     tc_fence_after_sync();
-    pdl_wait();                        // nothing above touches global memory
+    // The weights of the first ring of stages are requested before the wait for the kernel before this one: no kernel that
+    // lets its successor start early writes them.
+    int early = 0;
+    if (warp == 0 && lane == 0) {
+        int tile = pair, k = 0;
+        for (; early < p.S && tile < p.n_tiles; ++early) {
+            if (rank == 0) mbar_arrive_expect_tx(&bars->full[early], 2u * p.stage_bytes);
+            tma_load_2d_pair(smem + (size_t)early * p.stage_bytes + kXBytes, &tmap_w, map_to_cta(smem_u32(&bars->full[early]), 0u), k * 64,
+                             (tile % p.nNT) * p.BN + (int)rank * (p.BN / 2));
+            if (++k == p.nK) { k = 0; tile += n_pairs; }
+        }
+    }
+    pdl_wait();                        // nothing else above touches global memory
     // the biases: staged by the epilogue warps, which meet again before the first use
     if (warp >= kFirstEpiWarp && warp < kResWarp) {
         for (int i = tid - kFirstEpiWarp * 32; i < p.O; i += kEpiWarps * 32) bias_s[i] = bias ? bias[i] : 0.f;
@@ -134,9 +146,9 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 for (int k = 0; k < p.nK; ++k) {
                     if (lap >= 1 && !pair_wait(&bars->empty[s], (lap & 1u) ^ 1u, abort_flag, peer_abort, ws, 0x8100)) { ok = false; break; }
                     uint8_t *st = smem + (size_t)s * p.stage_bytes;
-                    if (rank == 0) mbar_arrive_expect_tx(&bars->full[s], 2u * p.stage_bytes);
+                    if (rank == 0 && early <= 0) mbar_arrive_expect_tx(&bars->full[s], 2u * p.stage_bytes);
                     tma_load_2d_pair(st, &tmap_x, full0 + s * 8u, k * 64, mt * kRows);     // rows past M read as zeros
-                    tma_load_2d_pair(st + kXBytes, &tmap_w, full0 + s * 8u, k * 64, nt * p.BN + (int)rank * (p.BN / 2));
+                    if (early-- <= 0) tma_load_2d_pair(st + kXBytes, &tmap_w, full0 + s * 8u, k * 64, nt * p.BN + (int)rank * (p.BN / 2));
                     if (++s == (uint32_t)p.S) { s = 0; ++lap; }
                 }
             }

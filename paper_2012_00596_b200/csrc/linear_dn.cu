@@ -110,7 +110,18 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    pdl_wait();                        // nothing above touches global memory
+    // The weights of the first ring of stages are requested before the wait for the kernel before this one: no kernel that
+    // lets its successor start early writes them.
+    int early = 0;
+    if (warp == 0 && lane == 0) {
+        int tile = blockIdx.x, k = 0;
+        for (; early < p.S && tile < p.n_tiles; ++early) {
+            mbar_arrive_expect_tx(&bars->full[early], p.stage_bytes);
+            tma_load_2d(smem + (size_t)early * p.stage_bytes + kXBytes, &tmap_w, &bars->full[early], k * 64, (tile % p.nNT) * p.BN);
+            if (++k == p.nK) { k = 0; tile += gridDim.x; }
+        }
+    }
+    pdl_wait();                        // nothing else above touches global memory
     // the biases: staged by the epilogue warps, which meet again before the first use
     if (warp >= kFirstEpiWarp && warp < kResWarp) {
         for (int i = tid - kFirstEpiWarp * 32; i < p.nNT * p.BN; i += kEpiWarps * 32) bias_s[i] = (bias && i < p.O) ? bias[i] : 0.f;
@@ -130,9 +141,9 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 for (int k = 0; k < p.nK; ++k) {
                     if (lap >= 1 && !mbar_wait(&bars->empty[s], (lap & 1u) ^ 1u, abort_flag, ws, 0x5100)) { ok = false; break; }
                     uint8_t *st = smem + (size_t)s * p.stage_bytes;
-                    mbar_arrive_expect_tx(&bars->full[s], p.stage_bytes);
+                    if (early <= 0) mbar_arrive_expect_tx(&bars->full[s], p.stage_bytes);
                     tma_load_2d(st, &tmap_x, &bars->full[s], k * 64, mt * kRows);
-                    tma_load_2d(st + kXBytes, &tmap_w, &bars->full[s], k * 64, nt * p.BN);
+                    if (early-- <= 0) tma_load_2d(st + kXBytes, &tmap_w, &bars->full[s], k * 64, nt * p.BN);
                     if (++s == (uint32_t)p.S) { s = 0; ++lap; }
                 }
             }
