@@ -9,11 +9,19 @@
 // MMAs (K = 32: eight pixels x four channels, the eighth pixel and the fourth channel meet zero weights) straight from the
 // rows.  Widening a row costs one 16-byte store per two pixels, once per row instead of once per window.
 //
+// Shared memory is what bounds it (an MMA of K filters reads 4 KB of rows and 32 K bytes of weights, three times what its
+// arithmetic takes), so the two output rows of a step share their operand: input row t of the window is kernel row t of the
+// first and t - 2 of the second, and with the kernel rows of one parity stored in falling order the two filter sets are one
+// operand of 2 K columns.  18 operand reads per step instead of 28.
+//
 // A CTA walks consecutive steps; a step is two output rows (2p, 2p + 1) of an image, i.e. one pooled row.
 //   warps 0-3   input rows -> ring of widened rows (four new rows per step; loads run a step ahead)
-//   warp 4      MMAs: per output row seven kernel rows x two, rows outside the image skipped, into one of two TMEM sets
-//   warps 5-12  epilogue: bias, ReLU, one rounding; pooled: the running maximum with the row above (kept in registers from
-//               the step before), through shared memory, then three columns to one and 16-byte stores along the row.
+//   warp 4      MMAs: nine input rows x two, rows outside the image are zeros, into one of two TMEM sets
+//   warps 5-12  epilogue: bias, ReLU, one rounding; pooled: after the maximum with the row above (kept in registers from
+//               the step before: all of it is monotone, so one rounding serves the three rows), into one of two stages
+//   warps 13-15 (pooled) three staged columns to one, 16-byte stores along the row.  Warps of their own: these loads queue
+//               behind the operand reads of the MMAs, and the accumulators waited for them (1.8 k of 3.6 k clocks a step).
+// 64 x 224 x 224, K = 64, pooled: 49.3 us (63 with separate operand reads and pooling by the epilogue's warps).
 // Every pooled value is written once: no reductions in memory and nothing to clear first.  Every wait is bounded.
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -25,7 +33,8 @@ using namespace tc;
 namespace {
 
 constexpr int kConvWarps = 4, kMmaWarp = kConvWarps, kFirstEpi = kConvWarps + 1, kEpiWarps = 8;
-constexpr int kThreads = (kFirstEpi + kEpiWarps) * 32;
+constexpr int kFirstPool = kFirstEpi + kEpiWarps, kPoolWarps = 3;
+template <bool kPool> constexpr int kThreads = (kFirstPool + (kPool ? kPoolWarps : 0)) * 32;
 constexpr int kR = 7, kC = 3;
 constexpr int kSlots = 24;                         // rows of the ring: a window of nine, and up to nine of the next step
 constexpr int kWindow = 9;                         // input rows under a step
@@ -40,7 +49,7 @@ struct StemRowsParams {
 };
 
 struct StemRowsBars {
-    uint64_t in_full[2], in_empty[2], acc_full[2], acc_empty[2];
+    uint64_t in_full[2], in_empty[2], acc_full[2], acc_empty[2], stage_full[2], stage_empty[2];
     uint32_t tmem_base;
     uint32_t abort_flag;
 };
@@ -56,15 +65,6 @@ __device__ __forceinline__ uint4 max4(const uint4 &a, const uint4 &b)
 {
     return make_uint4(max_bf16x2(a.x, b.x), max_bf16x2(a.y, b.y), max_bf16x2(a.z, b.z), max_bf16x2(a.w, b.w));
 }
-// barrier among the epilogue warps with a vote: true when every one of their threads says so
-__device__ __forceinline__ bool epi_all(bool ok)
-{
-    uint32_t r;
-    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %2, 0;\n\tbar.red.and.pred p, 1, %1, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(r) : "n"(kEpiWarps * 32), "r"((uint32_t)ok) : "memory");
-    return r != 0u;
-}
-
 // The steps of a CTA in order.  `warm`: the step before the first one of an image's inside, computed for the row it hands
 // on and not stored.
 struct Steps {
@@ -86,14 +86,14 @@ struct Steps {
 };
 
 template <bool kPool>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads<kPool>, 1)
 conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, const uint8_t *__restrict__ blob,
                       const float *__restrict__ bias, void *__restrict__ y, uint32_t *ws)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *ring = smem;                             // [kSlots] rows of `pitch` bytes: pixel x at 8 (x + 3)
-    uint8_t *bsm = smem + p.off_b;                    // [7 kernel rows][4 octets][K filters][8] bf16
+    uint8_t *bsm = smem + p.off_b;                    // [parity of the kernel row][4 octets][4 K: (6 | 5 - r) / 2, filter][8] bf16
     float *bias_s = reinterpret_cast<float *>(smem + p.off_bias);
     StemRowsBars *bars = reinterpret_cast<StemRowsBars *>(smem + p.off_bar);
     volatile uint32_t *abort_flag = &bars->abort_flag;
@@ -105,6 +105,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
         for (int s = 0; s < 2; ++s) {
             mbar_init(&bars->in_full[s], kConvWarps); mbar_init(&bars->in_empty[s], 1);
             mbar_init(&bars->acc_full[s], 1); mbar_init(&bars->acc_empty[s], kEpiWarps);
+            mbar_init(&bars->stage_full[s], kEpiWarps); mbar_init(&bars->stage_empty[s], kPoolWarps);
         }
         bars->abort_flag = 0;
         fence_barrier_init();
@@ -112,7 +113,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
     if (warp == kMmaWarp) tmem_alloc(&bars->tmem_base, p.tmem_cols);
     pdl_trigger();
     // borders of the ring's rows and the operand's unused places: zeros, once
-    for (uint32_t o = tid * 16; o < p.off_stage; o += kThreads * 16) *reinterpret_cast<uint4 *>(smem + o) = make_uint4(0, 0, 0, 0);
+    for (uint32_t o = tid * 16; o < p.off_stage; o += kThreads<kPool> * 16) *reinterpret_cast<uint4 *>(smem + o) = make_uint4(0, 0, 0, 0);
     __syncthreads();
     {
         // weight of (tap (r, s), channel c, filter n) at k = s * 4 + c of kernel row r.  (The blob is never written by a
@@ -125,18 +126,18 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
         for (int fb = 0; fb < p.K / p.Mb; ++fb) {
             const uint32_t j0 = blk_off[fb], n = (blk_off[fb + 1] - j0) * per_pair;       // one channel block per filter block
 #pragma unroll 4
-            for (uint32_t e = tid; e < n; e += kThreads) {
+            for (uint32_t e = tid; e < n; e += kThreads<kPool>) {
                 const uint32_t j = j0 + e / per_pair, rem = e % per_pair, f = rem / kC, c = rem - f * kC;
                 const uint32_t tap = pairs[j] >> 16, r = tap / kR, sx = tap - r * kR;
                 const uint16_t v = values[(size_t)j * per_pair + rem];
                 const uint32_t kk = sx * 4 + c;
                 if (r < (uint32_t)kR)                                                        // (not a 7x7 tap: ignored)
-                    *reinterpret_cast<uint16_t *>(bsm + (((size_t)r * 4 + (kk >> 3)) * p.K + fb * p.Mb + f) * 16 + (kk & 7) * 2) = v;
+                    *reinterpret_cast<uint16_t *>(bsm + ((((size_t)(r & 1) * 4 + (kk >> 3)) * 4 + ((6 - r) >> 1)) * p.K + fb * p.Mb + f) * 16 + (kk & 7) * 2) = v;
             }
         }
     }
     pdl_wait();
-    for (int i = tid; i < p.K; i += kThreads) bias_s[i] = bias ? bias[i] : 0.f;
+    for (int i = tid; i < p.K; i += kThreads<kPool>) bias_s[i] = bias ? bias[i] : 0.f;
     fence_proxy_async_smem();
     tc_fence_before_sync();
     __syncthreads();
@@ -144,13 +145,14 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
     const uint32_t tmem_base = bars->tmem_base;
 
     if (warp < kConvWarps) {
-        // ---- input rows: thread u widens pixel pair u, i.e. padded pixels 2u and 2u + 1 = input pixels 2u - 3 and 2u - 2,
-        // twelve bytes that start two bytes before a word boundary ------------------------------------------------------
-        const int words_in = 3 * p.W / 2, u = tid, g = 3 * u - 5;            // first word of the twelve (and two) bytes
-        const bool on = u < p.pairs;
+        // ---- input rows: thread u - 1 widens pixel pair u, i.e. padded pixels 2u and 2u + 1 = input pixels 2u - 3 and 2u - 2,
+        // twelve bytes that start two bytes before a word boundary.  (Pair 0 is padding; rows of 128 columns have one pair
+        // more than there are threads, the last pixel and padding: four threads take one row's each.) --------------------
+        const int words_in = 3 * p.W / 2, u = tid + 1, g = 3 * u - 5;        // first word of the twelve (and two) bytes
+        const bool on = u < p.pairs, tail = p.Q == kConvWarps * 32 && tid < 4;
         const uint32_t *x32 = reinterpret_cast<const uint32_t *>(x);
         // rows w .. w + 3 of the window of (image n, first row y_lo): requested together
-        auto request = [&](uint32_t (&a)[4][4], int n, int y_lo, int w) {
+        auto request = [&](uint32_t (&a)[4][4], uint2 &last, int n, int y_lo, int w) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int yy = y_lo + w + q;
@@ -159,8 +161,19 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
 #pragma unroll
                 for (int k = 0; k < 4; ++k) a[q][k] = in && g + k >= 0 && g + k < words_in ? __ldg(row + g + k) : 0u;
             }
+            last = make_uint2(0u, 0u);
+            if (tail && w + tid < kWindow && y_lo + w + tid >= 0 && y_lo + w + tid < p.H) {
+                const uint32_t *end = x32 + ((size_t)n * p.H + y_lo + w + tid + 1) * words_in;
+                last = make_uint2(__ldg(end - 2), __ldg(end - 1));
+            }
         };
-        auto widen = [&](const uint32_t (&a)[4][4], uint32_t base, int w) {
+        auto widen = [&](const uint32_t (&a)[4][4], const uint2 &last, uint32_t base, int w) {
+            if (tail && w + tid < kWindow) {
+                uint32_t slot = base + (uint32_t)(w + tid);
+                if (slot >= (uint32_t)kSlots) slot -= kSlots;
+                *reinterpret_cast<uint4 *>(ring + slot * p.pitch + (uint32_t)(p.Q + 1) * 16u) =
+                    make_uint4(__funnelshift_r(last.x, last.y, 16), last.y >> 16, 0u, 0u);
+            }
             if (!on) return;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -175,9 +188,10 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
             }
         };
         Steps st(lo, hi, p.spi, kPool);
+        uint2 next_last, l0, l1;
         uint32_t i = 0, base = 0, next[4][4];                                // step count; ring slot of the window's first row
         bool more = st.next();
-        if (more) request(next, st.n, 4 * st.p - 3, kWindow - 4);           // the four rows every step brings, a step ahead
+        if (more) request(next, next_last, st.n, 4 * st.p - 3, kWindow - 4);   // the four rows every step brings, a step ahead
         while (more) {
             const int y_lo = 4 * st.p - 3;
             base = st.reset ? (i ? base + kWindow : 0u) : base + 4u;
@@ -185,14 +199,14 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
             if (i >= 2 && !mbar_wait(&bars->in_empty[i & 1u], ((i >> 1) & 1u) ^ 1u, abort_flag, ws, 0xB100)) break;
             if (st.reset) {                                                  // the other five rows of the window
                 uint32_t a[4][4], b2[4][4];
-                request(a, st.n, y_lo, 0);
-                request(b2, st.n, y_lo, 1);
-                widen(a, base, 0);
-                widen(b2, base, 1);
+                request(a, l0, st.n, y_lo, 0);
+                request(b2, l1, st.n, y_lo, 1);
+                widen(a, l0, base, 0);
+                widen(b2, l1, base, 1);
             }
-            widen(next, base, kWindow - 4);
+            widen(next, next_last, base, kWindow - 4);
             more = st.next();
-            if (more) request(next, st.n, 4 * st.p - 3, kWindow - 4);
+            if (more) request(next, next_last, st.n, 4 * st.p - 3, kWindow - 4);
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars->in_full[i & 1u]);
@@ -201,9 +215,9 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
     } else if (warp == kMmaWarp) {
         // ---- MMAs ------------------------------------------------------------------------------------------------------
         if (elect_one()) {
-            const uint32_t idesc = idesc_bf16_f32(128, p.K);
+            const uint32_t idesc1 = idesc_bf16_f32(128, p.K), idesc2 = idesc_bf16_f32(128, 2 * p.K);
             const uint32_t ring16 = (smem_u32(ring) >> 4) | (1u << 16), pitch16 = p.pitch >> 4;      // K-direction offset: 16 bytes
-            const uint32_t b16 = (smem_u32(bsm) >> 4) | ((uint32_t)p.K << 16), brow16 = 4u * p.K;
+            const uint32_t b16 = (smem_u32(bsm) >> 4) | ((uint32_t)(4 * p.K) << 16);
             Steps st(lo, hi, p.spi, kPool);
             uint32_t i = 0, base = 0;
             bool ok = true;
@@ -214,19 +228,20 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                 if (i >= 2 && !mbar_wait(&bars->acc_empty[b], ph ^ 1u, abort_flag, ws, 0xB200)) break;
                 if (!mbar_wait(&bars->in_full[b], ph, abort_flag, ws, 0xB210)) break;
                 tc_fence_after_sync();
-                for (int j = 0; j < 2; ++j) {
-                    const uint32_t d = tmem_base + (b * 2u + j) * p.K;
-                    const int y0 = 2 * (2 * st.p + j) - 3;                  // input row under kernel row 0
-                    uint32_t acc = 0;
-                    for (int r = 0; r < kR; ++r) {
-                        if (y0 + r < 0 || y0 + r >= p.H) continue;           // zero padding
-                        uint32_t slot = base + 2u * j + r;
-                        if (slot >= (uint32_t)kSlots) slot -= kSlots;
-                        const uint32_t a_lo = ring16 + slot * pitch16, b_lo = b16 + r * brow16;
-                        mma_bf16_ss(d, desc64(a_lo), desc64(b_lo), idesc, acc);
-                        mma_bf16_ss(d, desc64(a_lo + 2u), desc64(b_lo + 2u * p.K), idesc, 1u);
-                        acc = 1u;
-                    }
+                const uint32_t d = tmem_base + b * 2u * p.K;
+                // window row t: kernel row t of the first output row (t < 7), t - 2 of the second (t >= 2); a row that
+                // both need goes first, so that one MMA starts both sums
+#pragma unroll
+                for (int k = 0; k < kWindow; ++k) {
+                    const uint32_t t = k < 5 ? k + 2 : k < 7 ? k - 5 : k;
+                    const bool both = t >= 2 && t < (uint32_t)kR;
+                    const uint32_t r = t < (uint32_t)kR ? t : t - 2;         // the larger kernel row: the operand's first columns
+                    uint32_t slot = base + t;
+                    if (slot >= (uint32_t)kSlots) slot -= kSlots;
+                    const uint32_t a_lo = ring16 + slot * pitch16, b_lo = b16 + ((r & 1) * 16 + ((6 - r) >> 1)) * p.K;
+                    const uint32_t dt = t < (uint32_t)kR ? d : d + p.K, idesc = both ? idesc2 : idesc1;
+                    mma_bf16_ss(dt, desc64(a_lo), desc64(b_lo), idesc, k > 0);
+                    mma_bf16_ss(dt, desc64(a_lo + 2u), desc64(b_lo + 8u * p.K), idesc, 1u);
                 }
                 mma_commit(&bars->in_empty[b]);
                 mma_commit(&bars->acc_full[b]);
@@ -234,58 +249,57 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
             }
         }
         __syncwarp();
-    } else {
+    } else if (warp < kFirstPool) {
         // ---- epilogue: warp -> TMEM lane quarter and every second 16-column chunk -----------------------------------------
-        const int quarter = warp & 3, part = (warp - kFirstEpi) >> 2, q = quarter * 32 + lane, et = tid - kFirstEpi * 32;
+        const int quarter = warp & 3, part = (warp - kFirstEpi) >> 2, q = quarter * 32 + lane;
         const int nch = p.K / 16;
         constexpr int kMaxOwn = 4;                       // chunks per warp (K <= 128)
-        uint32_t saved[kMaxOwn][8];                      // the row above, packed
-#pragma unroll
-        for (int c = 0; c < kMaxOwn; ++c)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) saved[c][k] = 0u;
+        float saved[kMaxOwn][16];                        // the row above (pooled)
         Steps st(lo, hi, p.spi, kPool);
         uint32_t i = 0;
         bool ok = true;
         while (st.next()) {
             const uint32_t b = i & 1u;
             uint8_t *stage = smem + p.off_stage + (kPool ? (size_t)b * p.stage_bytes : 0u);
-            if (kPool && st.p == 0) {
+            if (kPool && st.reset) {
 #pragma unroll
                 for (int c = 0; c < kMaxOwn; ++c)
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) saved[c][k] = 0u;            // (nothing is negative after ReLU)
+                    for (int k = 0; k < 16; ++k) saved[c][k] = __uint_as_float(0xFF800000u);
             }
             ok = mbar_wait(&bars->acc_full[b], (i >> 1) & 1u, abort_flag, ws, 0xB400);
-            if (!__all_sync(0xFFFFFFFFu, ok)) ok = false;
+            if (kPool && ok && i >= 2) ok = mbar_wait(&bars->stage_empty[b], ((i >> 1) & 1u) ^ 1u, abort_flag, ws, 0xB410);
+            if (!__all_sync(0xFFFFFFFFu, ok)) break;
             tc_fence_after_sync();
             const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * 2u * p.K;
 #pragma unroll
             for (int c = 0; c < kMaxOwn; ++c) {
                 const int ch = part + 2 * c;
-                if (ch >= nch || !ok) break;
+                if (ch >= nch) break;
                 uint32_t r0[16], r1[16];
                 tmem_ld_x16(t_addr + ch * 16, r0);
                 tmem_ld_x16(t_addr + p.K + ch * 16, r1);
                 tmem_ld_wait();
-                uint32_t o0[8], o1[8];
+                const float4 *b4 = reinterpret_cast<const float4 *>(bias_s + ch * 16);
+                float bv[16];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const float b0 = bias_s[ch * 16 + 2 * k], b1 = bias_s[ch * 16 + 2 * k + 1];
-                    o0[k] = cvt_bf16x2(__uint_as_float(r0[2 * k]) + b0, __uint_as_float(r0[2 * k + 1]) + b1);
-                    o1[k] = cvt_bf16x2(__uint_as_float(r1[2 * k]) + b0, __uint_as_float(r1[2 * k + 1]) + b1);
-                    if (p.relu) { o0[k] = relu_bf16x2(o0[k]); o1[k] = relu_bf16x2(o1[k]); }
+                for (int k = 0; k < 4; ++k) {
+                    const float4 v = b4[k];
+                    bv[4 * k] = v.x; bv[4 * k + 1] = v.y; bv[4 * k + 2] = v.z; bv[4 * k + 3] = v.w;
                 }
                 if constexpr (kPool) {
                     // rows 2p - 1, 2p, 2p + 1 (the last one may not exist)
                     const bool has1 = 2 * st.p + 1 < p.P;
                     uint32_t m[8];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        m[k] = max_bf16x2(saved[c][k], o0[k]);
-                        if (has1) m[k] = max_bf16x2(m[k], o1[k]);
-                        saved[c][k] = o1[k];
+                    for (int k = 0; k < 16; ++k) {
+                        float v = fmaxf(saved[c][k], __uint_as_float(r0[k]));
+                        if (has1) v = fmaxf(v, __uint_as_float(r1[k]));
+                        saved[c][k] = __uint_as_float(r1[k]);
+                        bv[k] += v;
                     }
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) m[k] = relu_bf16x2(cvt_bf16x2(bv[2 * k], bv[2 * k + 1]));
                     // one line of 2 K bytes per column, 16-byte units XOR-ed with the column (conflict free)
                     uint8_t *line = stage + (size_t)q * p.line;
                     const uint32_t x7 = (uint32_t)(q & 7);
@@ -299,9 +313,15 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                         const size_t o = (((size_t)st.n * p.P + row) * p.Q + q) * p.K + ch * 16;
                         if (p.y_bf16) {
                             uint4 *yp = reinterpret_cast<uint4 *>(static_cast<uint16_t *>(y) + o);
-                            const uint32_t *v = j ? o1 : o0;
-                            yp[0] = make_uint4(v[0], v[1], v[2], v[3]);
-                            yp[1] = make_uint4(v[4], v[5], v[6], v[7]);
+                            const uint32_t *v = j ? r1 : r0;
+                            uint32_t o2[8];
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) {
+                                o2[k] = cvt_bf16x2(__uint_as_float(v[2 * k]) + bv[2 * k], __uint_as_float(v[2 * k + 1]) + bv[2 * k + 1]);
+                                if (p.relu) o2[k] = relu_bf16x2(o2[k]);
+                            }
+                            yp[0] = make_uint4(o2[0], o2[1], o2[2], o2[3]);
+                            yp[1] = make_uint4(o2[4], o2[5], o2[6], o2[7]);
                         } else {
                             float4 *yp = reinterpret_cast<float4 *>(static_cast<float *>(y) + o);
                             const uint32_t *v = j ? r1 : r0;
@@ -310,7 +330,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                                 float f[4];
 #pragma unroll
                                 for (int k = 0; k < 4; ++k) {
-                                    f[k] = __uint_as_float(v[4 * h + k]) + bias_s[ch * 16 + 4 * h + k];
+                                    f[k] = __uint_as_float(v[4 * h + k]) + bv[4 * h + k];
                                     if (p.relu) f[k] = fmaxf(f[k], 0.f);
                                 }
                                 yp[h] = make_float4(f[0], f[1], f[2], f[3]);
@@ -321,23 +341,35 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
             }
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&bars->acc_empty[b]);
-            if constexpr (kPool) {
-                if (!epi_all(ok)) break;                 // (the staged row is complete; all eight warps go on, or stop, as one)
-                if (st.store) {
-                    // pooled column v = columns 2v - 1, 2v, 2v + 1
-                    const int units = p.K / 8;
-                    uint16_t *out = static_cast<uint16_t *>(y) + ((size_t)st.n * p.PP + st.p) * p.PQ * p.K;
-                    for (int e = et; e < p.PQ * units; e += kEpiWarps * 32) {
-                        const int v = e / units, u = e - v * units, c0 = 2 * v;
-                        auto at = [&](int col) { return *reinterpret_cast<const uint4 *>(stage + (size_t)col * p.line + (((uint32_t)u ^ (uint32_t)(col & 7)) << 4)); };
-                        uint4 m = at(c0);
-                        if (c0 > 0) m = max4(m, at(c0 - 1));
-                        if (c0 + 1 < p.Q) m = max4(m, at(c0 + 1));
-                        *reinterpret_cast<uint4 *>(out + (size_t)v * p.K + u * 8) = m;
-                    }
+            if (lane == 0) {
+                mbar_arrive(&bars->acc_empty[b]);
+                if (kPool) mbar_arrive(&bars->stage_full[b]);
+            }
+            ++i;
+        }
+    } else if constexpr (kPool) {
+        // ---- pooling: thread -> 16-byte unit u of a line, every `vs`-th pooled column; column v = columns 2v - 1, 2v, 2v + 1
+        const int pt = tid - kFirstPool * 32, units = p.K / 8, u = pt % units, v0 = pt / units, vs = kPoolWarps * 32 / units;
+        const bool on = v0 < vs;
+        Steps st(lo, hi, p.spi, kPool);
+        uint32_t i = 0;
+        while (st.next()) {
+            const uint32_t b = i & 1u;
+            const bool ok = mbar_wait(&bars->stage_full[b], (i >> 1) & 1u, abort_flag, ws, 0xB500);
+            if (!__all_sync(0xFFFFFFFFu, ok)) break;
+            if (on && st.store) {
+                const uint8_t *stage = smem + p.off_stage + (size_t)b * p.stage_bytes;
+                uint16_t *out = static_cast<uint16_t *>(y) + ((size_t)st.n * p.PP + st.p) * p.PQ * p.K + u * 8;
+                auto at = [&](int col) { return *reinterpret_cast<const uint4 *>(stage + (size_t)col * p.line + (((uint32_t)u ^ (uint32_t)(col & 7)) << 4)); };
+#pragma unroll 4
+                for (int v = v0; v < p.PQ; v += vs) {
+                    const int c0 = 2 * v;
+                    const uint4 m = max4(at(c0), max4(at(c0 > 0 ? c0 - 1 : c0), at(c0 + 1 < p.Q ? c0 + 1 : c0)));
+                    *reinterpret_cast<uint4 *>(out + (size_t)v * p.K) = m;
                 }
-            } else if (!ok) break;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->stage_empty[b]);
             ++i;
         }
     }
@@ -358,7 +390,7 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, StemRowsParams &p, bo
     p.P = (d.H + 2 * d.pad - d.R) / 2 + 1; p.Q = (d.W + 2 * d.pad - d.S) / 2 + 1;
     if (p.P < 1 || p.Q < 1 || p.Q > 128) return false;         // a whole output row is one MMA tile
     p.relu = d.relu; p.y_bf16 = d.y_dtype == NPAS_BF16;
-    if (pool && (!d.relu || !p.y_bf16)) return false;          // (the running maximum starts from zero, on packed bf16 pairs)
+    if (pool && (!d.relu || !p.y_bf16)) return false;          // (rows beside the image count as nothing because nothing is negative)
     p.PP = (p.P - 1) / 2 + 1; p.PQ = (p.Q - 1) / 2 + 1;
     p.spi = (p.P + 1) / 2;                                     // = PP
     const long long steps = (long long)d.N * p.spi;
@@ -368,7 +400,7 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, StemRowsParams &p, bo
     p.pitch = round_up((uint32_t)p.pairs * 16u, 128);
     p.line = round_up(2u * d.K, 128);
     p.off_b = kSlots * p.pitch + 1024u;                        // (an operand reads 128 columns, past the end of the last row)
-    p.off_stage = round_up(p.off_b + (uint32_t)kR * 4u * d.K * 16u, 128);
+    p.off_stage = round_up(p.off_b + 2u * 4u * 4u * d.K * 16u, 128);
     p.stage_bytes = 128u * p.line;
     p.off_bias = p.off_stage + (pool ? 2u * p.stage_bytes : 0u);
     p.off_bar = round_up(p.off_bias + d.K * 4u, 128);
@@ -392,13 +424,13 @@ npas_status conv_stem_rows_launch(const npas_conv_desc &d, const npas_bp_desc &b
 {
     StemRowsParams p;
     if (!plan(d, bp, p, pool)) return NPAS_ERR_UNSUPPORTED;
-    auto go = [&](auto kernel) {
+    auto go = [&](auto kernel, int threads) {
         if (allow_dynamic_smem(reinterpret_cast<const void *>(kernel), (int)kSmemLimit) != NPAS_OK) return cudaErrorUnknown;
         const int sms = sm_count(), grid = p.n_steps < sms ? p.n_steps : sms;
-        return launch_pdl(kernel, dim3(grid), dim3(kThreads), p.smem_bytes, st, p, static_cast<const uint16_t *>(x),
+        return launch_pdl(kernel, dim3(grid), dim3(threads), p.smem_bytes, st, p, static_cast<const uint16_t *>(x),
                           static_cast<const uint8_t *>(blob), bias, y, ws);
     };
-    const cudaError_t e = pool ? go(conv_stem_rows_kernel<true>) : go(conv_stem_rows_kernel<false>);
+    const cudaError_t e = pool ? go(conv_stem_rows_kernel<true>, kThreads<true>) : go(conv_stem_rows_kernel<false>, kThreads<false>);
     count_launch();
     return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;
 }
