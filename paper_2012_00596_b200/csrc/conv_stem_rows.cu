@@ -2,11 +2,11 @@
 // pad-1 max-pool.
 //
 // conv_stem.cu builds the im2col operand of 128 pixels in shared memory: 90 KB of traffic per tile, more time than the
-// MMAs take.  Here the operand is never built.  Input rows are stored with FOUR channels per pixel (the fourth zero), 8
+// MMAs take.  Here the operand is never built.  Input rows are stored with FOUR channels per pixel (the fourth is one), 8
 // bytes each, so that output column q (stride 2) starts 16 q bytes into a row: eight consecutive columns are one core
 // matrix of the unswizzled K-major layout, and the next two pixels of the window are the core matrix 16 bytes further on.
 // The K-direction offset of the operand descriptor is therefore 16 bytes, core matrices overlap, and a kernel row is two
-// MMAs (K = 32: eight pixels x four channels, the eighth pixel and the fourth channel meet zero weights) straight from the
+// MMAs (K = 32: eight pixels x four channels, the eighth pixel meets zero weights, the fourth channel the bias) straight from the
 // rows.  Widening a row costs one 16-byte store per two pixels, once per row instead of once per window.
 //
 // Shared memory is what bounds it (an MMA of K filters reads 4 KB of rows and 32 K bytes of weights, three times what its
@@ -17,12 +17,15 @@
 // A CTA walks consecutive steps; a step is two output rows (2p, 2p + 1) of an image, i.e. one pooled row.
 //   warps 0-3   input rows -> ring of widened rows (four new rows per step; loads run a step ahead)
 //   warp 4      MMAs: nine input rows x two, rows outside the image are zeros, into one of two TMEM sets
-//   warps 5-12  epilogue: bias, ReLU, one rounding; pooled: after the maximum with the row above (kept in registers from
+//   warps 5-12  epilogue: ReLU, one rounding; pooled: after the maximum with the row above (kept in registers from
 //               the step before: all of it is monotone, so one rounding serves the three rows), into one of two stages
 //   warps 13-15 (pooled) three staged columns to one, 16-byte stores along the row.  Warps of their own: these loads queue
 //               behind the operand reads of the MMAs, and the accumulators waited for them (1.8 k of 3.6 k clocks a step).
-// 64 x 224 x 224, K = 64, pooled: 49.3 us (63 with separate operand reads and pooling by the epilogue's warps).
+// 64 x 224 x 224, K = 64, pooled: 39.6 us (63 with separate operand reads, the bias from shared memory and pooling by the
+// epilogue's warps).
 // Every pooled value is written once: no reductions in memory and nothing to clear first.  Every wait is bounded.
+#include <type_traits>
+
 #include "common.cuh"
 #include "tc_common.cuh"
 
@@ -38,6 +41,7 @@ template <bool kPool> constexpr int kThreads = (kFirstPool + (kPool ? kPoolWarps
 constexpr int kR = 7, kC = 3;
 constexpr int kSlots = 24;                         // rows of the ring: a window of nine, and up to nine of the next step
 constexpr int kWindow = 9;                         // input rows under a step
+constexpr uint32_t kOne = 0x3F800000u;              // bf16 one as the second of a pair
 constexpr uint32_t kSmemLimit = 232448;
 constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);   // SBO = 128 bytes, descriptor version bit
 
@@ -45,7 +49,7 @@ struct StemRowsParams {
     int N, H, W, K, P, Q, Mb, relu, y_bf16;
     int PP, PQ, pairs, n_steps;                    // pooled height / width; pixel pairs of a row; steps in all (images x row pairs)
     int spi;                                       // steps per image
-    uint32_t pitch, line, off_b, off_stage, stage_bytes, off_bias, off_bar, smem_bytes, tmem_cols;
+    uint32_t pitch, line, off_b, off_stage, stage_bytes, off_bar, smem_bytes, tmem_cols;
 };
 
 struct StemRowsBars {
@@ -94,7 +98,6 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *ring = smem;                             // [kSlots] rows of `pitch` bytes: pixel x at 8 (x + 3)
     uint8_t *bsm = smem + p.off_b;                    // [parity of the kernel row][4 octets][4 K: (6 | 5 - r) / 2, filter][8] bf16
-    float *bias_s = reinterpret_cast<float *>(smem + p.off_bias);
     StemRowsBars *bars = reinterpret_cast<StemRowsBars *>(smem + p.off_bar);
     volatile uint32_t *abort_flag = &bars->abort_flag;
 
@@ -122,22 +125,54 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
         const uint32_t *blk_off = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_BLK]);
         const uint32_t *pairs = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_PAIRS]);
         const uint16_t *values = reinterpret_cast<const uint16_t *>(blob + hdr[BP_OFF_VALUES]);
-        const int per_pair = p.Mb * kC;
-        for (int fb = 0; fb < p.K / p.Mb; ++fb) {
-            const uint32_t j0 = blk_off[fb], n = (blk_off[fb + 1] - j0) * per_pair;       // one channel block per filter block
-#pragma unroll 4
-            for (uint32_t e = tid; e < n; e += kThreads<kPool>) {
-                const uint32_t j = j0 + e / per_pair, rem = e % per_pair, f = rem / kC, c = rem - f * kC;
-                const uint32_t tap = pairs[j] >> 16, r = tap / kR, sx = tap - r * kR;
-                const uint16_t v = values[(size_t)j * per_pair + rem];
-                const uint32_t kk = sx * 4 + c;
-                if (r < (uint32_t)kR)                                                        // (not a 7x7 tap: ignored)
-                    *reinterpret_cast<uint16_t *>(bsm + ((((size_t)(r & 1) * 4 + (kk >> 3)) * 4 + ((6 - r) >> 1)) * p.K + fb * p.Mb + f) * 16 + (kk & 7) * 2) = v;
+        const uint32_t per_pair = p.Mb * kC, nfb = p.K / p.Mb;
+        auto put = [&](uint32_t tap, uint32_t n, uint32_t c, uint16_t v) {
+            const uint32_t r = tap / kR, kk = (tap - r * kR) * 4 + c;
+            if (r < (uint32_t)kR)                                                            // (not a 7x7 tap: ignored)
+                *reinterpret_cast<uint16_t *>(bsm + ((((r & 1) * 4 + (kk >> 3)) * 4 + ((6 - r) >> 1)) * p.K + n) * 16 + (kk & 7) * 2) = v;
+        };
+        if (per_pair % 8 == 0) {
+            // eight weights of a pair per thread: one load, no division per weight
+            const uint32_t upp = per_pair / 8, n_units = blk_off[nfb] * upp;
+            for (uint32_t e = tid; e < n_units; e += kThreads<kPool>) {
+                const uint32_t j = e / upp, rem = (e - j * upp) * 8, tap = pairs[j] >> 16;
+                const uint4 q = *reinterpret_cast<const uint4 *>(values + (size_t)j * per_pair + rem);
+                uint32_t fb = 0;
+                while (fb + 1 < nfb && blk_off[fb + 1] <= j) ++fb;                           // one channel block per filter block
+                const uint32_t v[4] = {q.x, q.y, q.z, q.w};
+                uint32_t f = rem / kC, c = rem - f * kC;
+                f += fb * p.Mb;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    put(tap, f, c, (uint16_t)(v[k >> 1] >> (16 * (k & 1))));
+                    if (++c == (uint32_t)kC) { c = 0; ++f; }
+                }
+            }
+        } else {
+            for (uint32_t fb = 0; fb < nfb; ++fb) {
+                const uint32_t j0 = blk_off[fb], n = (blk_off[fb + 1] - j0) * per_pair;
+                for (uint32_t e = tid; e < n; e += kThreads<kPool>) {
+                    const uint32_t j = j0 + e / per_pair, rem = e % per_pair, f = rem / kC;
+                    put(pairs[j] >> 16, fb * p.Mb + f, rem - f * kC, values[(size_t)j * per_pair + rem]);
+                }
             }
         }
     }
     pdl_wait();
-    for (int i = tid; i < p.K; i += kThreads<kPool>) bias_s[i] = bias ? bias[i] : 0.f;
+    // bias: the fourth channel of every pixel is one, and a window's pixels 2 .. 4 of kernel row 3 (never outside the image)
+    // weigh it with the bias' upper, middle and lower eight bits, so that the sum is exact
+    for (int f = tid; bias && f < p.K; f += kThreads<kPool>) {
+        const float v = bias[f];
+        const bool finite = fabsf(v) <= 3.0e38f;
+        const uint32_t hi16 = finite ? __float_as_uint(v) >> 16 : cvt_bf16x2(v, 0.f) & 0xFFFFu;
+        const float rest = finite ? v - __uint_as_float(hi16 << 16) : 0.f;
+        const uint32_t mid16 = __float_as_uint(rest) >> 16, lo16 = __float_as_uint(rest - __uint_as_float(mid16 << 16)) >> 16;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t kk = 4 * (2 + k) + 3;
+            *reinterpret_cast<uint16_t *>(bsm + (((4 + (kk >> 3)) * 4 + 1) * p.K + f) * 16 + (kk & 7) * 2) = (uint16_t)(k == 0 ? hi16 : k == 1 ? mid16 : lo16);
+        }
+    }
     fence_proxy_async_smem();
     tc_fence_before_sync();
     __syncthreads();
@@ -172,7 +207,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                 uint32_t slot = base + (uint32_t)(w + tid);
                 if (slot >= (uint32_t)kSlots) slot -= kSlots;
                 *reinterpret_cast<uint4 *>(ring + slot * p.pitch + (uint32_t)(p.Q + 1) * 16u) =
-                    make_uint4(__funnelshift_r(last.x, last.y, 16), last.y >> 16, 0u, 0u);
+                    make_uint4(__funnelshift_r(last.x, last.y, 16), (last.y >> 16) | kOne, 0u, kOne);
             }
             if (!on) return;
 #pragma unroll
@@ -184,7 +219,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                 const uint32_t e01 = __funnelshift_r(a[q][0], a[q][1], 16), e23 = __funnelshift_r(a[q][1], a[q][2], 16),
                                e45 = __funnelshift_r(a[q][2], a[q][3], 16);
                 *reinterpret_cast<uint4 *>(ring + slot * p.pitch + (uint32_t)u * 16u) =
-                    make_uint4(e01, e23 & 0xFFFFu, (e23 >> 16) | (e45 << 16), e45 >> 16);
+                    make_uint4(e01, (e23 & 0xFFFFu) | kOne, (e23 >> 16) | (e45 << 16), (e45 >> 16) | kOne);
             }
         };
         Steps st(lo, hi, p.spi, kPool);
@@ -280,26 +315,19 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                 tmem_ld_x16(t_addr + ch * 16, r0);
                 tmem_ld_x16(t_addr + p.K + ch * 16, r1);
                 tmem_ld_wait();
-                const float4 *b4 = reinterpret_cast<const float4 *>(bias_s + ch * 16);
-                float bv[16];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float4 v = b4[k];
-                    bv[4 * k] = v.x; bv[4 * k + 1] = v.y; bv[4 * k + 2] = v.z; bv[4 * k + 3] = v.w;
-                }
                 if constexpr (kPool) {
                     // rows 2p - 1, 2p, 2p + 1 (the last one may not exist)
                     const bool has1 = 2 * st.p + 1 < p.P;
+                    float v[16];
                     uint32_t m[8];
 #pragma unroll
                     for (int k = 0; k < 16; ++k) {
-                        float v = fmaxf(saved[c][k], __uint_as_float(r0[k]));
-                        if (has1) v = fmaxf(v, __uint_as_float(r1[k]));
+                        v[k] = fmaxf(saved[c][k], __uint_as_float(r0[k]));
+                        if (has1) v[k] = fmaxf(v[k], __uint_as_float(r1[k]));
                         saved[c][k] = __uint_as_float(r1[k]);
-                        bv[k] += v;
                     }
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) m[k] = relu_bf16x2(cvt_bf16x2(bv[2 * k], bv[2 * k + 1]));
+                    for (int k = 0; k < 8; ++k) m[k] = relu_bf16x2(cvt_bf16x2(v[2 * k], v[2 * k + 1]));
                     // one line of 2 K bytes per column, 16-byte units XOR-ed with the column (conflict free)
                     uint8_t *line = stage + (size_t)q * p.line;
                     const uint32_t x7 = (uint32_t)(q & 7);
@@ -317,7 +345,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                             uint32_t o2[8];
 #pragma unroll
                             for (int k = 0; k < 8; ++k) {
-                                o2[k] = cvt_bf16x2(__uint_as_float(v[2 * k]) + bv[2 * k], __uint_as_float(v[2 * k + 1]) + bv[2 * k + 1]);
+                                o2[k] = cvt_bf16x2(__uint_as_float(v[2 * k]), __uint_as_float(v[2 * k + 1]));
                                 if (p.relu) o2[k] = relu_bf16x2(o2[k]);
                             }
                             yp[0] = make_uint4(o2[0], o2[1], o2[2], o2[3]);
@@ -330,7 +358,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                                 float f[4];
 #pragma unroll
                                 for (int k = 0; k < 4; ++k) {
-                                    f[k] = __uint_as_float(v[4 * h + k]) + bv[4 * h + k];
+                                    f[k] = __uint_as_float(v[4 * h + k]);
                                     if (p.relu) f[k] = fmaxf(f[k], 0.f);
                                 }
                                 yp[h] = make_float4(f[0], f[1], f[2], f[3]);
@@ -357,19 +385,34 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
             const uint32_t b = i & 1u;
             const bool ok = mbar_wait(&bars->stage_full[b], (i >> 1) & 1u, abort_flag, ws, 0xB500);
             if (!__all_sync(0xFFFFFFFFu, ok)) break;
-            if (on && st.store) {
-                const uint8_t *stage = smem + p.off_stage + (size_t)b * p.stage_bytes;
-                uint16_t *out = static_cast<uint16_t *>(y) + ((size_t)st.n * p.PP + st.p) * p.PQ * p.K + u * 8;
-                auto at = [&](int col) { return *reinterpret_cast<const uint4 *>(stage + (size_t)col * p.line + (((uint32_t)u ^ (uint32_t)(col & 7)) << 4)); };
-#pragma unroll 4
-                for (int v = v0; v < p.PQ; v += vs) {
-                    const int c0 = 2 * v;
-                    const uint4 m = max4(at(c0), max4(at(c0 > 0 ? c0 - 1 : c0), at(c0 + 1 < p.Q ? c0 + 1 : c0)));
-                    *reinterpret_cast<uint4 *>(out + (size_t)v * p.K) = m;
+            const uint8_t *stage = smem + p.off_stage + (size_t)b * p.stage_bytes;
+            uint16_t *out = static_cast<uint16_t *>(y) + ((size_t)st.n * p.PP + st.p) * p.PQ * p.K + u * 8;
+            auto at = [&](int col) { return *reinterpret_cast<const uint4 *>(stage + (size_t)col * p.line + (((uint32_t)u ^ (uint32_t)(col & 7)) << 4)); };
+            const int v_end = on && st.store ? p.PQ : 0;
+            // loads of a batch are in flight together and not branched around (a row of 56 columns, 64 filters: five at a time
+            // 39.6 us for 64 images, three 44.5, one after the other 46; 32 columns fit three: 22.1 against 26.2)
+            auto batches = [&](auto size) {
+                constexpr int kBatch = decltype(size)::value;
+                for (int vb = 0; vb < p.PQ; vb += kBatch * vs) {
+                    uint4 m[kBatch];
+#pragma unroll
+                    for (int k = 0; k < kBatch; ++k) {
+                        const int c0 = 2 * min(vb + v0 + k * vs, p.PQ - 1);
+                        m[k] = max4(at(c0), max4(at(c0 > 0 ? c0 - 1 : c0), at(c0 + 1 < p.Q ? c0 + 1 : c0)));
+                    }
+                    if (vb + kBatch * vs >= p.PQ) {      // all read: the stage is free before the row is on its way
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&bars->stage_empty[b]);
+                    }
+#pragma unroll
+                    for (int k = 0; k < kBatch; ++k) {
+                        const int v = vb + v0 + k * vs;
+                        if (v < v_end) *reinterpret_cast<uint4 *>(out + (size_t)v * p.K) = m[k];
+                    }
                 }
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bars->stage_empty[b]);
+            };
+            if (p.PQ <= 3 * vs) batches(std::integral_constant<int, 3>{});
+            else batches(std::integral_constant<int, 5>{});
             ++i;
         }
     }
@@ -402,8 +445,7 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, StemRowsParams &p, bo
     p.off_b = kSlots * p.pitch + 1024u;                        // (an operand reads 128 columns, past the end of the last row)
     p.off_stage = round_up(p.off_b + 2u * 4u * 4u * d.K * 16u, 128);
     p.stage_bytes = 128u * p.line;
-    p.off_bias = p.off_stage + (pool ? 2u * p.stage_bytes : 0u);
-    p.off_bar = round_up(p.off_bias + d.K * 4u, 128);
+    p.off_bar = p.off_stage + (pool ? 2u * p.stage_bytes : 0u);
     p.smem_bytes = p.off_bar + (uint32_t)sizeof(StemRowsBars) + 1024u;
     if (p.smem_bytes > kSmemLimit) return false;
     p.tmem_cols = 32;
