@@ -73,7 +73,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *m, const void *s
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
@@ -112,7 +111,8 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     if (warp == 1) tmem_alloc_pair(&bars->tmem_base, p.tmem_cols);     // both CTAs
     pdl_trigger();
     tc_fence_before_sync();
-    cluster_sync_all();                 // barriers of both CTAs exist before anything arrives on them
+    __syncthreads();
+    cluster_sync_relaxed();             // barriers of both CTAs exist before anything arrives on them
     tc_fence_after_sync();
     // The weights of the first ring of stages are requested before the wait for the kernel before this one: no kernel that
     // lets its successor start early writes them.
@@ -168,7 +168,8 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             // the leader needs the accumulator only a tile later)
             const uint32_t acc_empty0 = map_to_cta(smem_u32(&bars->acc_empty[0]), 0u);
             uint32_t it = 0;
-            for (int tile = pair; tile < p.n_tiles; tile += n_pairs, ++it) {
+            // (only where the leader waits for it, two tiles on: an arrival nobody waits for could outlive the leader)
+            for (int tile = pair; tile + 2 * n_pairs < p.n_tiles; tile += n_pairs, ++it) {
                 const uint32_t acc = it & 1u;
                 if (!mbar_wait(&bars->acc_done[acc], (it >> 1) & 1u, abort_flag, ws, 0x8700)) break;
                 tc_fence_after_sync();
@@ -237,7 +238,7 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     if (++slot == (uint32_t)p.NS) { slot = 0; ph ^= 1u; }
                 }
             }
-            bulk_wait_all();                            // the slots stay valid until the last store has read them
+            bulk_wait_read<0>();                        // the slots stay valid until the last store has read them
         }
     } else if (p.NS) {
         // ---- epilogue through shared memory: warp -> TMEM lane quarter (warp % 4) and the 16 columns
@@ -402,7 +403,7 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         const long long t0 = clock64();
         while (clock64() - t0 < 400000ll) { }
     }
-    cluster_sync_all();                 // neither CTA retires (or frees TMEM) while the other may still use it
+    cluster_sync_relaxed();             // neither CTA retires (or frees TMEM) while the other may still use it
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc_pair(tmem_base, p.tmem_cols);
@@ -421,8 +422,8 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinD2Params &p)
     // Column tile BN: the widest divisor of O that leaves room for enough stages (three once the K loop has
     // three or more steps), else the widest with two (measured: narrower tiles never won, the kernel is
     // bound by what the SMs take in from L2, and wide tiles take in the least per MAC).  Epilogue slots
-    // (bf16 output, BN % 64 == 0, and the output side at least as large as the input side): three when
-    // only stores pass through them, six when the residual is prefetched into them.
+    // (bf16 output, BN % 64 == 0): three when only stores pass through them, six when the residual is prefetched
+    // into them.
     // (the call descriptor's `variant` restricts the choice to one width)
     const int want = p.nK >= 3 ? 3 : 2;
     const int want_bn = d.variant;
@@ -432,7 +433,7 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinD2Params &p)
             if (d.O % bn || (want_bn && bn != want_bn)) continue;
             // with so few tiles that half of the pairs would idle, the narrower tile doubles their number
             if (bn == 256 && !want_bn && (long long)((p.nMT + 1) / 2) * (d.O / 256) <= 37) continue;
-            const int ns = (p.y_bf16 && bn % 64 == 0 && (d.has_residual || d.O >= d.I)) ? (d.has_residual ? kMaxSlots : 3) : 0;
+            const int ns = p.y_bf16 && bn % 64 == 0 ? (d.has_residual ? kMaxSlots : 3) : 0;
             const uint32_t stage = round_up(kXBytes + (uint32_t)(bn / 2) * 128u, 1024);   // multiples of 1024: swizzled tiles stay aligned
             const uint32_t need = fixed + (uint32_t)ns * kSlotBytes;
             if (need + 2 * stage > kSmemLimit) continue;

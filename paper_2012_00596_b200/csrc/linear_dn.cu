@@ -77,7 +77,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *m, const void *s
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 __global__ void __launch_bounds__(kThreads, 1)
 linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
@@ -93,35 +92,42 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+    // The producer starts by itself: it initialises the barriers it signals and requests the first ring of stages before the
+    // other warps have set up theirs and tensor memory (0.4 us).  The weights do not wait for the kernel before this one: no
+    // kernel that lets its successor start early writes them.
+    int early = 0;
     if (tid == 0) {
         for (int s = 0; s < p.S; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&bars->acc_full[a], 1); mbar_init(&bars->acc_empty[a], kEpiWarps); }
-        for (int s = 0; s < p.NS; ++s) {
-            mbar_init(&bars->res_full[s], 1); mbar_init(&bars->res_empty[s], 1); mbar_init(&bars->slot_done[s], kEpiWarps);
-        }
-        bars->abort_flag = 0;
         fence_barrier_init();
-        prefetch_tensormap(&tmap_x);
-        prefetch_tensormap(&tmap_w);
-        if (p.NS) { prefetch_tensormap(&tmap_y); if (res) prefetch_tensormap(&tmap_r); }
-    }
-    if (warp == 1) tmem_alloc(&bars->tmem_base, p.tmem_cols);
-    pdl_trigger();
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    // The weights of the first ring of stages are requested before the wait for the kernel before this one: no kernel that
-    // lets its successor start early writes them.
-    int early = 0;
-    if (warp == 0 && lane == 0) {
+        fence_proxy_async_smem();
         int tile = blockIdx.x, k = 0;
         for (; early < p.S && tile < p.n_tiles; ++early) {
             mbar_arrive_expect_tx(&bars->full[early], p.stage_bytes);
             tma_load_2d(smem + (size_t)early * p.stage_bytes + kXBytes, &tmap_w, &bars->full[early], k * 64, (tile % p.nNT) * p.BN);
             if (++k == p.nK) { k = 0; tile += gridDim.x; }
         }
+        pdl_wait();
+        tile = blockIdx.x; k = 0;
+        for (int e = 0; e < early; ++e) {
+            tma_load_2d(smem + (size_t)e * p.stage_bytes, &tmap_x, &bars->full[e], k * 64, (tile / p.nNT) * kRows);
+            if (++k == p.nK) { k = 0; tile += gridDim.x; }
+        }
+    } else if (tid == kFirstEpiWarp * 32) {
+        for (int a = 0; a < 2; ++a) { mbar_init(&bars->acc_full[a], 1); mbar_init(&bars->acc_empty[a], kEpiWarps); }
+        for (int s = 0; s < p.NS; ++s) {
+            mbar_init(&bars->res_full[s], 1); mbar_init(&bars->res_empty[s], 1); mbar_init(&bars->slot_done[s], kEpiWarps);
+        }
+        bars->abort_flag = 0;
+        fence_barrier_init();
+        if (p.NS) { prefetch_tensormap(&tmap_y); if (res) prefetch_tensormap(&tmap_r); }
     }
-    pdl_wait();                        // nothing else above touches global memory
+    __syncwarp();
+    if (warp == 1) tmem_alloc(&bars->tmem_base, p.tmem_cols);
+    pdl_trigger();
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    pdl_wait();                        // nothing above but the producer's copies touches global memory
     // the biases: staged by the epilogue warps, which meet again before the first use
     if (warp >= kFirstEpiWarp && warp < kResWarp) {
         for (int i = tid - kFirstEpiWarp * 32; i < p.nNT * p.BN; i += kEpiWarps * 32) bias_s[i] = (bias && i < p.O) ? bias[i] : 0.f;
@@ -141,9 +147,11 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 for (int k = 0; k < p.nK; ++k) {
                     if (lap >= 1 && !mbar_wait(&bars->empty[s], (lap & 1u) ^ 1u, abort_flag, ws, 0x5100)) { ok = false; break; }
                     uint8_t *st = smem + (size_t)s * p.stage_bytes;
-                    if (early <= 0) mbar_arrive_expect_tx(&bars->full[s], p.stage_bytes);
-                    tma_load_2d(st, &tmap_x, &bars->full[s], k * 64, mt * kRows);
-                    if (early-- <= 0) tma_load_2d(st + kXBytes, &tmap_w, &bars->full[s], k * 64, nt * p.BN);
+                    if (early-- <= 0) {                          // (the first ring is already on its way)
+                        mbar_arrive_expect_tx(&bars->full[s], p.stage_bytes);
+                        tma_load_2d(st, &tmap_x, &bars->full[s], k * 64, mt * kRows);
+                        tma_load_2d(st + kXBytes, &tmap_w, &bars->full[s], k * 64, nt * p.BN);
+                    }
                     if (++s == (uint32_t)p.S) { s = 0; ++lap; }
                 }
             }
@@ -211,7 +219,7 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     if (++slot == (uint32_t)p.NS) { slot = 0; ph ^= 1u; }
                 }
             }
-            bulk_wait_all();                            // the slots stay valid until the last store has read them
+            bulk_wait_read<0>();                        // the slots stay valid until the last store has read them
         }
     } else if (p.NS) {
         // ---- epilogue through shared memory: warp -> TMEM lane quarter (warp % 4) and the 16 columns
@@ -399,8 +407,8 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinDnParams &p)
     // Column tile BN: the widest divisor of O that leaves room for enough stages (three once the K loop has
     // three or more steps), else the widest with two (measured: narrower tiles never won, the kernel is
     // bound by what the SMs take in from L2, and wide tiles take in the least per MAC).  Epilogue slots
-    // (bf16 output, BN % 64 == 0, and the output side at least as large as the input side): three when
-    // only stores pass through them, six when the residual is prefetched into them.
+    // (bf16 output, BN % 64 == 0): three when only stores pass through them, six when the residual is prefetched
+    // into them.
     // (the call descriptor's `variant` restricts the choice to one width)
     const int want = p.nK >= 3 ? 3 : 2;
     const int want_bn = d.variant;
@@ -410,7 +418,7 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinDnParams &p)
             if (want_bn && bn != want_bn) continue;
             // (an output width that 16 does not divide: tiles of 128, the last one cut short by the tensor map and the store)
             if (d.O % 16 ? (!want_bn && bn != 128) : (d.O % bn != 0)) continue;
-            const int ns = (p.y_bf16 && bn % 64 == 0 && (d.has_residual || d.O >= d.I)) ? (d.has_residual ? kMaxSlots : 3) : 0;
+            const int ns = p.y_bf16 && bn % 64 == 0 ? (d.has_residual ? kMaxSlots : 3) : 0;
             const uint32_t stage = round_up(kXBytes + (uint32_t)bn * 128u, 1024);   // multiples of 1024: swizzled tiles stay aligned
             const uint32_t need = fixed + (uint32_t)ns * kSlotBytes;
             if (need + 2 * stage > kSmemLimit) continue;
