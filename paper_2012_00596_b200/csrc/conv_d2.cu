@@ -122,6 +122,9 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     const uint32_t rank = cluster_ctarank();                  // 0: leader (issues the MMAs), 1: its peer
     const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
+    // (the header's words on their way while the barriers are set up: the blob is never written by a kernel that lets its
+    // successor start early)
+    const uint32_t off_tapu = hdr[BP_OFF_TAPU], off_image = hdr[BP_OFF_IMAGE], image_gi = hdr[BP_GI];
     const uint32_t peer_abort = map_to_cta(smem_u32(&bars->abort_flag), rank ^ 1u);
 
     if (tid == 0) {
@@ -143,17 +146,16 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     if (warp == 1) tmem_alloc_pair(&bars->tmem_base, p.tmem_cols);      // both CTAs; warp 1 also frees it
     pdl_trigger();
     tc_fence_before_sync();
-    cluster_sync_all();                 // barriers of both CTAs exist before anything arrives on them
+    __syncthreads();
+    cluster_sync_relaxed();             // barriers of both CTAs exist before anything arrives on them
     tc_fence_after_sync();
-    // Nothing above touches global memory.  The weight producer does not wait: it reads the blob only, which no kernel that
-    // lets its successor start early writes, so the first ring of weights is on its way while the kernel before this one ends.
-    if (warp != 2) pdl_wait();
+    // Only the activations, the biases and the residual may come from the kernel before this one: the weight producer and the
+    // tap unions do not wait for its end.
     const uint32_t tmem_base = bars->tmem_base;
-    // the two producers start at once; the other warps first stage the biases and the tap unions
+    if (warp == 0) pdl_wait();
+    // the two producers start at once; the other warps first stage the tap unions
     if (warp != 0 && warp != 2) {
         const int t = tid < 64 ? tid - 32 : tid - 64;         // 0 .. kThreads - 65 over warps 1, 3, 4, ...
-        for (int i = t; i < p.K; i += kThreads - 64) bias_s[i] = bias ? bias[i] : 0.f;
-        const uint32_t off_tapu = hdr[BP_OFF_TAPU];
         const uint32_t *tapu = reinterpret_cast<const uint32_t *>(blob + off_tapu);
         for (int i = t; i < (p.K / p.GI) * p.nCh; i += kThreads - 64) tapu_s[i] = off_tapu ? tapu[i] : 0xFFFFFFFFu;
         if (p.IT > 1 && p.act_stride > p.slab_bytes) {
@@ -168,6 +170,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             fence_proxy_async_smem();
         }
         consumers_sync();
+        pdl_wait();
     }
 
     if (warp == 0) {
@@ -208,11 +211,10 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         }
     } else if (warp == 2) {
         // ---- weight producer: this CTA's half of the weight tile of every 16-channel chunk ----------------
-        const uint32_t off_image = hdr[BP_OFF_IMAGE];
         bool ok = true;
         // the blob must carry the operand image in the groups the plan assumed; if not, nothing is requested
         // and the other roles leave their waits through the abort flag
-        if (off_image == 0u || (off_image & 2047u) || hdr[BP_GI] != (uint32_t)p.GI) {
+        if (off_image == 0u || (off_image & 2047u) || image_gi != (uint32_t)p.GI) {
             if (lane == 0) {
                 bars->abort_flag = 2;
                 st_remote_u32(peer_abort, 2u);
@@ -319,6 +321,8 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         }
     } else {
         // ---- epilogue: warp -> TMEM lane quarter (warp % 4) and every kParts-th 16-column chunk -----------
+        for (int i = tid - kFirstEpiWarp * 32; i < p.K; i += kEpiWarps * 32) bias_s[i] = bias ? bias[i] : 0.f;
+        asm volatile("bar.sync 2, %0;" ::"n"(kEpiWarps * 32) : "memory");
         const int quarter = warp & 3, part = (warp - kFirstEpiWarp) >> 2, m = quarter * 32 + lane;
         const int il = p.IT > 1 ? m / p.img_pitch : 0, mr = m - il * p.img_pitch;    // image of the tile, position inside it
         const int oy = mr / p.Wp, ox = mr - oy * p.Wp;
@@ -423,8 +427,8 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(rank == 0 ? &bars->acc_empty[acc] : &bars->acc_done[acc]);
-            if (rank == 1 && warp == kFirstEpiWarp && lane == 0) {
-                // peer: once all its epilogue warps have read the accumulator, ONE arrival on the leader's barrier
+            if (rank == 1 && warp == kFirstEpiWarp && lane == 0 && item + p.nacc * n_pairs < p.n_items) {
+                // peer, where the leader will wait for it (an arrival nobody waits for could outlive the leader): once all its epilogue warps have read the accumulator, ONE arrival on the leader's barrier
                 // with release semantics at cluster scope (the leader needs the accumulator an item later)
                 if (!mbar_wait(&bars->acc_done[acc], lap_acc & 1u, abort_flag, ws, 0x7520)) { ok = false; }
                 else {
@@ -443,7 +447,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         const long long t0 = clock64();
         while (clock64() - t0 < 400000ll) { }
     }
-    cluster_sync_all();                 // neither CTA retires (or frees TMEM) while the other may still use it
+    cluster_sync_relaxed();             // neither CTA retires (or frees TMEM) while the other may still use it
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc_pair(tmem_base, p.tmem_cols);
