@@ -2,8 +2,8 @@
 // pairs (paper Sec. 3: inside a block the kept kernel positions are shared by all kernels, so a kept
 // pair is a dense [Mb filters x Nb channels] sub-contraction).  bf16 in, fp32 accumulation in TMEM.
 //
-// Mapping.  A CTA owns up to 128 consecutive "padded-linear" output positions of one image (M of
-// the MMA) and one group of GS filter blocks (<= 256 filters = 256 fp32 accumulator columns).  For a
+// Mapping.  A CTA owns 128 consecutive output positions (M of the MMA), counted through rows and images without gaps
+// because the stagers below read the slab by position and any position may lie anywhere in it, and one group of GS filter blocks (<= 256 filters = 256 fp32 accumulator columns).  For a
 // 16-channel chunk and a tap, the activation operand (128 positions x 16 channels, shifted by the
 // tap) is the same for every filter block that keeps the tap.  Measured on B200, what an MMA with
 // a small N costs is the fetch of that operand, not the math: about 39 cycles from shared memory
@@ -19,8 +19,8 @@
 // MMAs from one thread in program order (bitwise reproducible sums).
 //
 // Pipeline (18 warps, persistent CTA over the tiles of its filter group):
-//   warp 0      activation slabs by TMA, [channel octet][padded position][8 channels], zero fill
-//               outside the image = padding; a tap shift is an address offset of whole positions
+//   warp 0      activation slabs by TMA, one copy per input row under the tile: [row][channel octet][padded column][8
+//               channels], zero fill outside the image = padding; a tap shift is an address offset of rows and columns
 //   warp 1      the chunk's tiles of the group: ONE bulk copy per chunk into a ring of weight slots
 //   warps 2-9   stagers: slab -> registers -> TMEM staging buffer (ring of 2 or 3), one warp per
 //               TMEM lane quarter, two sets of four warps taking alternate chunks
@@ -32,7 +32,14 @@
 // blob's index sections, while the producers already run).  Per chunk an issuing warp fetches its
 // records, waits for the staging buffer and the weight slot, issues, and commits once: that commit
 // frees both the staging buffer and the weight slot.
+// What a CTA works on: whole tiles while there is one for every CTA; a last round that would leave half of them idle is
+// split by filters, each part issued by a share of the issuing warps.  64x28x28x512 -> 512, blocks of 16 x 16, three taps
+// of nine: 131 us (147 with tiles of whole rows of one image, an eighth of the lanes on padding and seven rounds of items).
+// What is left: a chunk takes 940 cycles, 40 MMAs of 24; shared memory is busy for 710 of them (288 for the stagers' reads, 190
+// each for the weights' arrival and for the MMAs' reading them).
 // Every wait is bounded; a blob that breaks the descriptor's promises is reported, not computed.
+#include <numeric>
+
 #include "common.cuh"
 #include "tc_common.cuh"
 
@@ -56,10 +63,12 @@ constexpr uint32_t kDescHiB = (256u >> 4) | (1u << 14);   // B operand: 256 byte
 
 struct ConvKrParams {
     int N, H, W, C, K, R, S, pad, P, Q;
-    int Wp, TR, tiles_per_img, n_tiles, slab_rows;
+    int Wp, n_tiles;
+    int per, grp_pos, tiles_per_grp;     // positions per tile; positions and tiles of a group: all images, or one image
+    int n_pos, slots, NQ;                // output positions; rows of a slab; parts a tile of the last round is split into
     int Mb, GS, SEG, NA, RS, nGrp;
     int nChunks, cps, nStages, PPS, SA, NWS, nabuf, NP, cpb, nCB, max_taps;
-    uint32_t plane_bytes, act_stage_bytes, act_tx_bytes, wcap, bufcols, tile_bytes;
+    uint32_t oct_bytes, row_bytes, row_pitch, act_stage_bytes, wcap, bufcols, tile_bytes;
     int relu, y_bf16;
     uint32_t off_act, off_w, off_cm, off_kto, off_rec, off_bar, smem_bytes;
     int RW;                      // words per (issuing warp, chunk) record list: count + MMAs, a multiple of 4
@@ -75,13 +84,39 @@ struct Bars {
     uint32_t tmem_base;
     uint32_t abort_flag;
     uint32_t tapoff[kMaxTaps];       // byte offset of a tap's shift inside a slab plane
-    float bias[256];
+    alignas(16) float bias[256];
 };
 
 struct Ring {
     int idx, lap;
     __device__ __forceinline__ void next(int n) { if (++idx == n) { idx = 0; ++lap; } }
 };
+
+// The item number `it` of CTA x of `step` in its filter group: a tile and the issuing warps [lo, hi) that work on it.
+__device__ __forceinline__ bool get_item(const ConvKrParams &p, int it, int &tile, int &lo, int &hi)
+{
+    const int x = blockIdx.x, step = gridDim.x, full = p.NQ > 1 ? p.n_tiles / step : 0x7FFFFFFF;
+    lo = 0; hi = p.NA;
+    if (it < full) { tile = x + it * step; return tile < p.n_tiles; }
+    if (it > full || x >= (p.n_tiles - full * step) * p.NQ) return false;
+    const int q = x % p.NQ, share = p.NA / p.NQ;
+    tile = full * step + x / p.NQ;
+    lo = q * share; hi = lo + share;
+    return true;
+}
+// where a tile starts (image, row) and how many positions it has
+struct TileAt { int first, count, n, y, slots; };
+__device__ __forceinline__ TileAt tile_at(const ConvKrParams &p, int tile)
+{
+    TileAt t;
+    const int g = tile / p.tiles_per_grp, j = tile - g * p.tiles_per_grp, pq = p.P * p.Q;
+    t.first = g * p.grp_pos + j * p.per;
+    t.count = min(p.per, p.grp_pos - j * p.per);
+    t.n = t.first / pq; t.y = (t.first - t.n * pq) / p.Q;
+    const int last = t.first + t.count - 1, n1 = last / pq, y1 = (last - n1 * pq) / p.Q;
+    t.slots = (n1 - t.n) * (p.P + p.R - 1) + y1 - t.y + p.R;
+    return t;
+}
 
 // D[tmem] += A[tmem] * B[smem]
 __device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc)
@@ -116,14 +151,7 @@ __device__ __forceinline__ void tmem_st_x32(uint32_t taddr, const uint4 (&u)[8])
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void mma_warps_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kMmaWarps * 32) : "memory"); }
-// barrier among the four epilogue warps that share one half of the filter columns (ids 2 and 3)
-__device__ __forceinline__ void part_sync(int part)
-{
-    if (part == 0) asm volatile("bar.sync 2, 128;" ::: "memory");
-    else asm volatile("bar.sync 3, 128;" ::: "memory");
-}
-// the same barriers with a vote: true when `pred` holds in every thread that arrives (a group of warps then
-// enters or skips a region with barriers inside as one)
+// barrier with a vote: true when `pred` holds in every thread that arrives
 template <int kId, int kCount>
 __device__ __forceinline__ bool bar_all(bool pred)
 {
@@ -132,21 +160,19 @@ __device__ __forceinline__ bool bar_all(bool pred)
                  : "=r"(r) : "n"(kId), "n"(kCount), "r"((uint32_t)pred) : "memory");
     return r != 0u;
 }
-// [rows][padded columns][64 filters] in shared memory (128-byte swizzled) -> Y[n][y0 + row][column][k0 ..]; what lies
-// outside the tensor (the padding columns of a row, rows past the last) is not written
-__device__ __forceinline__ void tma_store_4d(const CUtensorMap *m, uint32_t src, int c0, int c1, int c2, int c3)
+// 32 positions x 64 filters in shared memory (128-byte swizzled) -> Y
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *m, uint32_t src, int c0, int c1)
 {
-    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
-                 ::"l"(reinterpret_cast<uint64_t>(m)), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
+                 ::"l"(reinterpret_cast<uint64_t>(m)), "r"(src), "r"(c0), "r"(c1) : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
-constexpr uint32_t kEpiBufBytes = 128u * 128u;          // 128 positions x 64 bf16 filters
+constexpr uint32_t kEpiBufBytes = 32u * 128u;           // a warp's 32 positions x 64 bf16 filters
 
 
 // One MMA = one run of neighbouring kept blocks inside a segment at one tap: first tile of the
@@ -157,21 +183,28 @@ __device__ __forceinline__ uint32_t make_rec(uint32_t tile, uint32_t tap, uint32
 }
 
 // Staged epilogue of one warp (bf16 output, whole 64-filter slabs): registers -> shared memory (one 128-byte line
-// per position, 16-byte units swizzled by the line number) -> one tensor store per slab and column half, which writes
-// whole lines where a thread's own stores would be 16-byte requests (measured: 2 k of the 4 k cycles of an epilogue
-// over 256 filters).  A function of its own so that its registers do not weigh on the issue loop.
+// per position, 16-byte units swizzled by the line number) -> one tensor store per slab, which writes whole lines where a
+// thread's own stores would be 16-byte requests.  A warp's buffer is its own: no barrier, and the next slab leaves tensor
+// memory while the store reads (256 filters, one tap of nine: 1.9 us, 2.6 with a buffer and two barriers per slab for four
+// warps; three taps 3.2 either way, because the next tile's operands arrive in shared memory meanwhile).  A warp whose last
+// positions lie past the tile's end stores from its registers.
 __device__ __forceinline__ void epilogue_staged(const CUtensorMap *tmap_y, uint32_t ebuf, const float *bias_s, const uint16_t *res_row,
-                                             bool relu, uint32_t t_addr, int part, bool leader, int m, int col_lo, int col_hi,
-                                             int k0, int y0, int n)
+                                             bool relu, uint32_t t_addr, int lane, int col_lo, int col_hi, int k0, int pos, int rows,
+                                             uint16_t *y_row)
 {
-    const uint32_t line = ebuf + (uint32_t)m * 128u, sw = (uint32_t)(m & 7) << 4;
+    const uint32_t line = ebuf + (uint32_t)lane * 128u, sw = (uint32_t)(lane & 7) << 4;
+    const bool whole = rows >= 32;
     auto finish16 = [&](const uint32_t *r, int c0, int u) {
         float v[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
         if (bias_s) {
+            const float4 *b4 = reinterpret_cast<const float4 *>(bias_s + c0);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] += bias_s[c0 + i];
+            for (int h = 0; h < 4; ++h) {
+                const float4 b = b4[h];
+                v[4 * h] += b.x; v[4 * h + 1] += b.y; v[4 * h + 2] += b.z; v[4 * h + 3] += b.w;
+            }
         }
         if (res_row) {
             const uint4 *rp = reinterpret_cast<const uint4 *>(res_row + c0);
@@ -194,24 +227,34 @@ __device__ __forceinline__ void epilogue_staged(const CUtensorMap *tmap_y, uint3
 #pragma unroll
             for (int i = 0; i < 8; ++i) o[i] = relu_bf16x2(o[i]);
         }
-        st_shared_v4(line + (((uint32_t)(2 * u) << 4) ^ sw), o[0], o[1], o[2], o[3]);
-        st_shared_v4(line + (((uint32_t)(2 * u + 1) << 4) ^ sw), o[4], o[5], o[6], o[7]);
+        if (whole) {
+            st_shared_v4(line + (((uint32_t)(2 * u) << 4) ^ sw), o[0], o[1], o[2], o[3]);
+            st_shared_v4(line + (((uint32_t)(2 * u + 1) << 4) ^ sw), o[4], o[5], o[6], o[7]);
+        } else if (lane < rows) {
+            uint4 *yp = reinterpret_cast<uint4 *>(y_row + c0);
+            yp[0] = make_uint4(o[0], o[1], o[2], o[3]);
+            yp[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        }
     };
     uint32_t ra[32];
-    for (int c0 = col_lo; c0 < col_hi; c0 += 64) {
-        if (leader) bulk_wait_read_all();            // the slab before this one has left the buffer
-        part_sync(part);
+    for (int c0 = col_lo; c0 < col_hi; c0 += 64 * (kMmaWarps / 4)) {
 #pragma unroll 1
         for (int u = 0; u < 2; ++u) {
             __syncwarp();
             tmem_ld_x32(t_addr + c0 + 32 * u, ra);
+            if (u == 0) {
+                if (lane == 0) bulk_wait_read_all();     // the slab before this one has left the buffer
+                __syncwarp();
+            }
             tmem_ld_wait();
             finish16(ra, c0 + 32 * u, 2 * u);
             finish16(ra + 16, c0 + 32 * u + 16, 2 * u + 1);
         }
-        fence_proxy_async_smem();
-        part_sync(part);
-        if (leader) { tma_store_4d(tmap_y, ebuf, k0 + c0, 0, y0, n); bulk_commit(); }
+        if (whole) {
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) { tma_store_2d(tmap_y, ebuf, k0 + c0, pos); bulk_commit(); }
+        }
     }
 }
 
@@ -232,7 +275,6 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int grp = blockIdx.y, fb0 = grp * p.GS;
-    const int tile0 = blockIdx.x, tile_step = gridDim.x;
 
     const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
 
@@ -250,10 +292,9 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     if (warp == 1) tmem_alloc(&bars->tmem_base, 512);
     for (int i = tid; i < p.nChunks * 16; i += kThreads) colmask[i] = 0u;
     pdl_trigger();
-    pdl_wait();                          // nothing above touches global memory
-    for (int i = tid; i < p.GS * p.Mb; i += kThreads) bars->bias[i] = bias ? bias[fb0 * p.Mb + i] : 0.f;
-    if (tid < kMaxTaps) bars->tapoff[tid] = tid < p.RS ? (uint32_t)((tid / p.S) * p.Wp + (tid % p.S)) * 16u : 0u;
+    if (tid < kMaxTaps) bars->tapoff[tid] = tid < p.RS ? (uint32_t)(tid / p.S) * p.row_pitch + (uint32_t)(tid % p.S) * 16u : 0u;
     __syncthreads();
+    // (the blob is never written by a kernel that lets its successor start early: no need to wait for the kernel before)
     // the blob must be what the descriptor says: version, the tile section and its grouping
     const bool hdr_ok = hdr[BP_MAGIC] == kMagicBP && hdr[BP_VERSION] == kVersion && hdr[BP_OFF_KT] != 0u &&
                         hdr[BP_GS] == (uint32_t)p.GS && hdr[BP_MB] == (uint32_t)p.Mb && hdr[BP_NCB] == (uint32_t)p.nCB;
@@ -285,6 +326,8 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             if (b < a || b - a > (uint32_t)(p.GS * p.max_taps)) bars->abort_flag = 2;   // would overflow a weight slot
         }
     }
+    pdl_wait();
+    for (int i = tid; i < p.GS * p.Mb; i += kThreads) bars->bias[i] = bias ? bias[fb0 * p.Mb + i] : 0.f;
     fence_proxy_async_smem();
     tc_fence_before_sync();
     __syncthreads();
@@ -297,16 +340,22 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         // nothing is copied or computed
     } else if (warp == 0) {
         // ---- activation producer ------------------------------------------------------------------
-        if (lane == 0) {
-            Ring ring{0, 0};
-            bool ok = true;
-            for (int tile = tile0; tile < p.n_tiles && ok; tile += tile_step) {
-                const int n = tile / p.tiles_per_img, y0 = (tile - n * p.tiles_per_img) * p.TR;
-                for (int s = 0; s < p.nStages; ++s, ring.next(p.SA)) {
-                    if (ring.lap >= 1 && !mbar_wait(&bars->act_empty[ring.idx], (ring.lap & 1) ^ 1, abort_flag, ws, 0x7100 + s)) { ok = false; break; }
-                    mbar_arrive_expect_tx(&bars->act_full[ring.idx], p.act_tx_bytes);
-                    tma_load_5d(act + (size_t)ring.idx * p.act_stage_bytes, &tmap_x, &bars->act_full[ring.idx], 0, -p.pad,
-                                y0 - p.pad, s * p.PPS, n);
+        Ring ring{0, 0};
+        bool ok = true;
+        int tile, lo, hi;
+        for (int it = 0; ok && get_item(p, it, tile, lo, hi); ++it) {
+            const TileAt t = tile_at(p, tile);
+            const int img_rows = p.P + p.R - 1, head = img_rows - t.y;       // input rows under an image; under the first one's rest
+            for (int s = 0; s < p.nStages; ++s, ring.next(p.SA)) {
+                ok = ring.lap < 1 || mbar_wait(&bars->act_empty[ring.idx], (ring.lap & 1) ^ 1, abort_flag, ws, 0x7100 + s);
+                if (!__all_sync(0xFFFFFFFFu, ok)) { ok = false; break; }
+                if (lane == 0) mbar_arrive_expect_tx(&bars->act_full[ring.idx], (uint32_t)t.slots * p.row_bytes);
+                __syncwarp();
+                for (int r = lane; r < t.slots; r += 32) {
+                    const int over = r - head, more = over < 0 ? 0 : 1 + over / img_rows;
+                    const int yy = over < 0 ? t.y + r : over - (more - 1) * img_rows;
+                    tma_load_5d(act + (size_t)ring.idx * p.act_stage_bytes + (size_t)r * p.row_pitch, &tmap_x, &bars->act_full[ring.idx], 0, -p.pad,
+                                yy - p.pad, s * p.PPS, t.n + more);
                 }
             }
         }
@@ -316,7 +365,8 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             const uint8_t *kt = blob + hdr[BP_OFF_KT];
             bool ok = true;
             uint32_t use = 0;
-            for (int tile = tile0; tile < p.n_tiles && ok; tile += tile_step) {
+            int tile, lo, hi;
+            for (int it = 0; ok && get_item(p, it, tile, lo, hi); ++it) {
                 for (int c = 0; c < p.nChunks; ++c, ++use) {
                     const uint32_t slot = use & (p.NWS - 1);
                     if (use >= (uint32_t)p.NWS) {
@@ -343,7 +393,12 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             uint32_t use = 0;
             Ring ar{0, 0};                                 // activation stage
             uint32_t buf = 0;                              // TMEM staging buffer of chunk `use`
-            for (int tile = tile0; tile < p.n_tiles && ok; tile += tile_step) {
+            int tile, lo, hi;
+            for (int it = 0; ok && get_item(p, it, tile, lo, hi); ++it) {
+                // this thread's position inside the slab (lanes past the tile's end repeat its last position)
+                const TileAt t = tile_at(p, tile);
+                const int pos = t.first + min((int)m, t.count - 1), n = pos / (p.P * p.Q), rem = pos - n * p.P * p.Q, oy = rem / p.Q;
+                const uint32_t at = (uint32_t)((n - t.n) * (p.P + p.R - 1) + oy - t.y) * p.row_pitch + (uint32_t)(rem - oy * p.Q) * 16u;
                 for (int st = 0; st < p.nStages && ok; ++st, ar.next(p.SA)) {
                     for (int in_stage = 0; in_stage < p.cps; ++in_stage, ++use, buf = buf + 1 == (uint32_t)p.nabuf ? 0u : buf + 1) {
                         if ((int)(use & (uint32_t)(p.NP - 1)) != phase) continue;
@@ -354,7 +409,7 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                             if (!mbar_wait(&bars->done[prev & (kMaxRing - 1)], (prev >> 2) & 1u, abort_flag, ws, 0x7400 + c)) { ok = false; break; }
                         }
                         tc_fence_after_sync();
-                        const uint8_t *src = act + (size_t)ar.idx * p.act_stage_bytes + (size_t)in_stage * 2u * p.plane_bytes + m * 16u;
+                        const uint8_t *src = act + (size_t)ar.idx * p.act_stage_bytes + (size_t)in_stage * 2u * p.oct_bytes + at;
                         const uint32_t tb = tmem_base + lane_base + 256 + buf * p.bufcols;
                         if (p.RS == 9) {
                             // 3x3 kernels: all eighteen loads in flight together, then three stores
@@ -363,12 +418,12 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                             for (int k = 0; k < 4; ++k) {
                                 const uint8_t *q = src + tapoff[k], *q2 = src + tapoff[4 + k];
                                 u[2 * k] = *reinterpret_cast<const uint4 *>(q);
-                                u[2 * k + 1] = *reinterpret_cast<const uint4 *>(q + p.plane_bytes);
+                                u[2 * k + 1] = *reinterpret_cast<const uint4 *>(q + p.oct_bytes);
                                 v[2 * k] = *reinterpret_cast<const uint4 *>(q2);
-                                v[2 * k + 1] = *reinterpret_cast<const uint4 *>(q2 + p.plane_bytes);
+                                v[2 * k + 1] = *reinterpret_cast<const uint4 *>(q2 + p.oct_bytes);
                             }
                             w0 = *reinterpret_cast<const uint4 *>(src + tapoff[8]);
-                            w1 = *reinterpret_cast<const uint4 *>(src + tapoff[8] + p.plane_bytes);
+                            w1 = *reinterpret_cast<const uint4 *>(src + tapoff[8] + p.oct_bytes);
                             tmem_st_x32(tb, u);
                             tmem_st_x32(tb + 32, v);
                             tmem_st_x8(tb + 64, w0, w1);
@@ -379,14 +434,14 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                             for (int k = 0; k < 4; ++k) {
                                 const uint8_t *q = src + bars->tapoff[4 * g + k];
                                 u[2 * k] = *reinterpret_cast<const uint4 *>(q);
-                                u[2 * k + 1] = *reinterpret_cast<const uint4 *>(q + p.plane_bytes);
+                                u[2 * k + 1] = *reinterpret_cast<const uint4 *>(q + p.oct_bytes);
                             }
                             tmem_st_x32(tb + g * 32, u);
                         }
                         for (int t = full_groups * 4; t < p.RS; ++t) {
                             const uint8_t *q = src + bars->tapoff[t];
                             const uint4 u0 = *reinterpret_cast<const uint4 *>(q);
-                            const uint4 u1 = *reinterpret_cast<const uint4 *>(q + p.plane_bytes);
+                            const uint4 u1 = *reinterpret_cast<const uint4 *>(q + p.oct_bytes);
                             tmem_st_x8(tb + t * 8, u0, u1);
                         }
                         }
@@ -427,8 +482,8 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             out[0] = n;
         }
         const int quarter = warp & 3, part = wq >> 2;
-        const int ncol = p.GS * p.Mb, per_part = ((ncol + kMmaWarps / 4 - 1) / (kMmaWarps / 4) + 15) / 16 * 16;
-        const int col_lo = min(ncol, part * per_part), col_hi = min(ncol, col_lo + per_part);
+        // an item's columns: in slabs (staged) or chunks that the two warps of a lane quarter take in turn
+        const int step = p.epi_tma ? 64 : 16, jump = step * (kMmaWarps / 4);
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
         const uint32_t idesc0 = idesc_bf16_f32(128, 0);
         const uint32_t w16 = smem_u32(wring) >> 4, wcap16 = p.wcap >> 4, tile16 = p.tile_bytes >> 4;
@@ -439,14 +494,17 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                         idesc0 | (((r >> 16) & 0xFFu) << 18));
         };
         const int k0 = fb0 * p.Mb;
-        const int m = quarter * 32 + lane, oy = m / p.Wp, ox = m - oy * p.Wp;
+        const int m = quarter * 32 + lane;
         uint32_t use = 0;
         Ring br{0, 0};                                  // TMEM staging buffer
         bool ok = true;
-        int it = 0;
-        for (int tile = tile0; tile < p.n_tiles && ok; tile += tile_step, ++it) {
+        int tile, seg_lo, seg_hi;
+        for (int it = 0; ok && get_item(p, it, tile, seg_lo, seg_hi); ++it) {
+            const int col_lo = seg_lo * p.SEG * p.Mb, col_hi = seg_hi * p.SEG * p.Mb;
+            const uint32_t issues = wq >= seg_lo && wq < seg_hi ? 0xFFFFFFFFu : 0u;
             // zero this tile's accumulators (every MMA accumulates), then let no MMA start early
-            for (int c0 = col_lo; c0 < col_hi; c0 += 16) tmem_st_zero_x16(tmem_base + lane_base + c0);
+            for (int cs = col_lo + part * step; cs < col_hi; cs += jump)
+                for (int c0 = cs; c0 < cs + step; c0 += 16) tmem_st_zero_x16(tmem_base + lane_base + c0);
             tmem_st_wait();
             tc_fence_before_sync();
             mma_warps_sync();
@@ -470,7 +528,7 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                     tc_fence_after_sync();
                     const uint32_t wb = (w16 + slot * wcap16) | (8u << 16);          // 128 bytes between the two channel octets
                     const uint32_t ab = tmem_base + 256 + buf * p.bufcols;
-                    const uint32_t n = v0.x;
+                    const uint32_t n = v0.x & issues;            // (a warp without a share still frees what it waited for)
                     if (elect_one()) {
                         if (n > 0) issue(v0.y, wb, ab);
                         if (n > 1) issue(v0.z, wb, ab);
@@ -490,20 +548,19 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             ok = __all_sync(0xFFFFFFFFu, ok && !*abort_flag);      // the warp goes on, or stops, as one (elect.sync needs all its lanes)
 
             // fused epilogue: the warps that share a TMEM lane quarter split the filter columns
-            const int n = tile / p.tiles_per_img, y0 = (tile - n * p.tiles_per_img) * p.TR;
-            const int yy = y0 + oy;
-            const bool valid = oy < p.TR && yy < p.P && ox < p.Q;
-            const size_t o0 = (((size_t)n * p.P + yy) * p.Q + ox) * p.K + k0;
-            bool go = __all_sync(0xFFFFFFFFu, ok && mbar_wait(&bars->acc_full, it & 1, abort_flag, ws, 0x7700));    // (tcgen05.ld needs the whole warp)
-            if (p.epi_tma) go = part == 0 ? bar_all<2, 128>(go) : bar_all<3, 128>(go);        // (the staged epilogue has barriers among the four warps of a column half)
+            const TileAt t = tile_at(p, tile);
+            const bool valid = m < t.count;
+            const size_t o0 = ((size_t)t.first + m) * p.K + k0;
+            const bool go = __all_sync(0xFFFFFFFFu, ok && mbar_wait(&bars->acc_full, it & 1, abort_flag, ws, 0x7700));    // (tcgen05.ld needs the whole warp)
             if (go) {
                 tc_fence_after_sync();
                 if (p.epi_tma) {
-                    epilogue_staged(&tmap_y, smem_u32(smem + p.off_epi) + (uint32_t)part * kEpiBufBytes, bias ? bars->bias : nullptr,
+                    epilogue_staged(&tmap_y, smem_u32(smem + p.off_epi) + (uint32_t)wq * kEpiBufBytes, bias ? bars->bias : nullptr,
                                     (res && valid) ? static_cast<const uint16_t *>(res) + o0 : nullptr, p.relu != 0,
-                                    tmem_base + lane_base, part, (wq & 3) == 0 && lane == 0, m, col_lo, col_hi, k0, y0, n);
+                                    tmem_base + lane_base, lane, col_lo + part * 64, col_hi, k0, t.first + quarter * 32, t.count - quarter * 32,
+                                    static_cast<uint16_t *>(y) + o0);
                 } else
-                for (int c0 = col_lo; c0 < col_hi; c0 += 16) {
+                for (int c0 = col_lo + part * 16; c0 < col_hi; c0 += jump) {
                     uint32_t r[16];
                     __syncwarp();
                     tmem_ld_x16(tmem_base + lane_base + c0, r);
@@ -563,11 +620,13 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             } else {
                 ok = false;
             }
-            // (at the top of the loop every warp zeroes exactly the lanes and columns it has just read.)  All eight warps go
-            // on, or stop, as one: there are barriers among them in the loop
+            // All eight warps go on, or stop, as one: there are barriers among them in the loop.  (At the top of it accumulators
+            // are zeroed that another warp may have read.)
+            tc_fence_before_sync();
             ok = bar_all<1, kMmaWarps * 32>(ok && !*abort_flag);
+            tc_fence_after_sync();
         }
-        if (p.epi_tma && (wq & 3) == 0 && lane == 0) bulk_wait_all();    // the staging buffers stay valid until the stores have read them
+        if (p.epi_tma && lane == 0) bulk_wait_read_all();                // the staging buffers stay valid until the stores have read them
     }
 
     // ---- tear-down ---------------------------------------------------------------------------
@@ -585,6 +644,13 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     }
 }
 
+// rows of the slab of tile t
+int rows_under(const ConvKrParams &p, int t)
+{
+    const int pq = p.P * p.Q, first = t * p.per, last = min(first + p.per, p.n_pos) - 1;
+    return (last / pq - first / pq) * (p.P + p.R - 1) + last % pq / p.Q - first % pq / p.Q + p.R;
+}
+
 bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvKrParams &p, dim3 &grid)
 {
     if (d.x_dtype != NPAS_BF16 || bp.w_packed != NPAS_BF16) return false;
@@ -598,11 +664,8 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvKrParams &p, dim3
     if (p.P < 1 || p.Q < 1) return false;
     p.Wp = d.W + 2 * d.pad;
     if (p.Wp > 128) return false;
-    p.TR = min(p.P, 128 / p.Wp);
-    p.tiles_per_img = (p.P + p.TR - 1) / p.TR;
-    p.n_tiles = d.N * p.tiles_per_img;
-    p.slab_rows = p.TR + d.R - 1;
-    if (p.slab_rows > 256 || p.TR * p.Wp <= d.S - 1) return false;
+    if ((long long)d.N * p.P * p.Q > 0x7FFFFF00ll) return false;
+    p.n_pos = d.N * p.P * p.Q;
     p.Mb = bp.Mb; p.GS = (int)L.GS; p.nGrp = (int)L.nGrp; p.nCB = d.C / bp.Nb; p.cpb = bp.Nb / 16;
     if (p.GS > 32 || p.GS * p.Mb > 256) return false;
     p.max_taps = bp.max_taps > 0 ? min(bp.max_taps, d.R * d.S) : d.R * d.S;
@@ -621,42 +684,66 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvKrParams &p, dim3
     // per (issuing warp, chunk): a count and at most (SEG + 1) / 2 runs per tap
     p.RW = (1 + p.RS * ((p.SEG + 1) / 2) + 3) & ~3;
     if (p.RW < 8) p.RW = 8;
-    p.plane_bytes = (uint32_t)p.slab_rows * p.Wp * 16u;
+    p.oct_bytes = (uint32_t)p.Wp * 16u;
     p.relu = d.relu; p.y_bf16 = d.y_dtype == NPAS_BF16;
-    const uint32_t reach = (128u + (d.R - 1) * p.Wp + d.S) * 16u;
-    const uint32_t slack = reach > p.plane_bytes ? round_up(reach - p.plane_bytes, 128) : 0u;
+    const int pq = p.P * p.Q;
+    // Tiles of 128 positions counted through all images: no lane idles.  Where their slab (the rows under a tile, those between
+    // two images apart) is too large for shared memory or for one copy per lane, tiles of whole rows of one image.
     bool fits = false;
-    for (int nws = kMaxRing; nws >= 2 && !fits; nws /= 2)
-        for (int cps = 4; cps >= p.NP && !fits; cps /= 2) {
-            if (cps % p.NP || p.nChunks % min(cps, p.nChunks)) continue;
-            p.NWS = nws;
-            p.cps = min(cps, p.nChunks);
-            p.PPS = p.cps * 2;
-            p.nStages = (p.nChunks + p.cps - 1) / p.cps;
-            p.act_tx_bytes = p.plane_bytes * p.PPS;
-            p.act_stage_bytes = round_up(p.act_tx_bytes, 128);
-            for (p.SA = 3; p.SA >= 2 && !fits; --p.SA) {
-                p.off_act = 0;
-                p.off_w = round_up(p.SA * p.act_stage_bytes + slack, 128);
-                p.off_cm = p.off_w + p.NWS * p.wcap;
-                p.off_kto = p.off_cm + round_up(64u * p.nChunks, 128);
-                p.off_rec = p.off_kto + round_up(8u * p.nChunks, 128);
-                p.off_bar = p.off_rec + round_up(4u * p.NA * p.nChunks * p.RW, 128);
-                // bf16 output in whole 64-filter slabs per column half: staged for tensor stores when there is room
-                const bool want_epi = p.y_bf16 && (p.GS * p.Mb) % 128 == 0;
-                for (p.epi_tma = want_epi ? 1 : 0; p.epi_tma >= 0 && !fits; --p.epi_tma) {
-                    p.off_epi = round_up(p.off_bar + (uint32_t)sizeof(Bars), 1024);
-                    p.smem_bytes = (p.epi_tma ? p.off_epi + 2u * kEpiBufBytes : p.off_bar + (uint32_t)sizeof(Bars)) + 1024u;
-                    fits = p.smem_bytes <= kSmemLimit && p.plane_bytes * (uint32_t)p.PPS < (1u << 18);
+    for (int by_rows = 0; by_rows <= 1 && !fits; ++by_rows) {
+        const int TR = min(p.P, 128 / p.Wp);
+        p.per = by_rows ? TR * p.Q : 128;
+        p.grp_pos = by_rows ? pq : p.n_pos;
+        p.tiles_per_grp = (p.grp_pos + p.per - 1) / p.per;
+        p.n_tiles = (by_rows ? d.N : 1) * p.tiles_per_grp;
+        p.slots = 0;
+        if (by_rows) p.slots = TR + d.R - 1;
+        else {
+            // (the place of a tile inside an image repeats)
+            const int period = pq / std::gcd(pq, 128);
+            for (int t = 0; t < min(p.n_tiles, period); ++t) p.slots = max(p.slots, rows_under(p, t));
+            if (p.slots > 32) continue;
+        }
+        for (int nws = kMaxRing; nws >= 2 && !fits; nws /= 2)
+            for (int cps = 4; cps >= p.NP && !fits; cps /= 2) {
+                if (cps % p.NP || p.nChunks % min(cps, p.nChunks)) continue;
+                p.NWS = nws;
+                p.cps = min(cps, p.nChunks);
+                p.PPS = p.cps * 2;
+                p.nStages = (p.nChunks + p.cps - 1) / p.cps;
+                p.row_bytes = p.oct_bytes * p.PPS;
+                p.row_pitch = round_up(p.row_bytes, 128);
+                p.act_stage_bytes = p.row_pitch * (uint32_t)p.slots;
+                for (p.SA = 3; p.SA >= 2 && !fits; --p.SA) {
+                    p.off_act = 0;
+                    p.off_w = p.SA * p.act_stage_bytes;
+                    p.off_cm = p.off_w + p.NWS * p.wcap;
+                    p.off_kto = p.off_cm + round_up(64u * p.nChunks, 128);
+                    p.off_rec = p.off_kto + round_up(8u * p.nChunks, 128);
+                    p.off_bar = p.off_rec + round_up(4u * p.NA * p.nChunks * p.RW, 128);
+                    // bf16 output in whole 64-filter slabs per column half: staged for tensor stores when there is room
+                    const bool want_epi = p.y_bf16 && (p.GS * p.Mb) % 128 == 0;
+                    for (p.epi_tma = want_epi ? 1 : 0; p.epi_tma >= 0 && !fits; --p.epi_tma) {
+                        p.off_epi = round_up(p.off_bar + (uint32_t)sizeof(Bars), 1024);
+                        p.smem_bytes = (p.epi_tma ? p.off_epi + kMmaWarps * kEpiBufBytes : p.off_bar + (uint32_t)sizeof(Bars)) + 1024u;
+                        fits = p.smem_bytes <= kSmemLimit && p.act_stage_bytes < (1u << 18);
+                        if (fits) break;
+                    }
                     if (fits) break;
                 }
-                if (fits) break;
             }
-        }
+    }
     if (!fits) return false;
     const int ctas_x = min(p.n_tiles, max(1, sm_count() / p.nGrp));
     if (p.nGrp > 65535) return false;
     grid = dim3(ctas_x, p.nGrp);
+    // the tiles of a last round that leaves at least half of the CTAs idle are split by filters, as long as a part is whole
+    // issuing warps and whole slabs of the epilogue
+    p.NQ = 1;
+    const int rest = p.n_tiles % ctas_x;
+    while (rest && p.n_tiles > ctas_x && 2 * p.NQ * rest <= ctas_x && p.NA % (2 * p.NQ) == 0 &&
+           (p.GS * p.Mb / (2 * p.NQ)) % (p.epi_tma ? 64 : 16) == 0)
+        p.NQ *= 2;
     return true;
 }
 
@@ -701,25 +788,24 @@ npas_status conv_kr_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return NPAS_ERR_CUDA;
     // X[N][H][W][C] bf16 seen as (8 channels, W, H, C/8, N): a box lands in shared memory as
-    // [octet][row][column][8 channels]
+    // [octet][column][8 channels], one row of the image
     CUtensorMap tmap;
     const cuuint64_t dims[5] = {8, (cuuint64_t)d.W, (cuuint64_t)d.H, (cuuint64_t)(d.C / 8), (cuuint64_t)d.N};
     const cuuint64_t strides[4] = {(cuuint64_t)d.C * 2, (cuuint64_t)d.W * d.C * 2, 16, (cuuint64_t)d.H * d.W * d.C * 2};
-    const cuuint32_t box[5] = {8, (cuuint32_t)p.Wp, (cuuint32_t)p.slab_rows, (cuuint32_t)p.PPS, 1};
+    const cuuint32_t box[5] = {8, (cuuint32_t)p.Wp, 1, (cuuint32_t)p.PPS, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(x), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return NPAS_ERR_CUDA;
-    // Y[N][P][Q][K] bf16 seen as (K, Q, P, N): a box of 64 filters x Wp columns x TR rows is the tile's positions
-    // in the order the accumulator lanes hold them; the padding columns fall outside the tensor
+    // Y[N][P][Q][K] bf16 seen as (K, positions): a box of 64 filters x a warp's 32 positions
     CUtensorMap tmy = tmap;
     if (p.epi_tma) {
-        const cuuint64_t ydims[4] = {(cuuint64_t)d.K, (cuuint64_t)p.Q, (cuuint64_t)p.P, (cuuint64_t)d.N};
-        const cuuint64_t ystr[3] = {(cuuint64_t)d.K * 2, (cuuint64_t)p.Q * d.K * 2, (cuuint64_t)p.P * p.Q * d.K * 2};
-        const cuuint32_t ybox[4] = {64, (cuuint32_t)p.Wp, (cuuint32_t)p.TR, 1};
-        const cuuint32_t yes[4] = {1, 1, 1, 1};
-        if (enc(&tmy, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, y, ydims, ystr, ybox, yes, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        const cuuint64_t ydims[2] = {(cuuint64_t)d.K, (cuuint64_t)p.n_pos};
+        const cuuint64_t ystr[1] = {(cuuint64_t)d.K * 2};
+        const cuuint32_t ybox[2] = {64, 32};
+        const cuuint32_t yes[2] = {1, 1};
+        if (enc(&tmy, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, y, ydims, ystr, ybox, yes, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return NPAS_ERR_CUDA;
     }
