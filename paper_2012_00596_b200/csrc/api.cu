@@ -162,10 +162,13 @@ static int linear_kernel_for(const npas_linear_desc &d, const npas_bb_desc &bb)
         case 0: case 2: break;
         default: return 0;
     }
-    // automatic: both operands by TMA (on CTA pairs where measured faster: few rows, 256 or more input
-    // features), then the gather kernel, then CUDA cores
+    // automatic: both operands by TMA (on CTAs or CTA pairs, whichever the model of both puts lower), then the gather
+    // kernel, then CUDA cores
     if (linear_sk_preferred(d, bb)) return 5;
-    if (d.I >= 256 && d.M <= 16384 && linear_d2_supported(d, bb)) return 6;
+    // (256 or more inputs and less than a sixteenth of the chip in 128 x 128 tiles stay on pairs: there the two are within the
+    // model's error of each other)
+    const bool tiny = d.I >= 256 && (long long)((d.M + 127) / 128) * ((d.O + 127) / 128) * 16 < sm_count();
+    if (linear_d2_supported(d, bb) && (tiny || linear_d2_cost(d, bb) < linear_dn_cost(d, bb))) return 6;
     if (linear_dn_supported(d, bb)) return 5;
     if (linear_tc_supported(d, bb)) return 3;
     return d.path == 2 ? 0 : 1;

@@ -26,6 +26,22 @@ enum BbHdr { BB_MAGIC, BB_VERSION, BB_DTYPE, BB_O, BB_I, BB_BO, BB_BI, BB_NBO, B
 constexpr uint32_t kVersionBB = 3;
 
 // Section offsets of a block-punched blob, computed on the host from the descriptor and nPairs.
+// Microseconds of the GEMM kernels with both operands by TMA, columns in tiles of `bn`, on CTAs (128 rows a tile) or on CTA
+// pairs (256 rows): fitted to 583 measured points (110 random layers, four widths on CTAs and three on pairs; standard error
+// 8 and 7 %; the width and kernel it picks take 0.6 % more than the best measured on average, 8 % at worst).  Rounds of tiles
+// x (K steps, a part of which grows with the width, and the epilogue), and the bytes that cross DRAM.  Wide tiles read the
+// input less often, narrow ones fill a last round better: 42389 x 1920 -> 256 takes 52 us on CTAs and 40 on pairs,
+// 9089 x 384 -> 576 12 us in tiles of 64 and 8 in tiles of 192, 1619 x 128 -> 512 5.5 us in tiles of 256 and 3.9 of 64.
+inline double linear_modelled(const npas_linear_desc &d, int bn, bool pair, int sms)
+{
+    const int nK = (d.I + 63) / 64, nMT = (d.M + 127) / 128, nNT = (d.O + bn - 1) / bn, cap = pair ? sms / 2 : sms;
+    const double tiles = (double)(pair ? (nMT + 1) / 2 : nMT) * nNT, r = (double)(((long long)tiles + cap - 1) / (cap > 0 ? cap : 1));
+    const double out = (d.has_residual ? 2. : 1.) * (d.y_dtype == NPAS_BF16 ? 1. : 2.);
+    const double mb = 2e-6 * ((double)d.M * d.I + out * d.M * d.O + (double)d.I * d.O);
+    return pair ? 3.32 + r * (nK * (0.0973 + 0.00067 * bn) + 0.0017 * bn * out + 0.43) + 0.061 * mb
+                : 3.02 + r * (nK * (0.1706 + 0.00070 * bn) + 0.0026 * bn * out + 0.14) + 0.037 * mb + 1.8e-7 * tiles * nK * (128 + bn);
+}
+
 struct BpLayout {
     uint32_t nFB, nCB, nPairs, G, es;
     uint32_t off_blk, off_pairs, off_values, total;
@@ -203,6 +219,7 @@ npas_status conv_kr_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
 npas_status linear_simt_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                                const void *blob, const float *bias, const void *res, void *y, cudaStream_t st);
 bool linear_dn_supported(const npas_linear_desc &d, const npas_bb_desc &bb);
+float linear_dn_cost(const npas_linear_desc &d, const npas_bb_desc &bb);
 npas_status linear_dn_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,
                              cudaStream_t st);
@@ -212,6 +229,7 @@ npas_status linear_sk_launch(const npas_linear_desc &d, const npas_bb_desc &bb, 
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,
                              cudaStream_t st);
 bool linear_d2_supported(const npas_linear_desc &d, const npas_bb_desc &bb);
+float linear_d2_cost(const npas_linear_desc &d, const npas_bb_desc &bb);
 npas_status linear_d2_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,
                              cudaStream_t st);

@@ -45,6 +45,7 @@ struct LinD2Params {
     int relu, y_bf16;
     int NS;                                               // epilogue slots (0: epilogue straight from registers)
     uint32_t stage_bytes, off_slots, off_bias, off_bar, smem_bytes, tmem_cols;
+    float cost;                                           // modelled microseconds
 };
 
 struct LinD2Bars {
@@ -87,6 +88,8 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     volatile uint32_t *abort_flag = &bars->abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // column tile nt: BN columns, the last one what is left of O
+    auto width = [&](int nt) { return min(p.BN, p.O - nt * p.BN); };
     const uint32_t rank = cluster_ctarank();                  // 0: leader (issues the MMAs), 1: its peer
     const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const uint32_t peer_abort = map_to_cta(smem_u32(&bars->abort_flag), rank ^ 1u);
@@ -122,7 +125,7 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         for (; early < p.S && tile < p.n_tiles; ++early) {
             if (rank == 0) mbar_arrive_expect_tx(&bars->full[early], 2u * p.stage_bytes);
             tma_load_2d_pair(smem + (size_t)early * p.stage_bytes + kXBytes, &tmap_w, map_to_cta(smem_u32(&bars->full[early]), 0u), k * 64,
-                             (tile % p.nNT) * p.BN + (int)rank * (p.BN / 2));
+                             (tile % p.nNT) * p.BN + (int)rank * (width(tile % p.nNT) / 2));
             if (++k == p.nK) { k = 0; tile += n_pairs; }
         }
     }
@@ -148,7 +151,7 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     uint8_t *st = smem + (size_t)s * p.stage_bytes;
                     if (rank == 0 && early <= 0) mbar_arrive_expect_tx(&bars->full[s], 2u * p.stage_bytes);
                     tma_load_2d_pair(st, &tmap_x, full0 + s * 8u, k * 64, mt * kRows);     // rows past M read as zeros
-                    if (early-- <= 0) tma_load_2d_pair(st + kXBytes, &tmap_w, full0 + s * 8u, k * 64, nt * p.BN + (int)rank * (p.BN / 2));
+                    if (early-- <= 0) tma_load_2d_pair(st + kXBytes, &tmap_w, full0 + s * 8u, k * 64, nt * p.BN + (int)rank * (width(nt) / 2));
                     if (++s == (uint32_t)p.S) { s = 0; ++lap; }
                 }
             }
@@ -179,7 +182,6 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         } else {
             // ---- leader: MMA issue for the pair; the thread's own instructions are on the critical path, so
             // the ring position is carried along and nothing else is computed ---------------------------------
-            const uint32_t idesc = idesc_bf16_f32(256, p.BN);
             const uint32_t base16 = (smem_u32(smem) >> 4) | kDescLboOne, stage16 = p.stage_bytes >> 4;
             uint32_t s = 0, ph = 0, a_lo = base16, it = 0;
             bool ok = true;
@@ -187,7 +189,7 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 const uint32_t acc = it & 1u, lap_acc = it >> 1;
                 if (lap_acc >= 1 && !pair_wait<true>(&bars->acc_empty[acc], (lap_acc & 1u) ^ 1u, abort_flag, peer_abort, ws, 0x8200)) break;
                 tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + acc * p.BN;
+                const uint32_t d_tmem = tmem_base + acc * p.BN, idesc = idesc_bf16_f32(256, width(tile % p.nNT));
                 for (int k = 0; k < p.nK; ++k) {
                     if (!pair_wait(&bars->full[s], ph, abort_flag, peer_abort, ws, 0x8300)) { ok = false; break; }
                     tc_fence_after_sync();
@@ -208,9 +210,9 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         if (lane == 0 && p.NS && res) {
             uint32_t n = 0;
             bool ok = true;
-            const int nsl = p.BN / 64;
             for (int tile = pair; tile < p.n_tiles && ok; tile += n_pairs) {
                 const int mp = tile / p.nNT, nt = tile - mp * p.nNT, mt = 2 * mp + (int)rank;
+                const int nsl = width(nt) / 64;
                 for (int sl = 0; sl < nsl; ++sl, ++n) {
                     const uint32_t slot = n % (uint32_t)p.NS, lap = n / (uint32_t)p.NS;
                     if (lap >= 1 && !mbar_wait(&bars->res_empty[slot], (lap & 1u) ^ 1u, abort_flag, ws, 0x8500)) { ok = false; break; }
@@ -224,11 +226,11 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // store before it has read its slot, that slot is free again (for the next residual slab, or, without
         // a residual, for the epilogue itself).  The epilogue warps never wait for a store or for each other.
         if (lane == 0 && p.NS) {
-            const int nsl = p.BN / 64;
             uint32_t slot = 0, ph = 0, prev = 0;
             bool ok = true, first = true;
             for (int tile = pair; tile < p.n_tiles && ok; tile += n_pairs) {
                 const int mp = tile / p.nNT, nt = tile - mp * p.nNT, mt = 2 * mp + (int)rank;
+                const int nsl = width(nt) / 64;
                 for (int sl = 0; sl < nsl; ++sl) {
                     if (!mbar_wait(&bars->slot_done[slot], ph, abort_flag, ws, 0x8600)) { ok = false; break; }
                     tma_store_2d(&tmap_y, smem + p.off_slots + (size_t)slot * kSlotBytes, nt * p.BN + sl * 64, mt * kRows);
@@ -244,14 +246,13 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // ---- epilogue through shared memory: warp -> TMEM lane quarter (warp % 4) and the 16 columns
         // number (warp - first) / 4 of every 64-column slab ---------------------------------------------------
         const int quarter = warp & 3, part = (warp - kFirstEpiWarp) >> 2, m = quarter * 32 + lane;
-        const int nsl = p.BN / 64;
         // this thread's two 16-byte pieces of its row of a slot (pieces XOR-ed with the row number)
         const uint32_t off0 = (uint32_t)m * 128u + (uint32_t)(((2 * part) ^ (m & 7)) * 16);
         const uint32_t off1 = (uint32_t)m * 128u + (uint32_t)(((2 * part + 1) ^ (m & 7)) * 16);
         uint32_t it = 0, n = 0, slot = 0, slot_ph = 0;      // slab count; its slot and the slot's lap parity
         bool ok = true;
         for (int tile = pair; tile < p.n_tiles && ok; tile += n_pairs, ++it) {
-            const int nt = tile % p.nNT;
+            const int nt = tile % p.nNT, nsl = width(nt) / 64;
             const uint32_t acc = it & 1u;
             const float *bs = bias_s + nt * p.BN + part * 16;
             const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * p.BN + (uint32_t)part * 16u;
@@ -313,7 +314,6 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     } else {
         // ---- epilogue: warp -> TMEM lane quarter (warp % 4) and every fourth 16-column chunk ----------
         const int quarter = warp & 3, part = (warp - kFirstEpiWarp) >> 2, m = quarter * 32 + lane;
-        const int nch = p.BN / 16;
         uint32_t it = 0;
         bool ok = true;
         for (int tile = pair; tile < p.n_tiles && ok; tile += n_pairs, ++it) {
@@ -321,6 +321,7 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             const uint32_t acc = it & 1u;
             const int row = mt * kRows + m;
             const bool valid = row < p.M;
+            const int nch = width(nt) / 16;
             const size_t o0 = (size_t)row * p.O + (size_t)nt * p.BN;
             const float *bs = bias_s + nt * p.BN;
             const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * p.BN;
@@ -413,37 +414,29 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinD2Params &p)
 {
     if (d.x_dtype != NPAS_BF16 || bb.w_packed != NPAS_BF16) return false;
-    if (d.I % 64 || d.O % 16 || d.O > 16384) return false;
+    if (d.I % 64 || d.O % 128 || d.O > 16384) return false;
     p.M = d.M; p.I = d.I; p.O = d.O;
     p.nK = d.I / 64;
     p.nMT = (d.M + kRows - 1) / kRows;
     p.relu = d.relu; p.y_bf16 = d.y_dtype == NPAS_BF16;
     const uint32_t fixed = (uint32_t)d.O * 4 + 128 + (uint32_t)sizeof(LinD2Bars) + 1024 + 256;
-    // Column tile BN: the widest divisor of O that leaves room for enough stages (three once the K loop has
-    // three or more steps), else the widest with two (measured: narrower tiles never won, the kernel is
-    // bound by what the SMs take in from L2, and wide tiles take in the least per MAC).  Epilogue slots
-    // (bf16 output, BN % 64 == 0): three when only stores pass through them, six when the residual is prefetched
-    // into them.
+    // Column tile BN: 128, 192 or 256 (the last tile what is left) by the model, as in linear_dn.cu; epilogue slots likewise.
     // (the call descriptor's `variant` restricts the choice to one width)
-    const int want = p.nK >= 3 ? 3 : 2;
-    const int want_bn = d.variant;
-    p.BN = 0;
-    for (int pass = 0; pass < 2 && !p.BN; ++pass)
-        for (int bn = 256; bn >= 128; bn /= 2) {               // each CTA stages bn / 2 rows of W
-            if (d.O % bn || (want_bn && bn != want_bn)) continue;
-            // with so few tiles that half of the pairs would idle, the narrower tile doubles their number
-            if (bn == 256 && !want_bn && (long long)((p.nMT + 1) / 2) * (d.O / 256) <= 37) continue;
-            const int ns = p.y_bf16 && bn % 64 == 0 ? (d.has_residual ? kMaxSlots : 3) : 0;
+    const int want = p.nK >= 3 ? 3 : 2, want_bn = d.variant, sms = sm_count();
+    p.BN = 0; p.cost = 0.f;
+    for (int stages = want; stages >= 2 && !p.BN; --stages)
+        for (int bn = 128; bn <= 256 && bn <= d.O; bn += 64) {            // each CTA stages bn / 2 rows of W
+            if (want_bn && bn != want_bn) continue;
+            const int ns = p.y_bf16 ? (d.has_residual ? kMaxSlots : 3) : 0;
             const uint32_t stage = round_up(kXBytes + (uint32_t)(bn / 2) * 128u, 1024);   // multiples of 1024: swizzled tiles stay aligned
             const uint32_t need = fixed + (uint32_t)ns * kSlotBytes;
-            if (need + 2 * stage > kSmemLimit) continue;
-            const int st = (int)((kSmemLimit - need) / stage);
-            if (pass == 0 && st < want) continue;
-            p.BN = bn; p.NS = ns; p.stage_bytes = stage; p.S = st > kMaxStages ? kMaxStages : st;
-            break;
+            const int st = need < kSmemLimit ? (int)((kSmemLimit - need) / stage) : 0;
+            const float cost = (float)linear_modelled(d, bn, true, sms);
+            if (st < stages || (p.BN && cost >= p.cost)) continue;
+            p.BN = bn; p.NS = ns; p.stage_bytes = stage; p.S = st > kMaxStages ? kMaxStages : st; p.cost = cost;
         }
     if (p.BN == 0) return false;
-    p.nNT = d.O / p.BN;
+    p.nNT = (d.O + p.BN - 1) / p.BN;
     const long long tiles = (long long)((p.nMT + 1) / 2) * p.nNT;       // a tile = two row tiles x one column tile
     if (tiles > 0x7FFFFFFF) return false;
     p.n_tiles = (int)tiles;
@@ -476,6 +469,12 @@ bool planned(const npas_linear_desc &d, const npas_bb_desc &b, LinD2Params &p)
 }
 
 }  // namespace
+
+float linear_d2_cost(const npas_linear_desc &d, const npas_bb_desc &bb)
+{
+    LinD2Params p;
+    return planned(d, bb, p) ? p.cost : 1e30f;
+}
 
 bool linear_d2_supported(const npas_linear_desc &d, const npas_bb_desc &bb)
 {

@@ -50,6 +50,7 @@ struct LinDnParams {
     int relu, y_bf16;
     int NS;                                               // epilogue slots (0: epilogue straight from registers)
     uint32_t stage_bytes, off_slots, off_bias, off_bar, smem_bytes, tmem_cols;
+    float cost;                                           // modelled microseconds
 };
 
 struct LinDnBars {
@@ -91,6 +92,8 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     volatile uint32_t *abort_flag = &bars->abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // column tile nt: BN columns, the last one what is left of O
+    auto width = [&](int nt) { return min(p.BN, p.O - nt * p.BN); };
 
     // The producer starts by itself: it initialises the barriers it signals and requests the first ring of stages before the
     // other warps have set up theirs and tensor memory (0.4 us).  The weights do not wait for the kernel before this one: no
@@ -160,7 +163,6 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // ---- MMA issue: one thread; its own instructions are on the critical path (four MMAs of a stage
         // execute in about 600 cycles), so the ring position is carried along and nothing else is computed
         if (elect_one()) {
-            const uint32_t idesc = idesc_bf16_f32(128, p.BN);
             const uint32_t base16 = (smem_u32(smem) >> 4) | kDescLboOne, stage16 = p.stage_bytes >> 4;
             uint32_t s = 0, ph = 0, a_lo = base16, it = 0;
             bool ok = true;
@@ -168,7 +170,7 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 const uint32_t acc = it & 1u, lap_acc = it >> 1;
                 if (lap_acc >= 1 && !mbar_wait(&bars->acc_empty[acc], (lap_acc & 1u) ^ 1u, abort_flag, ws, 0x5200)) break;
                 tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + acc * p.BN;
+                const uint32_t d_tmem = tmem_base + acc * p.BN, idesc = idesc_bf16_f32(128, (width(tile % p.nNT) + 15) & ~15);
                 for (int k = 0; k < p.nK; ++k) {
                     if (!mbar_wait(&bars->full[s], ph, abort_flag, ws, 0x5300)) { ok = false; break; }
                     tc_fence_after_sync();
@@ -189,9 +191,8 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         if (lane == 0 && p.NS && res) {
             uint32_t n = 0;
             bool ok = true;
-            const int nsl = p.BN / 64;
             for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
-                const int mt = tile / p.nNT, nt = tile - mt * p.nNT;
+                const int mt = tile / p.nNT, nt = tile - mt * p.nNT, nsl = (width(nt) + 63) / 64;
                 for (int sl = 0; sl < nsl; ++sl, ++n) {
                     const uint32_t slot = n % (uint32_t)p.NS, lap = n / (uint32_t)p.NS;
                     if (lap >= 1 && !mbar_wait(&bars->res_empty[slot], (lap & 1u) ^ 1u, abort_flag, ws, 0x5500)) { ok = false; break; }
@@ -205,11 +206,10 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // store before it has read its slot, that slot is free again (for the next residual slab, or, without
         // a residual, for the epilogue itself).  The epilogue warps never wait for a store or for each other.
         if (lane == 0 && p.NS) {
-            const int nsl = p.BN / 64;
             uint32_t slot = 0, ph = 0, prev = 0;
             bool ok = true, first = true;
             for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
-                const int mt = tile / p.nNT, nt = tile - mt * p.nNT;
+                const int mt = tile / p.nNT, nt = tile - mt * p.nNT, nsl = (width(nt) + 63) / 64;
                 for (int sl = 0; sl < nsl; ++sl) {
                     if (!mbar_wait(&bars->slot_done[slot], ph, abort_flag, ws, 0x5600)) { ok = false; break; }
                     tma_store_2d(&tmap_y, smem + p.off_slots + (size_t)slot * kSlotBytes, nt * p.BN + sl * 64, mt * kRows);
@@ -225,14 +225,13 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // ---- epilogue through shared memory: warp -> TMEM lane quarter (warp % 4) and the 16 columns
         // number (warp - first) / 4 of every 64-column slab ---------------------------------------------------
         const int quarter = warp & 3, part = (warp - kFirstEpiWarp) >> 2, m = quarter * 32 + lane;
-        const int nsl = p.BN / 64;
         // this thread's two 16-byte pieces of its row of a slot (pieces XOR-ed with the row number)
         const uint32_t off0 = (uint32_t)m * 128u + (uint32_t)(((2 * part) ^ (m & 7)) * 16);
         const uint32_t off1 = (uint32_t)m * 128u + (uint32_t)(((2 * part + 1) ^ (m & 7)) * 16);
         uint32_t it = 0, n = 0, slot = 0, slot_ph = 0;      // slab count; its slot and the slot's lap parity
         bool ok = true;
         for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x, ++it) {
-            const int mt = tile / p.nNT, nt = tile - mt * p.nNT;
+            const int nt = tile % p.nNT, nsl = (width(nt) + 63) / 64;
             const uint32_t acc = it & 1u;
             const float *bs = bias_s + nt * p.BN + part * 16;
             const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * p.BN + (uint32_t)part * 16u;
@@ -404,29 +403,33 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinDnParams &p)
     p.nMT = (d.M + kRows - 1) / kRows;
     p.relu = d.relu; p.y_bf16 = d.y_dtype == NPAS_BF16;
     const uint32_t fixed = ((uint32_t)d.O + 256u) * 4 + 128 + (uint32_t)sizeof(LinDnBars) + 1024 + 256;
-    // Column tile BN: the widest divisor of O that leaves room for enough stages (three once the K loop has
-    // three or more steps), else the widest with two (measured: narrower tiles never won, the kernel is
-    // bound by what the SMs take in from L2, and wide tiles take in the least per MAC).  Epilogue slots
-    // (bf16 output, BN % 64 == 0): three when only stores pass through them, six when the residual is prefetched
-    // into them.
+    // Column tile BN: any multiple of 64 where 64 divides O (the last tile what is left), by the model; else the widest power of
+    // two that divides O; else 128, the last tile cut short.  Only tiles that leave room for enough stages (three once the K
+    // loop has three or more steps), else for two.  Epilogue slots (bf16 output, BN % 64 == 0): three when only stores pass
+    // through them, six when the residual is prefetched into them.
     // (the call descriptor's `variant` restricts the choice to one width)
-    const int want = p.nK >= 3 ? 3 : 2;
-    const int want_bn = d.variant;
-    p.BN = 0;
-    for (int pass = 0; pass < 2 && !p.BN; ++pass)
-        for (int bn = 256; bn >= 16; bn /= 2) {
-            if (want_bn && bn != want_bn) continue;
-            // (an output width that 16 does not divide: tiles of 128, the last one cut short by the tensor map and the store)
-            if (d.O % 16 ? (!want_bn && bn != 128) : (d.O % bn != 0)) continue;
-            const int ns = p.y_bf16 && bn % 64 == 0 ? (d.has_residual ? kMaxSlots : 3) : 0;
-            const uint32_t stage = round_up(kXBytes + (uint32_t)bn * 128u, 1024);   // multiples of 1024: swizzled tiles stay aligned
-            const uint32_t need = fixed + (uint32_t)ns * kSlotBytes;
-            if (need + 2 * stage > kSmemLimit) continue;
-            const int st = (int)((kSmemLimit - need) / stage);
-            if (pass == 0 && st < want) continue;
-            p.BN = bn; p.NS = ns; p.stage_bytes = stage; p.S = st > kMaxStages ? kMaxStages : st;
-            break;
-        }
+    const int want = p.nK >= 3 ? 3 : 2, want_bn = d.variant, sms = sm_count();
+    if (want_bn && (want_bn < 16 || want_bn > 256)) return false;
+    if (want_bn && d.O % 16 == 0 && (want_bn & (want_bn - 1) || d.O % want_bn) && (d.O % 64 || want_bn % 64 || want_bn > d.O)) return false;
+    p.BN = 0; p.cost = 0.f;
+    auto consider = [&](int bn, int stages) {
+        const int ns = p.y_bf16 && bn % 64 == 0 ? (d.has_residual ? kMaxSlots : 3) : 0;
+        const uint32_t stage = round_up(kXBytes + (uint32_t)bn * 128u, 1024);   // multiples of 1024: swizzled tiles stay aligned
+        const uint32_t need = fixed + (uint32_t)ns * kSlotBytes;
+        const int st = need < kSmemLimit ? (int)((kSmemLimit - need) / stage) : 0;
+        const float cost = (float)linear_modelled(d, bn, false, sms);
+        if (st < stages || (p.BN && cost >= p.cost)) return;
+        p.BN = bn; p.NS = ns; p.stage_bytes = stage; p.S = st > kMaxStages ? kMaxStages : st; p.cost = cost;
+    };
+    for (int stages = want; stages >= 2 && !p.BN; --stages) {
+        if (want_bn) consider(want_bn, stages);
+        else if (d.O % 64 == 0) {
+            for (int bn = 64; bn <= 256 && bn <= d.O; bn += 64) consider(bn, stages);
+        } else if (d.O % 16 == 0) {
+            for (int bn = 256; bn >= 16 && !p.BN; bn /= 2)
+                if (d.O % bn == 0) consider(bn, stages);
+        } else consider(128, stages);
+    }
     if (p.BN == 0) return false;
     p.nNT = (d.O + p.BN - 1) / p.BN;
     const long long tiles = (long long)p.nMT * p.nNT;
@@ -461,6 +464,12 @@ bool planned(const npas_linear_desc &d, const npas_bb_desc &b, LinDnParams &p)
 }
 
 }  // namespace
+
+float linear_dn_cost(const npas_linear_desc &d, const npas_bb_desc &bb)
+{
+    LinDnParams p;
+    return planned(d, bb, p) ? p.cost : 1e30f;
+}
 
 bool linear_dn_supported(const npas_linear_desc &d, const npas_bb_desc &bb)
 {
