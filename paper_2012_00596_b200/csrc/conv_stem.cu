@@ -1,4 +1,5 @@
-// Few-channel first layer (7x7, stride 2, pad 3, C = 3) on the sm_100a tensor cores.
+// Few-channel first layer (7x7, stride 2, pad 3, C = 3) on the sm_100a tensor cores: images wider than 256 pixels and layers
+// of more than 128 filters (the others: conv_stem_rows.cu, whose operand needs no expansion and whose tile is a whole row).
 //
 // With three channels the operand of a kept (channel block, tap) pair is only three elements wide,
 // far below the tensor core's K = 16, so the generic block-punched kernels leave this layer to the
