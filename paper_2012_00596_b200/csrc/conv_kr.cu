@@ -766,16 +766,24 @@ bool conv_kr_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
     return planned(d, bp, p, grid);
 }
 
-// Where this kernel was measured faster than the dense-image kernels (64x28x28x512 -> 512 with random
-// tap sets): up to three taps in nine kept at blocks of 16 filters, up to four in nine at blocks of 32
-// filters or more; and only when there is at least one item per SM.
+// Whether this kernel is the better one: by a model of it (122 random 3x3 layers of 32 to 512 channels and filters, blocks of
+// 16 and 32, one to five taps kept; standard error 6 %) against one of the dense-image kernels (4 and 8 %).  What it picks is
+// 0.3 % above the better measured one on average; the rule on the taps kept alone (up to three of nine at blocks of 16, four
+// at 32, beyond which the two are level) picked the slower one by a fifth on average, mostly layers of few filters, whose staged slices serve few MMAs: 57x60x60x64 -> 64, one tap,
+// 41 us here against 19; 35x22x34x352 -> 352, three taps, 168 against 116; and the other way 28x18x18x512 -> 512, two taps,
+// 26 against 38.  Measured down to half an item per SM.
 bool conv_kr_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvKrParams p;
     dim3 grid;
     if (bp.max_taps <= 0 || !planned(d, bp, p, grid)) return false;
-    if (p.n_tiles * p.nGrp < sm_count()) return false;
-    return bp.Mb >= 32 ? 9 * bp.max_taps <= 4 * p.RS : 3 * bp.max_taps <= p.RS;
+    const long long items = (long long)p.n_tiles * p.nGrp;
+    if (items < sm_count() && (items * 2 < sm_count() || !conv_d2_preferred(d, bp))) return false;
+    if (bp.Mb >= 32 ? 9 * bp.max_taps > 4 * p.RS : 3 * bp.max_taps > p.RS) return false;
+    const int full = p.n_tiles / (int)grid.x, rest = p.n_tiles % (int)grid.x;
+    const double rounds = full + (rest == 0 ? 0. : p.NQ == 1 ? 1. : 0.45 + 0.55 / p.NQ);
+    const double us = 6.4 + rounds * (p.nChunks * (0.0448 * p.RS + 0.00473 * p.GS * p.max_taps) + 0.0087 * p.GS * p.Mb + 0.9);
+    return us < conv_dense_modelled(d, bp);
 }
 
 npas_status conv_kr_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
