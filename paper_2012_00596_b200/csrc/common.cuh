@@ -209,6 +209,7 @@ npas_status conv_sk_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
 bool conv_d2_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 bool conv_d2_preferred(const npas_conv_desc &d, const npas_bp_desc &bp);
 double conv_dense_modelled(const npas_conv_desc &d, const npas_bp_desc &bp);
+bool conv_sk_slower(const npas_conv_desc &d, const npas_bp_desc &bp);
 npas_status conv_d2_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
                            uint32_t *ws, cudaStream_t st);

@@ -606,27 +606,28 @@ bool conv_d2_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 // for the strided 3x3 geometry it computes by phases (a quarter of the MMAs); else as soon as there are
 // 64 items of 128 positions x 128 filters (half a wave of pairs): 11.4 against 13.7 us on 32x14x14x256 -> 256,
 // 17.5 against 22.0 on 64x28x28x128 -> 128, 26 against 36 on 64x7x7x512 -> 512.  Smaller problems stay on
-// independent CTAs.
+// independent CTAs unless the split form is modelled slower.
 bool conv_d2_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvD2Params p;
     const int pairs = pairs_available();
     if (pairs < 1 || !planned(d, bp, p)) return false;
     if (p.nph == 4) return true;
-    return (long long)p.n_tiles * ((d.K + 127) / 128) >= 64;
+    return (long long)p.n_tiles * ((d.K + 127) / 128) >= 64 || conv_sk_slower(d, bp);
 }
 
-// Microseconds of the dense-image kernels on a stride-1 layer of many items, fitted to 120 measured layers (standard error 4 % on
-// pairs, 8 % on independent CTAs): rounds of items x chunks x taps, and the bytes that cross DRAM.
+// Microseconds of the dense-image kernels on a stride-1 layer (or a strided one by phases), fitted to 120 measured layers
+// (standard error 4 % on pairs, 8 % on independent CTAs): rounds of items x chunks x taps, and the bytes that cross DRAM.
 double conv_dense_modelled(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     const double nCh = d.C / 16., taps = d.R * d.S / 9., sms = sm_count();
-    const int P = d.H + 2 * d.pad - d.R + 1, Q = d.W + 2 * d.pad - d.S + 1;
+    const int P = (d.H + 2 * d.pad - d.R) / d.stride + 1, Q = (d.W + 2 * d.pad - d.S) / d.stride + 1;
     const double mb = 2e-6 * d.N * ((double)d.H * d.W * d.C + (double)P * Q * d.K);
     ConvD2Params p;
     if (planned(d, bp, p)) {
         const long long pairs = pairs_available() > 0 ? pairs_available() : 1;
-        const long long items = d.K % 128 ? (long long)((p.n_tiles + 3) / 4) * (d.K / 64) : (long long)((p.n_tiles + 1) / 2) * (d.K / 128);
+        const int per = d.K % 128 && p.nph == 1 ? 4 : 2;
+        const long long items = (long long)((p.n_tiles + per - 1) / per) * (d.K / (d.K % 128 ? 64 : 128));
         const double r = (double)((items + pairs - 1) / pairs);
         return 4.4 + r * (d.K % 128 ? 0.354 * taps * nCh + 0.37 : 0.306 * taps * nCh + 0.67) + 0.089 * mb;
     }

@@ -424,7 +424,8 @@ bool conv_sk_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 // 54x6x33x160 -> 32 (108 position tiles) 8.0 against 6.9.  So: one wave, and no more position tiles than half the SMs.
 // Strided 3x3 layers that the pair kernel does not take by phases (it needs multiples of 64 channels and filters) always
 // come here: the single-CTA kernel computes every position (12x19x50x144 -> 208 8.9 against 36 us); those it takes, when
-// there are channels to split and one wave (14x14x512 -> 512 5.8 against 17.1 us).
+// there are channels to split, one wave, and the pair kernel is not modelled faster (14x14x512 -> 512 5.8 against 17.1 us;
+// 59x17x48x512 -> 64 38.6 against 19.3).
 bool conv_sk_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvSkParams p;
@@ -432,15 +433,27 @@ bool conv_sk_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
     if (d.variant) return false;
     const bool phases = d.stride == 2 && d.R == 3 && d.S == 3 && d.pad == 1;
     if (phases && (d.C % 64 || d.K % 64)) return planned(d, bp, p, false);
-    if (!planned(d, bp, p, true)) return false;
-    return phases ? p.nBlk > 1 : p.n_tiles * 2 <= sms;
+    const bool pairs = conv_d2_supported(d, bp);
+    if (planned(d, bp, p, true) && (phases ? p.nBlk > 1 && modelled(p, sms) <= conv_dense_modelled(d, bp) : p.n_tiles * 2 <= sms)) return true;
+    // several waves: against independent CTAs, whose tile is as narrow as the image's groups (11x15x25x416 -> 464 51 against 63 us)
+    return d.stride == 1 && !pairs && planned(d, bp, p, false) && 1.05 * modelled(p, sms) < conv_dense_modelled(d, bp);
+}
+
+// A stride-1 layer of this kernel's range that the pair kernel does sooner, by the models of both: many channels on just under
+// half a wave of position tiles, where one wave leaves too few CTAs to split the chain (6x30x30x512 -> 128 21.0 us here, 15.1
+// on pairs; 39x6x7x512 -> 128 15.6 and 14.2).
+bool conv_sk_slower(const npas_conv_desc &d, const npas_bp_desc &bp)
+{
+    ConvSkParams p;
+    return !d.variant && d.stride == 1 && planned(d, bp, p, true) && modelled(p, sm_count()) > conv_dense_modelled(d, bp);
 }
 
 npas_status conv_sk_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x, const void *blob, const float *bias,
                            const void *res, void *y, uint32_t *ws, cudaStream_t st)
 {
     ConvSkParams p;
-    if (!planned(d, bp, p, !d.variant) && !planned(d, bp, p, false)) return NPAS_ERR_UNSUPPORTED;
+    const bool one_wave = !d.variant && planned(d, bp, p, true) && (d.stride != 1 || p.n_tiles * 2 <= sm_count());     // (as it was chosen)
+    if (!one_wave && !planned(d, bp, p, false)) return NPAS_ERR_UNSUPPORTED;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return NPAS_ERR_CUDA;
     // X[N][H][W][C] as (C, W, H, N): a box of CB channels x Wp columns x slab rows (every other pixel for a parity class)
