@@ -156,8 +156,9 @@ typedef struct {
     int32_t relu, has_bias, has_residual;
     int32_t path;
     int32_t variant; /* 0 = the planner's choice; paths 5 and 6: the column-tile width BN (a power of two
-                        from 16 to 256 dividing O, or a multiple of 64 up to 256 where 64 divides O; path 6:
-                        128, 192 or 256); path 5 with KS << 16 added (KS = 1, 2, 4
+                        from 16 to 256 dividing O, a multiple of 64 up to 256 where 64 divides O, or a multiple of
+                        16 up to 256 where 16 does not divide O; path 6: 128, 192 or 256; other widths give
+                        NPAS_ERR_UNSUPPORTED); path 5 with KS << 16 added (KS = 1, 2, 4
                         or 8): the form for few output tiles, BN 16 to 128, in which a cluster of KS CTAs shares
                         a tile and splits the input columns; npas_tune_linear_bb measures them */
 } npas_linear_desc;

@@ -409,7 +409,9 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinDnParams &p)
     // through them, six when the residual is prefetched into them.
     // (the call descriptor's `variant` restricts the choice to one width)
     const int want = p.nK >= 3 ? 3 : 2, want_bn = d.variant, sms = sm_count();
-    if (want_bn && (want_bn < 16 || want_bn > 256)) return false;
+    // a requested width is whole 16-column chunks, whatever O: the MMA's width is rounded up to 16 while the two accumulators lie
+    // BN columns apart, and the direct epilogue walks BN / 16 chunks
+    if (want_bn && (want_bn < 16 || want_bn > 256 || want_bn % 16)) return false;
     if (want_bn && d.O % 16 == 0 && (want_bn & (want_bn - 1) || d.O % want_bn) && (d.O % 64 || want_bn % 64 || want_bn > d.O)) return false;
     p.BN = 0; p.cost = 0.f;
     auto consider = [&](int bn, int stages) {

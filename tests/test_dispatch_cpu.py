@@ -55,6 +55,22 @@ def test_linear_automatic_choice():
         assert _linear_query(kw, 0) == LINEAR_AUTO[i], i
 
 
+@pytest.mark.parametrize("O,Bo,takes", [(1000, 40, [16, 32, 48, 64, 80, 128, 144, 192, 240, 256]), (1024, 64, [16, 32, 64, 128, 192, 256]),
+                                        (1008, 48, [16]), (8, 8, [16, 128])])
+def test_linear_column_tile_is_whole_chunks_for_every_output_width(O, Bo, takes):
+    """`variant` of path 5: what the header promises for each width O and nothing else (a tile of 40 columns left 8 of 40 unwritten)."""
+    kw = dict(M=512, I=512, O=O, Bo=Bo, Bi=64, keep_cols=32)
+    for v in (1, 8, 15, 17, 20, 24, 40, 72, 100, 200, 250, 257, 264, 512, *takes):
+        if v in takes:
+            assert _linear_query(kw, 5, variant=v) == 5, v
+        else:
+            for path in (5, 6):
+                with pytest.raises(npas.NpasError) as e:
+                    _linear_query(kw, path, variant=v)
+                assert e.value.code == UNSUPPORTED, v
+            assert _linear_query(kw, 0, variant=v) not in (5, 6), v
+
+
 def test_sweep_shape_choices():
     """64x28x28x512 -> 512: kept pairs only where measured faster (up to 3 of 9 taps at 16x16 blocks, up to 4
     of 9 at 32x32), the CTA-pair dense-image kernel elsewhere, also for the block sizes below 16."""

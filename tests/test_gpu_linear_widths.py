@@ -26,3 +26,17 @@ def test_ragged_column_tiles(M, I, O, path, bn):
         npas.check_device_status(ws)
         assert floored_rel_err(host(y), ref) < TOL_BF16
         assert torch.equal(y, f())
+
+
+@pytest.mark.parametrize("bn", [16, 32, 48, 80, 112, 128, 144, 192, 240, 256])
+@pytest.mark.parametrize("M,O", [(300, 1000), (129, 24)])
+def test_requested_tiles_where_16_does_not_divide_the_outputs(M, O, bn):
+    c = inputs.linear_case(M=M, I=192, O=O, Bo=8, Bi=64, keep_rows=5, keep_cols=48, dtype="bf16", seed=1402)
+    r = torch.randn(M, O, generator=torch.Generator().manual_seed(9)).to(torch.bfloat16)
+    blob, ws = npas.pack_bb(dev(c.w, "bf16"), c.row_keep, c.col_keep, c.Bo, c.Bi), npas.workspace()
+    ref = oracle.linear_bb(c.x, c.w, c.row_keep, c.col_keep, Bo=c.Bo, Bi=c.Bi, bias=c.bias, residual=r.double().numpy(), relu=c.relu)
+    for odt in (torch.bfloat16, torch.float32):
+        y = torch.full((M, O), float("nan"), dtype=odt, device="cuda")          # every element is written
+        npas.linear_bb(dev(c.x, "bf16"), blob, dev(c.bias), r.to(odt).cuda(), relu=c.relu, out=y, ws=ws, path=5, variant=bn)
+        npas.check_device_status(ws)
+        assert floored_rel_err(host(y), ref) < TOL_BF16
