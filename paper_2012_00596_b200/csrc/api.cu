@@ -1,5 +1,6 @@
 // C-ABI entry points that validate arguments and pick a kernel; see npas.h for the contract.
 #include "common.cuh"
+#include "internal_api.h"
 
 namespace npas {
 
@@ -218,9 +219,25 @@ npas_status npas_linear_bb_kernel(const npas_linear_desc *d, const npas_bb_desc 
     return *kernel_id ? NPAS_OK : NPAS_ERR_UNSUPPORTED;
 }
 
+// where a call of a chain stands in it -> how its kernels are launched
+static Launch launch_of(int32_t chain)
+{
+    Launch how;
+    how.plain = chain == NPAS_CHAIN_FIRST;
+    how.blob_ready = chain != NPAS_CHAIN_NONE;
+    return how;
+}
+
 npas_status npas_conv2d_bp(const npas_conv_desc *d, const npas_bp_desc *bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y, void *ws,
                            size_t ws_bytes, void *stream)
+{
+    return npas_internal_conv2d_bp(d, bp, x, blob, bias, res, y, ws, ws_bytes, NPAS_CHAIN_NONE, stream);
+}
+
+npas_status npas_internal_conv2d_bp(const npas_conv_desc *d, const npas_bp_desc *bp, const void *x,
+                                    const void *blob, const float *bias, const void *res, void *y, void *ws,
+                                    size_t ws_bytes, int32_t chain, void *stream)
 {
     npas_status s = check_conv_args(d, bp);
     if (s != NPAS_OK) return s;
@@ -236,15 +253,16 @@ npas_status npas_conv2d_bp(const npas_conv_desc *d, const npas_bp_desc *bp, cons
     const float *b = d->has_bias ? bias : nullptr;
     const void *r = d->has_residual ? res : nullptr;
     uint32_t *w = static_cast<uint32_t *>(ws);
+    const Launch how = launch_of(chain);
     switch (conv_kernel_for(*d, *bp)) {
-        case 1: return conv_simt_launch(*d, *bp, x, blob, b, r, y, st);
+        case 1: return conv_simt_launch(*d, *bp, x, blob, b, r, y, st, how);
         case 3: return conv_tc_launch(*d, *bp, x, blob, b, r, y, w, st);
-        case 5: return conv_stem_launch(*d, *bp, x, blob, b, y, w, st);
+        case 5: return conv_stem_launch(*d, *bp, x, blob, b, y, w, st, false, how);
         case 6:
-            if (conv_split(*d, *bp)) return conv_sk_launch(*d, *bp, x, blob, b, r, y, w, st);
-            return conv_dn_launch(*d, *bp, x, blob, b, r, y, w, st);
-        case 7: return conv_d2_launch(*d, *bp, x, blob, b, r, y, w, st);
-        case 8: return conv_kr_launch(*d, *bp, x, blob, b, r, y, w, st);
+            if (conv_split(*d, *bp)) return conv_sk_launch(*d, *bp, x, blob, b, r, y, w, st, how);
+            return conv_dn_launch(*d, *bp, x, blob, b, r, y, w, st, how);
+        case 7: return conv_d2_launch(*d, *bp, x, blob, b, r, y, w, st, how);
+        case 8: return conv_kr_launch(*d, *bp, x, blob, b, r, y, w, st, how);
     }
     return NPAS_ERR_UNSUPPORTED;
 }
@@ -252,6 +270,14 @@ npas_status npas_conv2d_bp(const npas_conv_desc *d, const npas_bp_desc *bp, cons
 npas_status npas_conv2d_bp_maxpool(const npas_conv_desc *d, const npas_bp_desc *bp, int32_t pool_r, int32_t pool_stride,
                                    int32_t pool_pad, const void *x, const void *blob, const float *bias, void *y_pooled,
                                    void *ws, size_t ws_bytes, void *stream)
+{
+    return npas_internal_conv2d_bp_maxpool(d, bp, pool_r, pool_stride, pool_pad, x, blob, bias, y_pooled, ws, ws_bytes,
+                                           NPAS_CHAIN_NONE, stream);
+}
+
+npas_status npas_internal_conv2d_bp_maxpool(const npas_conv_desc *d, const npas_bp_desc *bp, int32_t pool_r, int32_t pool_stride,
+                                            int32_t pool_pad, const void *x, const void *blob, const float *bias, void *y_pooled,
+                                            void *ws, size_t ws_bytes, int32_t chain, void *stream)
 {
     npas_status s = check_conv_args(d, bp);
     if (s != NPAS_OK) return s;
@@ -268,12 +294,19 @@ npas_status npas_conv2d_bp_maxpool(const npas_conv_desc *d, const npas_bp_desc *
         !conv_stem_pool_supported(*d, *bp))
         return NPAS_ERR_UNSUPPORTED;
     return conv_stem_launch(*d, *bp, x, blob, d->has_bias ? bias : nullptr, y_pooled, static_cast<uint32_t *>(ws),
-                            static_cast<cudaStream_t>(stream), true);
+                            static_cast<cudaStream_t>(stream), true, launch_of(chain));
 }
 
 npas_status npas_linear_bb(const npas_linear_desc *d, const npas_bb_desc *bb, const void *x,
                            const void *blob, const float *bias, const void *residual, void *y, void *ws,
                            size_t ws_bytes, void *stream)
+{
+    return npas_internal_linear_bb(d, bb, x, blob, bias, residual, y, ws, ws_bytes, NPAS_CHAIN_NONE, stream);
+}
+
+npas_status npas_internal_linear_bb(const npas_linear_desc *d, const npas_bb_desc *bb, const void *x,
+                                    const void *blob, const float *bias, const void *residual, void *y, void *ws,
+                                    size_t ws_bytes, int32_t chain, void *stream)
 {
     npas_status s = check_linear_args(d, bb);
     if (s != NPAS_OK) return s;
@@ -289,13 +322,14 @@ npas_status npas_linear_bb(const npas_linear_desc *d, const npas_bb_desc *bb, co
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const float *b = d->has_bias ? bias : nullptr;
     uint32_t *w = static_cast<uint32_t *>(ws);
+    const Launch how = launch_of(chain);
     switch (linear_kernel_for(*d, *bb)) {
-        case 1: return linear_simt_launch(*d, *bb, x, blob, b, r, y, st);
+        case 1: return linear_simt_launch(*d, *bb, x, blob, b, r, y, st, how);
         case 3: return linear_tc_launch(*d, *bb, x, blob, b, r, y, w, st);
         case 5:
-            if (linear_split_k(*d, *bb)) return linear_sk_launch(*d, *bb, x, blob, b, r, y, w, st);
-            return linear_dn_launch(*d, *bb, x, blob, b, r, y, w, st);
-        case 6: return linear_d2_launch(*d, *bb, x, blob, b, r, y, w, st);
+            if (linear_split_k(*d, *bb)) return linear_sk_launch(*d, *bb, x, blob, b, r, y, w, st, how);
+            return linear_dn_launch(*d, *bb, x, blob, b, r, y, w, st, how);
+        case 6: return linear_d2_launch(*d, *bb, x, blob, b, r, y, w, st, how);
     }
     return NPAS_ERR_UNSUPPORTED;
 }

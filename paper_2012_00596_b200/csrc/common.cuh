@@ -178,13 +178,19 @@ inline bool cached_plan(const D &d, const B &b, int tag, P &p, F make)
 }
 npas_status allow_dynamic_smem(const void *kernel, int bytes);     // once per (kernel, device)
 
+// How a compute kernel follows what is ahead of it in its stream (launch_pdl in tc_common.cuh has the rule).
+struct Launch {
+    bool plain = false;            // after everything ahead of it has ended, instead of as a programmatic dependent
+    bool blob_ready = false;       // nothing has written the blob since before a launch of this chain that was `plain`
+};
+
 // Words of the caller's workspace.
 enum WsWord { WS_STATUS = 0, WS_DETAIL = 1 };
 
 // ---- kernels implemented in the other translation units (host launchers) ------------------------
 npas_status conv_simt_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                              const void *blob, const float *bias, const void *res, void *y,
-                             cudaStream_t st);
+                             cudaStream_t st, Launch how);
 bool conv_tc_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 npas_status conv_tc_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
@@ -193,48 +199,48 @@ bool conv_stem_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 bool conv_stem_pool_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 npas_status conv_stem_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                              const void *blob, const float *bias, void *y, uint32_t *ws, cudaStream_t st,
-                             bool pool = false);
+                             bool pool, Launch how);
 bool conv_stem_rows_supported(const npas_conv_desc &d, const npas_bp_desc &bp, bool pool);
 npas_status conv_stem_rows_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x, const void *blob,
-                                  const float *bias, void *y, uint32_t *ws, cudaStream_t st, bool pool);
+                                  const float *bias, void *y, uint32_t *ws, cudaStream_t st, bool pool, Launch how);
 bool conv_dn_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 npas_status conv_dn_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
-                           uint32_t *ws, cudaStream_t st);
+                           uint32_t *ws, cudaStream_t st, Launch how);
 bool conv_sk_preferred(const npas_conv_desc &d, const npas_bp_desc &bp);
 bool conv_sk_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 npas_status conv_sk_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
-                           uint32_t *ws, cudaStream_t st);
+                           uint32_t *ws, cudaStream_t st, Launch how);
 bool conv_d2_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 bool conv_d2_preferred(const npas_conv_desc &d, const npas_bp_desc &bp);
 double conv_dense_modelled(const npas_conv_desc &d, const npas_bp_desc &bp);
 bool conv_sk_slower(const npas_conv_desc &d, const npas_bp_desc &bp);
 npas_status conv_d2_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
-                           uint32_t *ws, cudaStream_t st);
+                           uint32_t *ws, cudaStream_t st, Launch how);
 bool conv_kr_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 bool conv_kr_preferred(const npas_conv_desc &d, const npas_bp_desc &bp);
 npas_status conv_kr_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
-                           uint32_t *ws, cudaStream_t st);
+                           uint32_t *ws, cudaStream_t st, Launch how);
 npas_status linear_simt_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
-                               const void *blob, const float *bias, const void *res, void *y, cudaStream_t st);
+                               const void *blob, const float *bias, const void *res, void *y, cudaStream_t st, Launch how);
 bool linear_dn_supported(const npas_linear_desc &d, const npas_bb_desc &bb);
 float linear_dn_cost(const npas_linear_desc &d, const npas_bb_desc &bb);
 npas_status linear_dn_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,
-                             cudaStream_t st);
+                             cudaStream_t st, Launch how);
 bool linear_sk_supported(const npas_linear_desc &d, const npas_bb_desc &bb);
 bool linear_sk_preferred(const npas_linear_desc &d, const npas_bb_desc &bb);
 npas_status linear_sk_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,
-                             cudaStream_t st);
+                             cudaStream_t st, Launch how);
 bool linear_d2_supported(const npas_linear_desc &d, const npas_bb_desc &bb);
 float linear_d2_cost(const npas_linear_desc &d, const npas_bb_desc &bb);
 npas_status linear_d2_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,
-                             cudaStream_t st);
+                             cudaStream_t st, Launch how);
 bool linear_tc_supported(const npas_linear_desc &d, const npas_bb_desc &bb);
 npas_status linear_tc_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,

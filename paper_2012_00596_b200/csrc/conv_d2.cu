@@ -55,7 +55,7 @@ struct ConvD2Params {
     int IT, img_pitch;                                        // small maps: IT whole images per tile, img_pitch positions apart
     int RS, nCh, nBlk, GH, NT, MT, CPW, n_fsets, n_items, SA, SB, nacc, dcols;   // GH: filters per CTA, NT = 2 GH per item; CPW: chunks per weight stage
     int GI;                                                   // filters per group of the blob's operand image (128, or 64 when 128 does not divide K)
-    int relu, y_bf16;
+    int relu, y_bf16, early;                                  // early: the blob may be read before the wait (Launch::blob_ready)
     uint32_t slab_bytes, act_stride, a_stage_bytes, w_bytes, off_w, off_tapu, off_bias, off_bar, smem_bytes, tmem_cols;
     uint32_t shift16[kMaxTapsD2];                             // operand start of every tap inside a tile's slabs, 16-byte units
     uint32_t w_box_rows;                                      // 128-byte rows of the blob per weight copy (the weight map's box)
@@ -121,10 +121,13 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_ctarank();                  // 0: leader (issues the MMAs), 1: its peer
     const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-    const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
-    // (the header's words on their way while the barriers are set up: the blob is never written by a kernel that lets its
-    // successor start early)
-    const uint32_t off_tapu = hdr[BP_OFF_TAPU], off_image = hdr[BP_OFF_IMAGE], image_gi = hdr[BP_GI];
+    // (in a chain of layers the header's words are on their way while the barriers are set up)
+    uint32_t off_tapu = 0, off_image = 0, image_gi = 0;
+    auto read_header = [&]() {
+        const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
+        off_tapu = hdr[BP_OFF_TAPU]; off_image = hdr[BP_OFF_IMAGE]; image_gi = hdr[BP_GI];
+    };
+    if (p.early) read_header();
     const uint32_t peer_abort = map_to_cta(smem_u32(&bars->abort_flag), rank ^ 1u);
 
     if (tid == 0) {
@@ -149,10 +152,11 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     __syncthreads();
     cluster_sync_relaxed();             // barriers of both CTAs exist before anything arrives on them
     tc_fence_after_sync();
-    // Only the activations, the biases and the residual may come from the kernel before this one: the weight producer and the
-    // tap unions do not wait for its end.
+    // In a chain of layers only the activations, the biases and the residual come from the kernel before this one: the weight
+    // producer and the tap unions do not wait for its end.
     const uint32_t tmem_base = bars->tmem_base;
-    if (warp == 0) pdl_wait();
+    if (warp == 0 || !p.early) pdl_wait();
+    if (!p.early) read_header();
     // the two producers start at once; the other warps first stage the tap unions
     if (warp != 0 && warp != 2) {
         const int t = tid < 64 ? tid - 32 : tid - 64;         // 0 .. kThreads - 65 over warps 1, 3, 4, ...
@@ -640,7 +644,7 @@ double conv_dense_modelled(const npas_conv_desc &d, const npas_bp_desc &bp)
 
 npas_status conv_d2_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
-                           uint32_t *ws, cudaStream_t st)
+                           uint32_t *ws, cudaStream_t st, Launch how)
 {
     ConvD2Params p;
     const int pairs = pairs_available();
@@ -696,7 +700,8 @@ npas_status conv_d2_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
     }
     if (allow_dynamic_smem(reinterpret_cast<const void *>(conv_bp_d2_kernel), (int)kSmemLimit) != NPAS_OK) return NPAS_ERR_CUDA;
     const int n_pairs = p.n_items < pairs ? p.n_items : pairs;
-    const cudaError_t e = launch_pdl(conv_bp_d2_kernel, dim3(2 * n_pairs), dim3(kThreads), p.smem_bytes, st, tmap, tmap_w, p,
+    p.early = how.blob_ready;
+    const cudaError_t e = launch_pdl(how, conv_bp_d2_kernel, dim3(2 * n_pairs), dim3(kThreads), p.smem_bytes, st, tmap, tmap_w, p,
                                      static_cast<const uint8_t *>(blob), bias, res, y, ws);
     count_launch();
     return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;

@@ -435,7 +435,7 @@ bool conv_dn_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 
 npas_status conv_dn_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
-                           uint32_t *ws, cudaStream_t st)
+                           uint32_t *ws, cudaStream_t st, Launch how)
 {
     ConvDnParams p;
     const int sms = sm_count();
@@ -455,7 +455,7 @@ npas_status conv_dn_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
         return NPAS_ERR_CUDA;
     if (allow_dynamic_smem(reinterpret_cast<const void *>(conv_bp_dn_kernel), (int)kSmemLimit) != NPAS_OK) return NPAS_ERR_CUDA;
     const int grid = p.n_items < sms ? p.n_items : sms;
-    const cudaError_t e = launch_pdl(conv_bp_dn_kernel, dim3(grid), dim3(kThreads), p.smem_bytes, st, tmap, p,
+    const cudaError_t e = launch_pdl(how, conv_bp_dn_kernel, dim3(grid), dim3(kThreads), p.smem_bytes, st, tmap, p,
                                      static_cast<const uint8_t *>(x), static_cast<const uint8_t *>(blob), bias, res, y, ws);
     count_launch();
     return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;

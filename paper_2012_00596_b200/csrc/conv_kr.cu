@@ -69,7 +69,7 @@ struct ConvKrParams {
     int Mb, GS, SEG, NA, RS, nGrp;
     int nChunks, cps, nStages, PPS, SA, NWS, nabuf, NP, cpb, nCB, max_taps;
     uint32_t oct_bytes, row_bytes, row_pitch, act_stage_bytes, wcap, bufcols, tile_bytes;
-    int relu, y_bf16;
+    int relu, y_bf16, early;     // early: the blob may be read before the wait (Launch::blob_ready)
     uint32_t off_act, off_w, off_cm, off_kto, off_rec, off_bar, smem_bytes;
     int RW;                      // words per (issuing warp, chunk) record list: count + MMAs, a multiple of 4
     int epi_tma;                 // bf16 output leaves through shared memory and tensor stores (64-filter slabs)
@@ -294,7 +294,7 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     pdl_trigger();
     if (tid < kMaxTaps) bars->tapoff[tid] = tid < p.RS ? (uint32_t)(tid / p.S) * p.row_pitch + (uint32_t)(tid % p.S) * 16u : 0u;
     __syncthreads();
-    // (the blob is never written by a kernel that lets its successor start early: no need to wait for the kernel before)
+    if (!p.early) pdl_wait();
     // the blob must be what the descriptor says: version, the tile section and its grouping
     const bool hdr_ok = hdr[BP_MAGIC] == kMagicBP && hdr[BP_VERSION] == kVersion && hdr[BP_OFF_KT] != 0u &&
                         hdr[BP_GS] == (uint32_t)p.GS && hdr[BP_MB] == (uint32_t)p.Mb && hdr[BP_NCB] == (uint32_t)p.nCB;
@@ -788,7 +788,7 @@ bool conv_kr_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
 
 npas_status conv_kr_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
-                           uint32_t *ws, cudaStream_t st)
+                           uint32_t *ws, cudaStream_t st, Launch how)
 {
     ConvKrParams p;
     dim3 grid;
@@ -818,7 +818,8 @@ npas_status conv_kr_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
             return NPAS_ERR_CUDA;
     }
     if (allow_dynamic_smem(reinterpret_cast<const void *>(conv_bp_kr_kernel), (int)kSmemLimit) != NPAS_OK) return NPAS_ERR_CUDA;
-    const cudaError_t e = launch_pdl(conv_bp_kr_kernel, grid, dim3(kThreads), p.smem_bytes, st, tmap, tmy, p,
+    p.early = how.blob_ready;
+    const cudaError_t e = launch_pdl(how, conv_bp_kr_kernel, grid, dim3(kThreads), p.smem_bytes, st, tmap, tmy, p,
                                      static_cast<const uint8_t *>(blob), bias, res, y, ws);
     count_launch();
     return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;

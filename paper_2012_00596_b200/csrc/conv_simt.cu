@@ -135,7 +135,7 @@ conv_bp_simt_kernel(npas_conv_desc d, int Mb, int Nb_, int P, int Q, int KW, con
 
 template <typename TX, typename TY>
 static npas_status launch(const npas_conv_desc &d, const npas_bp_desc &bp, int P, int Q, const void *x, const void *blob,
-                          const float *bias, const void *res, void *y, cudaStream_t st)
+                          const float *bias, const void *res, void *y, cudaStream_t st, Launch how)
 {
     const long long npix = (long long)d.N * P * Q, fgroups = (long long)(bp.K / bp.Mb) * ((bp.Mb + kFilters - 1) / kFilters);
     // shares of the pairs: as many as leave a warp eight steps, more while there are not two CTAs per SM
@@ -147,7 +147,7 @@ static npas_status launch(const npas_conv_desc &d, const npas_bp_desc &bp, int P
     const dim3 grid((unsigned)((npix + tile - 1) / tile), bp.K / bp.Mb, (bp.Mb + kFilters - 1) / kFilters);
     if (grid.y > 65535 || grid.z > 65535) return NPAS_ERR_UNSUPPORTED;
     auto go = [&](auto kernel) {
-        return tc::launch_pdl(kernel, grid, dim3(kWarps * 32), 0, st, d, (int)bp.Mb, (int)bp.Nb, P, Q, KW, static_cast<const TX *>(x),
+        return tc::launch_pdl(how, kernel, grid, dim3(kWarps * 32), 0, st, d, (int)bp.Mb, (int)bp.Nb, P, Q, KW, static_cast<const TX *>(x),
                               static_cast<const uint8_t *>(blob), bias, static_cast<const TY *>(res), static_cast<TY *>(y));
     };
     const cudaError_t e = bp.Nb == 4 ? go(conv_bp_simt_kernel<TX, TY, 4>) : bp.Nb == 8 ? go(conv_bp_simt_kernel<TX, TY, 8>) : go(conv_bp_simt_kernel<TX, TY, 0>);
@@ -157,12 +157,12 @@ static npas_status launch(const npas_conv_desc &d, const npas_bp_desc &bp, int P
 
 npas_status conv_simt_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                              const void *blob, const float *bias, const void *res, void *y,
-                             cudaStream_t st)
+                             cudaStream_t st, Launch how)
 {
     const int P = (d.H + 2 * d.pad - d.R) / d.stride + 1, Q = (d.W + 2 * d.pad - d.S) / d.stride + 1;
-    if (d.x_dtype == NPAS_F32 && d.y_dtype == NPAS_F32) return launch<float, float>(d, bp, P, Q, x, blob, bias, res, y, st);
-    if (d.x_dtype == NPAS_BF16 && d.y_dtype == NPAS_BF16) return launch<uint16_t, uint16_t>(d, bp, P, Q, x, blob, bias, res, y, st);
-    if (d.x_dtype == NPAS_BF16 && d.y_dtype == NPAS_F32) return launch<uint16_t, float>(d, bp, P, Q, x, blob, bias, res, y, st);
+    if (d.x_dtype == NPAS_F32 && d.y_dtype == NPAS_F32) return launch<float, float>(d, bp, P, Q, x, blob, bias, res, y, st, how);
+    if (d.x_dtype == NPAS_BF16 && d.y_dtype == NPAS_BF16) return launch<uint16_t, uint16_t>(d, bp, P, Q, x, blob, bias, res, y, st, how);
+    if (d.x_dtype == NPAS_BF16 && d.y_dtype == NPAS_F32) return launch<uint16_t, float>(d, bp, P, Q, x, blob, bias, res, y, st, how);
     return NPAS_ERR_DTYPE;
 }
 

@@ -15,8 +15,8 @@
 // groups x (chunk, tap, octet) rows lands as [tap][octet][NT filters][8], whatever the image's group width, so NT is any
 // multiple of 16 that groups can make up (one MMA covers 176 filters where the image has groups of 16).
 //
-// What bounds it is the latency of the chain copy, MMAs, exchange, store: the weights are requested before the
-// programmatic wait (no kernel that lets its successor start early writes them), the slabs right behind it.
+// What bounds it is the latency of the chain copy, MMAs, exchange, store: the weights are requested by a warp of their own, in
+// a chain of layers before the programmatic wait (`early`), the slabs right behind it.
 #include "common.cuh"
 #include "tc_pair.cuh"
 
@@ -42,7 +42,7 @@ struct ConvSkParams {
     int nph, Wp, TR, tiles_per_img, n_tiles, slab_rows;
     int RS, nCh, CB, nBlk, NT, nFT, KC, KT, bpr, tpr;     // bpr: channel blocks per CTA; tpr: taps per CTA
     int GI, lines, S, rpr;
-    int relu, y_bf16, use_taps;
+    int relu, y_bf16, use_taps, early;                    // early: the blob may be read before the wait (Launch::blob_ready)
     uint32_t desc_hi_a, slab_bytes, act_stride, w_chunk, stage_bytes, red_pitch, off_red, off_bias, off_bar, smem_bytes, tmem_cols;
     uint32_t shift16[kMaxTapsSk];                         // operand start of every tap inside a stage's slabs, 16-byte units
 };
@@ -109,6 +109,7 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
     cluster_arrive();                  // this CTA is running: its shared memory may be written by the others
+    if (!p.early) pdl_wait();
 
     if (warp == 2) {
         // ---- weights: one box per 16-channel chunk; the first ring of stages before anything else ------------------
@@ -449,7 +450,7 @@ bool conv_sk_slower(const npas_conv_desc &d, const npas_bp_desc &bp)
 }
 
 npas_status conv_sk_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x, const void *blob, const float *bias,
-                           const void *res, void *y, uint32_t *ws, cudaStream_t st)
+                           const void *res, void *y, uint32_t *ws, cudaStream_t st, Launch how)
 {
     ConvSkParams p;
     const bool one_wave = !d.variant && planned(d, bp, p, true) && (d.stride != 1 || p.n_tiles * 2 <= sm_count());     // (as it was chosen)
@@ -478,7 +479,8 @@ npas_status conv_sk_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
         return NPAS_ERR_CUDA;
     if (allow_dynamic_smem(reinterpret_cast<const void *>(conv_bp_sk_kernel), (int)kSmemLimit) != NPAS_OK) return NPAS_ERR_CUDA;
     const int KS = p.KC * p.KT;
-    const cudaError_t e = launch_pdl_cluster(conv_bp_sk_kernel, dim3(p.n_tiles * p.nFT * KS), dim3(kThreads), KS, p.smem_bytes, st, tmx, tmw, p,
+    p.early = how.blob_ready;
+    const cudaError_t e = launch_pdl_cluster(how, conv_bp_sk_kernel, dim3(p.n_tiles * p.nFT * KS), dim3(kThreads), KS, p.smem_bytes, st, tmx, tmw, p,
                                              static_cast<const uint8_t *>(blob), bias, res, y, ws);
     count_launch();
     return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;

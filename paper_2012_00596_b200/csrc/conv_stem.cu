@@ -383,10 +383,10 @@ bool conv_stem_pool_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 }
 
 npas_status conv_stem_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
-                             const void *blob, const float *bias, void *y, uint32_t *ws, cudaStream_t st, bool pool)
+                             const void *blob, const float *bias, void *y, uint32_t *ws, cudaStream_t st, bool pool, Launch how)
 {
     // whole rows per step where a row fits one MMA tile (W <= 256) and the filters fit (K <= 128)
-    if (conv_stem_rows_supported(d, bp, pool)) return conv_stem_rows_launch(d, bp, x, blob, bias, y, ws, st, pool);
+    if (conv_stem_rows_supported(d, bp, pool)) return conv_stem_rows_launch(d, bp, x, blob, bias, y, ws, st, pool, how);
     StemParams p;
     if (!plan(d, bp, p, pool)) return NPAS_ERR_UNSUPPORTED;
     // the pooled tensor is built by max-reductions: it starts as zeros (no value is negative after ReLU)

@@ -46,7 +46,7 @@ constexpr uint32_t kSmemLimit = 232448;
 constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);   // SBO = 128 bytes, descriptor version bit
 
 struct StemRowsParams {
-    int N, H, W, K, P, Q, Mb, relu, y_bf16;
+    int N, H, W, K, P, Q, Mb, relu, y_bf16, early;  // early: the blob may be read before the wait (Launch::blob_ready)
     int PP, PQ, pairs, n_steps;                    // pooled height / width; pixel pairs of a row; steps in all (images x row pairs)
     int spi;                                       // steps per image
     uint32_t pitch, line, off_b, off_stage, stage_bytes, off_bar, smem_bytes, tmem_cols;
@@ -119,8 +119,8 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
     for (uint32_t o = tid * 16; o < p.off_stage; o += kThreads<kPool> * 16) *reinterpret_cast<uint4 *>(smem + o) = make_uint4(0, 0, 0, 0);
     __syncthreads();
     {
-        // weight of (tap (r, s), channel c, filter n) at k = s * 4 + c of kernel row r.  (The blob is never written by a
-        // kernel that lets its successor start early: no need to wait for the kernel before this one.)
+        // weight of (tap (r, s), channel c, filter n) at k = s * 4 + c of kernel row r
+        if (!p.early) pdl_wait();
         const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
         const uint32_t *blk_off = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_BLK]);
         const uint32_t *pairs = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_PAIRS]);
@@ -462,14 +462,15 @@ bool conv_stem_rows_supported(const npas_conv_desc &d, const npas_bp_desc &bp, b
 }
 
 npas_status conv_stem_rows_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x, const void *blob, const float *bias,
-                                  void *y, uint32_t *ws, cudaStream_t st, bool pool)
+                                  void *y, uint32_t *ws, cudaStream_t st, bool pool, Launch how)
 {
     StemRowsParams p;
     if (!plan(d, bp, p, pool)) return NPAS_ERR_UNSUPPORTED;
+    p.early = how.blob_ready;
     auto go = [&](auto kernel, int threads) {
         if (allow_dynamic_smem(reinterpret_cast<const void *>(kernel), (int)kSmemLimit) != NPAS_OK) return cudaErrorUnknown;
         const int sms = sm_count(), grid = p.n_steps < sms ? p.n_steps : sms;
-        return launch_pdl(kernel, dim3(grid), dim3(threads), p.smem_bytes, st, p, static_cast<const uint16_t *>(x),
+        return launch_pdl(how, kernel, dim3(grid), dim3(threads), p.smem_bytes, st, p, static_cast<const uint16_t *>(x),
                           static_cast<const uint8_t *>(blob), bias, y, ws);
     };
     const cudaError_t e = pool ? go(conv_stem_rows_kernel<true>, kThreads<true>) : go(conv_stem_rows_kernel<false>, kThreads<false>);

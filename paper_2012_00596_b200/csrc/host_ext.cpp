@@ -22,7 +22,7 @@
 #include <vector>
 
 #include "npas.h"
-#include "pack_api.h"
+#include "internal_api.h"
 
 namespace {
 
@@ -668,6 +668,8 @@ PyObject *stack_forward(PyObject *, PyObject *const *a, Py_ssize_t nargs)
             const void *in = st.in_at < 0 ? xin : base + st.in_at, *res = st.res_at < 0 ? nullptr : base + st.res_at;
             void *out = st.out < 0 ? yout : base + st.out;
             at_layer = i;
+            // nothing in this call writes a blob, and a layer beside starts behind an event recorded after the first layer
+            const int32_t chain = i == 0 ? NPAS_CHAIN_FIRST : NPAS_CHAIN_LATER;
             const bool beside = from[(size_t)i] >= 0;
             void *stream = beside ? side.stream : main;
             if (pending >= 0 && join[(size_t)pending] == i) {
@@ -681,11 +683,11 @@ PyObject *stack_forward(PyObject *, PyObject *const *a, Py_ssize_t nargs)
                     if (s != NPAS_OK) break;
                     in = base + st.sub;
                 }
-                s = npas_linear_bb(&st.ld, &st.bb, in, st.blob, st.bias, res, out, w, wb, stream);
+                s = npas_internal_linear_bb(&st.ld, &st.bb, in, st.blob, st.bias, res, out, w, wb, chain, stream);
             } else if (r.kind == 0) {
-                s = npas_conv2d_bp_maxpool(&st.cd, &st.bp, 3, 2, 1, in, st.blob, st.bias, out, w, wb, stream);
+                s = npas_internal_conv2d_bp_maxpool(&st.cd, &st.bp, 3, 2, 1, in, st.blob, st.bias, out, w, wb, chain, stream);
             } else {
-                s = npas_conv2d_bp(&st.cd, &st.bp, in, st.blob, st.bias, res, out, w, wb, stream);
+                s = npas_internal_conv2d_bp(&st.cd, &st.bp, in, st.blob, st.bias, res, out, w, wb, chain, stream);
             }
             if (beside && s == NPAS_OK && cudaEventRecord(side.done, side.stream) != cudaSuccess) s = NPAS_ERR_CUDA;
             if (s == NPAS_OK && begins[(size_t)i] >= 0) {

@@ -47,8 +47,6 @@ npas_status allow_dynamic_smem(const void *kernel, int bytes)
 
 namespace tc {
 
-bool pdl_enabled() { return true; }
-
 EncodeTiledFn encode_tiled_fn()
 {
     static EncodeTiledFn fn = nullptr;

@@ -1,0 +1,34 @@
+// What the Python binding's native code calls beside the C ABI in npas.h.
+//
+// Packing without the read-back: for callers that have counted the very masks they pass, so that the blob's size is right by
+// construction and nothing has to be asked of the device.
+//
+// Chains: several compute calls that one caller makes in a row, with nothing in between that could write one of their blobs.
+// The first is launched after everything ahead of it in the stream has ended; the others may then fetch their weights while
+// the kernel ahead of them still runs (the rule is at launch_pdl in tc_common.cuh).  A call on another stream belongs to the
+// chain when that stream has waited for an event recorded after the chain's first call.
+#pragma once
+#include "npas.h"
+
+#ifdef __cplusplus
+extern "C" {
+#endif
+// size of the blob with n_pairs kept (block, tap) pairs / n_vals stored values (each block's rounded up to 8) and max_cols
+// kept columns in the fullest block
+npas_status npas_internal_bp_size(const npas_bp_desc *d, uint64_t n_pairs, size_t *blob_bytes);
+npas_status npas_internal_bb_size(const npas_bb_desc *d, uint64_t n_vals, uint32_t max_cols, size_t *blob_bytes);
+// the pack calls up to, but without, their synchronisation
+npas_status npas_internal_pack_bp(const npas_bp_desc *d, const void *w, const uint64_t *tap_mask, void *blob, size_t blob_bytes, void *stream);
+npas_status npas_internal_pack_bb(const npas_bb_desc *d, const void *w, const uint64_t *rk, const uint64_t *ck, void *blob,
+                                  size_t blob_bytes, void *stream);
+enum { NPAS_CHAIN_NONE = 0, NPAS_CHAIN_FIRST = 1, NPAS_CHAIN_LATER = 2 };
+npas_status npas_internal_conv2d_bp(const npas_conv_desc *d, const npas_bp_desc *bp, const void *x, const void *blob, const float *bias,
+                                    const void *residual, void *y, void *ws, size_t ws_bytes, int32_t chain, void *stream);
+npas_status npas_internal_conv2d_bp_maxpool(const npas_conv_desc *d, const npas_bp_desc *bp, int32_t pool_r, int32_t pool_stride,
+                                            int32_t pool_pad, const void *x, const void *blob, const float *bias, void *y_pooled,
+                                            void *ws, size_t ws_bytes, int32_t chain, void *stream);
+npas_status npas_internal_linear_bb(const npas_linear_desc *d, const npas_bb_desc *bb, const void *x, const void *blob, const float *bias,
+                                    const void *residual, void *y, void *ws, size_t ws_bytes, int32_t chain, void *stream);
+#ifdef __cplusplus
+}
+#endif

@@ -42,7 +42,7 @@ constexpr uint32_t kDescLboOne = 1u << 16;                // LBO is not used by 
 
 struct LinD2Params {
     int M, I, O, BN, nK, nMT, nNT, n_tiles, S;
-    int relu, y_bf16;
+    int relu, y_bf16, early;                              // early: the blob may be read before the wait (Launch::blob_ready)
     int NS;                                               // epilogue slots (0: epilogue straight from registers)
     uint32_t stage_bytes, off_slots, off_bias, off_bar, smem_bytes, tmem_cols;
     float cost;                                           // modelled microseconds
@@ -117,10 +117,10 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     __syncthreads();
     cluster_sync_relaxed();             // barriers of both CTAs exist before anything arrives on them
     tc_fence_after_sync();
-    // The weights of the first ring of stages are requested before the wait for the kernel before this one: no kernel that
-    // lets its successor start early writes them.
+    // The weights of the first ring of stages; in a chain of layers before the wait for the kernel before this one.
     int early = 0;
     if (warp == 0 && lane == 0) {
+        if (!p.early) pdl_wait();
         int tile = pair, k = 0;
         for (; early < p.S && tile < p.n_tiles; ++early) {
             if (rank == 0) mbar_arrive_expect_tx(&bars->full[early], 2u * p.stage_bytes);
@@ -484,7 +484,7 @@ bool linear_d2_supported(const npas_linear_desc &d, const npas_bb_desc &bb)
 
 npas_status linear_d2_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,
-                             cudaStream_t st)
+                             cudaStream_t st, Launch how)
 {
     LinD2Params p;
     if (!planned(d, bb, p)) return NPAS_ERR_UNSUPPORTED;
@@ -505,7 +505,8 @@ npas_status linear_d2_launch(const npas_linear_desc &d, const npas_bb_desc &bb, 
     const int sms = sm_count();
     const int n_pairs = p.n_tiles < sms / 2 ? p.n_tiles : sms / 2;
     if (n_pairs < 1) return NPAS_ERR_UNSUPPORTED;
-    const cudaError_t e = launch_pdl(linear_bb_d2_kernel, dim3(2 * n_pairs), dim3(kThreads), p.smem_bytes, st, tmx, tmw, tmy, tmr,
+    p.early = how.blob_ready;
+    const cudaError_t e = launch_pdl(how, linear_bb_d2_kernel, dim3(2 * n_pairs), dim3(kThreads), p.smem_bytes, st, tmx, tmw, tmy, tmr,
                                      p, bias, res, y, ws);
     count_launch();
     return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;

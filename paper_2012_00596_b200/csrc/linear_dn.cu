@@ -47,7 +47,7 @@ constexpr uint32_t kDescLboOne = 1u << 16;                // LBO is not used by 
 
 struct LinDnParams {
     int M, I, O, BN, nK, nMT, nNT, n_tiles, S;
-    int relu, y_bf16;
+    int relu, y_bf16, early;                              // early: the blob may be read before the wait (Launch::blob_ready)
     int NS;                                               // epilogue slots (0: epilogue straight from registers)
     uint32_t stage_bytes, off_slots, off_bias, off_bar, smem_bytes, tmem_cols;
     float cost;                                           // modelled microseconds
@@ -96,13 +96,14 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     auto width = [&](int nt) { return min(p.BN, p.O - nt * p.BN); };
 
     // The producer starts by itself: it initialises the barriers it signals and requests the first ring of stages before the
-    // other warps have set up theirs and tensor memory (0.4 us).  The weights do not wait for the kernel before this one: no
-    // kernel that lets its successor start early writes them.
+    // other warps have set up theirs and tensor memory (0.4 us).  In a chain of layers the weights do not wait for the kernel
+    // before this one.
     int early = 0;
     if (tid == 0) {
         for (int s = 0; s < p.S; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], 1); }
         fence_barrier_init();
         fence_proxy_async_smem();
+        if (!p.early) pdl_wait();
         int tile = blockIdx.x, k = 0;
         for (; early < p.S && tile < p.n_tiles; ++early) {
             mbar_arrive_expect_tx(&bars->full[early], p.stage_bytes);
@@ -481,7 +482,7 @@ bool linear_dn_supported(const npas_linear_desc &d, const npas_bb_desc &bb)
 
 npas_status linear_dn_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,
-                             cudaStream_t st)
+                             cudaStream_t st, Launch how)
 {
     LinDnParams p;
     if (!planned(d, bb, p)) return NPAS_ERR_UNSUPPORTED;
@@ -501,7 +502,8 @@ npas_status linear_dn_launch(const npas_linear_desc &d, const npas_bb_desc &bb, 
     if (allow_dynamic_smem(reinterpret_cast<const void *>(linear_bb_dn_kernel), (int)kSmemLimit) != NPAS_OK) return NPAS_ERR_CUDA;
     const int sms = sm_count();
     const int grid = p.n_tiles < sms ? p.n_tiles : sms;
-    const cudaError_t e = launch_pdl(linear_bb_dn_kernel, dim3(grid), dim3(kThreads), p.smem_bytes, st, tmx, tmw, tmy, tmr,
+    p.early = how.blob_ready;
+    const cudaError_t e = launch_pdl(how, linear_bb_dn_kernel, dim3(grid), dim3(kThreads), p.smem_bytes, st, tmx, tmw, tmy, tmr,
                                      p, bias, res, y, ws);
     count_launch();
     return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;

@@ -177,26 +177,26 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
 
 template <typename TX, typename TY>
 static npas_status launch(const npas_linear_desc &d, const npas_bb_desc &bb, const BbLayout &L, dim3 grid, const void *x,
-                          const void *blob, const float *bias, const void *res, void *y, cudaStream_t st)
+                          const void *blob, const float *bias, const void *res, void *y, cudaStream_t st, Launch how)
 {
     const LinSimtSmem S = smem_plan(bb);
     auto k = linear_bb_simt_kernel<TX, TY>;
     if (allow_dynamic_smem(reinterpret_cast<const void *>(k), (int)S.bytes) != NPAS_OK) return NPAS_ERR_CUDA;
-    const cudaError_t e = tc::launch_pdl(k, grid, dim3(S.group_threads * S.groups), S.bytes, st, d, (int)bb.Bo, (int)bb.Bi, L, S, static_cast<const TX *>(x),
+    const cudaError_t e = tc::launch_pdl(how, k, grid, dim3(S.group_threads * S.groups), S.bytes, st, d, (int)bb.Bo, (int)bb.Bi, L, S, static_cast<const TX *>(x),
                                          static_cast<const uint8_t *>(blob), bias, static_cast<const TY *>(res), static_cast<TY *>(y));
     count_launch();
     return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;
 }
 
 npas_status linear_simt_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
-                               const void *blob, const float *bias, const void *res, void *y, cudaStream_t st)
+                               const void *blob, const float *bias, const void *res, void *y, cudaStream_t st, Launch how)
 {
     const BbLayout L = bb_layout(bb);
     const dim3 grid((d.M + kBM - 1) / kBM, L.nBo);
     if (grid.y > 65535) return NPAS_ERR_UNSUPPORTED;
-    if (d.x_dtype == NPAS_F32 && d.y_dtype == NPAS_F32) return launch<float, float>(d, bb, L, grid, x, blob, bias, res, y, st);
-    if (d.x_dtype == NPAS_BF16 && d.y_dtype == NPAS_BF16) return launch<uint16_t, uint16_t>(d, bb, L, grid, x, blob, bias, res, y, st);
-    if (d.x_dtype == NPAS_BF16 && d.y_dtype == NPAS_F32) return launch<uint16_t, float>(d, bb, L, grid, x, blob, bias, res, y, st);
+    if (d.x_dtype == NPAS_F32 && d.y_dtype == NPAS_F32) return launch<float, float>(d, bb, L, grid, x, blob, bias, res, y, st, how);
+    if (d.x_dtype == NPAS_BF16 && d.y_dtype == NPAS_BF16) return launch<uint16_t, uint16_t>(d, bb, L, grid, x, blob, bias, res, y, st, how);
+    if (d.x_dtype == NPAS_BF16 && d.y_dtype == NPAS_F32) return launch<uint16_t, float>(d, bb, L, grid, x, blob, bias, res, y, st, how);
     return NPAS_ERR_DTYPE;
 }
 

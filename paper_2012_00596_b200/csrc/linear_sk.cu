@@ -10,8 +10,8 @@
 // rounds once and stores 16 bytes per thread along the row.
 //
 // What bounds it: the latency of one pass through the chain (copy, MMA, exchange, barrier, store), so the first copies
-// are as early as possible: the weights (never written by a kernel that lets its successor start early) are requested
-// before the programmatic wait, X right after it; only the rows that exist are copied.
+// are as early as possible: in a chain of layers (`early`) the weights are requested before the programmatic wait, X right
+// after it; only the rows that exist are copied.
 #include "common.cuh"
 #include "tc_pair.cuh"
 
@@ -32,7 +32,7 @@ constexpr uint32_t kDescLboOne = 1u << 16;
 
 struct LinSkParams {
     int M, I, O, BN, KS, nK, kpr, nMT, nNT, S, XR, rpr;   // kpr: steps per CTA; XR: rows of X per copy; rpr: rows a CTA owns
-    int relu, y_bf16;
+    int relu, y_bf16, early;                              // early: the blob may be read before the wait (Launch::blob_ready)
     uint32_t x_bytes, stage_bytes, red_pitch, off_red, off_bias, off_bar, smem_bytes, tmem_cols;
 };
 
@@ -74,8 +74,8 @@ linear_bb_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         fence_barrier_init();
         prefetch_tensormap(&tmap_x);
         prefetch_tensormap(&tmap_w);
-        // the weights of the first ring of steps: nothing that may still be running writes them
-        for (int k = 0; k < min(k_n, p.S); ++k) {
+        // the weights of the first ring of steps
+        for (int k = 0; p.early && k < min(k_n, p.S); ++k) {
             mbar_arrive_expect_tx(&bars->full[k], p.stage_bytes);
             tma_load_2d(smem + (size_t)k * p.stage_bytes + p.x_bytes, &tmap_w, &bars->full[k], (k_lo + k) * 64, nt * p.BN);
         }
@@ -96,8 +96,8 @@ linear_bb_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         if (lane == 0) {
             uint32_t s = 0, lap = 0;
             for (int k = 0; k < k_n; ++k) {
-                if (lap >= 1) {
-                    if (!mbar_wait(&bars->empty[s], (lap & 1u) ^ 1u, abort_flag, ws, 0x9100)) break;
+                if (lap >= 1 && !mbar_wait(&bars->empty[s], (lap & 1u) ^ 1u, abort_flag, ws, 0x9100)) break;
+                if (lap >= 1 || !p.early) {
                     mbar_arrive_expect_tx(&bars->full[s], p.stage_bytes);
                     tma_load_2d(smem + (size_t)s * p.stage_bytes + p.x_bytes, &tmap_w, &bars->full[s], (k_lo + k) * 64, nt * p.BN);
                 }
@@ -303,7 +303,7 @@ bool linear_sk_preferred(const npas_linear_desc &d, const npas_bb_desc &bb)
 }
 
 npas_status linear_sk_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x, const void *blob, const float *bias,
-                             const void *res, void *y, uint32_t *ws, cudaStream_t st)
+                             const void *res, void *y, uint32_t *ws, cudaStream_t st, Launch how)
 {
     LinSkParams p;
     if (!planned(d, bb, p, true)) return NPAS_ERR_UNSUPPORTED;
@@ -322,7 +322,8 @@ npas_status linear_sk_launch(const npas_linear_desc &d, const npas_bb_desc &bb, 
     if (!encode(&tmx, x, (uint64_t)d.M, (uint32_t)p.XR) || !encode(&tmw, static_cast<const uint8_t *>(blob) + L.off_dense, (uint64_t)d.O, (uint32_t)p.BN))
         return NPAS_ERR_CUDA;
     if (allow_dynamic_smem(reinterpret_cast<const void *>(linear_bb_sk_kernel), (int)kSmemLimit) != NPAS_OK) return NPAS_ERR_CUDA;
-    const cudaError_t e = launch_pdl_cluster(linear_bb_sk_kernel, dim3(p.nMT * p.nNT * p.KS), dim3(kThreads), p.KS, p.smem_bytes, st,
+    p.early = how.blob_ready;
+    const cudaError_t e = launch_pdl_cluster(how, linear_bb_sk_kernel, dim3(p.nMT * p.nNT * p.KS), dim3(kThreads), p.KS, p.smem_bytes, st,
                                              tmx, tmw, p, bias, res, y, ws);
     count_launch();
     return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;

@@ -5,7 +5,7 @@
 // sections), then a grid writes the sections 16 bytes per thread.  (Clearing the blob first and placing two-byte values
 // one by one took twice the bytes and partial writes: 512x3x3x512 with 16x8 blocks 14 us of placing after 10 of scanning.)
 #include "common.cuh"
-#include "pack_api.h"
+#include "internal_api.h"
 #include "tc_common.cuh"
 
 namespace npas {
@@ -554,7 +554,7 @@ npas_status npas_internal_pack_bp(const npas_bp_desc *d, const void *w, const ui
         const uint32_t units = (uint32_t)d->K * d->R * d->S * (d->C / 8), unit_ctas = (units + 255) / 256;
         const uint32_t items = (uint32_t)(d->K / L.GI) * (d->C / 16), grid = unit_ctas + (items + 7) / 8;
         cudaError_t e = cudaSuccess;
-        auto go = [&](auto kernel, auto *wp) { e = tc::launch_pdl(kernel, dim3(grid), dim3(256), 0, st, *d, L, wp, tap_mask, b8, unit_ctas); };
+        auto go = [&](auto kernel, auto *wp) { e = tc::launch_pdl({}, kernel, dim3(grid), dim3(256), 0, st, *d, L, wp, tap_mask, b8, unit_ctas); };
         if (d->w_in == NPAS_F32) {
             if (d->Nb % 8 == 0) go(bp_expand_kernel<uint32_t, 8>, w32);
             else if (d->Nb % 4 == 0) go(bp_expand_kernel<uint32_t, 4>, w32);
@@ -660,7 +660,7 @@ npas_status npas_internal_pack_bb(const npas_bb_desc *d, const void *w, const ui
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     uint8_t *b8 = static_cast<uint8_t *>(blob);
     bb_scan_kernel<<<1, 1024, 0, st>>>(*d, rk, ck, b8, (uint32_t)blob_bytes, L);
-    auto go = [&](auto kernel, auto *wp) { return tc::launch_pdl(kernel, dim3(L.nBlk), dim3(256), 0, st, *d, wp, rk, ck, b8, L); };
+    auto go = [&](auto kernel, auto *wp) { return tc::launch_pdl({}, kernel, dim3(L.nBlk), dim3(256), 0, st, *d, wp, rk, ck, b8, L); };
     const uint32_t *w32 = static_cast<const uint32_t *>(w);
     const cudaError_t e = d->w_packed == NPAS_F32 ? go(bb_gather_kernel<uint32_t, uint32_t>, w32)
                           : d->w_in == NPAS_F32 ? go(bb_gather_kernel<uint32_t, uint16_t>, w32)

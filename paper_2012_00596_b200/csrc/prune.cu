@@ -369,7 +369,7 @@ npas_status npas_prune_bp_magnitude_global(const npas_bp_desc *d, const void *w,
     const int in_smem = most <= kSelSmemKeys;
     const size_t smem = in_smem ? (size_t)most * 8 : 0;
     if (allow_dynamic_smem(reinterpret_cast<const void *>(prune_select_kernel), (int)(kSelSmemKeys * 8)) != NPAS_OK) return NPAS_ERR_CUDA;
-    if (tc::launch_pdl_cluster(prune_select_kernel, dim3(ctas), dim3(kSelThreads), ctas, smem, st, reinterpret_cast<const unsigned long long *>(scores),
+    if (tc::launch_pdl_cluster({}, prune_select_kernel, dim3(ctas), dim3(kSelThreads), ctas, smem, st, reinterpret_cast<const unsigned long long *>(scores),
                                (long long)n_keep, RS, masks, nBlk, ctas, in_smem) != cudaSuccess)
         return NPAS_ERR_CUDA;
     count_launch(2);

@@ -9,6 +9,8 @@
 #include <stdint.h>
 #include <utility>
 
+#include "common.cuh"
+
 namespace npas {
 namespace tc {
 
@@ -218,23 +220,29 @@ __device__ __forceinline__ uint32_t relu_bf16x2(uint32_t v)
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Launch with the attribute set.  Only for kernels that execute pdl_wait() before their first
-// access to global memory.
-bool pdl_enabled();
+// Launch with the attribute set (unless `how.plain`).  What a kernel so launched may read before pdl_wait() is only what was
+// complete before the kernel ahead of it STARTED: that one may still be running, or have ended without its stores being
+// visible yet, whether it triggers or not.  So
+//   * by themselves the compute kernels touch no global memory before the wait, blobs included: the kernel ahead of them may
+//     be a packer, or a copy into the blob;
+//   * in a chain of launches that one call makes, the first of them plain, nothing writes a blob, and whatever did before is
+//     complete when the first one starts: the later ones are given `blob_ready` and fetch weights before the wait;
+//   * the second packing kernels read masks and weights before the wait (never the blob): the scan ahead of them is
+//     launched plainly and writes the blob only.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
+inline cudaError_t launch_pdl(Launch how, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = pdl_enabled() ? 1 : 0;
+    cfg.attrs = at; cfg.numAttrs = how.plain ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 // the same with clusters of `cluster` CTAs
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t st, Args &&...args)
+inline cudaError_t launch_pdl_cluster(Launch how, void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t st, Args &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
@@ -243,7 +251,7 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 
     at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = pdl_enabled() ? 2 : 1;
+    cfg.attrs = at; cfg.numAttrs = how.plain ? 1 : 2;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
