@@ -6,8 +6,12 @@
 // bytes each, so that output column q (stride 2) starts 16 q bytes into a row: eight consecutive columns are one core
 // matrix of the unswizzled K-major layout, and the next two pixels of the window are the core matrix 16 bytes further on.
 // The K-direction offset of the operand descriptor is therefore 16 bytes, core matrices overlap, and a kernel row is two
-// MMAs (K = 32: eight pixels x four channels, the eighth pixel meets zero weights, the fourth channel the bias) straight from the
-// rows.  Widening a row costs one 16-byte store per two pixels, once per row instead of once per window.
+// MMAs (K = 32: eight pixels x four channels, the fourth channel meets the bias) straight from the rows.  Widening a row costs
+// one 16-byte store per two pixels, once per row instead of once per window.
+//
+// The eighth pixel lies outside the window and its weights are zero, but zero times an infinity is not: the second MMA's second
+// core matrix (pixels seven and eight) is read from a copy of the row in which the second pixel of every pair is zero, by a
+// K-direction offset from one row to the other.  That costs 8 more bytes stored per two pixels, and no more operand reads.
 //
 // Shared memory is what bounds it (an MMA of K filters reads 4 KB of rows and 32 K bytes of weights, three times what its
 // arithmetic takes), so the two output rows of a step share their operand: input row t of the window is kernel row t of the
@@ -21,8 +25,8 @@
 //               the step before: all of it is monotone, so one rounding serves the three rows), into one of two stages
 //   warps 13-15 (pooled) three staged columns to one, 16-byte stores along the row.  Warps of their own: these loads queue
 //               behind the operand reads of the MMAs, and the accumulators waited for them (1.8 k of 3.6 k clocks a step).
-// 64 x 224 x 224, K = 64, pooled: 39.6 us (63 with separate operand reads, the bias from shared memory and pooling by the
-// epilogue's warps).
+// 64 x 224 x 224, K = 64, pooled, launches back to back in a captured graph: 40.8 us (40.6 without the copy of the rows; 63 with
+// separate operand reads, the bias from shared memory and pooling by the epilogue's warps).
 // Every pooled value is written once: no reductions in memory and nothing to clear first.  Every wait is bounded.
 #include <type_traits>
 
@@ -39,7 +43,7 @@ constexpr int kConvWarps = 4, kMmaWarp = kConvWarps, kFirstEpi = kConvWarps + 1,
 constexpr int kFirstPool = kFirstEpi + kEpiWarps, kPoolWarps = 3;
 template <bool kPool> constexpr int kThreads = (kFirstPool + (kPool ? kPoolWarps : 0)) * 32;
 constexpr int kR = 7, kC = 3;
-constexpr int kSlots = 24;                         // rows of the ring: a window of nine, and up to nine of the next step
+constexpr int kSlots = 18;                         // rows of the ring: a window of nine, and up to nine of the next step
 constexpr int kWindow = 9;                         // input rows under a step
 constexpr uint32_t kOne = 0x3F800000u;              // bf16 one as the second of a pair
 constexpr uint32_t kSmemLimit = 232448;
@@ -49,7 +53,7 @@ struct StemRowsParams {
     int N, H, W, K, P, Q, Mb, relu, y_bf16, early;  // early: the blob may be read before the wait (Launch::blob_ready)
     int PP, PQ, pairs, n_steps;                    // pooled height / width; pixel pairs of a row; steps in all (images x row pairs)
     int spi;                                       // steps per image
-    uint32_t pitch, line, off_b, off_stage, stage_bytes, off_bar, smem_bytes, tmem_cols;
+    uint32_t pitch, off_z, line, off_b, off_stage, stage_bytes, off_bar, smem_bytes, tmem_cols;
 };
 
 struct StemRowsBars {
@@ -96,7 +100,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t *ring = smem;                             // [kSlots] rows of `pitch` bytes: pixel x at 8 (x + 3)
+    uint8_t *ring = smem;                             // [kSlots] rows of `pitch` bytes: pixel x at 8 (x + 3); off_z further the same, odd x only
     uint8_t *bsm = smem + p.off_b;                    // [parity of the kernel row][4 octets][4 K: (6 | 5 - r) / 2, filter][8] bf16
     StemRowsBars *bars = reinterpret_cast<StemRowsBars *>(smem + p.off_bar);
     volatile uint32_t *abort_flag = &bars->abort_flag;
@@ -206,8 +210,10 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
             if (tail && w + tid < kWindow) {
                 uint32_t slot = base + (uint32_t)(w + tid);
                 if (slot >= (uint32_t)kSlots) slot -= kSlots;
-                *reinterpret_cast<uint4 *>(ring + slot * p.pitch + (uint32_t)(p.Q + 1) * 16u) =
-                    make_uint4(__funnelshift_r(last.x, last.y, 16), (last.y >> 16) | kOne, 0u, kOne);
+                uint8_t *at = ring + slot * p.pitch + (uint32_t)(p.Q + 1) * 16u;
+                const uint32_t e01 = __funnelshift_r(last.x, last.y, 16), e2 = (last.y >> 16) | kOne;
+                *reinterpret_cast<uint4 *>(at) = make_uint4(e01, e2, 0u, kOne);
+                *reinterpret_cast<uint2 *>(at + p.off_z) = make_uint2(e01, e2);
             }
             if (!on) return;
 #pragma unroll
@@ -218,8 +224,9 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                 // six elements e0 .. e5 = bytes 2 .. 13 of the four words
                 const uint32_t e01 = __funnelshift_r(a[q][0], a[q][1], 16), e23 = __funnelshift_r(a[q][1], a[q][2], 16),
                                e45 = __funnelshift_r(a[q][2], a[q][3], 16);
-                *reinterpret_cast<uint4 *>(ring + slot * p.pitch + (uint32_t)u * 16u) =
-                    make_uint4(e01, (e23 & 0xFFFFu) | kOne, (e23 >> 16) | (e45 << 16), (e45 >> 16) | kOne);
+                uint8_t *at = ring + slot * p.pitch + (uint32_t)u * 16u;
+                *reinterpret_cast<uint4 *>(at) = make_uint4(e01, (e23 & 0xFFFFu) | kOne, (e23 >> 16) | (e45 << 16), (e45 >> 16) | kOne);
+                *reinterpret_cast<uint2 *>(at + p.off_z) = make_uint2(e01, (e23 & 0xFFFFu) | kOne);
             }
         };
         Steps st(lo, hi, p.spi, kPool);
@@ -251,7 +258,8 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
         // ---- MMAs ------------------------------------------------------------------------------------------------------
         if (elect_one()) {
             const uint32_t idesc1 = idesc_bf16_f32(128, p.K), idesc2 = idesc_bf16_f32(128, 2 * p.K);
-            const uint32_t ring16 = (smem_u32(ring) >> 4) | (1u << 16), pitch16 = p.pitch >> 4;      // K-direction offset: 16 bytes
+            const uint32_t ring16 = smem_u32(ring) >> 4, pitch16 = p.pitch >> 4;
+            const uint32_t lbo1 = 1u << 16, lbo2 = ((p.off_z >> 4) + 1u) << 16;      // K-direction offsets: the next pair, here and in the copy
             const uint32_t b16 = (smem_u32(bsm) >> 4) | ((uint32_t)(4 * p.K) << 16);
             Steps st(lo, hi, p.spi, kPool);
             uint32_t i = 0, base = 0;
@@ -275,8 +283,8 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                     if (slot >= (uint32_t)kSlots) slot -= kSlots;
                     const uint32_t a_lo = ring16 + slot * pitch16, b_lo = b16 + ((r & 1) * 16 + ((6 - r) >> 1)) * p.K;
                     const uint32_t dt = t < (uint32_t)kR ? d : d + p.K, idesc = both ? idesc2 : idesc1;
-                    mma_bf16_ss(dt, desc64(a_lo), desc64(b_lo), idesc, k > 0);
-                    mma_bf16_ss(dt, desc64(a_lo + 2u), desc64(b_lo + 8u * p.K), idesc, 1u);
+                    mma_bf16_ss(dt, desc64(a_lo | lbo1), desc64(b_lo), idesc, k > 0);
+                    mma_bf16_ss(dt, desc64((a_lo + 2u) | lbo2), desc64(b_lo + 8u * p.K), idesc, 1u);
                 }
                 mma_commit(&bars->in_empty[b]);
                 mma_commit(&bars->acc_full[b]);
@@ -442,7 +450,8 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, StemRowsParams &p, bo
     p.pairs = p.Q + 3;
     p.pitch = round_up((uint32_t)p.pairs * 16u, 128);
     p.line = round_up(2u * d.K, 128);
-    p.off_b = kSlots * p.pitch + 1024u;                        // (an operand reads 128 columns, past the end of the last row)
+    p.off_z = kSlots * p.pitch;
+    p.off_b = 2u * p.off_z + 1024u;                            // (an operand reads 128 columns, past the end of the last row)
     p.off_stage = round_up(p.off_b + 2u * 4u * 4u * d.K * 16u, 128);
     p.stage_bytes = 128u * p.line;
     p.off_bar = p.off_stage + (pool ? 2u * p.stage_bytes : 0u);
