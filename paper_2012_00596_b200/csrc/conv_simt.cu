@@ -82,8 +82,9 @@ conv_bp_simt_kernel(npas_conv_desc d, int Mb, int Nb_, int P, int Q, int KW, con
         const int nj = (int)min((uint32_t)kMaxPairs, j_end - j0);
         if (j0 != j_begin) __syncthreads();
         for (int e = tid; e < nj; e += kWarps * 32) {
-            const uint32_t pw = pairs[j0 + e], tap = pw >> 16, r = tap / d.S, sx = tap - r * d.S;
-            pair_s[e] = make_uint2((r * d.W + sx) * d.C + (pw & 0xFFFFu) * Nb, r | (sx << 16));
+            const uint32_t pw = pairs[j0 + e], tap = pw >> 16, cb = pw & 0xFFFFu, r = tap / d.S, sx = tap - r * d.S;
+            // (a pair outside the layer counts for nothing: its tap lies beside every image)
+            pair_s[e] = r < (uint32_t)d.R && cb < nCB ? make_uint2((r * d.W + sx) * d.C + cb * Nb, r | (sx << 16)) : make_uint2(0u, 0xFFFFFFFFu);
         }
         __syncthreads();
         // this warp's share of the steps (contiguous, so that its sums have one order)

@@ -157,7 +157,8 @@ conv_bp_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvTcParams
                     uint32_t a_off = 0;
                     if ((uint32_t)lane < np) {
                         const uint32_t pw = pairs[s0 + lane];
-                        const uint32_t cbl = (pw & 0xFFFFu) - c * p.CBS, tap = pw >> 16;
+                        // (kept inside the stage whatever the blob says)
+                        const uint32_t cbl = min((pw & 0xFFFFu) - c * p.CBS, (uint32_t)p.CBS - 1u), tap = min(pw >> 16, (uint32_t)(p.R * p.S) - 1u);
                         a_off = cbl * p.q8 * p.plane_bytes + ((tap / p.S) * p.Wp + (tap % p.S)) * 16u;
                     }
                     if (!mbar_wait(&bars->w_full[st], (seg / p.SW) & 1, abort_flag, ws, 0x400)) { ok = false; break; }
@@ -167,7 +168,7 @@ conv_bp_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvTcParams
                         for (uint32_t i = 0; i < np; i += 2) {
                             const bool two = i + 1 < np;
                             const uint32_t a0 = __shfl_sync(0xFFFFFFFFu, a_off, i);
-                            const uint32_t a1 = __shfl_sync(0xFFFFFFFFu, a_off, two ? i + 1 : i);
+                            const uint32_t a1 = max(a0, __shfl_sync(0xFFFFFFFFu, a_off, two ? i + 1 : i));      // (pairs ascend; a damaged blob's too)
                             if (lane == 0) {
                                 const uint32_t b0 = b_stage + i * p.pair_bytes;
                                 const uint64_t ad = smem_desc_kmajor(a_stage + a0, a1 - a0, 128);

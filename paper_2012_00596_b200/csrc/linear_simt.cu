@@ -118,7 +118,7 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
             for (int r0 = (tg >> 5) * 8; r0 < nr || !waited; r0 += gt / 4) {      // eight kept rows per warp
                 const int r = r0 + q;
                 double d[kBM / 8][2] = {};
-                const int row = r < nr ? rl[r] : 0;
+                const int row = r < nr ? rl[r] : 0;                 // (a row or column number outside the block counts for nothing)
                 for (int c0 = 0; c0 < nc || !waited; c0 += 4 * kSteps) {
                     float wv[kSteps];
                     int col[kSteps];
@@ -127,6 +127,7 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
                         const int c = c0 + 4 * i + k;
                         wv[i] = (r < nr && c < nc) ? lin_load(w + r * nc + c) : 0.f;
                         col[i] = c < nc ? (int)cl[c] : -1;
+                        if (col[i] >= Bi) col[i] = -1;
                     }
                     if (!waited) {                                     // the rows of X of this phase (every thread comes here once)
                         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -142,7 +143,7 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
                         for (int m = 0; m < kBM / 8; ++m) mma_f64(d[m], a, col[i] >= 0 ? (double)xp[m * 8 * pitch] : 0.);
                     }
                 }
-                if (r < nr) {
+                if (r < nr && row < Bo) {
 #pragma unroll
                     for (int m = 0; m < kBM / 8; ++m) {
                         double2 *p = reinterpret_cast<double2 *>(acc + row * kAccPitch + m * 8 + 2 * k);

@@ -97,7 +97,7 @@ linear_bb_tc_kernel(const LinTcParams p, const uint16_t *__restrict__ x, const u
         const int bi = i / (p.BOG * p.Kp), r = i - bi * (p.BOG * p.Kp), g = r / p.Kp, j = r - g * p.Kp;
         const uint32_t b = (bo0 + g) * p.nBi + bi;
         const uint8_t c = j < p.Bi ? blob[p.L.off_cols + (size_t)b * p.Bi + j] : (uint8_t)0xFF;
-        cols_s[i] = c == 0xFF ? (uint8_t)p.Bi : c;
+        cols_s[i] = min(c, (uint8_t)p.Bi);
     }
     for (int i = tid; i < ncol; i += kThreads) bias_s[i] = bias ? bias[bo0 * p.Bo + i] : 0.f;
     const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);

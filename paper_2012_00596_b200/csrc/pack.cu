@@ -276,6 +276,7 @@ __global__ void bp_scatter_kernel(npas_bp_desc d, const uint8_t *__restrict__ bl
     uint64_t bits = 0;
     for (uint32_t j = blk_off[b]; j < blk_off[b + 1]; ++j) {
         const uint32_t tap = pairs[j] >> 16;
+        if (tap >= (uint32_t)(d.R * d.S)) continue;            // (no tap of the layer: ignored)
         bits |= 1ull << tap;
         if (!w_out) continue;
         for (uint32_t e = threadIdx.x; e < Mb * Nb; e += blockDim.x) {

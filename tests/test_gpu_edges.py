@@ -95,3 +95,59 @@ def test_empty_and_oversized_problems_are_refused():
     size = ctypes.c_size_t(0)
     tm = np.zeros(4, dtype=np.uint64)
     assert lib.npas_pack_bp_size(ctypes.byref(d), tm.ctypes.data_as(ctypes.c_void_p), ctypes.byref(size)) == 2
+
+
+def _header(blob):
+    return blob.data[:128].view(torch.int32).tolist()
+
+
+@pytest.mark.parametrize("dtype,path", [("f32", 1), ("bf16", 1), ("bf16", 3)])
+def test_gemm_ignores_list_entries_outside_their_block(dtype, path):
+    """Row and column numbers of a damaged blob index shared memory: one outside its block counts for nothing."""
+    c = inputs.linear_case(M=70, I=128, O=96, Bo=32, Bi=64, keep_rows=8, keep_cols=16, dtype=dtype, seed=811)
+    blob = npas.pack_bb(dev(c.w, dtype), c.row_keep, c.col_keep, 32, 64)
+    h, rk, ck = _header(blob), c.row_keep.copy(), c.col_keep.copy()
+    off_rows, off_cols = h[11], h[12]
+    drop = lambda m, i: np.uint64(int(m) & ~(1 << [t for t in range(64) if int(m) >> t & 1][i]))
+    rows = blob.data[off_rows: off_rows + 6 * 32].view(6, 32)
+    cols = blob.data[off_cols: off_cols + 6 * 64].view(6, 64)
+    if path == 1:                                    # (the gather kernel's tiles hold the rows in place: it reads no row list)
+        for b, i, v in ((0, 0, 32), (1, 7, 255), (5, 3, 200)):
+            rows[b, i] = v
+            rk.flat[b] = drop(c.row_keep.flat[b], i)
+    for b, i, v in ((0, 0, 64), (2, 15, 255), (4, 9, 128)):
+        cols[b, i] = v
+        ck.flat[b] = drop(c.col_keep.flat[b], i)
+    ws = npas.workspace()
+    y = npas.linear_bb(dev(c.x, dtype), blob, dev(c.bias), relu=c.relu, ws=ws, path=path)
+    npas.check_device_status(ws)
+    ref = oracle.linear_bb(c.x, c.w, rk, ck, Bo=32, Bi=64, bias=c.bias, relu=c.relu)
+    assert floored_rel_err(host(y), ref) < (TOL_F32 if dtype == "f32" else TOL_BF16)
+
+
+@pytest.mark.parametrize("dtype,path", [("f32", 1), ("bf16", 1), ("bf16", 3)])
+@pytest.mark.parametrize("Mb,Nb", [(16, 8), (16, 16)])
+def test_conv_ignores_pairs_outside_the_layer(dtype, path, Mb, Nb):
+    """Channel blocks and taps of a damaged blob: nothing is read or written outside, unpacking included."""
+    c = inputs.conv_case(N=2, H=9, W=11, C=48, K=32, Mb=Mb, Nb=Nb, keep=3, dtype=dtype, seed=812)
+    blob = npas.pack_bp(dev(c.w, dtype), c.tap_mask, Mb, Nb)
+    h = _header(blob)
+    nPairs, off = h[11], h[13]
+    pairs = blob.data[off: off + 4 * nPairs].view(torch.int32)
+    tm, w = c.tap_mask.copy(), c.w.copy()
+    for j, (cb, tap) in ((1, (0xFFFF, 0)), (3 * 2 + 2, (48 // Nb, 8)), (nPairs - 1, (0, 9)), (3 * 4, (0, 0x7FFF))):
+        old = int(pairs[j])
+        kept = [t for t in range(9) if int(c.tap_mask.flat[j // 3]) >> t & 1]
+        assert old >> 16 == kept[j % 3]
+        fb, ob = divmod(j // 3, 48 // Nb)
+        w[fb * Mb:(fb + 1) * Mb, kept[j % 3] // 3, kept[j % 3] % 3, ob * Nb:(ob + 1) * Nb] = 0
+        pairs[j] = (tap << 16 | cb) - (1 << 32 if tap >= 0x8000 else 0)
+    ws = npas.workspace()
+    y = npas.conv2d_bp(dev(c.x, dtype), blob, dev(c.bias), relu=c.relu, ws=ws, path=path)
+    npas.check_device_status(ws)
+    if path == 1:
+        ref = oracle.conv2d_bp(c.x, w, tm, Mb=Mb, Nb=Nb, bias=c.bias, relu=c.relu)
+        assert floored_rel_err(host(y), ref) < (TOL_F32 if dtype == "f32" else TOL_BF16)
+    assert torch.isfinite(y).all()
+    _, masks = npas.unpack_bp(blob)
+    assert (npas.mask_to_numpy(masks) < 1 << 9).all()
