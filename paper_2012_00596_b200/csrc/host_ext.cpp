@@ -284,21 +284,26 @@ __attribute__((target_clones("popcnt", "default"))) MaskSums count_values(const 
 }
 uint64_t low_bits(int n) { return n >= 64 ? ~0ull : (1ull << n) - 1; }
 
-// Mask words on both sides: a CUDA tensor is copied to pinned memory (the caller synchronises), a CPU tensor to the GPU.
+// Mask words on both sides: a CUDA tensor is copied to pinned memory (the caller synchronises), a CPU tensor to the GPU.  The
+// size of a blob is counted on the host side and its content follows the device side, so both are one copy of the caller's
+// words, which another stream or thread may change meanwhile (the packers' kernels read them more than once, too).
 struct Mask { at::Tensor dev, host; };
+bool snapshot(const uint64_t *words, size_t n, const at::Device &dev, cudaStream_t st, Mask &out)
+{
+    out.dev = new_tensor({(int64_t)n}, at::kLong, dev);
+    out.host = at::empty({(int64_t)n}, at::TensorOptions().dtype(at::kLong).pinned_memory(true));
+    if (npas_internal_copy_masks(words, static_cast<uint64_t *>(out.dev.data_ptr()), static_cast<uint64_t *>(out.host.data_ptr()), n, st) == NPAS_OK) return true;
+    PyErr_SetString(PyExc_RuntimeError, "copy of the masks failed");
+    return false;
+}
 bool both_sides(const at::Tensor &m, int64_t n, const at::Device &dev, cudaStream_t st, Mask &out)
 {
     if (m.scalar_type() != at::kLong || !m.is_contiguous() || m.numel() < n) return fail_assert("mask words: contiguous int64, one per block");
-    cudaError_t e;
-    if (m.is_cuda()) {
-        out.dev = m;
-        out.host = at::empty({n}, at::TensorOptions().dtype(at::kLong).pinned_memory(true));
-        e = cudaMemcpyAsync(out.host.data_ptr(), m.data_ptr(), (size_t)n * 8, cudaMemcpyDeviceToHost, st);
-    } else {
-        out.host = m;
-        out.dev = new_tensor({n}, at::kLong, dev);
-        e = cudaMemcpyAsync(out.dev.data_ptr(), m.data_ptr(), (size_t)n * 8, cudaMemcpyHostToDevice, st);
-    }
+    if (m.is_cuda()) return snapshot(static_cast<const uint64_t *>(m.data_ptr()), (size_t)n, dev, st, out);
+    out.host = at::empty({n}, at::TensorOptions().dtype(at::kLong));
+    memcpy(out.host.data_ptr(), m.data_ptr(), (size_t)n * 8);
+    out.dev = new_tensor({n}, at::kLong, dev);
+    const cudaError_t e = cudaMemcpyAsync(out.dev.data_ptr(), out.host.data_ptr(), (size_t)n * 8, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) { PyErr_SetString(PyExc_RuntimeError, cudaGetErrorString(e)); return false; }
     return true;
 }
@@ -366,20 +371,17 @@ PyObject *pack_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
         const cudaStream_t st = c10::cuda::getCurrentCUDAStream().stream();
         const int64_t blocks = (int64_t)(d.O / d.Bo) * (d.I / d.Bi);
         Mask rows, cols;
-        const uint64_t *hr, *hc;
+        const uint64_t *hr, *hc, *dc;
         if (mr->is_cuda() && mc->is_cuda() && mr->numel() == blocks && mc->numel() == blocks &&
             static_cast<const int64_t *>(mc->data_ptr()) == static_cast<const int64_t *>(mr->data_ptr()) + blocks && mr->scalar_type() == at::kLong &&
             mc->scalar_type() == at::kLong && mr->is_contiguous() && mc->is_contiguous()) {
-            rows.dev = *mr; cols.dev = *mc;
-            rows.host = at::empty({2 * blocks}, at::TensorOptions().dtype(at::kLong).pinned_memory(true));
-            if (cudaMemcpyAsync(rows.host.data_ptr(), mr->data_ptr(), (size_t)blocks * 16, cudaMemcpyDeviceToHost, st) != cudaSuccess) {
-                PyErr_SetString(PyExc_RuntimeError, "copy of the masks failed");
-                return nullptr;
-            }
+            if (!snapshot(static_cast<const uint64_t *>(mr->data_ptr()), (size_t)blocks * 2, w->device(), st, rows)) return nullptr;
+            dc = static_cast<const uint64_t *>(rows.dev.data_ptr()) + blocks;
             hr = static_cast<const uint64_t *>(rows.host.data_ptr()); hc = hr + blocks;
         } else {
             if (!both_sides(*mr, blocks, w->device(), st, rows) || !both_sides(*mc, blocks, w->device(), st, cols)) return nullptr;
             hr = static_cast<const uint64_t *>(rows.host.data_ptr()); hc = static_cast<const uint64_t *>(cols.host.data_ptr());
+            dc = static_cast<const uint64_t *>(cols.dev.data_ptr());
         }
         if ((mr->is_cuda() || mc->is_cuda()) && !wait_for(st)) return nullptr;
         const MaskSums sums = count_values(hr, hc, (size_t)blocks, low_bits(d.Bo), low_bits(d.Bi));
@@ -388,8 +390,7 @@ PyObject *pack_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
         if (s != NPAS_OK) return packed(s, at::Tensor(), 0);
         at::Tensor blob = new_tensor({(int64_t)bytes}, at::kByte, w->device());
         Py_BEGIN_ALLOW_THREADS
-        s = npas_internal_pack_bb(&d, w->data_ptr(), static_cast<const uint64_t *>(rows.dev.data_ptr()),
-                                  static_cast<const uint64_t *>(cols.dev.data_ptr()), blob.data_ptr(), bytes, st);
+        s = npas_internal_pack_bb(&d, w->data_ptr(), static_cast<const uint64_t *>(rows.dev.data_ptr()), dc, blob.data_ptr(), bytes, st);
         Py_END_ALLOW_THREADS
         return packed(s, std::move(blob), (uint32_t)d.max_cols);
     });

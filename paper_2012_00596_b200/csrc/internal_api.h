@@ -17,6 +17,9 @@ extern "C" {
 // kept columns in the fullest block
 npas_status npas_internal_bp_size(const npas_bp_desc *d, uint64_t n_pairs, size_t *blob_bytes);
 npas_status npas_internal_bb_size(const npas_bb_desc *d, uint64_t n_vals, uint32_t max_cols, size_t *blob_bytes);
+// n mask words on the device to a device buffer and to page-locked host memory, each word read once: what the host counts is
+// what the packers see
+npas_status npas_internal_copy_masks(const uint64_t *words, uint64_t *dev, uint64_t *host, size_t n, void *stream);
 // the pack calls up to, but without, their synchronisation
 npas_status npas_internal_pack_bp(const npas_bp_desc *d, const void *w, const uint64_t *tap_mask, void *blob, size_t blob_bytes, void *stream);
 npas_status npas_internal_pack_bb(const npas_bb_desc *d, const void *w, const uint64_t *rk, const uint64_t *ck, void *blob,

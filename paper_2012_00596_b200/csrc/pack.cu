@@ -59,6 +59,22 @@ template <typename TIn, typename TOut> __device__ __forceinline__ TOut convert(T
     else return f32_bits_to_bf16(v);
 }
 
+// Two words per thread, to the device and over PCIe in one pass.  One launch, and no copy engine: prune + pack of 512x3x3x512
+// takes 40 us with it, 48 with a copy on the device and one to the host behind it, 44 with the copy to the host alone.
+__global__ void __launch_bounds__(256)
+copy_masks_kernel(const uint64_t *words, uint64_t *__restrict__ dev, uint64_t *__restrict__ host, size_t n)
+{
+    auto load = [](const uint64_t *p) { return *reinterpret_cast<const volatile uint64_t *>(p); };      // (once: they may be changing)
+    const size_t i = ((size_t)blockIdx.x * 256u + threadIdx.x) * 2u;
+    if (i + 1 < n) {
+        const ulonglong2 v = make_ulonglong2(load(words + i), load(words + i + 1));
+        *reinterpret_cast<ulonglong2 *>(dev + i) = v;
+        *reinterpret_cast<ulonglong2 *>(host + i) = v;
+    } else if (i < n) {
+        host[i] = dev[i] = load(words + i);
+    }
+}
+
 // ---- block-punched ---------------------------------------------------------------------------
 
 __global__ void __launch_bounds__(1024)
@@ -515,6 +531,16 @@ using namespace npas;
 
 // ================================================================================================
 extern "C" {
+
+npas_status npas_internal_copy_masks(const uint64_t *words, uint64_t *dev, uint64_t *host, size_t n, void *stream)
+{
+    if (!words || !dev || !host || n == 0 || !aligned16(dev) || !aligned16(host)) return NPAS_ERR_NULL;
+    void *mapped = nullptr;
+    if (cudaHostGetDevicePointer(&mapped, host, 0) != cudaSuccess) return NPAS_ERR_CUDA;
+    copy_masks_kernel<<<(unsigned)((n + 511) / 512), 256, 0, static_cast<cudaStream_t>(stream)>>>(words, dev, static_cast<uint64_t *>(mapped), n);
+    count_launch();
+    return launch_status();
+}
 
 npas_status npas_internal_bp_size(const npas_bp_desc *d, uint64_t n_pairs, size_t *blob_bytes)
 {

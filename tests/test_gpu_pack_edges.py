@@ -1,6 +1,8 @@
 """Packing and pruning where their kernels change shape: block widths that are not whole octets beside the operand image,
 filter groups narrower than a warp, more taps than a word, more groups than a cluster's shared memory holds, and device
-masks handed over without a copy."""
+masks that change while a layer is being packed."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -53,3 +55,45 @@ def test_pack_bb_and_pruning_at_the_edges(Bo, Bi, kr, kc):
         assert np.array_equal(blob.data.cpu().numpy(), oracle.pack_bb(w, rk0, ck0, Bo, Bi, dtype))
         wd, r2, c2 = npas.unpack_bb(blob)
         assert torch.equal(wd.float(), torch.from_numpy(oracle.bb_element_mask(rk0, ck0, O, I, Bo, Bi) * w).cuda().to(wd.dtype).float())
+
+
+def test_masks_that_change_while_they_are_packed():
+    """Another stream rewrites the caller's masks all the time, from nothing kept to everything and back: every blob is whole, its
+    size, its header and its sections being those of one state of the masks (each word's own)."""
+    stop, side = threading.Event(), torch.cuda.Stream()
+    rng = inputs.rng_for(1004)
+    w = dev(rng.standard_normal((64, 3, 3, 64), dtype=np.float32), "bf16")
+    tm = torch.zeros((4, 8), dtype=torch.int64, device="cuda")
+    m = dev(rng.standard_normal((128, 192), dtype=np.float32), "bf16")
+    both = torch.zeros((2, 2, 3), dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+
+    def flip():
+        with torch.cuda.stream(side):
+            while not stop.is_set():
+                for v in (-1, 0, 0x155):
+                    tm.fill_(v)
+                    both.fill_(v)
+                side.synchronize()
+
+    t = threading.Thread(target=flip)
+    t.start()
+    try:
+        for _ in range(300):
+            blob = npas.pack_bp(w, tm, 16, 8)
+            npas.blob_check(blob)
+            wd, masks = npas.unpack_bp(blob)
+            assert blob.data[:128].view(torch.int32)[15].item() == blob.data.numel()
+            words = npas.mask_to_numpy(masks)
+            assert set(words.ravel().tolist()) <= {0x1FF, 0, 0x155}
+            kept = torch.from_numpy(oracle.bp_element_mask(words, 64, 64, 3, 3, 16, 8)).cuda()
+            assert torch.equal(wd, torch.where(kept.bool(), w, torch.zeros_like(w)))
+            blob = npas.pack_bb(m, both[0], both[1], 64, 64)
+            npas.blob_check(blob)
+            assert blob.data[:128].view(torch.int32)[15].item() == blob.data.numel()
+            wd, rk, ck = npas.unpack_bb(blob)
+            em = oracle.bb_element_mask(npas.mask_to_numpy(rk), npas.mask_to_numpy(ck), 128, 192, 64, 64)
+            assert torch.equal(wd, torch.where(torch.from_numpy(em).cuda().bool(), m, torch.zeros_like(m)))
+    finally:
+        stop.set()
+        t.join()
