@@ -427,9 +427,9 @@ bool conv_sk_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 // come here: the single-CTA kernel computes every position (12x19x50x144 -> 208 8.9 against 36 us); those it takes, when
 // there are channels to split, one wave, and the pair kernel is not modelled faster (14x14x512 -> 512 5.8 against 17.1 us;
 // 59x17x48x512 -> 64 38.6 against 19.3).
-bool conv_sk_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
+// The plan is part of the answer: what is launched is what was compared.
+static bool chosen(const npas_conv_desc &d, const npas_bp_desc &bp, ConvSkParams &p)
 {
-    ConvSkParams p;
     const int sms = sm_count();
     if (d.variant) return false;
     const bool phases = d.stride == 2 && d.R == 3 && d.S == 3 && d.pad == 1;
@@ -438,6 +438,12 @@ bool conv_sk_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
     if (planned(d, bp, p, true) && (phases ? p.nBlk > 1 && modelled(p, sms) <= conv_dense_modelled(d, bp) : p.n_tiles * 2 <= sms)) return true;
     // several waves: against independent CTAs, whose tile is as narrow as the image's groups (11x15x25x416 -> 464 51 against 63 us)
     return d.stride == 1 && !pairs && planned(d, bp, p, false) && 1.05 * modelled(p, sms) < conv_dense_modelled(d, bp);
+}
+
+bool conv_sk_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
+{
+    ConvSkParams p;
+    return chosen(d, bp, p);
 }
 
 // A stride-1 layer of this kernel's range that the pair kernel does sooner, by the models of both: many channels on just under
@@ -453,8 +459,7 @@ npas_status conv_sk_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
                            const void *res, void *y, uint32_t *ws, cudaStream_t st, Launch how)
 {
     ConvSkParams p;
-    const bool one_wave = !d.variant && planned(d, bp, p, true) && (d.stride != 1 || p.n_tiles * 2 <= sm_count());     // (as it was chosen)
-    if (!one_wave && !planned(d, bp, p, false)) return NPAS_ERR_UNSUPPORTED;
+    if (d.variant ? !planned(d, bp, p, false) : !chosen(d, bp, p)) return NPAS_ERR_UNSUPPORTED;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return NPAS_ERR_CUDA;
     // X[N][H][W][C] as (C, W, H, N): a box of CB channels x Wp columns x slab rows (every other pixel for a parity class)
