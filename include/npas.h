@@ -258,9 +258,10 @@ npas_status npas_conv2d_bp_kernel(const npas_conv_desc *d, const npas_bp_desc *b
 npas_status npas_linear_bb_kernel(const npas_linear_desc *d, const npas_bb_desc *bb, int32_t *kernel_id);
 
 /* Auto-tuning (paper Sec. 3, "Compiler Optimizations": the generated code is tuned per layer).  Runs
- * every kernel and tile shape that takes the layer on the caller's own buffers (one warm-up and `reps`
- * timed launches each, CUDA events on `stream`), and returns the fastest as the (path, variant) pair to
- * put into the call descriptor; *us_out (nullable) receives its time per launch in microseconds.  The
+ * the automatic choice and every kernel and tile shape that takes the layer on the caller's own buffers
+ * (of the many shapes of path 6's split form those modelled within a quarter of its best; one warm-up and
+ * `reps` timed launches each, CUDA events on `stream`; what beats the automatic choice is timed against
+ * it twice more), and returns the fastest as the (path, variant) pair to put into the call descriptor; *us_out (nullable) receives its time per launch in microseconds.  The
  * plan is these two integers: the caller keeps them with the layer.  Synchronises the stream several
  * times (not for use inside a stream capture); y_dev holds the layer's result afterwards.  d->path and
  * d->variant are ignored.  Arguments as in the compute calls. */

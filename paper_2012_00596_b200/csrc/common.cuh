@@ -209,6 +209,8 @@ npas_status conv_dn_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
                            uint32_t *ws, cudaStream_t st, Launch how);
 bool conv_sk_preferred(const npas_conv_desc &d, const npas_bp_desc &bp);
 bool conv_sk_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
+int32_t conv_sk_variant(const npas_conv_desc &d, const npas_bp_desc &bp);
+int conv_sk_shapes(const npas_conv_desc &d, const npas_bp_desc &bp, int32_t *variants, int cap);
 npas_status conv_sk_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
                            uint32_t *ws, cudaStream_t st, Launch how);
@@ -233,6 +235,7 @@ npas_status linear_dn_launch(const npas_linear_desc &d, const npas_bb_desc &bb, 
                              cudaStream_t st, Launch how);
 bool linear_sk_supported(const npas_linear_desc &d, const npas_bb_desc &bb);
 bool linear_sk_preferred(const npas_linear_desc &d, const npas_bb_desc &bb);
+int32_t linear_sk_variant(const npas_linear_desc &d, const npas_bb_desc &bb);
 npas_status linear_sk_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,
                              cudaStream_t st, Launch how);

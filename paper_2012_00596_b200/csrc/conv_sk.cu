@@ -455,6 +455,36 @@ bool conv_sk_slower(const npas_conv_desc &d, const npas_bp_desc &bp)
     return !d.variant && d.stride == 1 && planned(d, bp, p, true) && modelled(p, sm_count()) > conv_dense_modelled(d, bp);
 }
 
+static int32_t shape_of(const ConvSkParams &p) { return p.NT | (p.KC << 16) | (p.KT << 24); }
+
+// the shape an automatic choice of this kernel runs, as a `variant` (0: none)
+int32_t conv_sk_variant(const npas_conv_desc &d, const npas_bp_desc &bp)
+{
+    ConvSkParams p;
+    return chosen(d, bp, p) ? shape_of(p) : 0;
+}
+
+// Shapes worth timing, as `variant`s: those that the model (9 % standard error) puts within a quarter of its best one, where that
+// is not modelled half as slow again as the other dense-image kernels.
+int conv_sk_shapes(const npas_conv_desc &d, const npas_bp_desc &bp, int32_t *variants, int cap)
+{
+    npas_conv_desc q = d;
+    q.variant = 0;
+    ConvSkParams p;
+    const int sms = sm_count();
+    if (!planned(q, bp, p, false)) return 0;
+    const double best = modelled(p, sms);
+    if (best > 1.5 * conv_dense_modelled(q, bp)) return 0;
+    int n = 0;
+    for (int nt = 16; nt <= 128; nt += 16)
+        for (int kc = 1; kc <= kMaxSplit; ++kc)
+            for (int kt = 1; kc * kt <= kMaxSplit && kt <= 4; ++kt) {
+                q.variant = nt | (kc << 16) | (kt << 24);
+                if (n < cap && plan(q, bp, p, sms, false) && modelled(p, sms) <= 1.25 * best) variants[n++] = q.variant;
+            }
+    return n;
+}
+
 npas_status conv_sk_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x, const void *blob, const float *bias,
                            const void *res, void *y, uint32_t *ws, cudaStream_t st, Launch how)
 {

@@ -302,6 +302,13 @@ bool linear_sk_preferred(const npas_linear_desc &d, const npas_bb_desc &bb)
     return planned(d, bb, p, true);
 }
 
+// the shape an automatic choice of this kernel runs, as a `variant` (0: none)
+int32_t linear_sk_variant(const npas_linear_desc &d, const npas_bb_desc &bb)
+{
+    LinSkParams p;
+    return planned(d, bb, p, true) ? p.BN | (p.KS << 16) : 0;
+}
+
 npas_status linear_sk_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x, const void *blob, const float *bias,
                              const void *res, void *y, uint32_t *ws, cudaStream_t st, Launch how)
 {

@@ -82,6 +82,46 @@ def test_tuned_linear_plan_is_valid_and_not_slower():
     assert t_plan <= 1.25 * t_auto, (path, variant, t_plan, t_auto)
 
 
+def _graph_us(f, reps=20):
+    """Microseconds per call of a captured chain of calls (no host time in it), the best of several replays."""
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        f()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        for _ in range(reps):
+            f()
+    for _ in range(20):
+        g.replay()
+    return min(_time_once(g.replay, 5) for _ in range(5)) / reps
+
+
+@pytest.mark.parametrize("M,I,O", [(9089, 384, 576), (2000, 960, 1984), (64, 2048, 1000), (300, 512, 640)])
+def test_tuned_linear_plan_keeps_up_with_the_automatic_choice(M, I, O):
+    """Layers whose automatic choice is a tile of 192 columns or a split: the plan may not be slower than no plan (5 % for the noise
+    of two measurements of a kernel of a few microseconds)."""
+    c = inputs.linear_case(M=M, I=I, O=O, Bo=8 if O == 1000 else 64, Bi=64, keep_rows=4, keep_cols=32, dtype="bf16", seed=502)
+    x, blob, bias, ws = dev(c.x, "bf16"), npas.pack_bb(dev(c.w, "bf16"), c.row_keep, c.col_keep, c.Bo, c.Bi), dev(c.bias), npas.workspace()
+    y = torch.empty((M, O), dtype=torch.bfloat16, device="cuda")
+    path, variant, us = npas.tune_linear_bb(x, blob, bias, relu=True, out=y, ws=ws, reps=50)
+    run = lambda **kw: npas.linear_bb(x, blob, bias, relu=True, out=y, ws=ws, **kw)
+    t_plan, t_auto = _graph_us(lambda: run(path=path, variant=variant)), _graph_us(run)
+    assert t_plan <= 1.05 * t_auto, (path, variant, us, t_plan, t_auto)
+
+
+@pytest.mark.parametrize("N,H,C,K,stride", [(7, 45, 96, 176, 2), (4, 14, 256, 256, 1), (1, 7, 512, 512, 1), (11, 25, 416, 464, 1), (6, 30, 512, 128, 1)])
+def test_tuned_conv_plan_keeps_up_with_the_automatic_choice(N, H, C, K, stride):
+    """The same for convolutions whose automatic choice splits taps, takes odd channel splits or odd filter tiles."""
+    c = inputs.conv_case(N=N, H=H, W=H, C=C, K=K, Mb=16, Nb=8, keep=3, stride=stride, dtype="bf16", seed=503)
+    x, blob, bias, ws = dev(c.x, "bf16"), npas.pack_bp(dev(c.w, "bf16"), c.tap_mask, c.Mb, c.Nb), dev(c.bias), npas.workspace()
+    y = torch.empty((c.N, c.P, c.Q, c.K), dtype=torch.bfloat16, device="cuda")
+    path, variant, us = npas.tune_conv2d_bp(x, blob, bias, stride=stride, relu=True, out=y, ws=ws, reps=50)
+    run = lambda **kw: npas.conv2d_bp(x, blob, bias, stride=stride, relu=True, out=y, ws=ws, **kw)
+    t_plan, t_auto = _graph_us(lambda: run(path=path, variant=variant)), _graph_us(run)
+    assert t_plan <= 1.05 * t_auto, (path, variant, us, t_plan, t_auto)
+
+
 def test_tuner_rejects_bad_arguments_without_launching():
     c = inputs.conv_case(N=1, H=14, W=14, C=64, K=64, Mb=16, Nb=8, keep=3, dtype="bf16", seed=501)
     x, w = dev(c.x, "bf16"), dev(c.w, "bf16")
