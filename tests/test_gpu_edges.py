@@ -151,3 +151,16 @@ def test_conv_ignores_pairs_outside_the_layer(dtype, path, Mb, Nb):
     assert torch.isfinite(y).all()
     _, masks = npas.unpack_bp(blob)
     assert (npas.mask_to_numpy(masks) < 1 << 9).all()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("N,H,W,C,K,Mb,Nb,R,stride", [(4, 150, 151, 6, 40, 20, 6, 3, 1), (4, 161, 129, 8, 18, 9, 8, 3, 1), (1, 9, 9, 512, 16, 16, 16, 3, 1),
+                                                      (2, 131, 133, 3, 32, 16, 3, 3, 1), (3, 60, 60, 36, 24, 12, 12, 5, 2), (1, 40, 41, 100, 16, 8, 4, 3, 1)])
+def test_float64_convolution_at_its_edges(dtype, N, H, W, C, K, Mb, Nb, R, stride):
+    """Sixteen filters per CTA with ragged filter blocks, more steps than are described at a time, every number of shares of the
+    pairs, blocks of channels that are not whole steps; the same sums in float64 whatever the split."""
+    c = inputs.conv_case(N=N, H=H, W=W, C=C, K=K, Mb=Mb, Nb=Nb, R=R, S=R, stride=stride, pad=1,
+                         keep=(R * R if C in (3, 512) else lambda fb, cb: (5 * fb + 3 * cb) % (R * R + 1)), dtype=dtype, residual=True, seed=821)
+    y = _conv(c, 1)
+    assert floored_rel_err(host(y), _conv_ref(c)) < (TOL_F32 if dtype == "f32" else TOL_BF16)
+    assert torch.equal(y, _conv(c, 1))
