@@ -39,6 +39,26 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 
+// a warp copies `width` elements of a row of X, widened; `pairs`: the row and every piece of it start on even elements
+__device__ __forceinline__ void stage_row(float *dst, const float *src, int width, bool, int lane)
+{
+#pragma unroll 4
+    for (int c = lane; c < width; c += 32) dst[c] = src[c];
+}
+__device__ __forceinline__ void stage_row(float *dst, const uint16_t *src, int width, bool pairs, int lane)
+{
+    if (pairs) {
+#pragma unroll 4
+        for (int c = 2 * lane; c < width; c += 64) {
+            const uint32_t v = *reinterpret_cast<const uint32_t *>(src + c);
+            *reinterpret_cast<float2 *>(dst + c) = make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
+        }
+    } else {
+#pragma unroll 4
+        for (int c = lane; c < width; c += 32) dst[c] = bf16_bits_to_f32(src[c]);
+    }
+}
+
 __device__ __forceinline__ void group_sync(int g, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(threads) : "memory"); }
 
 // D[8 x 8] += A[8 x 4] * B[4 x 8]; lane l holds A(l / 4, l % 4), B(l % 4, l / 4), D(l / 4, 2 (l % 4) + {0, 1})
@@ -69,8 +89,9 @@ inline LinSimtSmem smem_plan(const npas_bb_desc &bb)
 
 }  // namespace
 
+// (registers for a second CTA wherever the groups leave threads for it)
 template <typename TX, typename TY>
-__global__ void __launch_bounds__(kMaxWarps * 32)
+__global__ void __maxnreg__(104)
 linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSmem S, const TX *__restrict__ x,
                       const uint8_t *__restrict__ blob, const float *__restrict__ bias, const TY *__restrict__ res,
                       TY *__restrict__ y)
@@ -84,6 +105,7 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
     const uint32_t *voff = reinterpret_cast<const uint32_t *>(blob + L.off_voff);
     const TX *vals = reinterpret_cast<const TX *>(blob + L.off_values);
     const bool x16 = sizeof(TX) == 4 && (d.I & 3) == 0 && (Bi & 3) == 0;
+    const bool x2 = (d.I & 1) == 0 && (Bi & 1) == 0;
     const int per_phase = (int)S.phase_cols / Bi;
 
     tc::pdl_trigger();
@@ -96,7 +118,7 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
             const TX *src = x + (size_t)(m0 + r) * d.I + (size_t)b0 * Bi;
             float *dst = xraw + r * pitch;
             if (x16) for (int c = (t & 31) * 4; c < width; c += 128) cp_async16(dst + c, src + c);
-            else for (int c = t & 31; c < width; c += 32) dst[c] = lin_load(src + c);
+            else stage_row(dst, src, width, x2, t & 31);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
         bool waited = false;
@@ -176,10 +198,175 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
     }
 }
 
+// ---- blocks of up to 32 rows --------------------------------------------------------------------------------------------------
+// Many blocks, each a header, lists and a few weights: a chain of loads for a handful of matrix instructions, whose latency is
+// what bounds it.  So here a block belongs to one warp, which has the next block's lists and first weights (and the header of the
+// one after) on their way, accumulates in a tile of its own and meets the others only between phases of 256 columns; with
+// three CTAs per SM and `gb` rows of blocks on the same staged rows of X.  The warps' sums are added in order at the end.
+struct LinRowsPlan { uint32_t warps, gb, phase_cols, pitch, off_acc, bytes; };
+constexpr int kRowsWarps = 8;
+constexpr int kRowsOutputs = 16;            // outputs per CTA where a row of blocks has fewer
+constexpr int kRowsCols = 256;              // columns of X staged at a time
+
+static LinRowsPlan rows_plan(const npas_linear_desc &d, const npas_bb_desc &bb)
+{
+    LinRowsPlan p;
+    const uint32_t nBo = bb.O / bb.Bo, nBi = bb.I / bb.Bi, mt = (uint32_t)(d.M + kBM - 1) / kBM;
+    p.gb = bb.Bo < kRowsOutputs ? kRowsOutputs / bb.Bo : 1u;
+    while (p.gb > 1 && (uint64_t)mt * ((nBo + p.gb - 1) / p.gb) < 4ull * sm_count()) --p.gb;
+    p.phase_cols = bb.I < kRowsCols ? (uint32_t)bb.I : kRowsCols / bb.Bi * bb.Bi;
+    p.pitch = round_up(p.phase_cols, 8) + 4;
+    p.warps = p.gb * nBi < kRowsWarps ? p.gb * nBi : kRowsWarps;
+    p.off_acc = round_up(kBM * p.pitch * 4u, 16);
+    p.bytes = p.off_acc + p.warps * p.gb * bb.Bo * kAccPitch * 8u;
+    return p;
+}
+
+// Against the kernel above, whose CTA gives a block to several warps: here where there are two CTAs per SM and a row of blocks has
+// work for the warps (392x512 -> 512 in 16x16 blocks keeping 8x8 24 us there, 12 here; 3136x508 -> 508 in 4x4 keeping 2x2 1030 and
+// 497), or four per SM in any case (705x128 -> 960, two blocks of 20x64 in a row, 17 and 9).  On smaller grids the kernel
+// above is the better one more often than not (100x64 -> 128 4.2 and 9.1, 1x508 -> 508 in 4x4 12.4 and 16.3, 615x20 -> 170, two
+// blocks in a row, 5.6 and 7.7).
+static bool rows_preferred(const npas_linear_desc &d, const npas_bb_desc &bb)
+{
+    const long long ctas = (long long)((d.M + kBM - 1) / kBM) * (bb.O / bb.Bo), sms = sm_count();
+    return bb.Bo <= 32 && (ctas >= 4 * sms || (ctas >= 2 * sms && bb.I / bb.Bi >= 4));
+}
+
+template <typename TX, typename TY>
+__global__ void __launch_bounds__(kRowsWarps * 32, 3)
+linear_bb_rows_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinRowsPlan S, const TX *__restrict__ x,
+                      const uint8_t *__restrict__ blob, const float *__restrict__ bias, const TY *__restrict__ res,
+                      TY *__restrict__ y)
+{
+    extern __shared__ __align__(16) uint8_t sm[];
+    const int t = threadIdx.x, nt = blockDim.x, warp = t >> 5, lane = t & 31, k = lane & 3, q = lane >> 2, W = (int)S.warps, pitch = (int)S.pitch;
+    const int bo0 = blockIdx.y * (int)S.gb, gb = min((int)S.gb, (int)L.nBo - bo0), outs = gb * Bo;
+    float *xs = reinterpret_cast<float *>(sm);                                                          // [kBM][pitch]
+    double *acc0 = reinterpret_cast<double *>(sm + S.off_acc), *acc = acc0 + (size_t)warp * outs * kAccPitch;   // [W][outs][kAccPitch]
+    const int m0 = blockIdx.x * kBM, rows_here = min(kBM, d.M - m0), nBi = (int)L.nBi, per_phase = (int)S.phase_cols / Bi;
+    const bool x16 = sizeof(TX) == 4 && (d.I & 3) == 0 && (Bi & 3) == 0, x2 = (d.I & 1) == 0 && (Bi & 1) == 0;
+    const uint32_t *voff = reinterpret_cast<const uint32_t *>(blob + L.off_voff);
+    const TX *vals = reinterpret_cast<const TX *>(blob + L.off_values);
+
+    tc::pdl_trigger();
+    for (int e = lane; e < outs * kAccPitch; e += 32) acc[e] = 0;
+    tc::pdl_wait();
+    for (int b0 = 0; b0 < nBi; b0 += per_phase) {
+        const int nb = min(per_phase, nBi - b0), width = nb * Bi;
+        if (b0) __syncthreads();                                       // the phase before has been read
+        for (int r = warp; r < rows_here; r += W) {                    // a warp per row
+            const TX *src = x + (size_t)(m0 + r) * d.I + (size_t)b0 * Bi;
+            float *dst = xs + r * pitch;
+            if (x16) for (int c = lane * 4; c < width; c += 128) cp_async16(dst + c, src + c);
+            else stage_row(dst, src, width, x2, lane);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        // the phase's blocks, a warp every W-th: row of blocks `hr`, block b0 + `hb` of it
+        struct Block { uint32_t blk, off, cnt; int at, base, row, c0, c1; float w[4]; };
+        int hr = 0, hb = warp;
+        while (hb >= nb) { hb -= nb; ++hr; }
+        auto header = [&](Block &n) {
+            n.off = n.cnt = 0; n.blk = ~0u;
+            if (hr >= gb) return;
+            n.blk = (uint32_t)(bo0 + hr) * L.nBi + (uint32_t)(b0 + hb);
+            n.at = hr * Bo * kAccPitch; n.base = hb * Bi;
+            n.off = voff[n.blk];
+            n.cnt = *reinterpret_cast<const uint16_t *>(blob + L.off_cnt + 2 * n.blk);
+            hb += W;
+            while (hb >= nb) { hb -= nb; ++hr; }
+        };
+        auto kept = [&](const Block &n, int &nr, int &nc) { nr = min((int)(n.cnt & 0xFFu), Bo); nc = min((int)(n.cnt >> 8), Bi); };
+        // rows r0 .. r0 + 7, columns c0 .. c0 + 15 of the block's weights
+        auto weights = [&](const Block &n, int nr, int nc, int r0, int c0, float (&w)[4]) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int c = c0 + 4 * i + k;
+                w[i] = r0 + q < nr && c < nc ? lin_load(vals + n.off + (r0 + q) * nc + c) : 0.f;
+            }
+        };
+        auto lists = [&](Block &n) {
+            if (n.blk == ~0u) return;
+            int nr, nc;
+            kept(n, nr, nc);
+            const uint8_t *rl = blob + L.off_rows + (size_t)n.blk * Bo, *cl = blob + L.off_cols + (size_t)n.blk * Bi;
+            n.row = lane < nr ? rl[lane] : Bo;                         // (a row or column number outside the block counts for nothing)
+            n.c0 = lane < nc ? cl[lane] : Bi;
+            n.c1 = lane + 32 < nc ? cl[lane + 32] : Bi;
+            weights(n, nr, nc, 0, 0, n.w);
+        };
+        Block now, next;
+        header(now);
+        lists(now);
+        header(next);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        while (now.blk != ~0u) {
+            const Block b = now;
+            now = next;
+            lists(now);
+            header(next);
+            int nr, nc;
+            kept(b, nr, nc);
+            for (int r0 = 0; r0 < nr; r0 += 8) {
+                const int row = __shfl_sync(0xFFFFFFFFu, b.row, (r0 + q) & 31);
+                double a[kBM / 8][2] = {};
+                for (int c0 = 0; c0 < nc; c0 += 16) {
+                    float w[4];
+                    if (r0 | c0) weights(b, nr, nc, r0, c0, w);
+                    else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) w[i] = b.w[i];
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (c0 + 4 * i >= nc) break;
+                        const int col = __shfl_sync(0xFFFFFFFFu, c0 < 32 ? b.c0 : b.c1, (c0 + 4 * i + k) & 31);
+                        const float *xp = xs + q * pitch + b.base + col;
+#pragma unroll
+                        for (int m = 0; m < kBM / 8; ++m) mma_f64(a[m], (double)w[i], col < Bi ? (double)xp[m * 8 * pitch] : 0.);
+                    }
+                }
+                if (r0 + q < nr && row < Bo) {
+#pragma unroll
+                    for (int m = 0; m < kBM / 8; ++m) {
+                        double2 *p = reinterpret_cast<double2 *>(acc + b.at + row * kAccPitch + m * 8 + 2 * k);
+                        double2 v = *p;
+                        v.x += a[m][0]; v.y += a[m][1];
+                        *p = v;
+                    }
+                }
+                __syncwarp();                                          // (two rows of the list may be one, in a damaged blob)
+            }
+        }
+    }
+    __syncthreads();
+    // the warps' sums in order, bias, residual, ReLU, one rounding; consecutive threads along the row of Y
+    for (int e = t; e < outs * rows_here; e += nt) {
+        const int m = e / outs, r = e - m * outs;
+        const size_t o = (size_t)(m0 + m) * d.O + (size_t)bo0 * Bo + r;
+        double v = acc0[r * kAccPitch + m];
+        for (int w = 1; w < W; ++w) v += acc0[((size_t)w * outs + r) * kAccPitch + m];
+        if (bias) v += (double)bias[bo0 * Bo + r];
+        if (res) v += (double)lin_load(res + o);
+        if (d.relu) v = v > 0 ? v : 0;
+        lin_store(y + o, (float)v);
+    }
+}
+
 template <typename TX, typename TY>
 static npas_status launch(const npas_linear_desc &d, const npas_bb_desc &bb, const BbLayout &L, dim3 grid, const void *x,
                           const void *blob, const float *bias, const void *res, void *y, cudaStream_t st, Launch how)
 {
+    if (rows_preferred(d, bb)) {
+        const LinRowsPlan p = rows_plan(d, bb);
+        auto k = linear_bb_rows_kernel<TX, TY>;
+        if (allow_dynamic_smem(reinterpret_cast<const void *>(k), (int)p.bytes) != NPAS_OK) return NPAS_ERR_CUDA;
+        const cudaError_t e = tc::launch_pdl(how, k, dim3(grid.x, (L.nBo + p.gb - 1) / p.gb), dim3(p.warps * 32), p.bytes, st, d, (int)bb.Bo, (int)bb.Bi, L, p,
+                                             static_cast<const TX *>(x), static_cast<const uint8_t *>(blob), bias, static_cast<const TY *>(res), static_cast<TY *>(y));
+        count_launch();
+        return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;
+    }
     const LinSimtSmem S = smem_plan(bb);
     auto k = linear_bb_simt_kernel<TX, TY>;
     if (allow_dynamic_smem(reinterpret_cast<const void *>(k), (int)S.bytes) != NPAS_OK) return NPAS_ERR_CUDA;

@@ -101,10 +101,10 @@ def _header(blob):
     return blob.data[:128].view(torch.int32).tolist()
 
 
-@pytest.mark.parametrize("dtype,path", [("f32", 1), ("bf16", 1), ("bf16", 3)])
-def test_gemm_ignores_list_entries_outside_their_block(dtype, path):
+@pytest.mark.parametrize("dtype,path,M", [("f32", 1, 70), ("bf16", 1, 70), ("bf16", 3, 70), ("f32", 1, 7000), ("bf16", 1, 7000)])
+def test_gemm_ignores_list_entries_outside_their_block(dtype, path, M):
     """Row and column numbers of a damaged blob index shared memory: one outside its block counts for nothing."""
-    c = inputs.linear_case(M=70, I=128, O=96, Bo=32, Bi=64, keep_rows=8, keep_cols=16, dtype=dtype, seed=811)
+    c = inputs.linear_case(M=M, I=128, O=96, Bo=32, Bi=64, keep_rows=8, keep_cols=16, dtype=dtype, seed=811)
     blob = npas.pack_bb(dev(c.w, dtype), c.row_keep, c.col_keep, 32, 64)
     h, rk, ck = _header(blob), c.row_keep.copy(), c.col_keep.copy()
     off_rows, off_cols = h[11], h[12]
@@ -164,3 +164,20 @@ def test_float64_convolution_at_its_edges(dtype, N, H, W, C, K, Mb, Nb, R, strid
     y = _conv(c, 1)
     assert floored_rel_err(host(y), _conv_ref(c)) < (TOL_F32 if dtype == "f32" else TOL_BF16)
     assert torch.equal(y, _conv(c, 1))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("M,I,O,Bo,Bi", [(3001, 508, 508, 4, 4), (2100, 520, 96, 32, 40), (9999, 66, 33, 33, 33), (1200, 1600, 160, 5, 64), (10000, 21, 30, 3, 7),
+                                         (4800, 320, 31, 31, 64), (2500, 128, 64, 1, 16)])
+def test_float64_gemm_of_small_blocks_at_its_edges(dtype, M, I, O, Bo, Bi):
+    """A warp per block: rows of blocks that do not divide the outputs per CTA, several phases of columns, ragged rows of X, odd
+    widths that no wide copy starts on, empty and full blocks; and the widest block rows it takes against the first it does not."""
+    c = inputs.linear_case(M=M, I=I, O=O, Bo=Bo, Bi=Bi, keep_rows=lambda a, b: (a * 29 + b * 13) % (Bo + 1), keep_cols=lambda a, b: (a * 7 + b * 23) % (Bi + 1),
+                           dtype=dtype, seed=831)
+    r = torch.randn(M, O, generator=torch.Generator().manual_seed(9)).to(torch.bfloat16)
+    blob, ws = npas.pack_bb(dev(c.w, dtype), c.row_keep, c.col_keep, Bo, Bi), npas.workspace()
+    run = lambda: npas.linear_bb(dev(c.x, dtype), blob, dev(c.bias), r.to(torch.float32 if dtype == "f32" else torch.bfloat16).cuda(), relu=c.relu, ws=ws, path=1)
+    y = run()
+    ref = oracle.linear_bb(c.x, c.w, c.row_keep, c.col_keep, Bo=Bo, Bi=Bi, bias=c.bias, residual=r.double().numpy(), relu=c.relu)
+    assert floored_rel_err(host(y), ref) < (TOL_F32 if dtype == "f32" else TOL_BF16)
+    assert torch.equal(y, run())
