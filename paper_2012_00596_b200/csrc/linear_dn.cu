@@ -96,21 +96,20 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     auto width = [&](int nt) { return min(p.BN, p.O - nt * p.BN); };
 
     // The producer starts by itself: it initialises the barriers it signals and requests the first ring of stages before the
-    // other warps have set up theirs and tensor memory (0.4 us).  In a chain of layers the weights do not wait for the kernel
-    // before this one.
+    // other warps have set up theirs and tensor memory (0.4 us); in a chain of layers only, where the weights do not wait for the
+    // kernel before this one (by itself, waiting here would hold up the others' set-up).
     int early = 0;
     if (tid == 0) {
         for (int s = 0; s < p.S; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], 1); }
         fence_barrier_init();
         fence_proxy_async_smem();
-        if (!p.early) pdl_wait();
         int tile = blockIdx.x, k = 0;
-        for (; early < p.S && tile < p.n_tiles; ++early) {
+        for (; p.early && early < p.S && tile < p.n_tiles; ++early) {
             mbar_arrive_expect_tx(&bars->full[early], p.stage_bytes);
             tma_load_2d(smem + (size_t)early * p.stage_bytes + kXBytes, &tmap_w, &bars->full[early], k * 64, (tile % p.nNT) * p.BN);
             if (++k == p.nK) { k = 0; tile += gridDim.x; }
         }
-        pdl_wait();
+        if (p.early) pdl_wait();
         tile = blockIdx.x; k = 0;
         for (int e = 0; e < early; ++e) {
             tma_load_2d(smem + (size_t)e * p.stage_bytes, &tmap_x, &bars->full[e], k * 64, (tile / p.nNT) * kRows);
