@@ -403,10 +403,13 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinDnParams &p)
     p.nMT = (d.M + kRows - 1) / kRows;
     p.relu = d.relu; p.y_bf16 = d.y_dtype == NPAS_BF16;
     const uint32_t fixed = ((uint32_t)d.O + 256u) * 4 + 128 + (uint32_t)sizeof(LinDnBars) + 1024 + 256;
-    // Column tile BN: any multiple of 64 where 64 divides O (the last tile what is left), by the model; else the widest power of
-    // two that divides O; else 128, the last tile cut short.  Only tiles that leave room for enough stages (three once the K
-    // loop has three or more steps), else for two.  Epilogue slots (bf16 output, BN % 64 == 0): three when only stores pass
-    // through them, six when the residual is prefetched into them.
+    // Column tile BN: any multiple of 64 where 64 divides O (the last tile what is left), by the model.  Where only 16 does, the
+    // widest power of two that divides O, unless a multiple of 64 with its last tile cut short is modelled faster: 12544x1024 -> 2000
+    // takes 348 us in 125 tiles of 16 that each read X again and 45 in tiles of 256, 30000x64 -> 160 7.4 and 5.8; with fp32 output,
+    // whose stores the model is too kind to, by a quarter (30000x128 -> 160 11.4 in tiles of 32 and 12.8 of 192).  Where not even 16
+    // does, 128.  Only tiles that leave room for enough stages (three once the K loop has three or more steps), else for two.
+    // Epilogue slots (bf16 output, BN % 64 == 0): three when only stores pass through them, six when the residual is prefetched
+    // into them.
     // (the call descriptor's `variant` restricts the choice to one width)
     const int want = p.nK >= 3 ? 3 : 2, want_bn = d.variant, sms = sm_count();
     // a requested width is whole 16-column chunks, whatever O: the MMA's width is rounded up to 16 while the two accumulators lie
@@ -414,13 +417,13 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinDnParams &p)
     if (want_bn && (want_bn < 16 || want_bn > 256 || want_bn % 16)) return false;
     if (want_bn && d.O % 16 == 0 && (want_bn & (want_bn - 1) || d.O % want_bn) && (d.O % 64 || want_bn % 64 || want_bn > d.O)) return false;
     p.BN = 0; p.cost = 0.f;
-    auto consider = [&](int bn, int stages) {
+    auto consider = [&](int bn, int stages, float times = 1.f) {
         const int ns = p.y_bf16 && bn % 64 == 0 ? (d.has_residual ? kMaxSlots : 3) : 0;
         const uint32_t stage = round_up(kXBytes + (uint32_t)bn * 128u, 1024);   // multiples of 1024: swizzled tiles stay aligned
         const uint32_t need = fixed + (uint32_t)ns * kSlotBytes;
         const int st = need < kSmemLimit ? (int)((kSmemLimit - need) / stage) : 0;
         const float cost = (float)linear_modelled(d, bn, false, sms);
-        if (st < stages || (p.BN && cost >= p.cost)) return;
+        if (st < stages || (p.BN && cost >= times * p.cost)) return;
         p.BN = bn; p.NS = ns; p.stage_bytes = stage; p.S = st > kMaxStages ? kMaxStages : st; p.cost = cost;
     };
     for (int stages = want; stages >= 2 && !p.BN; --stages) {
@@ -428,8 +431,9 @@ bool plan(const npas_linear_desc &d, const npas_bb_desc &bb, LinDnParams &p)
         else if (d.O % 64 == 0) {
             for (int bn = 64; bn <= 256 && bn <= d.O; bn += 64) consider(bn, stages);
         } else if (d.O % 16 == 0) {
-            for (int bn = 256; bn >= 16 && !p.BN; bn /= 2)
-                if (d.O % bn == 0) consider(bn, stages);
+            consider(d.O % 32 == 0 ? 32 : 16, stages);
+            const bool had = p.BN != 0;
+            for (int bn = 64; bn <= 256 && bn < d.O + 64; bn += 64) consider(bn, stages, had && p.BN < 64 && !p.y_bf16 ? 0.75f : 1.f);
         } else consider(128, stages);
     }
     if (p.BN == 0) return false;

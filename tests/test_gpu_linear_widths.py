@@ -40,3 +40,18 @@ def test_requested_tiles_where_16_does_not_divide_the_outputs(M, O, bn):
         npas.linear_bb(dev(c.x, "bf16"), blob, dev(c.bias), r.to(odt).cuda(), relu=c.relu, out=y, ws=ws, path=5, variant=bn)
         npas.check_device_status(ws)
         assert floored_rel_err(host(y), ref) < TOL_BF16
+
+
+@pytest.mark.parametrize("M,I,O", [(5000, 512, 1008), (20000, 64, 80), (3000, 256, 2000), (9000, 128, 48), (300, 1024, 16), (12000, 192, 208)])
+def test_widths_that_only_16_divides(M, I, O):
+    """Automatic column tiles there: a multiple of 64 with the last one cut, or a power of two."""
+    c = inputs.linear_case(M=M, I=I, O=O, Bo=16, Bi=64, keep_rows=8, keep_cols=48, dtype="bf16", seed=1403)
+    r = torch.randn(M, O, generator=torch.Generator().manual_seed(9)).to(torch.bfloat16)
+    blob, ws = npas.pack_bb(dev(c.w, "bf16"), c.row_keep, c.col_keep, c.Bo, c.Bi), npas.workspace()
+    ref = oracle.linear_bb(c.x, c.w, c.row_keep, c.col_keep, Bo=c.Bo, Bi=c.Bi, bias=c.bias, residual=r.double().numpy(), relu=c.relu)
+    for odt in (torch.bfloat16, torch.float32):
+        for path in (0, 5):
+            y = torch.full((M, O), float("nan"), dtype=odt, device="cuda")
+            npas.linear_bb(dev(c.x, "bf16"), blob, dev(c.bias), r.to(odt).cuda(), relu=c.relu, out=y, ws=ws, path=path)
+            npas.check_device_status(ws)
+            assert floored_rel_err(host(y), ref) < TOL_BF16
