@@ -261,7 +261,7 @@ npas_status npas_linear_bb_kernel(const npas_linear_desc *d, const npas_bb_desc 
  * the automatic choice and every kernel and tile shape that takes the layer on the caller's own buffers
  * (of the many shapes of path 6's split form those modelled within a quarter of its best; one warm-up and
  * `reps` timed launches each, CUDA events on `stream`; what beats the automatic choice is timed against
- * it twice more), and returns the fastest as the (path, variant) pair to put into the call descriptor; *us_out (nullable) receives its time per launch in microseconds.  The
+ * it twice more and must be 3 % faster), and returns the fastest as the (path, variant) pair to put into the call descriptor; *us_out (nullable) receives its time per launch in microseconds.  The
  * plan is these two integers: the caller keeps them with the layer.  Synchronises the stream several
  * times (not for use inside a stream capture); y_dev holds the layer's result afterwards.  d->path and
  * d->variant are ignored.  Arguments as in the compute calls. */
