@@ -115,7 +115,7 @@ typedef struct {
 
 /* Weight matrix of a block-based layer.  max_cols: the largest number of kept columns of any single
  * block, as the caller knows it from the masks (0 = unknown).  It fixes the width Kp of the blob's
- * tiles section; the tensor-core GEMM needs it (0 selects the CUDA-core kernel) and reports
+ * tiles section; the gathering tensor-core GEMM needs it (0 excludes that kernel) and reports
  * NPAS_ERR_BLOB through the device status words when it does not match the blob. */
 typedef struct {
     int32_t O, I, Bo, Bi;
@@ -124,8 +124,8 @@ typedef struct {
 } npas_bb_desc;
 
 /* One convolution call. x_dtype must equal the blob dtype; y_dtype may be f32 or (bf16 path) bf16.
- * path: 0 = automatic, 1 = force the CUDA-core kernel, 2 = automatic among the tcgen05 kernels,
- * 3 = force the tcgen05 kernel with both operands in shared memory, 5 = force the tcgen05 kernel
+ * path: 0 = automatic, 1 = force the float64 kernel (float64 matrix instructions; every geometry),
+ * 2 = automatic among the tcgen05 kernels, 3 = force the tcgen05 kernel with both operands in shared memory, 5 = force the tcgen05 kernel
  * for three-channel 7x7 stride-2 first layers, 6 = force the tcgen05 kernel that multiplies the
  * blob's dense operand image, 7 = force the variant of that kernel that runs on CTA pairs
  * (cta_group::2; C % 64 == 0, K % 64 == 0), 8 = force the tcgen05 kernel that multiplies kept
@@ -145,7 +145,7 @@ typedef struct {
                         npas_tune_conv2d_bp measures the candidates and returns the best (path, variant). */
 } npas_conv_desc;
 
-/* One block-based GEMM call.  path: 0 = automatic, 1 = force the CUDA-core kernel, 2 = automatic
+/* One block-based GEMM call.  path: 0 = automatic, 1 = force the float64 kernels, 2 = automatic
  * among the tcgen05 kernels, 3 = force the tcgen05 kernel that gathers the kept columns of X,
  * 5 = force the tcgen05 kernel that reads X and the blob's masked dense image by TMA, 6 = force
  * the variant of that kernel that runs on CTA pairs (cta_group::2; O a multiple of 128)
@@ -228,6 +228,12 @@ npas_status npas_unpack_bb(const npas_bb_desc *d, const void *blob_dev, size_t b
  *   npas_blob_check to verify a blob of unknown origin).  y must not alias x.
  *   ws_dev: NPAS_WORKSPACE_BYTES of device scratch, zeroed once by the caller before first use;
  *   a kernel whose bounded waits expire records NPAS_ERR_TIMEOUT there (npas_check_device_status).
+ *   The blob, like every input, is read in stream order: a packing call or a copy into it may be what
+ *   stands right ahead of the call.
+ *   Infinities and NaN in x: an output depends on nothing outside its own window (or row).  Inside it, the
+ *   kernels that multiply kept weights only (paths 1, 3 and 8 of the convolution, 1 of the GEMM) ignore
+ *   inputs that meet pruned weights; the others multiply them by zero, so that an infinity or a NaN there makes
+ *   the output NaN.  ReLU turns a NaN sum into zero.
  * npas_linear_bb: block-based pruned GEMM
  *   Y[m,o] = act(bias[o] + sum over kept i of X[m,i] W[o,i] (+ residual[m,o])); residual [M,O] in
  *   y_dtype, may not alias y.
@@ -242,16 +248,16 @@ npas_status npas_conv2d_bp(const npas_conv_desc *d, const npas_bp_desc *bp, cons
  * wins) of the convolution output, which is never written.  The result is bit for bit that of
  * npas_conv2d_bp followed by npas_maxpool2d.  Fused today: three-channel 7x7 stride-2 first layers
  * (path 5's envelope) with ReLU, bf16 output, no residual, and the 3x3 / stride-2 / pad-1 window;
- * any other combination returns NPAS_ERR_UNSUPPORTED and the caller issues the two calls.  The call
- * clears y_pooled_dev on `stream` before the kernel. */
+ * any other combination returns NPAS_ERR_UNSUPPORTED and the caller issues the two calls.  Images wider
+ * than 256 columns and layers of more than 128 filters clear y_pooled_dev on `stream` before the kernel. */
 npas_status npas_conv2d_bp_maxpool(const npas_conv_desc *d, const npas_bp_desc *bp, int32_t pool_r,
                                    int32_t pool_stride, int32_t pool_pad, const void *x_dev, const void *blob_dev,
                                    const float *bias_dev, void *y_pooled_dev, void *ws_dev, size_t ws_bytes,
                                    void *stream);
 
-/* Which kernel the call would run (the value `path` takes to force it): convolution 1 = CUDA cores,
+/* Which kernel the call would run (the value `path` takes to force it): convolution 1 = float64,
  * 3 = tcgen05 with both operands in shared memory, 5 = three-channel first layer, 6 = the blob's dense
- * operand image, 7 = the same on CTA pairs, 8 = kept (block, tap) pairs only; GEMM 1 = CUDA cores,
+ * operand image, 7 = the same on CTA pairs, 8 = kept (block, tap) pairs only; GEMM 1 = float64,
  * 3 = gathered kept columns, 5 = the blob's masked dense image by TMA, 6 = the same on CTA pairs.
  * Host only, nothing is launched; NPAS_ERR_UNSUPPORTED when the requested path declines the geometry. */
 npas_status npas_conv2d_bp_kernel(const npas_conv_desc *d, const npas_bp_desc *bp, int32_t *kernel_id);

@@ -381,8 +381,7 @@ def conv2d_bp_kernel(x_shape, blob: BpBlob, *, stride=1, pad=1, dtype=torch.bflo
 
 def conv2d_bp_workspace(x_shape, blob: BpBlob, *, stride=1, pad=1, dtype=torch.bfloat16, out_dtype=None, relu=False,
                         bias=False, residual=False, path=0, variant=0, device="cuda") -> torch.Tensor:
-    """npas_conv2d_bp_workspace: zeroed device scratch of the size the call can use for this layer (the status
-    words, plus room for the partial sums of a split last round where the kept-pairs kernel runs)."""
+    """npas_conv2d_bp_workspace: zeroed device scratch of the size the call needs for this layer (the status words)."""
     lib = load()
     N, H, W, C = x_shape
     d = blob.desc

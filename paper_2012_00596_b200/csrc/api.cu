@@ -110,7 +110,7 @@ npas_status npas_linear_bb_workspace(const npas_linear_desc *d, const npas_bb_de
     return NPAS_OK;
 }
 
-// Kernel ids (the values `path` takes to force one): 1 CUDA cores, 3 tcgen05 with both operands in
+// Kernel ids (the values `path` takes to force one): 1 float64, 3 tcgen05 with both operands in
 // shared memory, 5 three-channel first layer, 6 dense operand image, 7 the same on CTA pairs, 8 kept
 // pairs only.  Returns 0 when the requested path does not take the geometry.
 // Path 6 has two forms: the persistent kernel, and for few output tiles the one that splits channels and taps over a
@@ -136,7 +136,7 @@ static int conv_kernel_for(const npas_conv_desc &d, const npas_bp_desc &bp)
         default: return 0;
     }
     // automatic: the first-layer kernel; kept pairs only where that was measured faster (few taps kept,
-    // blocks of 16 channels or more); else the dense-image kernels; else shared-memory operands; else CUDA cores
+    // blocks of 16 channels or more); else the dense-image kernels; else shared-memory operands; else float64
     if (conv_stem_supported(d, bp)) return 5;
     if (conv_kr_preferred(d, bp)) return 8;
     if (conv_split(d, bp)) return 6;
@@ -154,7 +154,7 @@ static bool linear_split_k(const npas_linear_desc &d, const npas_bb_desc &bb)
     return (d.path == 0 || d.path == 2) && linear_sk_preferred(d, bb);
 }
 
-// 1 CUDA cores, 3 gathered X (kept columns only), 5 masked dense image by TMA, 6 the same on CTA pairs.
+// 1 float64, 3 gathered X (kept columns only), 5 masked dense image by TMA, 6 the same on CTA pairs.
 static int linear_kernel_for(const npas_linear_desc &d, const npas_bb_desc &bb)
 {
     switch (d.path) {
@@ -166,7 +166,7 @@ static int linear_kernel_for(const npas_linear_desc &d, const npas_bb_desc &bb)
         default: return 0;
     }
     // automatic: both operands by TMA (on CTAs or CTA pairs, whichever the model of both puts lower), then the gather
-    // kernel, then CUDA cores
+    // kernel, then float64
     if (linear_sk_preferred(d, bb)) return 5;
     // (256 or more inputs and less than a sixteenth of the chip in 128 x 128 tiles stay on pairs: there the two are within the
     // model's error of each other)
@@ -381,7 +381,7 @@ npas_status tune(const std::vector<Cand> &cands, R run, int reps, void *ws, cuda
     int best = -1;
     float best_us = 0.f, first_us = -1.f;
     for (size_t i = 0; i < cands.size(); ++i) {
-        if (cands[i].path == 1 && i > 0 && best >= 0) continue;          // CUDA cores only when nothing else takes the layer
+        if (cands[i].path == 1 && i > 0 && best >= 0) continue;          // the float64 kernels only when nothing else takes the layer
         if (i > 0 && cands[i].path == cands[0].path && cands[i].variant == cands[0].variant) continue;
         const float us = time(cands[i]);
         if (us < 0.f) continue;

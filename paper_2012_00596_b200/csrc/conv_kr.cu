@@ -33,10 +33,12 @@
 // records, waits for the staging buffer and the weight slot, issues, and commits once: that commit
 // frees both the staging buffer and the weight slot.
 // What a CTA works on: whole tiles while there is one for every CTA; a last round that would leave half of them idle is
-// split by filters, each part issued by a share of the issuing warps.  64x28x28x512 -> 512, blocks of 16 x 16, three taps
-// of nine: 131 us (147 with tiles of whole rows of one image, an eighth of the lanes on padding and seven rounds of items).
-// What is left: a chunk takes 940 cycles, 40 MMAs of 24; shared memory is busy for 710 of them (288 for the stagers' reads, 190
-// each for the weights' arrival and for the MMAs' reading them).
+// split by filters, each part issued by a share of the issuing warps.  64x28x28x512 -> 512, blocks of 16 x 16, back to back in
+// a captured graph: 104, 116 and 132 us for one, two and three taps of nine (117, 131 and 141 with tiles of whole rows of one
+// image, an eighth of the lanes on padding and seven rounds of items).
+// What is left: by those three figures some 90 us do not depend on the taps kept at all (the fit that the choice uses has 0.40
+// of a chunk's 0.63 us in that part): staging the nine shifted slices of every chunk and handing them over, and per tile an
+// epilogue that nothing overlaps.  The MMAs of three taps (40 of 24 cycles per chunk) are not what bounds it.
 // Every wait is bounded; a blob that breaks the descriptor's promises is reported, not computed.
 #include <numeric>
 

@@ -3,7 +3,8 @@
 // a row or a column of a block) is the sum of the squares of its weights, accumulated in fp64 in a
 // fixed order (filters / rows outer, channels / columns inner; a square of a float is exact in
 // fp64, so fused or separate multiply-add give the same bits); a block keeps its `keep`
-// highest-scoring groups, ties go to the lower index.  Offline step: one CTA per block.
+// highest-scoring groups, ties go to the lower index.  Offline step: one CTA per block for the per-block counts; for the
+// layer-wide budget a thread per group scores and a cluster selects.
 #include "common.cuh"
 #include "tc_common.cuh"
 

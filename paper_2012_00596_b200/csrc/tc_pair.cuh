@@ -23,11 +23,7 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// The same without making memory visible across the cluster: for "the other CTA is running and its barriers are initialised"
+// Cluster barrier that makes no memory visible across the cluster: for "the other CTA is running and its barriers are initialised"
 // (fence.mbarrier_init) and "the other CTA is done with this one's memory".  A release here waits for every store and copy of
 // the CTA still in flight: it took 0.7 us at either end of a kernel.
 __device__ __forceinline__ void cluster_sync_relaxed()

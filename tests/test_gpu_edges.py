@@ -181,3 +181,44 @@ def test_float64_gemm_of_small_blocks_at_its_edges(dtype, M, I, O, Bo, Bi):
     ref = oracle.linear_bb(c.x, c.w, c.row_keep, c.col_keep, Bo=Bo, Bi=Bi, bias=c.bias, residual=r.double().numpy(), relu=c.relu)
     assert floored_rel_err(host(y), ref) < (TOL_F32 if dtype == "f32" else TOL_BF16)
     assert torch.equal(y, run())
+
+
+@pytest.mark.parametrize("path", [0, 1, 3, 6, 7, 8])
+def test_conv_and_values_that_are_not_finite(path):
+    """Infinities and NaNs: nothing outside an output's window counts on any path, and what only pruned weights would meet counts
+    for nothing where kept pairs alone are multiplied."""
+    c = inputs.conv_case(N=2, H=12, W=13, C=64, K=128, Mb=16, Nb=16, keep=lambda fb, cb: (0 if cb == 2 and fb < 7 else 1 + (fb + cb) % 8), dtype="bf16",
+                         relu=False, seed=841)
+    x = dev(c.x, "bf16")
+    blob, ws = npas.pack_bp(dev(c.w, "bf16"), c.tap_mask, 16, 16), npas.workspace()
+    run = lambda v: npas.conv2d_bp(v, blob, dev(c.bias), ws=ws, path=path, out_dtype=torch.float32)
+    y0 = run(x)
+    for h, w in ((0, 0), (5, 6), (11, 12)):
+        for bad in (float("inf"), float("nan")):
+            v = x.clone()
+            v[1, h, w, 40] = bad                     # a channel that seven of the eight filter blocks have pruned at every tap
+            y = run(v)
+            near = ((torch.arange(12, device="cuda") - h).abs() <= 1)[:, None] & ((torch.arange(13, device="cuda") - w).abs() <= 1)[None, :]
+            assert torch.equal(y[0], y0[0]) and torch.equal(y[1][~near], y0[1][~near])
+            if path in (1, 3, 8):
+                assert torch.equal(y[1][..., :112], y0[1][..., :112])
+    npas.check_device_status(ws)
+
+
+@pytest.mark.parametrize("path", [0, 1, 3, 5, 6])
+def test_gemm_and_values_that_are_not_finite(path):
+    c = inputs.linear_case(M=200, I=192, O=256, Bo=64, Bi=64, keep_rows=32, keep_cols=32, dtype="bf16", relu=False, seed=842)
+    x = dev(c.x, "bf16")
+    blob, ws = npas.pack_bb(dev(c.w, "bf16"), c.row_keep, c.col_keep, 64, 64), npas.workspace()
+    run = lambda v: npas.linear_bb(v, blob, dev(c.bias), ws=ws, path=path, out_dtype=torch.float32)
+    y0, others = run(x), torch.arange(200, device="cuda") != 130
+    element = torch.from_numpy(oracle.bb_element_mask(c.row_keep, c.col_keep, 256, 192, 64, 64)).cuda().bool()
+    for i in (0, 77, 191):
+        for bad in (float("inf"), float("nan")):
+            v = x.clone()
+            v[130, i] = bad
+            y = run(v)
+            assert torch.equal(y[others], y0[others])
+            if path == 1:
+                assert torch.equal(y[130][~element[:, i]], y0[130][~element[:, i]])
+    npas.check_device_status(ws)
