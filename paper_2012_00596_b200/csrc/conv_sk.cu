@@ -420,7 +420,7 @@ bool conv_sk_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
     return planned(d, bp, p, false);
 }
 
-// Measured against the persistent kernels (this one, then the better of the two): 14x14x256 -> 256 one image 4.8 against
+// Measured against the persistent kernels (this one, then the better of the two, both in a chain of layers): 14x14x256 -> 256 one image 4.8 against
 // 9.9 us, four 6.7 against 10.1, eight 8.1 against 10.2; 7x7x512 -> 512 5.8 against 14.6; 7x27x29x96 -> 160 7.8 against 8.3;
 // 54x6x33x160 -> 32 (108 position tiles) 8.0 against 6.9.  So: one wave, and no more position tiles than half the SMs.
 // Strided 3x3 layers that the pair kernel does not take by phases (it needs multiples of 64 channels and filters) always

@@ -287,7 +287,7 @@ bool linear_sk_supported(const npas_linear_desc &d, const npas_bb_desc &bb)
 }
 
 // Where the persistent kernels leave most SMs idle: fewer tiles of 128 x 128 than a quarter of the SMs.  Measured (this
-// kernel against the better persistent one): 49x2048 -> 512 3.9 against 9.9 us, 64x2048 -> 1000 4.4 against 9.8,
+// kernel against the better persistent one, both in a chain of layers): 49x2048 -> 512 3.9 against 9.9 us, 64x2048 -> 1000 4.4 against 9.8,
 // 196x1024 -> 256 3.9 against 7.1, 784x512 -> 128 3.6 against 5.1, 1x128 -> 256 2.5 against 3.9; from about forty
 // tiles on they draw level (6272x512 -> 128 5.8 against 5.3).  Up to 256 columns there is little to split and the gain
 // is that of narrower tiles on more SMs: for a single row tile, or where 128 x 32 tiles fill a fifth of the chip.
