@@ -156,6 +156,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     // producer and the tap unions do not wait for its end.
     const uint32_t tmem_base = bars->tmem_base;
     if (warp == 0 || !p.early) pdl_wait();
+    blob = behind_wait(blob);
     if (!p.early) read_header();
     // the two producers start at once; the other warps first stage the tap unions
     if (warp != 0 && warp != 2) {
@@ -175,6 +176,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         }
         consumers_sync();
         pdl_wait();
+        bias = behind_wait(bias); res = behind_wait(res);
     }
 
     if (warp == 0) {

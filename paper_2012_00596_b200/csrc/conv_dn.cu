@@ -73,7 +73,6 @@ conv_bp_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDnParams
     volatile uint32_t *abort_flag = &bars->abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
 
     if (tid == 0) {
         const int nmma = p.MT * p.NG * p.TS;
@@ -90,6 +89,8 @@ conv_bp_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDnParams
     __syncthreads();
     tc_fence_after_sync();
     pdl_wait();                        // nothing above touches global memory
+    blob = behind_wait(blob); bias = behind_wait(bias); res = behind_wait(res);
+    const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
     const uint32_t tmem_base = bars->tmem_base;
     // Cold operands: the whole grid asks L2 for the operand image (one slice per CTA) and every CTA for the
     // input rows of its first item, so that DRAM latency is paid once, up front and in parallel, instead

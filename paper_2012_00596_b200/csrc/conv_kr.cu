@@ -278,8 +278,6 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int grp = blockIdx.y, fb0 = grp * p.GS;
 
-    const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
-
     // ---- set-up (once per CTA) ------------------------------------------------------------------
     if (tid == 0) {
         for (int s = 0; s < p.SA; ++s) { mbar_init(&bars->act_full[s], 1); mbar_init(&bars->act_empty[s], 4 * p.NP); }
@@ -297,6 +295,8 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     if (tid < kMaxTaps) bars->tapoff[tid] = tid < p.RS ? (uint32_t)(tid / p.S) * p.row_pitch + (uint32_t)(tid % p.S) * 16u : 0u;
     __syncthreads();
     if (!p.early) pdl_wait();
+    blob = behind_wait(blob);
+    const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
     // the blob must be what the descriptor says: version, the tile section and its grouping
     const bool hdr_ok = hdr[BP_MAGIC] == kMagicBP && hdr[BP_VERSION] == kVersion && hdr[BP_OFF_KT] != 0u &&
                         hdr[BP_GS] == (uint32_t)p.GS && hdr[BP_MB] == (uint32_t)p.Mb && hdr[BP_NCB] == (uint32_t)p.nCB;
@@ -329,6 +329,7 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         }
     }
     pdl_wait();
+    bias = behind_wait(bias); res = behind_wait(res);
     for (int i = tid; i < p.GS * p.Mb; i += kThreads) bars->bias[i] = bias ? bias[fb0 * p.Mb + i] : 0.f;
     fence_proxy_async_smem();
     tc_fence_before_sync();

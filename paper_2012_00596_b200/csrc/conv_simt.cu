@@ -58,6 +58,7 @@ conv_bp_simt_kernel(npas_conv_desc d, int Mb, int Nb_, int P, int Q, int KW, con
 
     tc::pdl_trigger();
     tc::pdl_wait();
+    x = tc::behind_wait(x); blob = tc::behind_wait(blob); bias = tc::behind_wait(bias); res = tc::behind_wait(res);
     const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
     const uint32_t nCB = d.C / Nb, G = NB ? NB : (Nb % 8 == 0) ? 8 : Nb;
     const uint32_t *blk_off = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_BLK]);

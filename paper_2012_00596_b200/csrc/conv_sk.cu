@@ -110,6 +110,7 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     const uint32_t tmem_base = bars->tmem_base;
     cluster_arrive();                  // this CTA is running: its shared memory may be written by the others
     if (!p.early) pdl_wait();
+    blob = behind_wait(blob);
 
     if (warp == 2) {
         // ---- weights: one box per 16-channel chunk; the first ring of stages before anything else ------------------
@@ -152,6 +153,7 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         __syncwarp();
     }
     pdl_wait();
+    bias = behind_wait(bias); res = behind_wait(res);
     if (warp > 2)
         for (int i = tid - 96; i < p.NT; i += kThreads - 96) bias_s[i] = (bias && k0 + i < p.K) ? bias[k0 + i] : 0.f;
 

@@ -125,6 +125,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
     {
         // weight of (tap (r, s), channel c, filter n) at k = s * 4 + c of kernel row r
         if (!p.early) pdl_wait();
+        blob = behind_wait(blob);
         const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
         const uint32_t *blk_off = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_BLK]);
         const uint32_t *pairs = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_PAIRS]);
@@ -163,6 +164,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
         }
     }
     pdl_wait();
+    x = behind_wait(x); bias = behind_wait(bias);
     // bias: the fourth channel of every pixel is one, and a window's pixels 2 .. 4 of kernel row 3 (never outside the image)
     // weigh it with the bias' upper, middle and lower eight bits, so that the sum is exact
     for (int f = tid; bias && f < p.K; f += kThreads<kPool>) {

@@ -131,6 +131,7 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     __syncthreads();
     tc_fence_after_sync();
     pdl_wait();                        // nothing above but the producer's copies touches global memory
+    bias = behind_wait(bias); res = behind_wait(res);
     // the biases: staged by the epilogue warps, which meet again before the first use
     if (warp >= kFirstEpiWarp && warp < kResWarp) {
         for (int i = tid - kFirstEpiWarp * 32; i < p.nNT * p.BN; i += kEpiWarps * 32) bias_s[i] = (bias && i < p.O) ? bias[i] : 0.f;

@@ -102,14 +102,15 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
     double *acc = reinterpret_cast<double *>(sm + S.off_grp + (size_t)g * S.grp_bytes);       // [Bo][kAccPitch]
 
     const int bo = blockIdx.y, m0 = blockIdx.x * kBM, rows_here = min(kBM, d.M - m0), nBi = (int)L.nBi;
-    const uint32_t *voff = reinterpret_cast<const uint32_t *>(blob + L.off_voff);
-    const TX *vals = reinterpret_cast<const TX *>(blob + L.off_values);
     const bool x16 = sizeof(TX) == 4 && (d.I & 3) == 0 && (Bi & 3) == 0;
     const bool x2 = (d.I & 1) == 0 && (Bi & 1) == 0;
     const int per_phase = (int)S.phase_cols / Bi;
 
     tc::pdl_trigger();
     tc::pdl_wait();
+    x = tc::behind_wait(x); blob = tc::behind_wait(blob); bias = tc::behind_wait(bias); res = tc::behind_wait(res);
+    const uint32_t *voff = reinterpret_cast<const uint32_t *>(blob + L.off_voff);
+    const TX *vals = reinterpret_cast<const TX *>(blob + L.off_values);
     for (int e = tg; e < Bo * kAccPitch; e += gt) acc[e] = 0;
     for (int b0 = 0; b0 < nBi; b0 += per_phase) {
         const int nb = min(per_phase, nBi - b0), width = nb * Bi, pitch = (int)round_up((uint32_t)width, 8) + 4;
@@ -246,12 +247,13 @@ linear_bb_rows_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinRowsPla
     double *acc0 = reinterpret_cast<double *>(sm + S.off_acc), *acc = acc0 + (size_t)warp * outs * kAccPitch;   // [W][outs][kAccPitch]
     const int m0 = blockIdx.x * kBM, rows_here = min(kBM, d.M - m0), nBi = (int)L.nBi, per_phase = (int)S.phase_cols / Bi;
     const bool x16 = sizeof(TX) == 4 && (d.I & 3) == 0 && (Bi & 3) == 0, x2 = (d.I & 1) == 0 && (Bi & 1) == 0;
-    const uint32_t *voff = reinterpret_cast<const uint32_t *>(blob + L.off_voff);
-    const TX *vals = reinterpret_cast<const TX *>(blob + L.off_values);
 
     tc::pdl_trigger();
     for (int e = lane; e < outs * kAccPitch; e += 32) acc[e] = 0;
     tc::pdl_wait();
+    x = tc::behind_wait(x); blob = tc::behind_wait(blob); bias = tc::behind_wait(bias); res = tc::behind_wait(res);
+    const uint32_t *voff = reinterpret_cast<const uint32_t *>(blob + L.off_voff);
+    const TX *vals = reinterpret_cast<const TX *>(blob + L.off_values);
     for (int b0 = 0; b0 < nBi; b0 += per_phase) {
         const int nb = min(per_phase, nBi - b0), width = nb * Bi;
         if (b0) __syncthreads();                                       // the phase before has been read

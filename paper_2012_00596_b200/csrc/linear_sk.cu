@@ -88,6 +88,7 @@ linear_bb_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     const uint32_t tmem_base = bars->tmem_base;
     cluster_arrive();                  // this CTA is running: its shared memory may be written by the others
     pdl_wait();
+    bias = behind_wait(bias); res = behind_wait(res);
 
     if (warp >= 2)
         for (int i = tid - 64; i < p.BN; i += kThreads - 64) bias_s[i] = (bias && i < cols) ? bias[nt * p.BN + i] : 0.f;

@@ -220,6 +220,11 @@ __device__ __forceinline__ uint32_t relu_bf16x2(uint32_t v)
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A pointer to what the kernel ahead may write, for use behind pdl_wait().  The compiler takes a `const __restrict__` argument
+// for memory that nothing writes while the kernel runs, and may move its loads in front of the wait (it did: two CTAs of a
+// cluster read the same scores, one of them before they were written); it cannot move a load whose address comes from here.
+template <typename T> __device__ __forceinline__ T *behind_wait(T *p) { asm volatile("" : "+l"(p)::"memory"); return p; }
+
 // Launch with the attribute set (unless `how.plain`).  What a kernel so launched may read before pdl_wait() is only what was
 // complete before the kernel ahead of it STARTED: that one may still be running, or have ended without its stores being
 // visible yet, whether it triggers or not.  So
