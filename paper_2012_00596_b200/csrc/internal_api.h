@@ -17,9 +17,17 @@ extern "C" {
 // kept columns in the fullest block
 npas_status npas_internal_bp_size(const npas_bp_desc *d, uint64_t n_pairs, size_t *blob_bytes);
 npas_status npas_internal_bb_size(const npas_bb_desc *d, uint64_t n_vals, uint32_t max_cols, size_t *blob_bytes);
-// n mask words on the device to a device buffer and to page-locked host memory, each word read once: what the host counts is
-// what the packers see
-npas_status npas_internal_copy_masks(const uint64_t *words, uint64_t *dev, uint64_t *host, size_t n, void *stream);
+// The plan of a blob: mask words on the device, each read once, to scratch memory (16-byte aligned, as many bytes as the first
+// call says) together with the prefix sums, and the counts that the blob's size follows from to a word of page-locked memory,
+// zero before: bit 63 set, above bit 32 the fullest block's taps / columns, below it the kept pairs / stored values.
+npas_status npas_internal_plan_bp_bytes(const npas_bp_desc *d, size_t *bytes);
+npas_status npas_internal_plan_bp(const npas_bp_desc *d, const uint64_t *words, void *scratch, uint64_t *host, void *stream);
+npas_status npas_internal_plan_bb_bytes(const npas_bb_desc *d, size_t *bytes);
+npas_status npas_internal_plan_bb(const npas_bb_desc *d, const uint64_t *rows, const uint64_t *cols, void *scratch, uint64_t *host, void *stream);
+// the blob of a plan, on the same stream, with the counts it posted
+npas_status npas_internal_pack_bp_planned(const npas_bp_desc *d, const void *w, void *scratch, uint64_t n_pairs, void *blob, size_t blob_bytes, void *stream);
+npas_status npas_internal_pack_bb_planned(const npas_bb_desc *d, const void *w, void *scratch, uint64_t n_vals, uint32_t max_cols, void *blob,
+                                          size_t blob_bytes, void *stream);
 // the pack calls up to, but without, their synchronisation
 npas_status npas_internal_pack_bp(const npas_bp_desc *d, const void *w, const uint64_t *tap_mask, void *blob, size_t blob_bytes, void *stream);
 npas_status npas_internal_pack_bb(const npas_bb_desc *d, const void *w, const uint64_t *rk, const uint64_t *ck, void *blob,

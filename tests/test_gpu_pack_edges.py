@@ -30,6 +30,18 @@ def test_pack_bp_sections_at_the_edges(K, C, R, Mb, Nb, w_in):
     assert blob.desc.max_taps == max(1, max(bin(int(v)).count("1") for v in c.tap_mask.ravel()))
 
 
+@pytest.mark.parametrize("K,C,R,Mb,Nb,w_in", [(3072, 3072, 1, 16, 16, "bf16"), (512, 512, 1, 1, 1, "f32"), (65536, 16, 1, 1, 16, "bf16")])
+def test_masks_on_the_device_and_on_the_host_give_the_same_blob(K, C, R, Mb, Nb, w_in):
+    """More blocks than the scan keeps counts of; the two ways to pack share no prefix sums."""
+    rng = inputs.rng_for(1005)
+    w = dev(rng.standard_normal((K, R, R, C), dtype=np.float32), w_in)
+    tm = rng.integers(0, 2, (K // Mb, C // Nb)).astype(np.int64)
+    on_gpu = npas.pack_bp(w, torch.from_numpy(tm).cuda(), Mb, Nb, torch.bfloat16)
+    assert torch.equal(on_gpu.data, npas.pack_bp(w, tm.view(np.uint64), Mb, Nb, torch.bfloat16).data)
+    wd, back = npas.unpack_bp(on_gpu)
+    assert torch.equal(back.cpu(), torch.from_numpy(tm))
+
+
 @pytest.mark.parametrize("rate", [1.5, 10.0])
 def test_global_pruning_of_more_groups_than_shared_memory_holds(rate):
     """204800 groups over eight CTAs; the scores of one filter block repeat in another, so equal keys meet the budget."""

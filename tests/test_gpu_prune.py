@@ -101,6 +101,36 @@ def test_prune_bp_global_extremes_and_all_ties():
     assert e.value.code == 2
 
 
+@pytest.mark.parametrize("kind", ["one value", "two values", "spread", "crowded", "outliers"])
+@pytest.mark.parametrize("K,C", [(64, 64), (128, 128)])              # 2304 groups on two CTAs, 9216 on eight
+def test_prune_bp_global_of_uneven_scores(K, C, kind):
+    """Scores that put many keys into one bin of the selection, or none where the sampled keys lie: equal keys that no
+    further division separates, a tail over many powers of two, a crowd of neighbouring values, values beyond the samples."""
+    rng = inputs.rng_for(905)
+    G = (K // 4) * (C // 4) * 9
+    if kind == "one value":
+        v = np.ones(G)
+    elif kind == "two values":
+        v = np.where(rng.random(G) < 0.5, 1.0, 2.0)
+    elif kind == "spread":
+        v = np.exp2(rng.integers(-60, 60, G))
+    elif kind == "crowded":
+        v = 1.0 + rng.integers(0, 1500, G) * 2.0 ** -23
+        v[::97] = 1000.0
+    else:
+        v = np.full(G, 3.0)
+        v[::256] += 0.5
+        v[5:900:7] = 2.0 ** 40
+        v[6:900:7] = 2.0 ** -40
+    # one weight per (block, tap) carries the score
+    w = np.zeros((K // 4, 4, 9, C // 4, 4), dtype=np.float32)
+    w[:, 0, :, :, 0] = v.reshape(K // 4, C // 4, 9).transpose(0, 2, 1)
+    w = w.reshape(K, 3, 3, C)
+    for n_keep in (1, G // 3, G // 2 + 1, G - 1, G):
+        tm = npas.prune_bp_magnitude_global(dev(w), 4, 4, n_keep=n_keep)
+        assert np.array_equal(to_u64(tm), oracle.prune_bp_global(w, Mb=4, Nb=4, n_keep=n_keep)), n_keep
+
+
 @pytest.mark.parametrize("rate,Mb,Nb", [(2.5, 16, 8), (7.0, 16, 16)])
 def test_rate_pruned_layer_end_to_end(rate, Mb, Nb):
     """A layer pruned to 2.5x / 7x (blocks keep different numbers of taps) through pack + convolution."""
