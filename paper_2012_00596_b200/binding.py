@@ -166,13 +166,8 @@ def pack_bp(w: torch.Tensor, tap_mask, Mb: int, Nb: int, packed_dtype=None) -> B
     """npas_pack_bp: dense KRSC weights + per-block tap bitsets -> blob (on w's device)."""
     if _host is None:
         load()
-    assert w.is_cuda and w.is_contiguous() and w.dim() == 4
-    K, R, S, C = w.shape
-    w_in = _dt(w)
-    w_packed = w_in if packed_dtype is None else _dt_code(packed_dtype)
-    code, blob, max_taps = _host.pack_bp(w, _mask_words(tap_mask, w.device), Mb, Nb, w_in, w_packed)
-    _check(code, "npas_pack_bp")
-    return BpBlob(blob, BpDesc(K, C, R, S, Mb, Nb, w_in, w_packed, max_taps))
+    r = _host.pack_bp(w, tap_mask, Mb, Nb, packed_dtype, _mask_words, BpDesc, BpBlob)
+    return r if type(r) is not int else _refused(r, "npas_pack_bp")
 
 
 def unpack_bp(blob: BpBlob):
@@ -189,13 +184,8 @@ def unpack_bp(blob: BpBlob):
 def pack_bb(w: torch.Tensor, row_keep, col_keep, Bo: int, Bi: int, packed_dtype=None) -> BbBlob:
     if _host is None:
         load()
-    assert w.is_cuda and w.is_contiguous() and w.dim() == 2
-    O, I = w.shape
-    w_in = _dt(w)
-    w_packed = w_in if packed_dtype is None else _dt_code(packed_dtype)
-    code, blob, max_cols = _host.pack_bb(w, _mask_words(row_keep, w.device), _mask_words(col_keep, w.device), Bo, Bi, w_in, w_packed)
-    _check(code, "npas_pack_bb")
-    return BbBlob(blob, BbDesc(O, I, Bo, Bi, w_in, w_packed, max_cols))
+    r = _host.pack_bb(w, row_keep, col_keep, Bo, Bi, packed_dtype, _mask_words, BbDesc, BbBlob)
+    return r if type(r) is not int else _refused(r, "npas_pack_bb")
 
 
 def unpack_bb(blob: BbBlob):
@@ -221,11 +211,7 @@ def prune_bp_magnitude_global(w: torch.Tensor, Mb: int, Nb: int, *, rate: float 
     layer (``rate``: n_keep = round(groups / rate), e.g. 2.5 or 7); tap bitsets as an int64 device tensor."""
     if _host is None:
         load()
-    assert w.is_cuda and w.is_contiguous() and w.dim() == 4 and (rate is None) != (n_keep is None)
-    K, R, S, C = w.shape
-    if n_keep is None:
-        n_keep = int(np.floor((K // Mb) * (C // Nb) * R * S / float(rate) + 0.5))
-    r = _host.prune_bp_global(w, Mb, Nb, _dt(w), int(n_keep))
+    r = _host.prune_bp_global(w, Mb, Nb, rate, n_keep)
     return r if type(r) is not int else _refused(r, "npas_prune_bp_magnitude_global")
 
 
@@ -233,7 +219,7 @@ def prune_bb_magnitude(w: torch.Tensor, Bo: int, Bi: int, keep_rows: int, keep_c
     """npas_prune_bb_magnitude: dense [O,I] weights -> (row bitsets, column bitsets), int64 tensors on the device."""
     if _host is None:
         load()
-    r = _host.prune_bb(w, Bo, Bi, _dt(w), int(keep_rows), int(keep_cols))
+    r = _host.prune_bb(w, Bo, Bi, keep_rows, keep_cols)
     return r if type(r) is not int else _refused(r, "npas_prune_bb_magnitude")
 
 

@@ -18,6 +18,7 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <atomic>
+#include <cmath>
 #include <mutex>
 #include <vector>
 
@@ -327,27 +328,84 @@ bool planned(cudaStream_t st, F launch, MaskSums &sums)
     sums = MaskSums{v & 0xFFFFFFFFu, (uint32_t)(v >> 32) & 0x7FFFFFFFu};
     return true;
 }
-PyObject *packed(npas_status s, at::Tensor &&blob, uint32_t most)
+// A blob object: blob_type(data, desc) with a desc_type instance that holds d; or the status as an int.
+template <typename D>
+PyObject *packed(npas_status s, at::Tensor &&blob, const D &d, PyObject *desc_type, PyObject *blob_type)
 {
-    PyObject *t = s == NPAS_OK ? THPVariable_Wrap(std::move(blob)) : (Py_INCREF(Py_None), Py_None);
-    return t ? Py_BuildValue("(iNI)", (int)s, t, most) : nullptr;
+    if (s != NPAS_OK) return PyLong_FromLong((long)s);
+    PyObject *desc = PyObject_CallNoArgs(desc_type);
+    if (!desc) return nullptr;
+    Py_buffer view;
+    bool ok = PyObject_GetBuffer(desc, &view, PyBUF_WRITABLE) == 0;
+    if (ok) {
+        ok = view.len == (Py_ssize_t)sizeof(D);
+        if (ok) memcpy(view.buf, &d, sizeof(D));
+        PyBuffer_Release(&view);
+        if (!ok) PyErr_SetString(PyExc_TypeError, "descriptor of the wrong type");
+    }
+    PyObject *data = ok ? THPVariable_Wrap(std::move(blob)) : nullptr, *r = nullptr;
+    if (data) {
+        PyObject *args[2] = {data, desc};
+        r = PyObject_Vectorcall(blob_type, args, 2, nullptr);
+    }
+    Py_XDECREF(data);
+    Py_DECREF(desc);
+    return r;
 }
 
-// pack_bp(w, mask, Mb, Nb, w_in, w_packed) -> (status, blob, fullest block's taps)
+// Mask words as the packers take them, an int64 tensor on w's device or on the CPU: the argument itself, or what the Python
+// function `words`(mask, device) makes of it.  `made` keeps what was made.
+struct Owned {
+    PyObject *p = nullptr;
+    ~Owned() { Py_XDECREF(p); }
+};
+bool mask_words(PyObject *o, PyObject *w_obj, const at::Tensor &w, PyObject *words, Owned &made, const at::Tensor *&m)
+{
+    if (THPVariable_Check(o)) {
+        m = &THPVariable_Unpack(o);
+        if (m->scalar_type() == at::kLong && m->device() == w.device() && m->is_contiguous()) return true;
+    }
+    Owned dev;
+    dev.p = PyObject_GetAttrString(w_obj, "device");
+    if (!dev.p) return false;
+    PyObject *args[2] = {o, dev.p};
+    made.p = PyObject_Vectorcall(words, args, 2, nullptr);
+    return made.p && tensor_arg(made.p, m, false, "mask");
+}
+
+// the types of the weights and of the packed weights (None: the same)
+bool weight_types(const at::Tensor &w, PyObject *packed_dtype, int32_t &in, int32_t &out)
+{
+    at::ScalarType t;
+    if (!dtype_of(w.scalar_type(), in)) return false;
+    if (packed_dtype != Py_None && !THPDtype_Check(packed_dtype)) { PyErr_Format(PyExc_TypeError, "unsupported dtype %R", packed_dtype); return false; }
+    return dtype_arg(packed_dtype, w.scalar_type(), t) && dtype_of(t, out);
+}
+
+bool whole_arg(PyObject *o, long long &v)             // int(o)
+{
+    Owned i;
+    i.p = PyNumber_Long(o);
+    if (!i.p) return false;
+    v = PyLong_AsLongLong(i.p);
+    return !(v == -1 && PyErr_Occurred());
+}
+
+// pack_bp(w, mask, Mb, Nb, packed_dtype, words, desc_type, blob_type) -> blob, or the status
 PyObject *pack_bp(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return guarded([&]() -> PyObject * {
         const at::Tensor *w, *m;
+        Owned made;
         npas_bp_desc d = {};
-        if (n != 6) { PyErr_SetString(PyExc_TypeError, "pack_bp takes 6 arguments"); return nullptr; }
-        if (!tensor_arg(a[0], w, false, "w") || !tensor_arg(a[1], m, false, "mask") || !int_arg(a[2], d.Mb) || !int_arg(a[3], d.Nb) ||
-            !int_arg(a[4], d.w_in) || !int_arg(a[5], d.w_packed))
-            return nullptr;
+        if (n != 8) { PyErr_SetString(PyExc_TypeError, "pack_bp takes 8 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], w, false, "w")) return nullptr;
         if (!(w->is_cuda() && w->is_contiguous() && w->dim() == 4)) { fail_assert("w must be a contiguous 4-D CUDA tensor"); return nullptr; }
         d.K = (int32_t)w->size(0); d.R = (int32_t)w->size(1); d.S = (int32_t)w->size(2); d.C = (int32_t)w->size(3);
+        if (!weight_types(*w, a[4], d.w_in, d.w_packed) || !mask_words(a[1], a[0], *w, a[5], made, m) || !int_arg(a[2], d.Mb) || !int_arg(a[3], d.Nb)) return nullptr;
         size_t bytes = 0;
         npas_status s = npas_internal_bp_size(&d, 0, &bytes);
-        if (s != NPAS_OK) return packed(s, at::Tensor(), 0);
+        if (s != NPAS_OK) return PyLong_FromLong((long)s);
         const cudaStream_t st = c10::cuda::getCurrentCUDAStream().stream();
         const int64_t blocks = (int64_t)(d.K / d.Mb) * (d.C / d.Nb);
         if (!mask_arg(*m, blocks)) return nullptr;
@@ -365,31 +423,33 @@ PyObject *pack_bp(PyObject *, PyObject *const *a, Py_ssize_t n)
         }
         d.max_taps = sums.most ? (int32_t)sums.most : 1;
         s = npas_internal_bp_size(&d, sums.total, &bytes);
-        if (s != NPAS_OK) return packed(s, at::Tensor(), 0);
+        if (s != NPAS_OK) return PyLong_FromLong((long)s);
         at::Tensor blob = new_tensor({(int64_t)bytes}, at::kByte, w->device());
         Py_BEGIN_ALLOW_THREADS
         s = m->is_cuda() ? npas_internal_pack_bp_planned(&d, w->data_ptr(), scratch.data_ptr(), sums.total, blob.data_ptr(), bytes, st)
                          : npas_internal_pack_bp(&d, w->data_ptr(), static_cast<const uint64_t *>(mask.dev.data_ptr()), blob.data_ptr(), bytes, st);
         Py_END_ALLOW_THREADS
-        return packed(s, std::move(blob), (uint32_t)d.max_taps);
+        return packed(s, std::move(blob), d, a[6], a[7]);
     });
 }
 
-// pack_bb(w, rows, cols, Bo, Bi, w_in, w_packed) -> (status, blob, fullest block's columns)
+// pack_bb(w, rows, cols, Bo, Bi, packed_dtype, words, desc_type, blob_type) -> blob, or the status
 PyObject *pack_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return guarded([&]() -> PyObject * {
         const at::Tensor *w, *mr, *mc;
+        Owned made_r, made_c;
         npas_bb_desc d = {};
-        if (n != 7) { PyErr_SetString(PyExc_TypeError, "pack_bb takes 7 arguments"); return nullptr; }
-        if (!tensor_arg(a[0], w, false, "w") || !tensor_arg(a[1], mr, false, "row_keep") || !tensor_arg(a[2], mc, false, "col_keep") ||
-            !int_arg(a[3], d.Bo) || !int_arg(a[4], d.Bi) || !int_arg(a[5], d.w_in) || !int_arg(a[6], d.w_packed))
-            return nullptr;
+        if (n != 9) { PyErr_SetString(PyExc_TypeError, "pack_bb takes 9 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], w, false, "w")) return nullptr;
         if (!(w->is_cuda() && w->is_contiguous() && w->dim() == 2)) { fail_assert("w must be a contiguous 2-D CUDA tensor"); return nullptr; }
         d.O = (int32_t)w->size(0); d.I = (int32_t)w->size(1);
+        if (!weight_types(*w, a[5], d.w_in, d.w_packed) || !mask_words(a[1], a[0], *w, a[6], made_r, mr) || !mask_words(a[2], a[0], *w, a[6], made_c, mc) ||
+            !int_arg(a[3], d.Bo) || !int_arg(a[4], d.Bi))
+            return nullptr;
         size_t bytes = 0;
         npas_status s = npas_internal_bb_size(&d, 0, 0, &bytes);
-        if (s != NPAS_OK) return packed(s, at::Tensor(), 0);
+        if (s != NPAS_OK) return PyLong_FromLong((long)s);
         const cudaStream_t st = c10::cuda::getCurrentCUDAStream().stream();
         const int64_t blocks = (int64_t)(d.O / d.Bo) * (d.I / d.Bi);
         if (!mask_arg(*mr, blocks) || !mask_arg(*mc, blocks)) return nullptr;
@@ -412,29 +472,42 @@ PyObject *pack_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
         }
         d.max_cols = sums.most ? (int32_t)sums.most : 1;
         s = npas_internal_bb_size(&d, sums.total, sums.most, &bytes);
-        if (s != NPAS_OK) return packed(s, at::Tensor(), 0);
+        if (s != NPAS_OK) return PyLong_FromLong((long)s);
         at::Tensor blob = new_tensor({(int64_t)bytes}, at::kByte, w->device());
         Py_BEGIN_ALLOW_THREADS
         s = plan ? npas_internal_pack_bb_planned(&d, w->data_ptr(), scratch.data_ptr(), sums.total, sums.most, blob.data_ptr(), bytes, st)
                  : npas_internal_pack_bb(&d, w->data_ptr(), dr, dc, blob.data_ptr(), bytes, st);
         Py_END_ALLOW_THREADS
-        return packed(s, std::move(blob), (uint32_t)d.max_cols);
+        return packed(s, std::move(blob), d, a[7], a[8]);
     });
 }
 
-// prune_bp_global(w, Mb, Nb, w_in, n_keep) -> masks, or the status
+// prune_bp_global(w, Mb, Nb, rate, n_keep) -> masks, or the status; one of the last two is None
 PyObject *prune_bp_global(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return guarded([&]() -> PyObject * {
         const at::Tensor *w;
         npas_bp_desc d = {};
         if (n != 5) { PyErr_SetString(PyExc_TypeError, "prune_bp_global takes 5 arguments"); return nullptr; }
-        if (!tensor_arg(a[0], w, false, "w") || !int_arg(a[1], d.Mb) || !int_arg(a[2], d.Nb) || !int_arg(a[3], d.w_in)) return nullptr;
-        const long long n_keep = PyLong_AsLongLong(a[4]);
-        if (n_keep == -1 && PyErr_Occurred()) return nullptr;
+        if (!tensor_arg(a[0], w, false, "w")) return nullptr;
         if (!(w->is_cuda() && w->is_contiguous() && w->dim() == 4)) { fail_assert("w must be a contiguous 4-D CUDA tensor"); return nullptr; }
+        if ((a[3] == Py_None) == (a[4] == Py_None)) { fail_assert("either rate or n_keep"); return nullptr; }
+        if (!int_arg(a[1], d.Mb) || !int_arg(a[2], d.Nb) || !dtype_of(w->scalar_type(), d.w_in)) return nullptr;
         d.K = (int32_t)w->size(0); d.R = (int32_t)w->size(1); d.S = (int32_t)w->size(2); d.C = (int32_t)w->size(3);
         d.w_packed = d.w_in;
+        long long n_keep = 0;
+        if (a[3] == Py_None) {
+            if (!whole_arg(a[4], n_keep)) return nullptr;
+        } else {
+            Owned f;
+            f.p = PyNumber_Float(a[3]);
+            if (!f.p) return nullptr;
+            const double rate = PyFloat_AS_DOUBLE(f.p);
+            if (d.Mb == 0 || d.Nb == 0 || rate == 0.0) { PyErr_SetString(PyExc_ZeroDivisionError, "division by zero"); return nullptr; }
+            const double keep = std::floor((double)((long long)(d.K / d.Mb) * (d.C / d.Nb) * d.R * d.S) / rate + 0.5);
+            if (!(std::fabs(keep) < 9e18)) { PyErr_SetString(std::isnan(keep) ? PyExc_ValueError : PyExc_OverflowError, "cannot keep that many groups"); return nullptr; }
+            n_keep = (long long)keep;
+        }
         size_t bytes = 0;
         npas_status s = npas_prune_bp_global_workspace(&d, &bytes);
         if (s != NPAS_OK) return PyLong_FromLong((long)s);
@@ -447,27 +520,25 @@ PyObject *prune_bp_global(PyObject *, PyObject *const *a, Py_ssize_t n)
     });
 }
 
-// prune_bb(w, Bo, Bi, w_in, keep_rows, keep_cols) -> (rows, columns), or the status
+// prune_bb(w, Bo, Bi, keep_rows, keep_cols) -> (rows, columns), or the status
 PyObject *prune_bb(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return guarded([&]() -> PyObject * {
         const at::Tensor *w;
         npas_bb_desc d = {};
-        int32_t kr, kc;
-        if (n != 6) { PyErr_SetString(PyExc_TypeError, "prune_bb takes 6 arguments"); return nullptr; }
-        if (!tensor_arg(a[0], w, false, "w") || !int_arg(a[1], d.Bo) || !int_arg(a[2], d.Bi) || !int_arg(a[3], d.w_in) || !int_arg(a[4], kr) || !int_arg(a[5], kc))
+        long long kr, kc;
+        if (n != 5) { PyErr_SetString(PyExc_TypeError, "prune_bb takes 5 arguments"); return nullptr; }
+        if (!tensor_arg(a[0], w, false, "w") || !int_arg(a[1], d.Bo) || !int_arg(a[2], d.Bi) || !dtype_of(w->scalar_type(), d.w_in) || !whole_arg(a[3], kr) || !whole_arg(a[4], kc))
             return nullptr;
         if (!(w->is_cuda() && w->is_contiguous() && w->dim() == 2)) { fail_assert("w must be a contiguous 2-D CUDA tensor"); return nullptr; }
         d.O = (int32_t)w->size(0); d.I = (int32_t)w->size(1);
         d.w_packed = d.w_in;
         if (d.Bo == 0 || d.Bi == 0) { PyErr_SetString(PyExc_ZeroDivisionError, "block size is zero"); return nullptr; }
-        // one buffer for both
-        const at::Tensor both = new_tensor({2, d.O / d.Bo, d.I / d.Bi}, at::kLong, w->device());
-        at::Tensor rk = both[0], ck = both[1];
+        at::Tensor rk = new_tensor({d.O / d.Bo, d.I / d.Bi}, at::kLong, w->device()), ck = new_tensor({d.O / d.Bo, d.I / d.Bi}, at::kLong, w->device());
         void *st = c10::cuda::getCurrentCUDAStream().stream();
         npas_status s;
         Py_BEGIN_ALLOW_THREADS
-        s = npas_prune_bb_magnitude(&d, w->data_ptr(), kr, kc, static_cast<uint64_t *>(rk.data_ptr()), static_cast<uint64_t *>(ck.data_ptr()), st);
+        s = npas_prune_bb_magnitude(&d, w->data_ptr(), (int32_t)kr, (int32_t)kc, static_cast<uint64_t *>(rk.data_ptr()), static_cast<uint64_t *>(ck.data_ptr()), st);
         Py_END_ALLOW_THREADS
         if (s != NPAS_OK) return PyLong_FromLong((long)s);
         return Py_BuildValue("(NN)", THPVariable_Wrap(std::move(rk)), THPVariable_Wrap(std::move(ck)));
