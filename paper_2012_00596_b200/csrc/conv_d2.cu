@@ -162,7 +162,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     if (warp != 0 && warp != 2) {
         const int t = tid < 64 ? tid - 32 : tid - 64;         // 0 .. kThreads - 65 over warps 1, 3, 4, ...
         const uint32_t *tapu = reinterpret_cast<const uint32_t *>(blob + off_tapu);
-        for (int i = t; i < (p.K / p.GI) * p.nCh; i += kThreads - 64) tapu_s[i] = off_tapu ? tapu[i] : 0xFFFFFFFFu;
+        for (int i = t; i < (p.K / p.GI) * p.nCh; i += kThreads - 64) tapu_s[i] = off_tapu ? __ldg(tapu + i) : 0xFFFFFFFFu;
         if (p.IT > 1 && p.act_stride > p.slab_bytes) {
             // several images per tile: the last image's bottom-right taps read just past the slab, where no copy
             // ever writes: zeros, once, in every buffer of the ring (read by the tensor core: async proxy)
@@ -327,7 +327,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         }
     } else {
         // ---- epilogue: warp -> TMEM lane quarter (warp % 4) and every kParts-th 16-column chunk -----------
-        for (int i = tid - kFirstEpiWarp * 32; i < p.K; i += kEpiWarps * 32) bias_s[i] = bias ? bias[i] : 0.f;
+        for (int i = tid - kFirstEpiWarp * 32; i < p.K; i += kEpiWarps * 32) bias_s[i] = bias ? __ldg(bias + i) : 0.f;
         asm volatile("bar.sync 2, %0;" ::"n"(kEpiWarps * 32) : "memory");
         const int quarter = warp & 3, part = (warp - kFirstEpiWarp) >> 2, m = quarter * 32 + lane;
         const int il = p.IT > 1 ? m / p.img_pitch : 0, mr = m - il * p.img_pitch;    // image of the tile, position inside it
@@ -373,7 +373,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                         const uint4 *rp = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0);
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            const uint4 u = rp[h];
+                            const uint4 u = __ldg(rp + h);
                             const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
@@ -385,7 +385,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                         const float4 *rp = reinterpret_cast<const float4 *>(static_cast<const float *>(res) + o0);
 #pragma unroll
                         for (int h = 0; h < 4; ++h) {
-                            const float4 u = rp[h];
+                            const float4 u = __ldg(rp + h);
                             v[4 * h] += u.x; v[4 * h + 1] += u.y; v[4 * h + 2] += u.z; v[4 * h + 3] += u.w;
                         }
                     }

@@ -118,10 +118,10 @@ conv_bp_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDnParams
     }
     // the producer starts at once; the other warps first stage the biases and the tap unions
     if (warp != 0) {
-        for (int i = tid - 32; i < p.K; i += kThreads - 32) bias_s[i] = bias ? bias[i] : 0.f;
+        for (int i = tid - 32; i < p.K; i += kThreads - 32) bias_s[i] = bias ? __ldg(bias + i) : 0.f;
         const uint32_t off_tapu = hdr[BP_OFF_TAPU];
         const uint32_t *tapu = reinterpret_cast<const uint32_t *>(blob + off_tapu);
-        for (int i = tid - 32; i < (p.K / p.GI) * p.nCh; i += kThreads - 32) tapu_s[i] = off_tapu ? tapu[i] : 0xFFFFFFFFu;
+        for (int i = tid - 32; i < (p.K / p.GI) * p.nCh; i += kThreads - 32) tapu_s[i] = off_tapu ? __ldg(tapu + i) : 0xFFFFFFFFu;
         consumers_sync();
     }
 
@@ -273,7 +273,7 @@ conv_bp_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDnParams
                         const uint4 *rp = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0);
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            const uint4 u = rp[h];
+                            const uint4 u = __ldg(rp + h);
                             const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
@@ -285,7 +285,7 @@ conv_bp_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDnParams
                         const float4 *rp = reinterpret_cast<const float4 *>(static_cast<const float *>(res) + o0);
 #pragma unroll
                         for (int h = 0; h < 4; ++h) {
-                            const float4 u = rp[h];
+                            const float4 u = __ldg(rp + h);
                             v[4 * h] += u.x; v[4 * h + 1] += u.y; v[4 * h + 2] += u.z; v[4 * h + 3] += u.w;
                         }
                     }

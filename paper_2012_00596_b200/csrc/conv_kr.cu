@@ -212,7 +212,7 @@ __device__ __forceinline__ void epilogue_staged(const CUtensorMap *tmap_y, uint3
             const uint4 *rp = reinterpret_cast<const uint4 *>(res_row + c0);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const uint4 q = rp[h];
+                const uint4 q = __ldg(rp + h);
                 const uint32_t wv[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -310,12 +310,12 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         for (int i = tid; i < p.GS * p.nCB; i += kThreads) {
             const int g = i / p.nCB, cb = i - g * p.nCB;
             const uint32_t *bo = blk_off + (size_t)(fb0 + g) * p.nCB + cb;
-            const uint32_t lo = bo[0], hi = bo[1];
+            const uint32_t lo = __ldg(bo), hi = __ldg(bo + 1);
             if (hi - lo > (uint32_t)p.max_taps) { bars->abort_flag = 2; continue; }     // more kept taps than promised
             uint32_t bits = 0;
 #pragma unroll
             for (int j = 0; j < kMaxTaps; ++j)
-                if (lo + j < hi) bits |= 1u << (pairs[lo + j] >> 16);
+                if (lo + j < hi) bits |= 1u << (__ldg(pairs + lo + j) >> 16);
             if (bits >> p.RS) { bars->abort_flag = 2; continue; }
             for (uint32_t U = bits; U; U &= U - 1) {
                 const uint32_t t = __ffs(U) - 1;
@@ -323,14 +323,14 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             }
         }
         for (int c = tid; c < p.nChunks; c += kThreads) {
-            const uint32_t a = kt_off[c * p.nGrp + grp], b = kt_off[c * p.nGrp + grp + 1];
+            const uint32_t a = __ldg(kt_off + c * p.nGrp + grp), b = __ldg(kt_off + c * p.nGrp + grp + 1);
             kto[2 * c] = a; kto[2 * c + 1] = b - a;
             if (b < a || b - a > (uint32_t)(p.GS * p.max_taps)) bars->abort_flag = 2;   // would overflow a weight slot
         }
     }
     pdl_wait();
     bias = behind_wait(bias); res = behind_wait(res);
-    for (int i = tid; i < p.GS * p.Mb; i += kThreads) bars->bias[i] = bias ? bias[fb0 * p.Mb + i] : 0.f;
+    for (int i = tid; i < p.GS * p.Mb; i += kThreads) bars->bias[i] = bias ? __ldg(bias + fb0 * p.Mb + i) : 0.f;
     fence_proxy_async_smem();
     tc_fence_before_sync();
     __syncthreads();
@@ -581,7 +581,7 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                             const uint4 *rp = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0 + c0);
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
-                                const uint4 u = rp[h];
+                                const uint4 u = __ldg(rp + h);
                                 const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
                                 for (int i = 0; i < 4; ++i) {
@@ -593,7 +593,7 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                             const float4 *rp = reinterpret_cast<const float4 *>(static_cast<const float *>(res) + o0 + c0);
 #pragma unroll
                             for (int h = 0; h < 4; ++h) {
-                                const float4 u = rp[h];
+                                const float4 u = __ldg(rp + h);
                                 v[4 * h] += u.x; v[4 * h + 1] += u.y; v[4 * h + 2] += u.z; v[4 * h + 3] += u.w;
                             }
                         }

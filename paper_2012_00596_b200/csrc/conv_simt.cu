@@ -83,7 +83,7 @@ conv_bp_simt_kernel(npas_conv_desc d, int Mb, int Nb_, int P, int Q, int KW, con
         }
     }
     double acc[FG][kPixels / 8][2] = {};
-    const uint32_t j_begin = blk_off[(size_t)fb * nCB], j_end = blk_off[(size_t)(fb + 1) * nCB];
+    const uint32_t j_begin = __ldg(blk_off + (size_t)fb * nCB), j_end = __ldg(blk_off + (size_t)(fb + 1) * nCB);
     const uint32_t spp = (Nb + 3) / 4;                                   // matrix steps per pair
     const uint32_t s_all = (j_end - j_begin) * spp;
     const TX *wp = vals + ((size_t)j_begin * Nb * Mb + (f0 + q8) * G + k);
@@ -91,7 +91,7 @@ conv_bp_simt_kernel(npas_conv_desc d, int Mb, int Nb_, int P, int Q, int KW, con
         const int steps = (int)min((uint32_t)kMaxSteps, s_all - b0);
         if (b0) __syncthreads();
         for (int e = tid; e < steps; e += kWarps * 32) {
-            const uint32_t j = (b0 + e) / spp, c0 = (b0 + e - j * spp) * 4, pw = pairs[j_begin + j], tap = pw >> 16, cb = pw & 0xFFFFu;
+            const uint32_t j = (b0 + e) / spp, c0 = (b0 + e - j * spp) * 4, pw = __ldg(pairs + j_begin + j), tap = pw >> 16, cb = pw & 0xFFFFu;
             const uint32_t r = tap / d.S, sx = tap - r * d.S, wo = (j * (Nb / G) + c0 / G) * Mb * G + c0 % G;
             // (a pair outside the layer counts for nothing: its tap lies beside every image)
             step_s[e] = r < (uint32_t)d.R && cb < nCB ? make_uint4((r * d.W + sx) * d.C + cb * Nb + c0, r | (sx << 16), wo, Nb - c0)

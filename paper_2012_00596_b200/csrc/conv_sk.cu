@@ -148,14 +148,14 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 #pragma unroll 4
             for (int e = lane; e < own_chunks * ng; e += 32) {
                 const int g = e / own_chunks, i = e - g * own_chunks;
-                atomicOr(&bars->taps[i], tapu[(g0 + g) * p.nCh + blk_lo * cpb + i]);
+                atomicOr(&bars->taps[i], __ldg(tapu + (g0 + g) * p.nCh + blk_lo * cpb + i));
             }
         __syncwarp();
     }
     pdl_wait();
     bias = behind_wait(bias); res = behind_wait(res);
     if (warp > 2)
-        for (int i = tid - 96; i < p.NT; i += kThreads - 96) bias_s[i] = (bias && k0 + i < p.K) ? bias[k0 + i] : 0.f;
+        for (int i = tid - 96; i < p.NT; i += kThreads - 96) bias_s[i] = (bias && k0 + i < p.K) ? __ldg(bias + k0 + i) : 0.f;
 
     if (warp == 0) {
         // ---- slabs -----------------------------------------------------------------------------------------------
@@ -269,7 +269,7 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         for (int j = 0; j < 8; ++j) v[j] += bias_s[c0 + j];
         if (p.y_bf16) {
             if (res) {
-                const uint4 u = *reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0);
+                const uint4 u = __ldg(reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0));
                 const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -287,7 +287,7 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         } else {
             if (res) {
                 const float4 *rp = reinterpret_cast<const float4 *>(static_cast<const float *>(res) + o0);
-                const float4 a = rp[0], b = rp[1];
+                const float4 a = __ldg(rp + 0), b = __ldg(rp + 1);
                 v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
                 v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
             }

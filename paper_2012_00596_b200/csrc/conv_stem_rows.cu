@@ -138,12 +138,12 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
         };
         if (per_pair % 8 == 0) {
             // eight weights of a pair per thread: one load, no division per weight
-            const uint32_t upp = per_pair / 8, n_units = blk_off[nfb] * upp;
+            const uint32_t upp = per_pair / 8, n_units = __ldg(blk_off + nfb) * upp;
             for (uint32_t e = tid; e < n_units; e += kThreads<kPool>) {
-                const uint32_t j = e / upp, rem = (e - j * upp) * 8, tap = pairs[j] >> 16;
-                const uint4 q = *reinterpret_cast<const uint4 *>(values + (size_t)j * per_pair + rem);
+                const uint32_t j = e / upp, rem = (e - j * upp) * 8, tap = __ldg(pairs + j) >> 16;
+                const uint4 q = __ldg(reinterpret_cast<const uint4 *>(values + (size_t)j * per_pair + rem));
                 uint32_t fb = 0;
-                while (fb + 1 < nfb && blk_off[fb + 1] <= j) ++fb;                           // one channel block per filter block
+                while (fb + 1 < nfb && __ldg(blk_off + fb + 1) <= j) ++fb;                           // one channel block per filter block
                 const uint32_t v[4] = {q.x, q.y, q.z, q.w};
                 uint32_t f = rem / kC, c = rem - f * kC;
                 f += fb * p.Mb;
@@ -158,7 +158,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
                 const uint32_t j0 = blk_off[fb], n = (blk_off[fb + 1] - j0) * per_pair;
                 for (uint32_t e = tid; e < n; e += kThreads<kPool>) {
                     const uint32_t j = j0 + e / per_pair, rem = e % per_pair, f = rem / kC;
-                    put(pairs[j] >> 16, fb * p.Mb + f, rem - f * kC, values[(size_t)j * per_pair + rem]);
+                    put(__ldg(pairs + j) >> 16, fb * p.Mb + f, rem - f * kC, __ldg(values + (size_t)j * per_pair + rem));
                 }
             }
         }
@@ -168,7 +168,7 @@ conv_stem_rows_kernel(const StemRowsParams p, const uint16_t *__restrict__ x, co
     // bias: the fourth channel of every pixel is one, and a window's pixels 2 .. 4 of kernel row 3 (never outside the image)
     // weigh it with the bias' upper, middle and lower eight bits, so that the sum is exact
     for (int f = tid; bias && f < p.K; f += kThreads<kPool>) {
-        const float v = bias[f];
+        const float v = __ldg(bias + f);
         const bool finite = fabsf(v) <= 3.0e38f;
         const uint32_t hi16 = finite ? __float_as_uint(v) >> 16 : cvt_bf16x2(v, 0.f) & 0xFFFFu;
         const float rest = finite ? v - __uint_as_float(hi16 << 16) : 0.f;

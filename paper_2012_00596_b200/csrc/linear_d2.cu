@@ -133,7 +133,7 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     bias = behind_wait(bias); res = behind_wait(res);
     // the biases: staged by the epilogue warps, which meet again before the first use
     if (warp >= kFirstEpiWarp && warp < kResWarp) {
-        for (int i = tid - kFirstEpiWarp * 32; i < p.O; i += kEpiWarps * 32) bias_s[i] = bias ? bias[i] : 0.f;
+        for (int i = tid - kFirstEpiWarp * 32; i < p.O; i += kEpiWarps * 32) bias_s[i] = bias ? __ldg(bias + i) : 0.f;
         epi_sync();
     }
     const uint32_t tmem_base = bars->tmem_base;
@@ -343,7 +343,7 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         const uint4 *rp = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0 + c0);
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            const uint4 u = rp[h];
+                            const uint4 u = __ldg(rp + h);
                             const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
@@ -355,7 +355,7 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         const float4 *rp = reinterpret_cast<const float4 *>(static_cast<const float *>(res) + o0 + c0);
 #pragma unroll
                         for (int h = 0; h < 4; ++h) {
-                            const float4 u = rp[h];
+                            const float4 u = __ldg(rp + h);
                             v[4 * h] += u.x; v[4 * h + 1] += u.y; v[4 * h + 2] += u.z; v[4 * h + 3] += u.w;
                         }
                     }

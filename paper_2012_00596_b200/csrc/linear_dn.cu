@@ -134,7 +134,7 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     bias = behind_wait(bias); res = behind_wait(res);
     // the biases: staged by the epilogue warps, which meet again before the first use
     if (warp >= kFirstEpiWarp && warp < kResWarp) {
-        for (int i = tid - kFirstEpiWarp * 32; i < p.nNT * p.BN; i += kEpiWarps * 32) bias_s[i] = (bias && i < p.O) ? bias[i] : 0.f;
+        for (int i = tid - kFirstEpiWarp * 32; i < p.nNT * p.BN; i += kEpiWarps * 32) bias_s[i] = (bias && i < p.O) ? __ldg(bias + i) : 0.f;
         epi_sync();
     }
     const uint32_t tmem_base = bars->tmem_base;
@@ -324,7 +324,7 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             if (8 * h >= left) break;
-                            const uint4 u = rp[h];
+                            const uint4 u = __ldg(rp + h);
                             const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
@@ -337,7 +337,7 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 #pragma unroll
                         for (int h = 0; h < 4; ++h) {
                             if (4 * h >= left) break;
-                            const float4 u = rp[h];
+                            const float4 u = __ldg(rp + h);
                             v[4 * h] += u.x; v[4 * h + 1] += u.y; v[4 * h + 2] += u.z; v[4 * h + 3] += u.w;
                         }
                     }

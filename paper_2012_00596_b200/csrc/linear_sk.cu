@@ -91,7 +91,7 @@ linear_bb_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     bias = behind_wait(bias); res = behind_wait(res);
 
     if (warp >= 2)
-        for (int i = tid - 64; i < p.BN; i += kThreads - 64) bias_s[i] = (bias && i < cols) ? bias[nt * p.BN + i] : 0.f;
+        for (int i = tid - 64; i < p.BN; i += kThreads - 64) bias_s[i] = (bias && i < cols) ? __ldg(bias + nt * p.BN + i) : 0.f;
 
     if (warp == 0) {
         if (lane == 0) {
@@ -181,7 +181,7 @@ linear_bb_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         for (int j = 0; j < 8; ++j) v[j] += bias_s[c0 + j];
         if (p.y_bf16) {
             if (res) {
-                const uint4 u = *reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0);
+                const uint4 u = __ldg(reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0));
                 const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -199,7 +199,7 @@ linear_bb_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         } else {
             if (res) {
                 const float4 *rp = reinterpret_cast<const float4 *>(static_cast<const float *>(res) + o0);
-                const float4 a = rp[0], b = rp[1];
+                const float4 a = __ldg(rp + 0), b = __ldg(rp + 1);
                 v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
                 v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
             }

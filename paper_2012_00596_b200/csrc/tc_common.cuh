@@ -223,7 +223,10 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // A pointer to what the kernel ahead may write, for use behind pdl_wait().  The compiler takes a `const __restrict__` argument
 // for memory that nothing writes while the kernel runs, and may move its loads in front of the wait (it did: two CTAs of a
 // cluster read the same scores, one of them before they were written); it cannot move a load whose address comes from here.
+// (Such loads are written as __ldg where they are to overtake stores to shared memory.)  Where every address is computed from
+// one index, a zero that the compiler does not know is enough, and the pointers stay what they were.
 template <typename T> __device__ __forceinline__ T *behind_wait(T *p) { asm volatile("" : "+l"(p)::"memory"); return p; }
+__device__ __forceinline__ int zero_behind_wait() { int z = 0; asm volatile("" : "+r"(z)::"memory"); return z; }
 
 // Launch with the attribute set (unless `how.plain`).  What a kernel so launched may read before pdl_wait() is only what was
 // complete before the kernel ahead of it STARTED: that one may still be running, or have ended without its stores being
