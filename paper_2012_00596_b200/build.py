@@ -12,7 +12,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnpas.so")
 HOST_SOURCE = os.path.join(CSRC, "host_ext.cpp")
 HOST_LIB = os.path.join(HERE, "_npas_host.so")
-SOURCES = ["api.cu", "host_util.cu", "pack.cu", "conv_simt.cu", "linear_simt.cu", "conv_tc.cu", "conv_kr.cu", "conv_stem.cu", "conv_stem_rows.cu", "conv_dn.cu", "conv_d2.cu", "conv_sk.cu", "linear_tc.cu", "linear_dn.cu", "linear_d2.cu", "linear_sk.cu",
+SOURCES = ["api.cu", "host_util.cu", "pack.cu", "conv_simt.cu", "linear_simt.cu", "conv_tc.cu", "conv_kr.cu", "conv_stem.cu", "conv_stem_rows.cu", "conv_dn.cu", "conv_d2.cu", "conv_sk.cu", "linear_tc.cu", "linear_dn.cu", "linear_d2.cu", "linear_sk.cu", "linear_two.cu",
            "prune.cu", "static_ws.cu"]
 
 

@@ -336,6 +336,24 @@ npas_status npas_internal_linear_bb(const npas_linear_desc *d, const npas_bb_des
     return NPAS_ERR_UNSUPPORTED;
 }
 
+int32_t npas_internal_linear_two_preferred(const npas_linear_desc *a, const npas_linear_desc *b) { return linear_two_preferred(*a, *b); }
+
+npas_status npas_internal_linear_two(const npas_linear_desc *a, const npas_bb_desc *bba, const npas_linear_desc *b, const npas_bb_desc *bbb,
+                                     const void *x, const void *blob1, const float *bias1, const void *residual, void *y1, const void *blob2,
+                                     const float *bias2, void *y2, void *ws, size_t ws_bytes, int32_t chain, void *stream)
+{
+    npas_status s = check_linear_args(a, bba);
+    if (s == NPAS_OK) s = check_linear_args(b, bbb);
+    if (s != NPAS_OK) return s;
+    if (!x || !blob1 || !y1 || !blob2 || !y2 || !ws || (a->has_bias && !bias1) || (b->has_bias && !bias2) || (a->has_residual && !residual)) return NPAS_ERR_NULL;
+    for (const void *q : {x, blob1, static_cast<const void *>(y1), blob2, static_cast<const void *>(y2), static_cast<const void *>(ws), residual,
+                          static_cast<const void *>(bias1), static_cast<const void *>(bias2)})
+        if (q && !aligned16(q)) return NPAS_ERR_ALIGNMENT;
+    if (ws_bytes < NPAS_WORKSPACE_BYTES) return NPAS_ERR_BUFFER_TOO_SMALL;
+    return linear_two_launch(*a, *bba, *b, *bbb, x, blob1, a->has_bias ? bias1 : nullptr, a->has_residual ? residual : nullptr, y1, blob2,
+                             b->has_bias ? bias2 : nullptr, y2, static_cast<uint32_t *>(ws), static_cast<cudaStream_t>(stream), launch_of(chain));
+}
+
 }  // extern "C"
 
 // ---- auto-tuning: measure every kernel / tile shape that takes the layer, keep the fastest --------

@@ -244,6 +244,10 @@ float linear_d2_cost(const npas_linear_desc &d, const npas_bb_desc &bb);
 npas_status linear_d2_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,
                              cudaStream_t st, Launch how);
+bool linear_two_preferred(const npas_linear_desc &a, const npas_linear_desc &b);
+npas_status linear_two_launch(const npas_linear_desc &a, const npas_bb_desc &bba, const npas_linear_desc &b, const npas_bb_desc &bbb, const void *x,
+                              const void *blob1, const float *bias1, const void *res, void *y1, const void *blob2, const float *bias2, void *y2,
+                              uint32_t *ws, cudaStream_t st, Launch how);
 bool linear_tc_supported(const npas_linear_desc &d, const npas_bb_desc &bb);
 npas_status linear_tc_launch(const npas_linear_desc &d, const npas_bb_desc &bb, const void *x,
                              const void *blob, const float *bias, const void *res, void *y, uint32_t *ws,

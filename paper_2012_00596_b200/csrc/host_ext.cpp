@@ -693,6 +693,15 @@ PyObject *stack_forward(PyObject *, PyObject *const *a, Py_ssize_t nargs)
             if (!free_between) continue;
             from[(size_t)i] = s; join[(size_t)i] = j; begins[(size_t)s] = i;
         }
+        // Two 1x1 layers behind one another, the second reading nothing but the first: one launch where that is the faster way.
+        // Its outputs are written while its inputs are still being read, so what is free behind the first layer is given back
+        // behind the second only.
+        std::vector<char> two((size_t)L, 0);
+        std::vector<int64_t> held;
+        auto give = [&](int i, int64_t at) {
+            if (two[(size_t)i]) held.push_back(at);
+            else arena.give(at);
+        };
         for (int i = 0; i < L; ++i) {
             const LayerRow &r = rows[i];
             Step &st = steps[(size_t)i];
@@ -726,15 +735,25 @@ PyObject *stack_forward(PyObject *, PyObject *const *a, Py_ssize_t nargs)
                 if (r.kind == 0) { st.p = (st.p + 2 - 3) / 2 + 1; st.q = (st.q + 2 - 3) / 2 + 1; }      // the pooled tensor
             }
             if (from[(size_t)i] < 0) st.out = i == L - 1 ? -1 : arena.take(N * st.p * st.q * r.cout * 2);
+            if (r.kind == 2 && r.stride == 1 && from[(size_t)i] < 0 && i + 1 < L && a[5] == Py_None) {
+                const LayerRow &t = rows[i + 1];
+                const npas_linear_desc b{st.ld.M, r.cout, t.cout, NPAS_BF16, NPAS_BF16, t.relu, 1, 0, 0, 0};
+                two[(size_t)i] = t.kind == 2 && t.stride == 1 && t.src == i && t.res == -3 && from[(size_t)i + 1] < 0 && begins[(size_t)i + 1] < 0 && (i == 0 || !two[(size_t)i - 1]) &&
+                                 npas_internal_linear_two_preferred(&st.ld, &b);
+            }
             made[(size_t)i] = Shape{st.p, st.q, r.cout, st.out};
             if (r.kind == 0) pooled = made[(size_t)i];
-            if (st.sub >= 0 && from[(size_t)i] < 0) arena.give(st.sub);
+            if (st.sub >= 0 && from[(size_t)i] < 0) give(i, st.sub);
             // buffers that no later layer reads (the pooled tensor has one of its own name)
             for (int j = 0; j <= i; ++j)
-                if (made[(size_t)j].at >= 0 && j != L - 1 && rows[j].kind != 0 && last[(size_t)j] <= i && (last[(size_t)j] == i || j == i)) { arena.give(made[(size_t)j].at); }
-            if (pooled.at >= 0 && pooled_last == i) arena.give(pooled.at);
+                if (made[(size_t)j].at >= 0 && j != L - 1 && rows[j].kind != 0 && last[(size_t)j] <= i && (last[(size_t)j] == i || j == i)) give(i, made[(size_t)j].at);
+            if (pooled.at >= 0 && pooled_last == i) give(i, pooled.at);
             for (int k = 0; k < i; ++k)                     // a layer beside these ends here: its subsampled input is free
-                if (from[(size_t)k] >= 0 && join[(size_t)k] == i && steps[(size_t)k].sub >= 0) arena.give(steps[(size_t)k].sub);
+                if (from[(size_t)k] >= 0 && join[(size_t)k] == i && steps[(size_t)k].sub >= 0) give(i, steps[(size_t)k].sub);
+            if (i > 0 && two[(size_t)i - 1]) {
+                for (const int64_t at : held) arena.give(at);
+                held.clear();
+            }
             const int f = begins[(size_t)i];
             if (f >= 0) {
                 const Shape &o = made[(size_t)i];
@@ -775,7 +794,12 @@ PyObject *stack_forward(PyObject *, PyObject *const *a, Py_ssize_t nargs)
                 pending = -1;
                 if (s != NPAS_OK) break;
             }
-            if (r.kind == 2) {
+            if (i > 0 && two[(size_t)i - 1]) continue;     // (done together with the layer before)
+            if (two[(size_t)i]) {
+                const Step &t = steps[(size_t)i + 1];
+                s = npas_internal_linear_two(&st.ld, &st.bb, &t.ld, &t.bb, in, st.blob, st.bias, res, out, t.blob, t.bias, t.out < 0 ? yout : base + t.out, w, wb,
+                                             chain, stream);
+            } else if (r.kind == 2) {
                 if (st.sub >= 0) {
                     s = npas_subsample2d((int32_t)N, (int32_t)st.h, (int32_t)st.w, st.ld.I, r.stride, 2, in, base + st.sub, stream);
                     if (s != NPAS_OK) break;

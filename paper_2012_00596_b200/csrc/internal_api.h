@@ -40,6 +40,12 @@ npas_status npas_internal_conv2d_bp_maxpool(const npas_conv_desc *d, const npas_
                                             void *ws, size_t ws_bytes, int32_t chain, void *stream);
 npas_status npas_internal_linear_bb(const npas_linear_desc *d, const npas_bb_desc *bb, const void *x, const void *blob, const float *bias,
                                     const void *residual, void *y, void *ws, size_t ws_bytes, int32_t chain, void *stream);
+// Two GEMMs behind one another, b's input being a's output (which is written all the same), as one launch: whether that is the
+// faster way, and the call.  None of y1, y2 may lie on x or the residual.
+int32_t npas_internal_linear_two_preferred(const npas_linear_desc *a, const npas_linear_desc *b);
+npas_status npas_internal_linear_two(const npas_linear_desc *a, const npas_bb_desc *bba, const npas_linear_desc *b, const npas_bb_desc *bbb,
+                                     const void *x, const void *blob1, const float *bias1, const void *residual, void *y1, const void *blob2,
+                                     const float *bias2, void *y2, void *ws, size_t ws_bytes, int32_t chain, void *stream);
 #ifdef __cplusplus
 }
 #endif
