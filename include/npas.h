@@ -128,7 +128,7 @@ typedef struct {
  * 2 = automatic among the tcgen05 kernels, 3 = force the tcgen05 kernel with both operands in shared memory, 5 = force the tcgen05 kernel
  * for three-channel 7x7 stride-2 first layers, 6 = force the tcgen05 kernel that multiplies the
  * blob's dense operand image, 7 = force the variant of that kernel that runs on CTA pairs
- * (cta_group::2; C % 64 == 0, K % 64 == 0), 8 = force the tcgen05 kernel that multiplies kept
+ * (cta_group::2; C % 64 == 0, K % 64 == 0; in its wide form, by `variant`, multiples of 16), 8 = force the tcgen05 kernel that multiplies kept
  * (block, tap) pairs only (stride 1, Mb and Nb multiples of 16, at most 16 taps)
  * (NPAS_ERR_UNSUPPORTED when the geometry is outside the requested kernel's envelope). */
 typedef struct {
@@ -138,7 +138,8 @@ typedef struct {
     int32_t path;
     int32_t variant; /* 0 = the kernel's own planner chooses its tile shape; path 7: NT + (MT << 16), NT =
                         64 (only when 128 does not divide K), 128 or 256 filters per item, MT = 1 or 2 position tiles per CTA (a combination the
-                        geometry does not allow gives NPAS_ERR_UNSUPPORTED); path 6: NT + (KC << 16) +
+                        geometry does not allow gives NPAS_ERR_UNSUPPORTED), + (1 << 24) asks for the wide form, which
+                        takes C and K in multiples of 16 and NT in multiples of 32 (0: its planner's choice); path 6: NT + (KC << 16) +
                         (KT << 24) asks for the form for few output tiles, in which a cluster of KC * KT <= 8
                         CTAs shares 128 positions x NT filters (16 to 128) and splits the channels into KC and
                         the taps into KT ranges; other paths ignore it.

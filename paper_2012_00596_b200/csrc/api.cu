@@ -116,11 +116,35 @@ npas_status npas_linear_bb_workspace(const npas_linear_desc *d, const npas_bb_de
 // Path 6 has two forms: the persistent kernel, and for few output tiles the one that splits channels and taps over a
 // cluster (asked for by `variant`, or chosen when no kernel was asked for; where the pair kernel has half a wave of its
 // stride-1 items, that one stays the choice).
+// Path 7 likewise: the form for channels and filters off multiples of 64 and 128 is asked for by a bit of `variant`, or chosen.
+struct ConvChoice { int kernel; bool split, wide; };
+
+static ConvChoice conv_choose(const npas_conv_desc &d, const npas_bp_desc &bp)
+{
+    // automatic: the first-layer kernel; kept pairs only where that was measured faster (few taps kept,
+    // blocks of 16 channels or more); else the dense-image kernels; else shared-memory operands; else float64
+    if (conv_stem_supported(d, bp)) return {5, false, false};
+    if (conv_kr_preferred(d, bp)) return {8, false, false};
+    if (conv_d2_wide_preferred(d, bp)) return {7, false, true};
+    if (!(d.stride == 1 && conv_d2_preferred(d, bp)) && conv_sk_preferred(d, bp)) return {6, true, false};
+    if (conv_d2_preferred(d, bp)) return {7, false, false};
+    if (conv_dn_supported(d, bp)) return {6, false, false};
+    if (conv_tc_supported(d, bp)) return {3, false, false};
+    return {d.path == 2 ? 0 : 1, false, false};
+}
+
+// (kept per thread like the plans: up to ten of them are compared)
+static ConvChoice conv_choice(const npas_conv_desc &d, const npas_bp_desc &bp)
+{
+    ConvChoice c{};
+    cached_plan(d, bp, 0, c, [&](ConvChoice &q) { q = conv_choose(d, bp); return true; });
+    return c;
+}
+
 static bool conv_split(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     if (d.path == 6) return d.variant != 0;
-    if ((d.path != 0 && d.path != 2) || (d.stride == 1 && conv_d2_preferred(d, bp))) return false;
-    return conv_sk_preferred(d, bp);
+    return (d.path == 0 || d.path == 2) && conv_choice(d, bp).split;
 }
 
 static int conv_kernel_for(const npas_conv_desc &d, const npas_bp_desc &bp)
@@ -135,15 +159,7 @@ static int conv_kernel_for(const npas_conv_desc &d, const npas_bp_desc &bp)
         case 0: case 2: break;
         default: return 0;
     }
-    // automatic: the first-layer kernel; kept pairs only where that was measured faster (few taps kept,
-    // blocks of 16 channels or more); else the dense-image kernels; else shared-memory operands; else float64
-    if (conv_stem_supported(d, bp)) return 5;
-    if (conv_kr_preferred(d, bp)) return 8;
-    if (conv_split(d, bp)) return 6;
-    if (conv_d2_preferred(d, bp)) return 7;
-    if (conv_dn_supported(d, bp)) return 6;
-    if (conv_tc_supported(d, bp)) return 3;
-    return d.path == 2 ? 0 : 1;
+    return conv_choice(d, bp).kernel;
 }
 
 // Path 5 has two forms: the persistent kernel, and for few output tiles the one that splits the input over a cluster
@@ -263,7 +279,8 @@ npas_status npas_internal_conv2d_bp(const npas_conv_desc *d, const npas_bp_desc 
         case 6:
             if (conv_split(*d, *bp)) return conv_sk_launch(*d, *bp, x, blob, b, r, y, w, st, how);
             return conv_dn_launch(*d, *bp, x, blob, b, r, y, w, st, how);
-        case 7: return conv_d2_launch(*d, *bp, x, blob, b, r, y, w, st, how);
+        case 7: return conv_d2_launch(*d, *bp, x, blob, b, r, y, w, st, how,
+                                      d->path == 7 ? (d->variant & conv_d2_wide_variant()) != 0 : conv_choice(*d, *bp).wide);
         case 8: return conv_kr_launch(*d, *bp, x, blob, b, r, y, w, st, how);
     }
     return NPAS_ERR_UNSUPPORTED;
@@ -437,10 +454,10 @@ npas_status npas_tune_conv2d_bp(const npas_conv_desc *d, const npas_bp_desc *bp,
     q.path = 0; q.variant = 0;
     const int kid = conv_kernel_for(q, *bp);
     std::vector<Cand> cands;
-    cands.push_back({kid, kid == 6 && conv_split(q, *bp) ? conv_sk_variant(q, *bp) : 0});
+    cands.push_back({kid, kid == 6 && conv_split(q, *bp) ? conv_sk_variant(q, *bp) : kid == 7 && conv_d2_wide_preferred(q, *bp) ? conv_d2_wide_variant() : 0});
     // every item shape of the pair kernel: filters per item 64, 128 or 256, position tiles per CTA 1 or 2
     for (const Cand &c : {Cand{5, 0}, Cand{8, 0}, Cand{7, 64 | (1 << 16)}, Cand{7, 64 | (2 << 16)}, Cand{7, 128 | (1 << 16)}, Cand{7, 128 | (2 << 16)},
-                          Cand{7, 256 | (1 << 16)}, Cand{7, 256 | (2 << 16)}, Cand{6, 0}, Cand{3, 0}})
+                          Cand{7, 256 | (1 << 16)}, Cand{7, 256 | (2 << 16)}, Cand{7, conv_d2_wide_variant()}, Cand{6, 0}, Cand{3, 0}})
         cands.push_back(c);
     int32_t split[64];
     const int n = conv_sk_shapes(q, *bp, split, 64);

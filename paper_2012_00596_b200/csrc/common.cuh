@@ -218,9 +218,13 @@ bool conv_d2_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 bool conv_d2_preferred(const npas_conv_desc &d, const npas_bp_desc &bp);
 double conv_dense_modelled(const npas_conv_desc &d, const npas_bp_desc &bp);
 bool conv_sk_slower(const npas_conv_desc &d, const npas_bp_desc &bp);
+double conv_sk_modelled(const npas_conv_desc &d, const npas_bp_desc &bp);
+double conv_d2_wide_modelled(const npas_conv_desc &d, const npas_bp_desc &bp);
+bool conv_d2_wide_preferred(const npas_conv_desc &d, const npas_bp_desc &bp);
+int32_t conv_d2_wide_variant();
 npas_status conv_d2_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
-                           uint32_t *ws, cudaStream_t st, Launch how);
+                           uint32_t *ws, cudaStream_t st, Launch how, bool wide);
 bool conv_kr_supported(const npas_conv_desc &d, const npas_bp_desc &bp);
 bool conv_kr_preferred(const npas_conv_desc &d, const npas_bp_desc &bp);
 npas_status conv_kr_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,

@@ -15,6 +15,12 @@
 //   pair halves the weight bytes every SM stages and reads per MMA, and every weight byte fetched
 //   from L2 serves twice the positions.
 //
+// The wide form (channels and filters in multiples of 16): the last slab of a position holds fewer than four chunks, the channels
+// past the end arriving as zeros that no MMA reads, and a CTA's half of the operand is several of the image's groups of 16, 32 or 64
+// filters, which one tensor copy lays next to one another (groups past the last one as zeros, their columns not stored).  Such
+// layers ran as the split form or on independent CTAs whose MMAs were as narrow as a group: 25x8x33x464 -> 480 73 -> 38 us,
+// 22x12x47x48 -> 432 33 -> 10.8, 17x64x21x320 -> 48 36 -> 12.5, 49x57x28x240 -> 96 strided 32 -> 21.
+//
 // Roles per CTA (384 threads): warp 0 loads the slabs (ring of 64-channel stages), warp 2 loads this CTA's
 // half of the weight tiles through a 2-D tensor map laid over the blob (ring of 16- or 32-channel stages),
 // warps 1 and 3 of the pair's leader (cluster rank 0) issue the MMAs, one warp per position tile and
@@ -44,6 +50,7 @@ constexpr int kThreads = (kFirstEpiWarp + kEpiWarps) * 32;
 constexpr int kMaxStages = 8;                    // weight ring
 constexpr int kMaxSlabStages = 3;
 constexpr int kMaxTapsD2 = 16;
+constexpr int32_t kWide = 1 << 24;               // in `variant`: the wide form (several groups of the image per CTA)
 constexpr uint32_t kSmemLimit = 232448;
 constexpr uint32_t kDescHiB = (128u >> 4) | (1u << 14);                      // B: no swizzle, SBO = 128 bytes, version bit
 constexpr uint32_t kDescHiA = (1024u >> 4) | (1u << 14) | (2u << 29);        // A: 128-byte swizzle, SBO = 1024 bytes, version bit
@@ -53,6 +60,7 @@ struct ConvD2Params {
     int nph, sh;                                              // input phases per slab (1, or 4: stride 2 by parity); store shift
     int Wp, TR, tiles_per_img, n_tiles, slab_rows;
     int IT, img_pitch;                                        // small maps: IT whole images per tile, img_pitch positions apart
+    int gathered, GG;                                         // a CTA's filters are GG whole groups of the image (else one group, or half of one)
     int RS, nCh, nBlk, GH, NT, MT, CPW, n_fsets, n_items, SA, SB, nacc, dcols;   // GH: filters per CTA, NT = 2 GH per item; CPW: chunks per weight stage
     int GI;                                                   // filters per group of the blob's operand image (128, or 64 when 128 does not divide K)
     int relu, y_bf16, early;                                  // early: the blob may be read before the wait (Launch::blob_ready)
@@ -113,7 +121,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint32_t *tapu_s = reinterpret_cast<uint32_t *>(smem + p.off_tapu);     // [K / GI][nCh]
+    uint32_t *tapu_s = reinterpret_cast<uint32_t *>(smem + p.off_tapu);     // [n_fsets][nCh]
     float *bias_s = reinterpret_cast<float *>(smem + p.off_bias);           // [K]
     ConvD2Bars *bars = reinterpret_cast<ConvD2Bars *>(smem + p.off_bar);
     volatile uint32_t *abort_flag = &bars->abort_flag;
@@ -162,7 +170,14 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     if (warp != 0 && warp != 2) {
         const int t = tid < 64 ? tid - 32 : tid - 64;         // 0 .. kThreads - 65 over warps 1, 3, 4, ...
         const uint32_t *tapu = reinterpret_cast<const uint32_t *>(blob + off_tapu);
-        for (int i = t; i < (p.K / p.GI) * p.nCh; i += kThreads - 64) tapu_s[i] = off_tapu ? __ldg(tapu + i) : 0xFFFFFFFFu;
+        const int ngrp = p.NT / p.GI, groups = p.K / p.GI;        // groups of the image per item
+        for (int i = t; i < p.n_fsets * p.nCh; i += kThreads - 64) {
+            const int fs = i / p.nCh, ch = i - fs * p.nCh;
+            uint32_t m = off_tapu ? 0u : 0xFFFFFFFFu;
+            if (off_tapu)
+                for (int g = fs * ngrp; g < min((fs + 1) * ngrp, groups); ++g) m |= __ldg(tapu + g * p.nCh + ch);
+            tapu_s[i] = m;
+        }
         if (p.IT > 1 && p.act_stride > p.slab_bytes) {
             // several images per tile: the last image's bottom-right taps read just past the slab, where no copy
             // ever writes: zeros, once, in every buffer of the ring (read by the tensor core: async proxy)
@@ -233,9 +248,13 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         // 2048 bytes: the weight map is then four-dimensional (128 bytes, 8 lines of a half, 2 halves, rows of
         // 2048 bytes) and ONE box (128, 8, 1, rows of the stage) brings the stage's halves back to back (36
         // separate 1 KB copies per stage cost the issuing warp 2.5 k cycles, more than the stage's MMAs take).
+        // One holding several groups (K off the multiples of 64, or 64 that fill no 128) has a map over (128 bytes, lines of
+        // a group's row, groups, rows of all (chunk, tap, octet)): ONE box puts the groups of every row next to one another,
+        // groups past the last one as zeros.
         const int rows_st = 2 * p.RS * p.CPW;                 // weight rows (chunk, tap, octet) of a stage
         const uint32_t copy_bytes = p.w_box_rows * 128u;      // 128 filters: one copy = one box of the weight map
-        const int n_copies = p.GH == 128 ? (int)(p.w_bytes / copy_bytes) : 1;
+        const bool runs = p.GH == 128 && !p.gathered;
+        const int n_copies = runs ? (int)(p.w_bytes / copy_bytes) : 1;
         const uint32_t grow = (uint32_t)p.GI * 16u;           // bytes of a (tap, octet) row of the image: GI filters x 8 channels
         const uint32_t w_full0 = map_to_cta(smem_u32(&bars->w_full[0]), 0u);      // the leader's barriers
         const uint32_t image_row0 = off_image >> 7;           // the weight map counts the blob in 128-byte rows
@@ -254,7 +273,11 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 if (!ok) break;
                 uint8_t *wdst = smem + p.off_w + (size_t)s * p.w_bytes;
                 const uint32_t src = wsrc + (uint32_t)wst * (uint32_t)rows_st * (grow >> 7);     // rows of the image, in 128-byte map rows
-                if (p.GH == 128) {
+                if (p.gathered) {
+                    if (lane == 0)
+                        tma_load_4d_pair(wdst, &tmap_w, w_full0 + s * 8u, 0, 0, fs * (p.NT / p.GI) + (int)rank * p.GG,
+                                         (int)(off_image / grow) + wst * rows_st);
+                } else if (runs) {
                     for (int i = lane; i < n_copies; i += 32)
                         tma_load_2d_pair(wdst + (size_t)i * copy_bytes, &tmap_w, w_full0 + s * 8u, 0, (int)(src + (uint32_t)i * p.w_box_rows));
                 } else if (lane == 0) {
@@ -269,7 +292,6 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             }
         }
     } else if (warp == 1 || warp == 3) {
-        const int wst_blk = 4 / p.CPW;                        // weight stages per 64-channel block
         // (the peer has no part in this role: its copies complete on the leader's barriers by themselves)
         if (rank == 0 && (warp >> 1) < p.MT) {
             // ---- leader: MMA issue for the pair; this warp owns the accumulator of position tile mt, so the
@@ -286,7 +308,6 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 for (int t = 0; t < kMaxTapsD2; ++t) shift[t] = p.shift16[t];
                 const uint32_t b_hi = (uint32_t)p.GH << 16, b_step = 2u * p.GH, chunk16 = (uint32_t)p.RS * b_step;
                 const uint32_t a_base = (base16 + (uint32_t)mt * tile16) | (1u << 16), b_base = (base16 + (p.off_w >> 4)) | b_hi;
-                const int ngrp = p.NT / p.GI;                   // groups of the image per item (1 or 2)
                 uint32_t sa = 0, pha = 0, a_st = a_base, sb = 0, phb = 0, b_st = b_base, it = 0;
                 bool ok = true;
                 for (int item = pair; item < p.n_items && ok; item += n_pairs, ++it) {
@@ -295,20 +316,21 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                     if (lap_acc >= 1 && !pair_wait<true>(&bars->acc_empty[acc], (lap_acc & 1u) ^ 1u, abort_flag, peer_abort, ws, 0x7200)) break;
                     tc_fence_after_sync();
                     const uint32_t d_tmem = tmem_base + acc * p.dcols + (uint32_t)mt * p.NT;
-                    const uint32_t *tu = tapu_s + (fs * ngrp) * p.nCh;
+                    const uint32_t *tu = tapu_s + fs * p.nCh;
                     int ch = 0;
                     for (int blk = 0; blk < p.nBlk && ok; ++blk) {
                         if (!pair_wait(&bars->a_full[sa], pha, abort_flag, peer_abort, ws, 0x7300)) { ok = false; break; }
                         uint32_t a16 = a_st;                    // 16 channels = 32 bytes inside the swizzled 128-byte row
-                        for (int q = 0; q < wst_blk; ++q) {
+                        // (the last block may hold fewer chunks: its slab's other channels are zeros that nothing reads)
+                        const int end = min(ch + 4, p.nCh);
+                        while (ch < end) {
                             if (!pair_wait(&bars->w_full[sb], phb, abort_flag, peer_abort, ws, 0x7320)) { ok = false; break; }
                             tc_fence_after_sync();
                             uint32_t b_lo = b_st;
                             for (int cc = 0; cc < p.CPW; ++cc, ++ch, a16 += 2u, b_lo += chunk16) {
                                 // a tap that no block of these (groups, chunk) keeps multiplies zeros: skipped, except
                                 // the very first MMA, which initialises the accumulator
-                                uint32_t m = tu[ch] | (ch == 0 ? 1u : 0u);
-                                if (ngrp == 2) m |= tu[p.nCh + ch];
+                                const uint32_t m = tu[ch] | (ch == 0 ? 1u : 0u);
                                 if (p.RS == 9) issue_taps<9>(d_tmem, a16, b_lo, b_step, shift, m, idesc, ch != 0);
                                 else issue_taps<kMaxTapsD2>(d_tmem, a16, b_lo, b_step, shift, m & ((1u << p.RS) - 1u), idesc, ch != 0);
                             }
@@ -359,6 +381,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 const int mt = j >= cpt ? 1 : 0, c0 = (j - mt * cpt) * 16;
                 if (!(mt ? val[1] : val[0])) return;
                 const int k0 = fs * p.NT + c0;
+                if (k0 >= p.K) return;                      // the last item's filters past the end
                 const size_t o0 = (mt ? obase[1] : obase[0]) + k0;
                 float v[16];
                 const float4 *b4 = reinterpret_cast<const float4 *>(bias_s + k0);
@@ -462,12 +485,25 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 
 int pairs_available() { return sm_count() / 2; }
 
-bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int pairs)
+// Microseconds of a plan of the wide form, fitted to 427 measured points (59 random layers, every item shape; standard error 12 %,
+// the shape it picks within 2 % of the best one): an MMA takes the pipe NT / 2 cycles and its issuing thread 70 (two warps issue for two
+// position tiles), the epilogue's columns, what leaves for DRAM.
+double modelled(const ConvD2Params &p, const npas_conv_desc &d, int pairs)
+{
+    const double rounds = (double)((p.n_items + pairs - 1) / pairs);
+    const double mma = p.MT == 2 ? (p.NT > 74 ? p.NT : 74.) : (p.NT > 140 ? p.NT / 2 : 70.);     // cycles per chunk and tap
+    const double out_mb = 2e-6 * p.N * p.Po * p.Qo * p.K * (d.has_residual ? 2. : 1.) * (p.y_bf16 ? 1. : 2.);
+    return 4.6 + rounds * (p.nCh * p.RS * mma / 1900. + 0.0068 * p.NT * p.MT) + 0.23 * out_mb;
+}
+
+// `wide`: channels and filters in multiples of 16, items of several of the image's groups (kWide).
+bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int pairs, bool wide)
 {
     if (d.x_dtype != NPAS_BF16 || bp.w_packed != NPAS_BF16) return false;
-    if ((d.stride != 1 && d.stride != 2) || d.pad < 0 || d.C % 64 || d.K % 64) return false;
-    p.GI = (int)bp_layout(bp, 0).GI;                      // 128, or 64 when 128 does not divide K
-    if (p.GI != 64 && p.GI != 128) return false;
+    if ((d.stride != 1 && d.stride != 2) || d.pad < 0 || d.C % 16 || d.K % 16) return false;
+    if (!wide && (d.C % 64 || d.K % 64)) return false;
+    p.GI = (int)bp_layout(bp, 0).GI;                      // 128, or the largest smaller power of two that divides K
+    if (p.GI < 16 || (!wide && p.GI < 64)) return false;
     p.RS = d.R * d.S;
     if (p.RS > kMaxTapsD2) return false;
     p.N = d.N; p.H = d.H; p.W = d.W; p.C = d.C; p.K = d.K; p.R = d.R; p.S = d.S; p.pad = d.pad; p.stride = d.stride;
@@ -515,7 +551,7 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             if (!phases) reach = (128u + (uint32_t)(d.R - 1) * p.Wp + d.S) * 128u;
         }
     }
-    p.nCh = d.C / 16; p.nBlk = d.C / 64;
+    p.nCh = d.C / 16; p.nBlk = (d.C + 63) / 64;
     p.relu = d.relu; p.y_bf16 = d.y_dtype == NPAS_BF16;
     p.slab_bytes = (uint32_t)(p.IT * p.slab_rows) * p.Wp * 128u;
     // a shifted operand reads 128 rows from its start: room behind the slab (what lies there only reaches
@@ -538,24 +574,28 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
     // filters per item (NT) and position tiles per CTA (MT): the combination with the least modelled time,
     // rounds of items over the pairs x (MMA cycles of an item + its epilogue where that is not overlapped)
     // (the call descriptor's `variant`, NT + (MT << 16), restricts the choice to one combination)
-    const int want_nt = d.variant & 0xFFFF, want_mt = (d.variant >> 16) & 0xFFFF;
+    const int want_nt = d.variant & 0xFFFF, want_mt = (d.variant & ~(wide ? kWide : 0)) >> 16;
     double best = 0.;
     bool found = false;
-    for (int NT = 256; NT >= 64; NT >>= 1) {
-        // an item is one or two groups of the image (with groups of 64 filters: one)
-        if (d.K % NT || (want_nt && NT != want_nt) || NT < p.GI || (p.GI == 64 && NT != 64)) continue;
+    for (int NT = 256; NT >= 32; NT -= 32) {
+        // an item is one or two groups of the image (with groups of 64 filters: one), or in the wide form every CTA of the pair
+        // holds the same number of whole groups
+        const bool gathered = p.GI < 128 && NT % (2 * p.GI) == 0;
+        if (want_nt && NT != want_nt) continue;
+        if (gathered ? !wide || NT >= d.K + 2 * p.GI : d.K % NT || NT < p.GI || NT < 64 || (NT & (NT - 1)) || p.GI < 64 || (p.GI == 64 && NT != 64)) continue;
         for (int MT = 1; MT <= 2; ++MT) {
             if (MT * NT > 512 || (want_mt && MT != want_mt)) continue;
             if (MT > 1 && p.n_tiles < 4) continue;
             ConvD2Params q = p;
-            q.NT = NT; q.GH = NT / 2; q.MT = MT; q.n_fsets = d.K / NT;
+            q.NT = NT; q.GH = NT / 2; q.MT = MT; q.n_fsets = (d.K + NT - 1) / NT;
+            q.gathered = gathered; q.GG = gathered ? q.GH / p.GI : 0;
             const long long items = (long long)((p.n_tiles + 2 * MT - 1) / (2 * MT)) * q.n_fsets;
             if (items > 0x7FFFFFFF) return false;
             q.n_items = (int)items;
             q.a_stage_bytes = (uint32_t)(MT * p.nph) * p.act_stride;
             // a weight stage holds two chunks of a 64-filter half (32 KB at nine taps, as one chunk of a
             // 128-filter half), one where the slabs leave no room for two such stages
-            q.CPW = q.GH == 64 ? 2 : q.GH == 32 ? 4 : 1;
+            q.CPW = q.GH > 64 ? 1 : q.GH > 32 ? 2 : 4;
             while (q.CPW > 1 && p.nCh % q.CPW) q.CPW /= 2;
             q.w_bytes = (uint32_t)q.CPW * p.RS * 2u * q.GH * 16u;
             while (q.CPW > 1 && 2u * q.a_stage_bytes + 2u * q.w_bytes > avail) { q.CPW /= 2; q.w_bytes /= 2; }
@@ -579,7 +619,7 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             // 56x56x64 -> 64, 23.7 us on two tiles per CTA against 26.5 on one)
             const double mma = (double)p.nCh * p.RS * (NT == 64 && MT == 2 ? per_mma : MT * per_mma);
             const double epi = (double)MT * NT * 16.;
-            const double cost = (rounds * (mma + (q.nacc == 2 ? 0. : epi)) + epi + 6000.) * ((NT == 128 && MT == 1) ? 0.9 : 1.);
+            const double cost = wide ? modelled(q, d, pairs) : (rounds * (mma + (q.nacc == 2 ? 0. : epi)) + epi + 6000.) * ((NT == 128 && MT == 1) ? 0.9 : 1.);
             if (!found || cost < best) { best = cost; p = q; found = true; }
         }
     }
@@ -595,18 +635,39 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
     return true;
 }
 
-bool planned(const npas_conv_desc &d, const npas_bp_desc &b, ConvD2Params &p)
+bool planned(const npas_conv_desc &d, const npas_bp_desc &b, ConvD2Params &p, bool wide = false)
 {
-    return cached_plan(d, b, 0, p, [&](ConvD2Params &q) { return plan(d, b, q, pairs_available()); });
+    return cached_plan(d, b, wide, p, [&](ConvD2Params &q) { return pairs_available() > 0 && plan(d, b, q, pairs_available(), wide); });
 }
 
 }  // namespace
 
+// forced: the wide form is asked for by a bit of `variant`
 bool conv_d2_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvD2Params p;
-    return planned(d, bp, p);
+    return planned(d, bp, p, (d.variant & kWide) != 0);
 }
+
+// Microseconds of the wide form where it may be chosen: layers that the other plan does not take, or only in items of 64 filters
+// (192, 320, 448 of them); strided ones by phases, not at every position.
+double conv_d2_wide_modelled(const npas_conv_desc &d, const npas_bp_desc &bp)
+{
+    ConvD2Params p;
+    if (d.variant || (d.C % 64 == 0 && (d.K % 128 == 0 || d.K == 64)) || !planned(d, bp, p, true)) return 1e30;
+    return d.stride != 1 && p.nph == 1 ? 1e30 : modelled(p, d, pairs_available());
+}
+
+// By the models of the kernels: against the split form where that is what would run (its model is fitted to layers of a chain; a call by
+// itself takes 1 us more, the wait for the blob), else against independent CTAs.  On 70 random layers of 16 to 512 channels and
+// filters what is chosen is 2.6 % above the better measured one, and 1.42 times faster than without this form (one with 22x15x22x48 ->
+// 192, 10.7 against 9.9 us, lies on the wrong side).
+bool conv_d2_wide_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
+{
+    const double us = conv_d2_wide_modelled(d, bp), split = us < 1e9 ? conv_sk_modelled(d, bp) : 0.;
+    return us < 1e9 && us < (split < 1e9 ? split + 1. : conv_dense_modelled(d, bp));
+}
+int32_t conv_d2_wide_variant() { return kWide; }
 
 // Whether the pair kernel is the better of the two dense-image kernels for this call (measured): always
 // for the strided 3x3 geometry it computes by phases (a quarter of the MMAs); else as soon as there are
@@ -646,11 +707,11 @@ double conv_dense_modelled(const npas_conv_desc &d, const npas_bp_desc &bp)
 
 npas_status conv_d2_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,
                            const void *blob, const float *bias, const void *res, void *y,
-                           uint32_t *ws, cudaStream_t st, Launch how)
+                           uint32_t *ws, cudaStream_t st, Launch how, bool wide)
 {
     ConvD2Params p;
     const int pairs = pairs_available();
-    if (pairs < 1 || !planned(d, bp, p)) return NPAS_ERR_UNSUPPORTED;
+    if (pairs < 1 || !planned(d, bp, p, wide)) return NPAS_ERR_UNSUPPORTED;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return NPAS_ERR_CUDA;
     // X[N][H][W][C] bf16 as (C, W, H, N): a box of 64 channels x Wp columns x slab rows lands in shared
@@ -675,7 +736,17 @@ npas_status conv_d2_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
     CUtensorMap tmap_w;
     const uint32_t all_pairs = (uint32_t)(bp.K / bp.Mb) * (uint32_t)(bp.C / bp.Nb) * (uint32_t)(bp.R * bp.S);
     const uint32_t blob_bytes = bp_layout(bp, all_pairs).total;
-    if (p.GH == 128) {
+    if (p.gathered) {
+        const uint32_t grow = (uint32_t)p.GI * 16u;
+        const cuuint64_t wdims[4] = {128, (cuuint64_t)(p.GI / 8), (cuuint64_t)(d.K / p.GI), (cuuint64_t)(blob_bytes / grow)};
+        const cuuint64_t wstrides[3] = {128, (cuuint64_t)p.nCh * p.RS * 2u * grow, grow};
+        const cuuint32_t wbox[4] = {128, (cuuint32_t)(p.GI / 8), (cuuint32_t)p.GG, (cuuint32_t)(2 * p.RS * p.CPW)};
+        const cuuint32_t westr[4] = {1, 1, 1, 1};
+        if (enc(&tmap_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(blob), wdims, wstrides, wbox, westr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return NPAS_ERR_CUDA;
+    } else if (p.GH == 128) {
         const uint32_t rows = p.w_bytes / 128u;
         p.w_box_rows = 256;
         while (rows % p.w_box_rows) --p.w_box_rows;

@@ -786,7 +786,7 @@ bool conv_kr_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
     const int full = p.n_tiles / (int)grid.x, rest = p.n_tiles % (int)grid.x;
     const double rounds = full + (rest == 0 ? 0. : p.NQ == 1 ? 1. : 0.45 + 0.55 / p.NQ);
     const double us = 6.4 + rounds * (p.nChunks * (0.0448 * p.RS + 0.00473 * p.GS * p.max_taps) + 0.0087 * p.GS * p.Mb + 0.9);
-    return us < conv_dense_modelled(d, bp);
+    return us < conv_dense_modelled(d, bp) && us < conv_d2_wide_modelled(d, bp);
 }
 
 npas_status conv_kr_launch(const npas_conv_desc &d, const npas_bp_desc &bp, const void *x,

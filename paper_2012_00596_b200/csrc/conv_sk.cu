@@ -425,12 +425,12 @@ bool conv_sk_supported(const npas_conv_desc &d, const npas_bp_desc &bp)
 // Measured against the persistent kernels (this one, then the better of the two, both in a chain of layers): 14x14x256 -> 256 one image 4.8 against
 // 9.9 us, four 6.7 against 10.1, eight 8.1 against 10.2; 7x7x512 -> 512 5.8 against 14.6; 7x27x29x96 -> 160 7.8 against 8.3;
 // 54x6x33x160 -> 32 (108 position tiles) 8.0 against 6.9.  So: one wave, and no more position tiles than half the SMs.
-// Strided 3x3 layers that the pair kernel does not take by phases (it needs multiples of 64 channels and filters) always
-// come here: the single-CTA kernel computes every position (12x19x50x144 -> 208 8.9 against 36 us); those it takes, when
+// Strided 3x3 layers off multiples of 64 channels or filters come here unless the pair kernel's wide form is modelled faster
+// (conv_d2.cu): the single-CTA kernel computes every position (12x19x50x144 -> 208 8.9 against 36 us); the others, when
 // there are channels to split, one wave, and the pair kernel is not modelled faster (14x14x512 -> 512 5.8 against 17.1 us;
 // 59x17x48x512 -> 64 38.6 against 19.3).
 // The plan is part of the answer: what is launched is what was compared.
-static bool chosen(const npas_conv_desc &d, const npas_bp_desc &bp, ConvSkParams &p)
+static bool choose(const npas_conv_desc &d, const npas_bp_desc &bp, ConvSkParams &p)
 {
     const int sms = sm_count();
     if (d.variant) return false;
@@ -440,6 +440,11 @@ static bool chosen(const npas_conv_desc &d, const npas_bp_desc &bp, ConvSkParams
     if (planned(d, bp, p, true) && (phases ? p.nBlk > 1 && modelled(p, sms) <= conv_dense_modelled(d, bp) : p.n_tiles * 2 <= sms)) return true;
     // several waves: against independent CTAs, whose tile is as narrow as the image's groups (11x15x25x416 -> 464 51 against 63 us)
     return d.stride == 1 && !pairs && planned(d, bp, p, false) && 1.05 * modelled(p, sms) < conv_dense_modelled(d, bp);
+}
+
+static bool chosen(const npas_conv_desc &d, const npas_bp_desc &bp, ConvSkParams &p)
+{
+    return cached_plan(d, bp, 0, p, [&](ConvSkParams &q) { return choose(d, bp, q); });
 }
 
 bool conv_sk_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
@@ -455,6 +460,13 @@ bool conv_sk_slower(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvSkParams p;
     return !d.variant && d.stride == 1 && planned(d, bp, p, true) && modelled(p, sm_count()) > conv_dense_modelled(d, bp);
+}
+
+// microseconds of the form that an automatic choice of this kernel would run; where it would not, more than any other takes
+double conv_sk_modelled(const npas_conv_desc &d, const npas_bp_desc &bp)
+{
+    ConvSkParams p;
+    return chosen(d, bp, p) ? modelled(p, sm_count()) : 1e30;
 }
 
 static int32_t shape_of(const ConvSkParams &p) { return p.NT | (p.KC << 16) | (p.KT << 24); }
