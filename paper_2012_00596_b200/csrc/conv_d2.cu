@@ -21,6 +21,9 @@
 // layers ran as the split form or on independent CTAs whose MMAs were as narrow as a group: 25x8x33x464 -> 480 73 -> 38 us,
 // 22x12x47x48 -> 432 33 -> 10.8, 17x64x21x320 -> 48 36 -> 12.5, 49x57x28x240 -> 96 strided 32 -> 21.
 //
+// Small layers with many tiles (64 to 128 channels and filters) keep an item's weights in shared memory for all of a pair's items, and two
+// tiles of an image share one slab: 59 + 36 KB per item came in for 64x56x56x64 -> 64, 44 now (23.0 -> 22.5 us; 28x28x64 -> 128 13.6 -> 13.2).
+//
 // Roles per CTA (384 threads): warp 0 loads the slabs (ring of 64-channel stages), warp 2 loads this CTA's
 // half of the weight tiles through a 2-D tensor map laid over the blob (ring of 16- or 32-channel stages),
 // warps 1 and 3 of the pair's leader (cluster rank 0) issue the MMAs, one warp per position tile and
@@ -60,6 +63,8 @@ struct ConvD2Params {
     int nph, sh;                                              // input phases per slab (1, or 4: stride 2 by parity); store shift
     int Wp, TR, tiles_per_img, n_tiles, slab_rows;
     int IT, img_pitch;                                        // small maps: IT whole images per tile, img_pitch positions apart
+    int NSL, resident;                                        // slabs per stage and phase; resident: all weight stages stay in shared memory
+    uint32_t tile16;                                          // from one position tile's slab to the next one's, 16-byte units
     int gathered, GG;                                         // a CTA's filters are GG whole groups of the image (else one group, or half of one)
     int RS, nCh, nBlk, GH, NT, MT, CPW, n_fsets, n_items, SA, SB, nacc, dcols;   // GH: filters per CTA, NT = 2 GH per item; CPW: chunks per weight stage
     int GI;                                                   // filters per group of the blob's operand image (128, or 64 when 128 does not divide K)
@@ -206,9 +211,10 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                     const uint32_t s = n % (uint32_t)p.SA, k = n / (uint32_t)p.SA;
                     if (k >= 1 && !pair_wait(&bars->a_empty[s], (k - 1u) & 1u, abort_flag, peer_abort, ws, 0x7100)) { ok = false; break; }
                     uint8_t *st = smem + (size_t)s * p.a_stage_bytes;
-                    if (rank == 0) mbar_arrive_expect_tx(&bars->a_full[s], 2u * (uint32_t)(p.MT * p.nph) * p.slab_bytes);
-                    for (int mt = 0; mt < p.MT; ++mt) {
-                        const int tile = min((ts * 2 + (int)rank) * p.MT + mt, p.n_tiles - 1);   // a missing tile repeats the last one
+                    if (rank == 0) mbar_arrive_expect_tx(&bars->a_full[s], 2u * (uint32_t)(p.NSL * p.nph) * p.slab_bytes);
+                    for (int mt = 0; mt < p.NSL; ++mt) {
+                        // a missing tile repeats the last one (two tiles of one slab: the last two)
+                        const int tile = min((ts * 2 + (int)rank) * p.MT + mt, p.n_tiles - 1 - (p.MT - p.NSL));
                         const int img = p.IT > 1 ? tile * p.IT : tile / p.tiles_per_img;
                         const int y0 = p.IT > 1 ? 0 : (tile - img * p.tiles_per_img) * p.TR;
                         uint8_t *dst = st + (size_t)(mt * p.nph) * p.act_stride;
@@ -284,8 +290,9 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                     tma_load_4d_pair(wdst, &tmap_w, w_full0 + s * 8u, 0, 0, (int)rank, (int)(src / (grow >> 7)));    // (src counts 128-byte rows)
                 }
             }
+            if (p.resident) break;                            // every item of this pair has the same filters
         }
-        if (lane == 0 && ok) {
+        if (lane == 0 && ok && !p.resident) {
             for (uint32_t e = n; e < n + (uint32_t)p.SB; ++e) {
                 const uint32_t s = e % (uint32_t)p.SB, k = e / (uint32_t)p.SB;
                 if (k >= 1 && !pair_wait(&bars->w_empty[s], (k - 1u) & 1u, abort_flag, peer_abort, ws, 0x7130)) break;
@@ -302,7 +309,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 const int mt = warp >> 1;
                 const uint32_t idesc = idesc_bf16_f32(256, p.NT);
                 const uint32_t base16 = smem_u32(smem) >> 4, a_stage16 = p.a_stage_bytes >> 4;
-                const uint32_t tile16 = (uint32_t)p.nph * (p.act_stride >> 4), w16 = p.w_bytes >> 4;
+                const uint32_t tile16 = p.tile16, w16 = p.w_bytes >> 4;
                 uint32_t shift[kMaxTapsD2];
 #pragma unroll
                 for (int t = 0; t < kMaxTapsD2; ++t) shift[t] = p.shift16[t];
@@ -324,7 +331,8 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                         // (the last block may hold fewer chunks: its slab's other channels are zeros that nothing reads)
                         const int end = min(ch + 4, p.nCh);
                         while (ch < end) {
-                            if (!pair_wait(&bars->w_full[sb], phb, abort_flag, peer_abort, ws, 0x7320)) { ok = false; break; }
+                            // (stages that stay are complete for good: the parity of their first and only phase)
+                            if (!pair_wait(&bars->w_full[sb], p.resident ? 0u : phb, abort_flag, peer_abort, ws, 0x7320)) { ok = false; break; }
                             tc_fence_after_sync();
                             uint32_t b_lo = b_st;
                             for (int cc = 0; cc < p.CPW; ++cc, ++ch, a16 += 2u, b_lo += chunk16) {
@@ -334,7 +342,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                                 if (p.RS == 9) issue_taps<9>(d_tmem, a16, b_lo, b_step, shift, m, idesc, ch != 0);
                                 else issue_taps<kMaxTapsD2>(d_tmem, a16, b_lo, b_step, shift, m & ((1u << p.RS) - 1u), idesc, ch != 0);
                             }
-                            mma_commit_pair(&bars->w_empty[sb]);
+                            if (!p.resident) mma_commit_pair(&bars->w_empty[sb]);
                             b_st += w16;
                             if (++sb == (uint32_t)p.SB) { sb = 0; phb ^= 1u; b_st = b_base; }
                         }
@@ -592,7 +600,16 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             const long long items = (long long)((p.n_tiles + 2 * MT - 1) / (2 * MT)) * q.n_fsets;
             if (items > 0x7FFFFFFF) return false;
             q.n_items = (int)items;
+            q.NSL = MT; q.tile16 = (uint32_t)p.nph * (p.act_stride >> 4);
             q.a_stage_bytes = (uint32_t)(MT * p.nph) * p.act_stride;
+            if (MT == 2 && p.nph == 1 && p.IT == 1 && p.tiles_per_img % 2 == 0 && 2 * p.TR + d.R - 1 <= 256) {
+                // two tiles that always follow one another in an image share a slab, and the rows between them
+                const uint32_t pitch = (uint32_t)(p.TR * p.Wp) * 128u;
+                q.NSL = 1; q.tile16 = pitch >> 4;
+                q.slab_rows = 2 * p.TR + d.R - 1;
+                q.slab_bytes = (uint32_t)q.slab_rows * p.Wp * 128u;
+                q.act_stride = q.a_stage_bytes = round_up(reach + pitch > q.slab_bytes ? reach + pitch : q.slab_bytes, 1024);
+            }
             // a weight stage holds two chunks of a 64-filter half (32 KB at nine taps, as one chunk of a
             // 128-filter half), one where the slabs leave no room for two such stages
             q.CPW = q.GH > 64 ? 1 : q.GH > 32 ? 2 : 4;
@@ -607,6 +624,15 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             q.SA = (p.nBlk >= 3 && 3u * q.a_stage_bytes + 4u * q.w_bytes <= avail) ? 3 : 2;
             q.SB = (int)((avail - (uint32_t)q.SA * q.a_stage_bytes) / q.w_bytes);
             if (q.SB > kMaxStages) q.SB = kMaxStages;
+            // Weights that stay: where a pair has several items, all of the same filters, and a whole item's weights fit beside two slab
+            // stages (three where there is room: the next items' slabs are then on their way).
+            const int w_stages = p.nCh / q.CPW;
+            q.resident = items > pairs && pairs % q.n_fsets == 0 && w_stages <= kMaxStages &&
+                         2u * q.a_stage_bytes + (uint32_t)w_stages * q.w_bytes <= avail;
+            if (q.resident) {
+                q.SB = w_stages;
+                q.SA = 3u * q.a_stage_bytes + (uint32_t)w_stages * q.w_bytes <= avail ? 3 : 2;
+            }
             if ((uint32_t)q.SA * q.a_stage_bytes + (uint32_t)q.SB * q.w_bytes >= (1u << 18)) continue;   // descriptor addresses are 14 bits of 16 bytes
             // An MMA of a pair takes the tensor pipe NT / 2 cycles, and its issuing thread 50 to 100.  The epilogue
             // of an item overlaps the next item's MMAs when two accumulators fit, and always costs once at the

@@ -54,3 +54,18 @@ def test_wide_form_is_chosen_and_agrees_with_the_shared_memory_form(kw, out_dtyp
     got, other = host(run_case(c, out_dtype=out_dtype)), host(run_case(c, path=6, out_dtype=out_dtype))
     # the same products summed in fp32 in another order, and at most one rounding to bf16 (2^-8 of a value) of each
     assert floored_rel_err(got, other) < (TOL_BF16 if out_dtype is None else 1e-3)
+
+
+@pytest.mark.parametrize("wide", [0, WIDE])
+@pytest.mark.parametrize("kw", [
+    dict(N=24, H=27, W=56, C=64, K=64, Mb=16, Nb=8, keep=3),                      # two tiles share a slab; the last row of an image's last tile is missing
+    dict(N=43, H=13, W=56, C=64, K=64, Mb=16, Nb=8, keep=9),                      # seven tiles per image: a slab each
+    dict(N=24, H=28, W=28, C=64, K=256, Mb=16, Nb=16, keep=3),                    # two sets of filters, a pair keeps one of them
+    dict(N=26, H=28, W=28, C=64, K=384, Mb=16, Nb=8, keep=2),                     # three sets, which do not divide the pairs: nothing stays
+    dict(N=75, H=14, W=14, C=256, K=128, Mb=16, Nb=8, keep=2),                    # weights that do not fit
+])
+def test_several_items_per_pair(kw, wide):
+    c = inputs.conv_case(dtype="bf16", residual=True, seed=312, **kw)
+    y = run_case(c, path=7, variant=wide)
+    assert floored_rel_err(host(y), oracle_case(c)) < TOL_BF16
+    assert torch.equal(y, run_case(c, path=7, variant=wide))
