@@ -270,23 +270,20 @@ conv_bp_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDnParams
                 }
                 if (res) {
                     if (p.y_bf16) {
-                        const uint4 *rp = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0);
+                        uint32_t wv[8];
+                        ld_sector(wv, static_cast<const uint16_t *>(res) + o0);
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const uint4 u = __ldg(rp + h);
-                            const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                v[8 * h + 2 * i] += __uint_as_float(wv[i] << 16);
-                                v[8 * h + 2 * i + 1] += __uint_as_float(wv[i] & 0xFFFF0000u);
-                            }
+                        for (int i = 0; i < 8; ++i) {
+                            v[2 * i] += __uint_as_float(wv[i] << 16);
+                            v[2 * i + 1] += __uint_as_float(wv[i] & 0xFFFF0000u);
                         }
                     } else {
-                        const float4 *rp = reinterpret_cast<const float4 *>(static_cast<const float *>(res) + o0);
 #pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            const float4 u = __ldg(rp + h);
-                            v[4 * h] += u.x; v[4 * h + 1] += u.y; v[4 * h + 2] += u.z; v[4 * h + 3] += u.w;
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t wv[8];
+                            ld_sector(wv, static_cast<const float *>(res) + o0 + 8 * h);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) v[8 * h + i] += __uint_as_float(wv[i]);
                         }
                     }
                 }
@@ -299,17 +296,19 @@ conv_bp_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDnParams
 #pragma unroll
                         for (int i = 0; i < 8; ++i) o[i] = relu_bf16x2(o[i]);
                     }
-                    uint4 *yp = reinterpret_cast<uint4 *>(static_cast<uint16_t *>(y) + o0);
-                    yp[0] = make_uint4(o[0], o[1], o[2], o[3]);
-                    yp[1] = make_uint4(o[4], o[5], o[6], o[7]);
+                    st_sector(static_cast<uint16_t *>(y) + o0, o);
                 } else {
                     if (p.relu) {
 #pragma unroll
                         for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i], 0.f);
                     }
-                    float4 *yp = reinterpret_cast<float4 *>(static_cast<float *>(y) + o0);
 #pragma unroll
-                    for (int h = 0; h < 4; ++h) yp[h] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t o[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(v[8 * h + i]);
+                        st_sector(static_cast<float *>(y) + o0 + 8 * h, o);
+                    }
                 }
             };
 

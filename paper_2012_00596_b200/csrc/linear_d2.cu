@@ -340,23 +340,20 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 }
                 if (res) {
                     if (p.y_bf16) {
-                        const uint4 *rp = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(res) + o0 + c0);
+                        uint32_t wv[8];
+                        ld_sector(wv, static_cast<const uint16_t *>(res) + o0 + c0);
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const uint4 u = __ldg(rp + h);
-                            const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                v[8 * h + 2 * i] += __uint_as_float(wv[i] << 16);
-                                v[8 * h + 2 * i + 1] += __uint_as_float(wv[i] & 0xFFFF0000u);
-                            }
+                        for (int i = 0; i < 8; ++i) {
+                            v[2 * i] += __uint_as_float(wv[i] << 16);
+                            v[2 * i + 1] += __uint_as_float(wv[i] & 0xFFFF0000u);
                         }
                     } else {
-                        const float4 *rp = reinterpret_cast<const float4 *>(static_cast<const float *>(res) + o0 + c0);
 #pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            const float4 u = __ldg(rp + h);
-                            v[4 * h] += u.x; v[4 * h + 1] += u.y; v[4 * h + 2] += u.z; v[4 * h + 3] += u.w;
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t wv[8];
+                            ld_sector(wv, static_cast<const float *>(res) + o0 + c0 + 8 * h);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) v[8 * h + i] += __uint_as_float(wv[i]);
                         }
                     }
                 }
@@ -365,13 +362,18 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i], 0.f);
                 }
                 if (p.y_bf16) {
-                    uint4 *yp = reinterpret_cast<uint4 *>(static_cast<uint16_t *>(y) + o0 + c0);
-                    yp[0] = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
-                    yp[1] = make_uint4(pack2(v[8], v[9]), pack2(v[10], v[11]), pack2(v[12], v[13]), pack2(v[14], v[15]));
-                } else {
-                    float4 *yp = reinterpret_cast<float4 *>(static_cast<float *>(y) + o0 + c0);
+                    uint32_t o[8];
 #pragma unroll
-                    for (int h = 0; h < 4; ++h) yp[h] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+                    for (int i = 0; i < 8; ++i) o[i] = pack2(v[2 * i], v[2 * i + 1]);
+                    st_sector(static_cast<uint16_t *>(y) + o0 + c0, o);
+                } else {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t o[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(v[8 * h + i]);
+                        st_sector(static_cast<float *>(y) + o0 + c0 + 8 * h, o);
+                    }
                 }
             };
 
