@@ -77,8 +77,8 @@ struct ConvD2Params {
 struct ConvD2Bars {
     uint64_t a_full[kMaxSlabStages], a_empty[kMaxSlabStages];     // slab ring
     uint64_t w_full[kMaxStages], w_empty[kMaxStages];             // weight ring
-    uint64_t acc_full[2], acc_empty[2];
-    uint64_t acc_done[2];                                         // peer only: its epilogue warps have read the accumulator
+    uint64_t acc_full[4], acc_empty[4];
+    uint64_t acc_done[4];                                         // peer only: its epilogue warps have read the accumulator
     uint32_t tmem_base;
     uint32_t abort_flag;
 };
@@ -151,7 +151,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         // the peer's single relayed arrival have come in.
         for (int s = 0; s < p.SA; ++s) { mbar_init(&bars->a_full[s], 1); mbar_init(&bars->a_empty[s], p.MT); }
         for (int s = 0; s < p.SB; ++s) { mbar_init(&bars->w_full[s], 1); mbar_init(&bars->w_empty[s], p.MT); }
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < 4; ++a) {
             mbar_init(&bars->acc_full[a], p.MT); mbar_init(&bars->acc_empty[a], kEpiWarps + 1); mbar_init(&bars->acc_done[a], kEpiWarps);
         }
         bars->abort_flag = 0;
@@ -319,7 +319,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 bool ok = true;
                 for (int item = pair; item < p.n_items && ok; item += n_pairs, ++it) {
                     const int fs = item % p.n_fsets;
-                    const uint32_t acc = p.nacc == 2 ? (it & 1u) : 0u, lap_acc = p.nacc == 2 ? (it >> 1) : it;
+                    const uint32_t acc = it & (uint32_t)(p.nacc - 1), lap_acc = p.nacc == 4 ? it >> 2 : p.nacc == 2 ? it >> 1 : it;
                     if (lap_acc >= 1 && !pair_wait<true>(&bars->acc_empty[acc], (lap_acc & 1u) ^ 1u, abort_flag, peer_abort, ws, 0x7200)) break;
                     tc_fence_after_sync();
                     const uint32_t d_tmem = tmem_base + acc * p.dcols + (uint32_t)mt * p.NT;
@@ -369,7 +369,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         bool ok = true;
         for (int item = pair; item < p.n_items && ok; item += n_pairs, ++it) {
             const int ts = item / p.n_fsets, fs = item - ts * p.n_fsets;
-            const uint32_t acc = p.nacc == 2 ? (it & 1u) : 0u, lap_acc = p.nacc == 2 ? (it >> 1) : it;
+            const uint32_t acc = it & (uint32_t)(p.nacc - 1), lap_acc = p.nacc == 4 ? it >> 2 : p.nacc == 2 ? it >> 1 : it;
             const int nch = p.MT * cpt;
             const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * p.dcols;
 
@@ -616,7 +616,9 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             q.w_bytes = (uint32_t)q.CPW * p.RS * 2u * q.GH * 16u;
             while (q.CPW > 1 && 2u * q.a_stage_bytes + 2u * q.w_bytes > avail) { q.CPW /= 2; q.w_bytes /= 2; }
             q.dcols = MT * NT;
-            q.nacc = 2 * q.dcols <= 512 ? 2 : 1;
+            // (an accumulator is handed back about as long after its item as the item itself took: with two, items of few MMAs waited for
+            // it: 64x56x56x64 -> 64 20.8 us with two and 18.5 with four, 28x28x64 -> 256 18.8 and 17.1)
+            q.nacc = 4 * q.dcols <= 512 ? 4 : 2 * q.dcols <= 512 ? 2 : 1;
             // two slab stages, the rest of shared memory for weight stages; a third slab stage if at least
             // four weight stages remain
             if (2u * q.a_stage_bytes + 2u * q.w_bytes > avail) continue;
@@ -641,10 +643,10 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             const double rounds = (double)((items + pairs - 1) / pairs);
             const double per_mma = NT / 2 > 70 ? NT / 2 : 70.;
             // (two position tiles have an issuing warp each; at 64 filters the pipe (32 cycles) keeps up with both:
-            // 56x56x64 -> 64, 23.7 us on two tiles per CTA against 26.5 on one)
+            // 56x56x64 -> 64, 18.5 us on two tiles per CTA against 22.3 on one)
             const double mma = (double)p.nCh * p.RS * (NT == 64 && MT == 2 ? per_mma : MT * per_mma);
             const double epi = (double)MT * NT * 16.;
-            const double cost = wide ? modelled(q, d, pairs) : (rounds * (mma + (q.nacc == 2 ? 0. : epi)) + epi + 6000.) * ((NT == 128 && MT == 1) ? 0.9 : 1.);
+            const double cost = wide ? modelled(q, d, pairs) : (rounds * (mma + (q.nacc >= 2 ? 0. : epi)) + epi + 6000.) * ((NT == 128 && MT == 1) ? 0.9 : 1.);
             if (!found || cost < best) { best = cost; p = q; found = true; }
         }
     }
@@ -721,7 +723,7 @@ double conv_dense_modelled(const npas_conv_desc &d, const npas_bp_desc &bp)
         const int per = d.K % 128 && p.nph == 1 ? 4 : 2;
         const long long items = (long long)((p.n_tiles + per - 1) / per) * (d.K / (d.K % 128 ? 64 : 128));
         const double r = (double)((items + pairs - 1) / pairs);
-        return 4.4 + r * (d.K % 128 ? 0.354 * taps * nCh + 0.37 : 0.306 * taps * nCh + 0.67) + 0.089 * mb;
+        return 4.4 + r * (d.K % 128 ? 0.354 * taps * nCh + 0.4 : 0.306 * taps * nCh + 0.25) + 0.07 * mb;
     }
     const int Wp = d.W + 2 * d.pad;
     if (Wp > 128) return 1e30;
