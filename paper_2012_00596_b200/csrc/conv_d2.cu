@@ -492,7 +492,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 
 int pairs_available() { return sm_count() / 2; }
 
-// Microseconds of a plan of the wide form, fitted to 427 measured points (59 random layers, every item shape; standard error 12 %,
+// Microseconds of a plan of the wide form, fitted to 420 measured points (59 random layers, every item shape; standard error 11 %,
 // the shape it picks within 2 % of the best one): an MMA takes the pipe NT / 2 cycles and its issuing thread 70 (two warps issue for two
 // position tiles), the epilogue's columns, what leaves for DRAM.
 double modelled(const ConvD2Params &p, const npas_conv_desc &d, int pairs)
@@ -500,7 +500,7 @@ double modelled(const ConvD2Params &p, const npas_conv_desc &d, int pairs)
     const double rounds = (double)((p.n_items + pairs - 1) / pairs);
     const double mma = p.MT == 2 ? (p.NT > 74 ? p.NT : 74.) : (p.NT > 140 ? p.NT / 2 : 70.);     // cycles per chunk and tap
     const double out_mb = 2e-6 * p.N * p.Po * p.Qo * p.K * (d.has_residual ? 2. : 1.) * (p.y_bf16 ? 1. : 2.);
-    return 4.6 + rounds * (p.nCh * p.RS * mma / 1900. + 0.0068 * p.NT * p.MT) + 0.23 * out_mb;
+    return 4.6 + rounds * (p.nCh * p.RS * mma / 1900. + 0.0044 * p.NT * p.MT) + 0.19 * out_mb;
 }
 
 // `wide`: channels and filters in multiples of 16, items of several of the image's groups (kWide).
@@ -687,8 +687,7 @@ double conv_d2_wide_modelled(const npas_conv_desc &d, const npas_bp_desc &bp)
 
 // By the models of the kernels: against the split form where that is what would run (its model is fitted to layers of a chain; a call by
 // itself takes 1 us more, the wait for the blob), else against independent CTAs.  On 70 random layers of 16 to 512 channels and
-// filters what is chosen is 2.6 % above the better measured one, and 1.42 times faster than without this form (one with 22x15x22x48 ->
-// 192, 10.7 against 9.9 us, lies on the wrong side).
+// filters what is chosen is 3 % above the better measured one in sum, and 1.45 times faster than without this form.
 bool conv_d2_wide_preferred(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     const double us = conv_d2_wide_modelled(d, bp), split = us < 1e9 ? conv_sk_modelled(d, bp) : 0.;
