@@ -332,6 +332,14 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                                 v[8 * h + 2 * i + 1] += __uint_as_float(wv[i] & 0xFFFF0000u);
                             }
                         }
+                    } else if (left >= 16) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t wv[8];
+                            ld_sector(wv, static_cast<const float *>(res) + o0 + c0 + 8 * h);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) v[8 * h + i] += __uint_as_float(wv[i]);
+                        }
                     } else {
                         const float4 *rp = reinterpret_cast<const float4 *>(static_cast<const float *>(res) + o0 + c0);
 #pragma unroll
@@ -350,6 +358,14 @@ linear_bb_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     uint4 *yp = reinterpret_cast<uint4 *>(static_cast<uint16_t *>(y) + o0 + c0);
                     yp[0] = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
                     if (left > 8) yp[1] = make_uint4(pack2(v[8], v[9]), pack2(v[10], v[11]), pack2(v[12], v[13]), pack2(v[14], v[15]));
+                } else if (left >= 16) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t o[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(v[8 * h + i]);
+                        st_sector(static_cast<float *>(y) + o0 + c0 + 8 * h, o);
+                    }
                 } else {
                     float4 *yp = reinterpret_cast<float4 *>(static_cast<float *>(y) + o0 + c0);
 #pragma unroll

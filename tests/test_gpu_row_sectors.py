@@ -31,11 +31,12 @@ def test_conv_outputs_off_a_sector(path, variant, out_dtype):
         assert torch.equal(y, want), (y_off, r_off)
 
 
-def test_gemm_outputs_off_a_sector():
+@pytest.mark.parametrize("path", [5, 6])
+def test_gemm_outputs_off_a_sector(path):
     c = inputs.config3(M=300)
     x, blob, bias = dev(c.x, "bf16"), npas.pack_bb(dev(c.w, "bf16"), c.row_keep, c.col_keep, 64, 64), dev(c.bias)
     res = torch.randn((300, c.w.shape[0]), device="cuda")
-    kw = dict(relu=True, out_dtype=torch.float32, path=6)
+    kw = dict(relu=True, out_dtype=torch.float32, path=path)
     want = npas.linear_bb(x, blob, bias, res, **kw)
     for y_off, r_off in ((16, 0), (0, 16), (16, 16)):
         y = _at(torch.zeros_like(want), y_off)
