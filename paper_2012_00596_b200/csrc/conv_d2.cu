@@ -257,7 +257,6 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         // One holding several groups (K off the multiples of 64, or 64 that fill no 128) has a map over (128 bytes, lines of
         // a group's row, groups, rows of all (chunk, tap, octet)): ONE box puts the groups of every row next to one another,
         // groups past the last one as zeros.
-        const int rows_st = 2 * p.RS * p.CPW;                 // weight rows (chunk, tap, octet) of a stage
         const uint32_t copy_bytes = p.w_box_rows * 128u;      // 128 filters: one copy = one box of the weight map
         const bool runs = p.GH == 128 && !p.gathered;
         const int n_copies = runs ? (int)(p.w_bytes / copy_bytes) : 1;
@@ -269,7 +268,8 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             const int fs = item % p.n_fsets;
             const int f0 = fs * p.NT + (int)rank * p.GH;      // first filter of this CTA's half
             const uint32_t wsrc = image_row0 + (uint32_t)(((size_t)(f0 / p.GI) * p.nCh * (2u * p.RS * grow) + (size_t)(f0 % p.GI) * 16u) >> 7);
-            for (int wst = 0; wst < p.nCh / p.CPW; ++wst, ++n) {
+            for (int c0 = 0; c0 < p.nCh; c0 += p.CPW, ++n) {
+                const int chunk = min(c0, p.nCh - p.CPW);     // a last stage of fewer chunks starts early: no row past the group's
                 const uint32_t s = n % (uint32_t)p.SB, k = n / (uint32_t)p.SB;
                 if (lane == 0) {
                     if (k >= 1 && !pair_wait(&bars->w_empty[s], (k - 1u) & 1u, abort_flag, peer_abort, ws, 0x7120)) ok = false;
@@ -278,11 +278,11 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
                 if (!ok) break;
                 uint8_t *wdst = smem + p.off_w + (size_t)s * p.w_bytes;
-                const uint32_t src = wsrc + (uint32_t)wst * (uint32_t)rows_st * (grow >> 7);     // rows of the image, in 128-byte map rows
+                const uint32_t src = wsrc + (uint32_t)(chunk * 2 * p.RS) * (grow >> 7);     // rows of the image, in 128-byte map rows
                 if (p.gathered) {
                     if (lane == 0)
                         tma_load_4d_pair(wdst, &tmap_w, w_full0 + s * 8u, 0, 0, fs * (p.NT / p.GI) + (int)rank * p.GG,
-                                         (int)(off_image / grow) + wst * rows_st);
+                                         (int)(off_image / grow) + chunk * 2 * p.RS);
                 } else if (runs) {
                     for (int i = lane; i < n_copies; i += 32)
                         tma_load_2d_pair(wdst + (size_t)i * copy_bytes, &tmap_w, w_full0 + s * 8u, 0, (int)(src + (uint32_t)i * p.w_box_rows));
@@ -335,7 +335,8 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                             if (!pair_wait(&bars->w_full[sb], p.resident ? 0u : phb, abort_flag, peer_abort, ws, 0x7320)) { ok = false; break; }
                             tc_fence_after_sync();
                             uint32_t b_lo = b_st;
-                            for (int cc = 0; cc < p.CPW; ++cc, ++ch, a16 += 2u, b_lo += chunk16) {
+                            if (ch + p.CPW > p.nCh) b_lo += (uint32_t)(ch + p.CPW - p.nCh) * chunk16;
+                            for (int cc = 0; cc < p.CPW && ch < end; ++cc, ++ch, a16 += 2u, b_lo += chunk16) {
                                 // a tap that no block of these (groups, chunk) keeps multiplies zeros: skipped, except
                                 // the very first MMA, which initialises the accumulator
                                 const uint32_t m = tu[ch] | (ch == 0 ? 1u : 0u);
@@ -611,8 +612,10 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             }
             // a weight stage holds two chunks of a 64-filter half (32 KB at nine taps, as one chunk of a
             // 128-filter half), one where the slabs leave no room for two such stages
+            // (whatever divides the chunks: a wait and a commit per chunk of nine MMAs made an odd number of chunks a third slower,
+            // 37x8x16x368 -> 80 15.6 us on stages of one chunk and 10.5, 3x42x51x240 -> 96 11.7 and 8.7)
             q.CPW = q.GH > 64 ? 1 : q.GH > 32 ? 2 : 4;
-            while (q.CPW > 1 && p.nCh % q.CPW) q.CPW /= 2;
+            while (q.CPW > p.nCh) q.CPW /= 2;
             q.w_bytes = (uint32_t)q.CPW * p.RS * 2u * q.GH * 16u;
             while (q.CPW > 1 && 2u * q.a_stage_bytes + 2u * q.w_bytes > avail) { q.CPW /= 2; q.w_bytes /= 2; }
             q.dcols = MT * NT;
@@ -627,7 +630,7 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             if (q.SB > kMaxStages) q.SB = kMaxStages;
             // Weights that stay: where a pair has several items, all of the same filters, and a whole item's weights fit beside two slab
             // stages (three where there is room: the next items' slabs are then on their way).
-            const int w_stages = p.nCh / q.CPW;
+            const int w_stages = (p.nCh + q.CPW - 1) / q.CPW;
             q.resident = items > pairs && pairs % q.n_fsets == 0 && w_stages <= kMaxStages &&
                          2u * q.a_stage_bytes + (uint32_t)w_stages * q.w_bytes <= avail;
             if (q.resident) {
