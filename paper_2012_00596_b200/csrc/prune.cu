@@ -6,6 +6,7 @@
 // highest-scoring groups, ties go to the lower index.  Offline step: one CTA per block for the per-block counts; for the
 // layer-wide budget a thread per group scores and a cluster selects.
 #include "common.cuh"
+#include "select_range.h"
 #include "tc_common.cuh"
 
 namespace npas {
@@ -182,7 +183,7 @@ prune_bp_scores_kernel(npas_bp_desc d, const T *__restrict__ w, double *scores)
 constexpr int kSelThreads = 256;
 constexpr uint32_t kSelSmemKeys = 24576;                        // 192 KB of keys per CTA
 constexpr uint32_t kSelRank = 512;                              // keys that are ranked directly
-constexpr int kSelBins = 4 * kSelThreads;                       // four neighbouring bins per thread
+static_assert(kSelBins == 4 * kSelThreads, "four neighbouring bins per thread");
 constexpr int kSelBatch = 10;                                   // keys of a thread whose loads are in flight together
 
 struct SelShared {
@@ -210,7 +211,6 @@ __device__ __forceinline__ uint4 sel_remote(const void *p, unsigned int rank)
     asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(sel_peer(p, rank)) : "memory");
     return v;
 }
-__device__ __forceinline__ int sel_bits(unsigned long long v) { return v ? 64 - __clzll((long long)v) : 0; }
 
 __global__ void __launch_bounds__(kSelThreads)
 prune_select_kernel(const unsigned long long *__restrict__ keys, long long n_keep, int RS, unsigned long long *tap_mask,
@@ -255,19 +255,20 @@ prune_select_kernel(const unsigned long long *__restrict__ keys, long long n_kee
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < kSelThreads / 32; ++i) { base = min(base, sh.warp_lo[i]); top = max(top, sh.warp_hi[i]); }
-    int shift = max(0, sel_bits(top - base) - 10);
-    if ((top - base) >> shift > kSelBins - 3) ++shift;
+    int shift = sel_first_shift(base, top);
 
     // the budget left, `need`, falls among the `have` keys in [lo, hi], of which CTAs of lower rank hold `before`
-    unsigned long long lo = 0, hi = ~0ull;
+    // (how many passes that takes at most is a property of the ranges alone, select_range.h; were a budget to fall among no keys, which
+    // takes scores that change under the kernel, the search would end there)
+    uint64_t lo = 0, hi = ~0ull;
     unsigned int need = (unsigned int)n_keep, have = (unsigned int)total, before = first;
-    for (int pass = 0; need != have && have > kSelRank && lo != hi; ++pass) {
+    for (int pass = 0; pass < kSelPasses && need != have && have > kSelRank && lo != hi; ++pass) {
         unsigned int *hist = sh.hist[pass & 1];
         if (pass == 0)
-            each([&](unsigned long long k, long long) { atomicAdd(&hist[k < base ? 0u : 1u + (unsigned int)min((unsigned long long)kSelBins - 2, (k - base) >> shift)], 1u); });
+            each([&](unsigned long long k, long long) { atomicAdd(&hist[sel_first_bin(k, base, shift)], 1u); });
         else {
-            shift = max(0, sel_bits(hi - lo) - 10);
-            each([&](unsigned long long k, long long) { if (k >= lo && k <= hi) atomicAdd(&hist[(unsigned int)((k - lo) >> shift)], 1u); });
+            shift = sel_shift(hi - lo);
+            each([&](unsigned long long k, long long) { if (k >= lo && k <= hi) atomicAdd(&hist[sel_bin(k, lo, shift)], 1u); });
         }
         sel_cluster_sync();
         {
@@ -286,6 +287,7 @@ prune_select_kernel(const unsigned long long *__restrict__ keys, long long n_kee
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) { const unsigned int v = __shfl_up_sync(0xFFFFFFFFu, up, d); if (lane >= d) up += v; }
             if (lane == 31) sh.warp_sums[wid] = up;
+            if (t == 0) sh.pick_have = 0;
             __syncthreads();
 #pragma unroll
             for (int i = 0; i < kSelThreads / 32; ++i) up += i < wid ? sh.warp_sums[i] : 0u;
@@ -299,18 +301,12 @@ prune_select_kernel(const unsigned long long *__restrict__ keys, long long n_kee
             *reinterpret_cast<uint4 *>(&sh.hist[(pass + 1) & 1][4 * t]) = zero4;      // (every CTA has read the counts of the pass before)
         }
         __syncthreads();
-        const unsigned long long bin = sh.pick_bin;
-        need -= sh.pick_above;
         have = sh.pick_have;
+        if (have == 0) { need = 0; break; }               // (every CTA has the same counts)
+        need -= sh.pick_above;
         before = sh.pick_before;
-        if (pass == 0) {
-            lo = bin == 0 ? 0 : base + ((bin - 1) << shift);
-            if (bin < kSelBins - 1) hi = base + (bin << shift) - 1;
-            if (hi < lo) hi = ~0ull;                  // (scores that are no numbers may wrap around)
-        } else {
-            lo += bin << shift;
-            hi = min(hi, lo + ((1ull << shift) - 1));
-        }
+        if (pass == 0) sel_first_range(sh.pick_bin, base, shift, lo, hi);
+        else sel_range(sh.pick_bin, shift, lo, hi);
         __syncthreads();
     }
     const bool all = need == have, ranked = !all && have <= kSelRank;

@@ -1,12 +1,14 @@
 """One-shot magnitude pruning on the GPU: masks bit-identical to the oracle's (both sides decide on fp64
 sums of exact squares taken in the same order), and the pruned layer runs through pack + kernel."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
 
 import oracle
 import paper_2012_00596_b200 as npas
-from paper_2012_00596_b200 import inputs
+from paper_2012_00596_b200 import binding as B, inputs
 from util import TOL_BF16, dev, floored_rel_err, host
 
 pytestmark = pytest.mark.gpu
@@ -129,6 +131,28 @@ def test_prune_bp_global_of_uneven_scores(K, C, kind):
     for n_keep in (1, G // 3, G // 2 + 1, G - 1, G):
         tm = npas.prune_bp_magnitude_global(dev(w), 4, 4, n_keep=n_keep)
         assert np.array_equal(to_u64(tm), oracle.prune_bp_global(w, Mb=4, Nb=4, n_keep=n_keep)), n_keep
+
+
+@pytest.mark.parametrize("bits", [0xFFFFFFFF, 0xFFC00000, 0x7FC00000, 0x7F800000])
+@pytest.mark.parametrize("K,C,block", [(128, 128, 4), (256, 256, 1)])        # keys in shared memory; more than fit there
+def test_prune_bp_global_of_scores_that_are_no_numbers(K, C, block, bits):
+    """Weights whose squares sum to no number (or to infinity) in most groups, with the budget falling among them: the sets are those
+    of the score bits in descending order, ties to the lower index.  The scores are read back from the call's workspace."""
+    rng = inputs.rng_for(906)
+    w = rng.standard_normal((K, 9, C), dtype=np.float32)
+    w.view(np.uint32)[rng.random(w.shape) < (0.1 if block > 1 else 0.7)] = bits
+    lib, G = npas.load(), (K // block) * (C // block) * 9
+    x, d = dev(w.reshape(K, 3, 3, C)), B.BpDesc(K, C, 3, 3, block, block, B.F32, B.F32)
+    assert np.array_equal(x.cpu().numpy().view(np.uint32), w.view(np.uint32).reshape(x.shape))
+    ws = torch.zeros(G * 8 + 256, dtype=torch.uint8, device="cuda")
+    for n_keep in (1, 600, G // 4, G // 2, G - 1):
+        tm = torch.zeros((K // block, C // block), dtype=torch.int64, device="cuda")
+        assert lib.npas_prune_bp_magnitude_global(ctypes.byref(d), B._p(x), ctypes.c_int64(n_keep), B._p(tm), B._p(ws), ctypes.c_size_t(ws.numel()), B._stream()) == 0
+        keys = ws.cpu().numpy()[: G * 8].view(np.uint64)
+        assert (keys >= np.uint64(0x7FF0000000000000)).sum() > G // 3
+        kept = np.zeros(G, dtype=np.uint64)
+        kept[np.argsort(~keys, kind="stable")[:n_keep]] = 1
+        assert np.array_equal(to_u64(tm).ravel(), (kept.reshape(-1, 9) << np.arange(9, dtype=np.uint64)).sum(axis=1).astype(np.uint64)), n_keep
 
 
 @pytest.mark.parametrize("rate,Mb,Nb", [(2.5, 16, 8), (7.0, 16, 16)])
