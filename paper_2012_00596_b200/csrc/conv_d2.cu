@@ -38,6 +38,7 @@
 #include <cstdlib>
 
 #include "common.cuh"
+#include "internal_api.h"
 #include "tc_pair.cuh"
 
 namespace npas {
@@ -585,6 +586,7 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
     const int want_nt = d.variant & 0xFFFF, want_mt = (d.variant & ~(wide ? kWide : 0)) >> 16;
     double best = 0.;
     bool found = false;
+    ConvD2Params chosen;                                  // (`p` stays the geometry that every combination starts from)
     for (int NT = 256; NT >= 32; NT -= 32) {
         // an item is one or two groups of the image (with groups of 64 filters: one), or in the wide form every CTA of the pair
         // holds the same number of whole groups
@@ -650,10 +652,11 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             const double mma = (double)p.nCh * p.RS * (NT == 64 && MT == 2 ? per_mma : MT * per_mma);
             const double epi = (double)MT * NT * 16.;
             const double cost = wide ? modelled(q, d, pairs) : (rounds * (mma + (q.nacc >= 2 ? 0. : epi)) + epi + 6000.) * ((NT == 128 && MT == 1) ? 0.9 : 1.);
-            if (!found || cost < best) { best = cost; p = q; found = true; }
+            if (!found || cost < best) { best = cost; chosen = q; found = true; }
         }
     }
     if (!found) return false;
+    p = chosen;
     p.off_w = (uint32_t)p.SA * p.a_stage_bytes;
     p.off_tapu = p.off_w + (uint32_t)p.SB * p.w_bytes;
     p.off_bias = p.off_tapu + round_up((uint32_t)(d.K / p.GI) * p.nCh * 4u, 128);
@@ -810,3 +813,13 @@ npas_status conv_d2_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
 }
 
 }  // namespace npas
+
+extern "C" npas_status npas_internal_conv_d2_plan(const npas_conv_desc *d, const npas_bp_desc *bp, int32_t shape[8])
+{
+    npas::ConvD2Params p;
+    if (!d || !bp || !shape) return NPAS_ERR_NULL;
+    if (!npas::planned(*d, *bp, p, (d->variant & npas::kWide) != 0)) return NPAS_ERR_UNSUPPORTED;
+    const int32_t v[8] = {p.NT, p.MT, p.slab_rows, (int32_t)p.a_stage_bytes, (int32_t)p.w_bytes, p.SA, p.SB, (int32_t)p.smem_bytes};
+    for (int i = 0; i < 8; ++i) shape[i] = v[i];
+    return NPAS_OK;
+}

@@ -1,4 +1,7 @@
 """Host-only checks of the kernel choice: the committed (case, path) table and the plan cache."""
+import ctypes
+import random
+
 import pytest
 
 import paper_2012_00596_b200 as npas
@@ -85,6 +88,33 @@ def test_sweep_shape_choices():
         assert _conv_query(kw, 7, nt | (mt << 16)) == 7
     with pytest.raises(npas.NpasError):
         _conv_query(kw, 7, 64 | (1 << 16))
+
+
+def _pair_plan(N, H, W, C, K, R, stride, pad, Nb, variant):
+    d = B.ConvDesc(N, H, W, C, K, R, R, stride, pad, B.BF16, B.BF16, 1, 1, 0, 7, variant)
+    shape = (ctypes.c_int32 * 8)()
+    s = npas.load().npas_internal_conv_d2_plan(ctypes.byref(d), ctypes.byref(B.BpDesc(K, C, R, R, 16, Nb, B.BF16, B.BF16, 0)), shape)
+    assert s in (0, UNSUPPORTED)
+    return list(shape) if s == 0 else None
+
+
+@pytest.mark.parametrize("wide", [0, 1 << 24])
+def test_plan_of_the_pair_kernel_is_that_of_its_shape_alone(wide):
+    """The item shape the planner picks among all is planned as when it is the only one allowed: no candidate leaves anything behind for
+    the ones after it (slabs of two tiles had left their rows and strides to shapes of one tile)."""
+    rng = random.Random(17)
+    layers = [(30, 11, 43, 16, 368, 1, 1, 0)]
+    while len(layers) < 4000:
+        R = rng.choice([1, 1, 3, 3, 4])
+        layers.append((rng.randint(1, 64), rng.randint(3, 64), rng.randint(3, 100), 16 * rng.randint(1, 32), 16 * rng.randint(1, 32), R, rng.choice([1, 1, 2]),
+                       rng.randint(0, R // 2)))
+    planned = 0
+    for lay in layers:
+        free = _pair_plan(*lay, 8, wide)
+        if free is not None:
+            planned += 1
+            assert free == _pair_plan(*lay, 8, wide | free[0] | (free[1] << 16)), lay
+    assert planned > (1500 if wide else 60)
 
 
 def test_plan_cache_round_trip_and_rejects_garbage():
