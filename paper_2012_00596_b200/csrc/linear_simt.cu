@@ -399,7 +399,7 @@ linear_bb_rows_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinRowsPla
     }
     __syncthreads();
     // the warps' sums in order, bias, residual, ReLU, one rounding; consecutive threads along the row of Y
-    for (int e = t; e < outs * rows_here; e += nt) {
+    for (int e = t + tc::zero_behind_wait(); e < outs * rows_here; e += nt) {
         const int m = e / outs, r = e - m * outs;
         const size_t o = (size_t)(m0 + m) * d.O + (size_t)bo0 * Bo + r;
         double v = acc0[r * kAccPitch + m];

@@ -84,6 +84,38 @@ def test_linear_after_a_copy_into_its_blob(name):
     npas.check_device_status(ws)
 
 
+@pytest.mark.parametrize("Bo", [16, 64])                   # a warp per block; warps that share a block
+def test_linear_f32_after_the_kernels_that_write_its_bias_and_residual(Bo):
+    """Both are results of the library's own kernels just ahead, which let their successors start before they have written anything."""
+    M, I, O = 1000, 512, 512
+    c = inputs.linear_case(M=M, I=I, O=O, Bo=Bo, Bi=64, keep_rows=Bo // 2, keep_cols=32, dtype="f32", seed=1506)
+    blob, ws = npas.pack_bb(dev(c.w), c.row_keep, c.col_keep, Bo, 64), npas.workspace()
+    x, others, heads = dev(c.x), [dev(c.x[::-1]), dev(c.x) * 3], [dev(c.x[:1]), dev(c.x[1:2])]
+    bias, res = torch.empty((1, O), device="cuda"), torch.empty((M, O), device="cuda")
+
+    def call(i, b, r):
+        npas.linear_bb(others[i], blob, out=r, ws=ws)
+        npas.linear_bb(heads[i], blob, out=b, ws=ws)
+        return npas.linear_bb(x, blob, b.view(O), r, ws=ws)
+
+    want = []
+    for i in range(2):
+        b, r = torch.empty_like(bias), torch.empty_like(res)
+        npas.linear_bb(others[i], blob, out=r, ws=ws)
+        npas.linear_bb(heads[i], blob, out=b, ws=ws)
+        torch.cuda.synchronize()
+        want.append(npas.linear_bb(x, blob, b.view(O), r, ws=ws))
+    assert not torch.equal(want[0], want[1])
+    g, out = _captured(lambda: [call(i % 2, bias, res) for i in range(12)])
+    for _ in range(5):
+        for o in out:
+            o.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(o, want[i % 2]) for i, o in enumerate(out))
+    npas.check_device_status(ws)
+
+
 def test_pack_then_convolve_in_one_graph():
     """The packers' two kernels and the convolution on what they write; the scan lets its successor start early."""
     lib = npas.load()
