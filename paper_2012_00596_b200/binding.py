@@ -430,6 +430,27 @@ def tune_linear_bb(x: torch.Tensor, blob: BbBlob, bias=None, residual=None, *, r
     return path.value, variant.value, us.value
 
 
+def tune_linear_two(x: torch.Tensor, blob1: BbBlob, bias1, residual, blob2: BbBlob, bias2, *, relu, plans=((0, 0), (0, 0)), ws=None, reps=10):
+    """Two GEMMs behind one another, the second on the first one's result: measures them as one launch and one by one on their
+    ``plans``.  (True where one launch is the faster way, microseconds of the faster way), or None where there is no such launch."""
+    lib = load()
+    M, I = x.shape
+    d1, d2 = blob1.desc, blob2.desc
+    a = LinearDesc(M, I, d1.O, BF16, BF16, int(bool(relu[0])), int(bias1 is not None), int(residual is not None), *plans[0])
+    b = LinearDesc(M, d1.O, d2.O, BF16, BF16, int(bool(relu[1])), int(bias2 is not None), 0, *plans[1])
+    if ws is None:
+        ws = workspace(x.device)
+    y1, y2 = (torch.empty((M, d.O), dtype=torch.bfloat16, device=x.device) for d in (d1, d2))
+    together, us = ctypes.c_int32(0), ctypes.c_float(0)
+    code = lib.npas_internal_tune_linear_two(ctypes.byref(a), ctypes.byref(d1), ctypes.byref(b), ctypes.byref(d2), _p(x), _p(blob1.data), _p(bias1), _p(residual),
+                                             _p(y1), _p(blob2.data), _p(bias2), _p(y2), _p(ws), ctypes.c_size_t(ws.numel()), int(reps), ctypes.byref(together),
+                                             ctypes.byref(us), _stream())
+    if code == 8:                                # NPAS_ERR_UNSUPPORTED
+        return None
+    _check(code, "npas_internal_tune_linear_two")
+    return bool(together.value), us.value
+
+
 class PlanCache:
     """Tuned (path, variant) pairs keyed by what the choice depends on: the call geometry, the block
     sizes and the mask statistic the kernels plan with (largest kept count of a block).  Plain JSON on
@@ -448,6 +469,11 @@ class PlanCache:
     def linear_key(M, blob: BbBlob, relu, has_bias, has_residual) -> str:
         d = blob.desc
         return "linear:" + ",".join(str(int(v)) for v in (M, d.I, d.O, d.Bo, d.Bi, d.max_cols, relu, has_bias, has_residual))
+
+    @staticmethod
+    def two_key(first: str, second: str) -> str:
+        """Two GEMMs behind one another, by their own keys; the plan is (2, 0) in one launch, (1, 0) one by one."""
+        return f"two:{first}|{second}"
 
     def get(self, key: str):
         v = self.plans.get(key)

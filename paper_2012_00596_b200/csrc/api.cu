@@ -514,6 +514,38 @@ npas_status npas_tune_linear_bb(const npas_linear_desc *d, const npas_bb_desc *b
     return tune(cands, run, reps, ws, static_cast<cudaStream_t>(stream), path_out, variant_out, us_out);
 }
 
+// One launch or two, each on the plan its descriptor names: the faster of three measurements of either, in turn.
+npas_status npas_internal_tune_linear_two(const npas_linear_desc *a, const npas_bb_desc *bba, const npas_linear_desc *b, const npas_bb_desc *bbb,
+                                          const void *x, const void *blob1, const float *bias1, const void *residual, void *y1, const void *blob2,
+                                          const float *bias2, void *y2, void *ws, size_t ws_bytes, int32_t reps, int32_t *together_out, float *us_out, void *stream)
+{
+    if (!a || !b || !together_out || !us_out) return NPAS_ERR_NULL;
+    if (reps < 1 || reps > 10000) return NPAS_ERR_SHAPE;
+    npas_linear_desc a0 = *a, b0 = *b;
+    a0.path = a0.variant = b0.path = b0.variant = 0;
+    if (!linear_two_preferred(a0, b0)) return NPAS_ERR_UNSUPPORTED;
+    Timer t;
+    if (!t.ok) return NPAS_ERR_CUDA;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    auto one = [&] {
+        return npas_internal_linear_two(&a0, bba, &b0, bbb, x, blob1, bias1, residual, y1, blob2, bias2, y2, ws, ws_bytes, NPAS_CHAIN_NONE, stream);
+    };
+    auto two = [&] {
+        const npas_status s = npas_linear_bb(a, bba, x, blob1, bias1, residual, y1, ws, ws_bytes, stream);
+        return s != NPAS_OK ? s : npas_linear_bb(b, bbb, y1, blob2, bias2, nullptr, y2, ws, ws_bytes, stream);
+    };
+    float us[2] = {-1.f, -1.f};
+    for (int round = 0; round < 3; ++round)
+        for (int i = 0; i < 2; ++i) {
+            const float u = i ? time_candidate(one, reps, ws, st, t) : time_candidate(two, reps, ws, st, t);
+            if (u >= 0.f && (us[i] < 0.f || u < us[i])) us[i] = u;
+        }
+    if (us[0] < 0.f && us[1] < 0.f) return NPAS_ERR_CUDA;
+    *together_out = us[0] < 0.f || (us[1] >= 0.f && us[1] < us[0]);
+    *us_out = us[*together_out];
+    return NPAS_OK;
+}
+
 npas_status npas_blob_check(const npas_bp_desc *bp, const npas_bb_desc *bb, const void *blob,
                             size_t blob_bytes, void *stream)
 {

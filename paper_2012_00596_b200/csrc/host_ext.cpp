@@ -600,6 +600,7 @@ private:
 };
 
 // One row of the topology: kind 0 first layer (followed by the max-pool), 1 convolution, 2 GEMM over the pixels.
+enum { kApart = 1, kTogether = 2 };
 struct LayerRow { int32_t kind, stride, pad, relu, cout, src, res, reserved; };
 
 // A second stream and the two events that tie it to the caller's, one set per thread (made for the device it last used, given
@@ -637,8 +638,10 @@ struct SideStream {
 };
 thread_local SideStream side;
 
-// stack_forward(x, rows, blobs, biases, ws, routes): rows = bytes of LayerRow; routes = None, or [path, variant] pairs as
-// a flat list.  src / res: index of a layer, -1 the network's input, -2 the pooled tensor, -3 (res only) none.
+// stack_forward(x, rows, blobs, biases, ws, routes): rows = bytes of LayerRow; routes = None, or [path, variant, with_next] of every
+// layer as a flat list.  src / res: index of a layer, -1 the network's input, -2 the pooled tensor, -3 (res only) none.
+// with_next: whether a layer and the one behind it were measured faster one by one (kApart) or in one launch (kTogether, whatever
+// their own plans); not measured (0), they share a launch where that is preferred and neither has a plan of its own.
 PyObject *stack_forward(PyObject *, PyObject *const *a, Py_ssize_t nargs)
 {
     return guarded([&]() -> PyObject * {
@@ -667,6 +670,8 @@ PyObject *stack_forward(PyObject *, PyObject *const *a, Py_ssize_t nargs)
                 if (s >= 0) last[(size_t)s] = i;
                 if (s == -2) pooled_last = i;
             }
+        if (a[5] != Py_None && (!PyList_Check(a[5]) || PyList_GET_SIZE(a[5]) != 3 * (Py_ssize_t)L)) { fail_assert("stack_forward: three numbers per layer in routes"); return nullptr; }
+        auto route = [&](int i, int which, int32_t &v) { return int_arg(PyList_GET_ITEM(a[5], 3 * i + which), v); };
         Shape pooled{0, 0, 0, -1};
         Arena arena;
         const int64_t N = x->size(0);
@@ -716,7 +721,7 @@ PyObject *stack_forward(PyObject *, PyObject *const *a, Py_ssize_t nargs)
             if (!tensor_arg(data, blob, false, "blob.data") || !tensor_arg(PyList_GET_ITEM(a[3], i), bias, false, "bias")) return nullptr;
             st.blob = blob->data_ptr(); st.bias = static_cast<const float *>(bias->data_ptr());
             int32_t path = 0, variant = 0;
-            if (a[5] != Py_None && (!int_arg(PyList_GetItem(a[5], 2 * i), path) || !int_arg(PyList_GetItem(a[5], 2 * i + 1), variant))) return nullptr;
+            if (a[5] != Py_None && (!route(i, 0, path) || !route(i, 1, variant))) return nullptr;
             const Shape in = r.src == -1 ? Shape{x->size(1), x->size(2), x->size(3), -1} : r.src == -2 ? pooled : made[(size_t)r.src];
             st.h = in.h; st.w = in.w; st.in_at = in.at;
             if (from[(size_t)i] < 0) st.sub = -1;
@@ -735,11 +740,17 @@ PyObject *stack_forward(PyObject *, PyObject *const *a, Py_ssize_t nargs)
                 if (r.kind == 0) { st.p = (st.p + 2 - 3) / 2 + 1; st.q = (st.q + 2 - 3) / 2 + 1; }      // the pooled tensor
             }
             if (from[(size_t)i] < 0) st.out = i == L - 1 ? -1 : arena.take(N * st.p * st.q * r.cout * 2);
-            if (r.kind == 2 && r.stride == 1 && from[(size_t)i] < 0 && i + 1 < L && a[5] == Py_None) {
+            if (i > 0 && two[(size_t)i - 1]) st.ld.path = st.ld.variant = 0;
+            else if (r.kind == 2 && r.stride == 1 && from[(size_t)i] < 0 && i + 1 < L) {
                 const LayerRow &t = rows[i + 1];
+                int32_t with_next = 0, path2 = 0, variant2 = 0;
+                if (a[5] != Py_None && (!route(i, 2, with_next) || !route(i + 1, 0, path2) || !route(i + 1, 1, variant2))) return nullptr;
+                npas_linear_desc one = st.ld;
+                one.path = one.variant = 0;
                 const npas_linear_desc b{st.ld.M, r.cout, t.cout, NPAS_BF16, NPAS_BF16, t.relu, 1, 0, 0, 0};
-                two[(size_t)i] = t.kind == 2 && t.stride == 1 && t.src == i && t.res == -3 && from[(size_t)i + 1] < 0 && begins[(size_t)i + 1] < 0 && (i == 0 || !two[(size_t)i - 1]) &&
-                                 npas_internal_linear_two_preferred(&st.ld, &b);
+                two[(size_t)i] = t.kind == 2 && t.stride == 1 && t.src == i && t.res == -3 && from[(size_t)i + 1] < 0 && begins[(size_t)i + 1] < 0 &&
+                                 (with_next == kTogether || (with_next == 0 && !path && !variant && !path2 && !variant2)) && npas_internal_linear_two_preferred(&one, &b);
+                if (two[(size_t)i]) st.ld = one;
             }
             made[(size_t)i] = Shape{st.p, st.q, r.cout, st.out};
             if (r.kind == 0) pooled = made[(size_t)i];

@@ -46,6 +46,11 @@ int32_t npas_internal_linear_two_preferred(const npas_linear_desc *a, const npas
 npas_status npas_internal_linear_two(const npas_linear_desc *a, const npas_bb_desc *bba, const npas_linear_desc *b, const npas_bb_desc *bbb,
                                      const void *x, const void *blob1, const float *bias1, const void *residual, void *y1, const void *blob2,
                                      const float *bias2, void *y2, void *ws, size_t ws_bytes, int32_t chain, void *stream);
+// Which of the two ways is the faster one on the caller's buffers, for layers whose descriptors name their own measured plans (like the
+// tuners in npas.h; not supported where the launch is not preferred): *together, and the microseconds of that way.
+npas_status npas_internal_tune_linear_two(const npas_linear_desc *a, const npas_bb_desc *bba, const npas_linear_desc *b, const npas_bb_desc *bbb,
+                                          const void *x, const void *blob1, const float *bias1, const void *residual, void *y1, const void *blob2,
+                                          const float *bias2, void *y2, void *ws, size_t ws_bytes, int32_t reps, int32_t *together, float *us, void *stream);
 // The plan of the pair convolution (path 7) for a call, as a forced `variant` restricts it: filters per item, position tiles per CTA,
 // rows of a slab, bytes of a slab stage and of a weight stage, stages of each, bytes of shared memory.
 npas_status npas_internal_conv_d2_plan(const npas_conv_desc *d, const npas_bp_desc *bp, int32_t shape[8]);

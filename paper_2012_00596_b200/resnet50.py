@@ -39,8 +39,9 @@ class Resnet50Stack:
 
     def tune(self, x: torch.Tensor, reps: int = 20) -> "npas.PlanCache":
         """One pass over the stack on input x in which every layer asks the library's tuner (it times each kernel
-        and tile shape that takes the layer, on the tensors the layer really sees) and keeps the answer; later
-        passes run every layer on its measured choice.  Returns the plan cache (JSON-serialisable)."""
+        and tile shape that takes the layer, on the tensors the layer really sees) and keeps the answer, and two 1x1
+        layers that may share a launch are timed that way too; later passes run everything on its measured choice.
+        Returns the plan cache (JSON-serialisable)."""
         self.plans = npas.PlanCache()
         self._tuning = int(reps)
         try:
@@ -76,17 +77,35 @@ class Resnet50Stack:
         return npas.conv2d_bp(x, self.blobs[i], self.biases[i], res, stride=lay.stride, pad=pad, relu=lay.relu,
                               out=out, ws=self.ws, path=pth, variant=var)
 
+    def _follows(self, i: int) -> bool:
+        """Whether layer i is a 1x1 layer that reads nothing but the 1x1 layer before it."""
+        a, b = self.layers[i - 1], self.layers[i]
+        return i > 0 and a.kind == b.kind == "pw" and a.stride == b.stride == 1 and b.src == i - 1 and b.res == -1
+
+    def _linear_key(self, i: int, M: int) -> str:
+        return npas.PlanCache.linear_key(M, self.blobs[i], self.layers[i].relu, True, self.layers[i].res != -1)
+
+    def _tune_two(self, i: int, x: torch.Tensor, res: torch.Tensor | None):
+        """Layer i, on input x and shortcut res, and the one behind it: as one launch or one by one."""
+        M = x.numel() // x.shape[3]
+        keys = [self._linear_key(j, M) for j in (i, i + 1)]
+        r = npas.tune_linear_two(x.view(M, x.shape[3]), self.blobs[i], self.biases[i], res, self.blobs[i + 1], self.biases[i + 1],
+                                 relu=(self.layers[i].relu, self.layers[i + 1].relu), plans=[self.plans.get(k) or (0, 0) for k in keys],
+                                 ws=self.ws, reps=self._tuning)
+        if r is not None:
+            self.plans.put(npas.PlanCache.two_key(*keys), 2 if r[0] else 1, 0, r[1])
+
     def _routes(self, x: torch.Tensor):
-        """Measured (kernel, tile shape) of every layer as a flat list, or None without measurements."""
+        """Measured (kernel, tile shape, with the next layer or not) of every layer as a flat list, or None without measurements."""
         if not self.plans.plans:
             return None
-        shapes, routes = {-1: tuple(x.shape)}, []
+        shapes, routes, keys = {-1: tuple(x.shape)}, [], []
         for i, lay in enumerate(self.layers):
             n, h, w, c = shapes[lay.src]
             has_res = lay.res != -1
             if lay.kind == "pw":
                 h, w = (h - 1) // lay.stride + 1, (w - 1) // lay.stride + 1
-                key = npas.PlanCache.linear_key(n * h * w, self.blobs[i], lay.relu, True, has_res)
+                key = self._linear_key(i, n * h * w)
             else:
                 pad, R = (3, 7) if lay.kind == "stem" else (1, 3)
                 key = npas.PlanCache.conv_key((n, h, w, c), self.blobs[i], lay.stride, pad, lay.relu, True, has_res)
@@ -94,9 +113,12 @@ class Resnet50Stack:
             shapes[i] = (n, h, w, lay.Cout)
             if lay.kind == "stem":
                 shapes[-2] = (n, (h - 1) // 2 + 1, (w - 1) // 2 + 1, lay.Cout)
-                routes += [0, 0]                       # (the fused first layer chooses its own kernel)
+                routes += [0, 0, 0]                    # (the fused first layer chooses its own kernel)
             else:
-                routes += self.plans.get(key) or (0, 0)
+                routes += [*(self.plans.get(key) or (0, 0)), 0]
+            keys.append(key)
+            if self._follows(i):
+                routes[3 * i - 1] = (self.plans.get(npas.PlanCache.two_key(*keys[-2:])) or (0, 0))[0]
         return routes
 
     def forward(self, x: torch.Tensor, keep: bool = False):
@@ -108,7 +130,7 @@ class Resnet50Stack:
             return y if type(y) is not tuple else npas._refused(y[0], f"layer {self.layers[y[1]].name}")
         last_use = {s: j for j, l in enumerate(self.layers) for s in (l.src, l.res)}
         outs: dict[int, torch.Tensor] = {}
-        seen = []
+        seen, before = [], (None, None)
         for i, lay in enumerate(self.layers):
             if lay.src == -1:
                 xin = x
@@ -124,6 +146,10 @@ class Resnet50Stack:
                 continue
             y = self.run_layer(i, xin, res)
             outs[i] = y
+            if self._tuning:
+                if self._follows(i):
+                    self._tune_two(i - 1, *before)
+                before = (xin, res)
             if keep:
                 seen.append((xin, res, y))
             if lay.kind == "stem":

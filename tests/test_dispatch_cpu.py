@@ -127,9 +127,10 @@ def test_plan_cache_round_trip_and_rejects_garbage():
                             False, False, False)                       # the mask statistic is part of the key
     c.put(k1, 7, 256 | (1 << 16), 155.25)
     c.put(k2, 6, 128, 11.5)
+    c.put(c.two_key(k2, k2), 2, 0, 20.0)
     text = c.to_json()
     d = npas.PlanCache.from_json(text)
-    assert d.get(k1) == (7, 256 | (1 << 16)) and d.get(k2) == (6, 128) and d.get("conv:other") is None
+    assert d.get(k1) == (7, 256 | (1 << 16)) and d.get(k2) == (6, 128) and d.get("conv:other") is None and d.get(d.two_key(k2, k2)) == (2, 0)
     assert d.to_json() == text
     for bad in ('{"version": 2, "plans": {}}', '{"plans": []}', '{"version": 1, "plans": {"k": [1, 2]}}'):
         with pytest.raises(ValueError):
