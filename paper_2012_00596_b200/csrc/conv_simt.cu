@@ -31,6 +31,16 @@ template <typename T> __device__ inline float load_as_f32(const T *p);
 template <> __device__ inline float load_as_f32<float>(const float *p) { return __ldg(p); }
 template <> __device__ inline float load_as_f32<uint16_t>(const uint16_t *p) { return bf16_bits_to_f32(__ldg(p)); }
 
+// Where a filter block's pairs begin or end.  Both forms read through the pointer the kernel was given, at an offset known behind the
+// wait only, and differ in nothing but where the compiler then places the kernel's loads: float32 layers are 2 to 4 % slower with __ldg
+// (32x56x56x20 -> 32 60.4 us against 57.9, 16x28x28x64 -> 64 with a residual 41.4 against 37.6), bf16 ones 0 to 6 % without
+// (16x14x14x36 -> 36 13.0 against 12.3).
+template <typename TX> __device__ __forceinline__ uint32_t pair_bound(const uint32_t *p)
+{
+    if constexpr (sizeof(TX) == 2) return __ldg(p);
+    else return *p;
+}
+
 template <typename T> __device__ inline void store_from_f32(T *p, float v);
 template <> __device__ inline void store_from_f32<float>(float *p, float v) { *p = v; }
 template <> __device__ inline void store_from_f32<uint16_t>(uint16_t *p, float v) { *p = f32_bits_to_bf16(__float_as_uint(v)); }
@@ -58,8 +68,8 @@ conv_bp_simt_kernel(npas_conv_desc d, int Mb, int Nb_, int P, int Q, int KW, con
 
     tc::pdl_trigger();
     tc::pdl_wait();
-    x = tc::behind_wait(x); blob = tc::behind_wait(blob); bias = tc::behind_wait(bias); res = tc::behind_wait(res);
-    const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
+    const int z = tc::zero_behind_wait();                                    // in the header's address, the bias', and every pixel number
+    const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob) + z;      // (lists and values lie at offsets that it holds)
     const uint32_t nCB = d.C / Nb, G = NB ? NB : (Nb % 8 == 0) ? 8 : Nb;
     const uint32_t *blk_off = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_BLK]);
     const uint32_t *pairs = reinterpret_cast<const uint32_t *>(blob + hdr[BP_OFF_PAIRS]);
@@ -67,7 +77,7 @@ conv_bp_simt_kernel(npas_conv_desc d, int Mb, int Nb_, int P, int Q, int KW, con
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, k = lane & 3, q8 = lane >> 2;
     const int kw = warp & (KW - 1), pt = warp / KW, fb = blockIdx.y, f0 = blockIdx.z * kFilters, nf = min(kFilters, Mb - f0);
-    const long long npix = (long long)d.N * P * Q, pix0 = (long long)blockIdx.x * (kPixels * (kWarps / KW));
+    const long long npix = (long long)d.N * P * Q, pix0 = (long long)blockIdx.x * (kPixels * (kWarps / KW)) + z;
 
     // this lane's four pixels (one of every group of eight): top-left input position and where it lies
     int h0[kPixels / 8], w0[kPixels / 8];
@@ -83,7 +93,7 @@ conv_bp_simt_kernel(npas_conv_desc d, int Mb, int Nb_, int P, int Q, int KW, con
         }
     }
     double acc[FG][kPixels / 8][2] = {};
-    const uint32_t j_begin = __ldg(blk_off + (size_t)fb * nCB), j_end = __ldg(blk_off + (size_t)(fb + 1) * nCB);
+    const uint32_t j_begin = pair_bound<TX>(blk_off + (size_t)fb * nCB), j_end = pair_bound<TX>(blk_off + (size_t)(fb + 1) * nCB);
     const uint32_t spp = (Nb + 3) / 4;                                   // matrix steps per pair
     const uint32_t s_all = (j_end - j_begin) * spp;
     const TX *wp = vals + ((size_t)j_begin * Nb * Mb + (f0 + q8) * G + k);
@@ -91,7 +101,7 @@ conv_bp_simt_kernel(npas_conv_desc d, int Mb, int Nb_, int P, int Q, int KW, con
         const int steps = (int)min((uint32_t)kMaxSteps, s_all - b0);
         if (b0) __syncthreads();
         for (int e = tid; e < steps; e += kWarps * 32) {
-            const uint32_t j = (b0 + e) / spp, c0 = (b0 + e - j * spp) * 4, pw = __ldg(pairs + j_begin + j), tap = pw >> 16, cb = pw & 0xFFFFu;
+            const uint32_t j = (b0 + e) / spp, c0 = (b0 + e - j * spp) * 4, pw = pairs[j_begin + j], tap = pw >> 16, cb = pw & 0xFFFFu;
             const uint32_t r = tap / d.S, sx = tap - r * d.S, wo = (j * (Nb / G) + c0 / G) * Mb * G + c0 % G;
             // (a pair outside the layer counts for nothing: its tap lies beside every image)
             step_s[e] = r < (uint32_t)d.R && cb < nCB ? make_uint4((r * d.W + sx) * d.C + cb * Nb + c0, r | (sx << 16), wo, Nb - c0)
@@ -134,7 +144,7 @@ conv_bp_simt_kernel(npas_conv_desc d, int Mb, int Nb_, int P, int Q, int KW, con
     // the shares in order, then bias, residual, ReLU, one rounding at the store
     const int f = tid & (kFilters - 1);
     if (f >= nf) return;
-    const double bv = bias ? (double)bias[fb * Mb + f0 + f] : 0.;
+    const double bv = bias ? (double)bias[fb * Mb + f0 + f + z] : 0.;
     for (int e = tid / kFilters; e < kPixels * (kWarps / KW); e += kWarps * 32 / kFilters) {
         const long long pix = pix0 + e;
         if (pix >= npix) return;

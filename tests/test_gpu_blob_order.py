@@ -116,6 +116,38 @@ def test_linear_f32_after_the_kernels_that_write_its_bias_and_residual(Bo):
     npas.check_device_status(ws)
 
 
+@pytest.mark.parametrize("path,dtype", [(1, "f32"), (1, "bf16"), (6, "bf16"), (7, "bf16"), (8, "bf16"), (0, "bf16")])
+def test_conv_after_the_kernels_that_write_its_input_and_residual(path, dtype):
+    """A chain of convolutions in which each reads two results of the ones just ahead; path 0 is the split form here."""
+    N, H, C = (1, 14, 256) if path == 0 else (2, 14, 64)
+    c = inputs.conv_case(N=N, H=H, W=H, C=C, K=C, Mb=16, Nb=16, keep=3, dtype=dtype, seed=1507)
+    blob, ws, xs = npas.pack_bp(dev(c.w, dtype), c.tap_mask, 16, 16), npas.workspace(), [dev(c.x, dtype), dev(c.x[:, ::-1], dtype)]
+    bufs = [torch.empty_like(xs[0]) for _ in range(3)]
+
+    def chain(wait):
+        out = []
+        for i in range(6):
+            r = xs[i % 2]
+            for j in range(3):                     # x -> a, (a, x) -> b, (b, a) -> c
+                src, res = (r, None) if j == 0 else (bufs[j - 1], r if j == 1 else bufs[j - 2])
+                npas.conv2d_bp(src, blob, None, res, relu=True, out=bufs[j], ws=ws, path=path)
+                wait()
+            out.append(npas.conv2d_bp(bufs[2], blob, None, bufs[1], relu=True, ws=ws, path=path))
+            wait()
+        return out
+
+    want = chain(torch.cuda.synchronize)
+    assert not torch.equal(want[0], want[1])
+    g, out = _captured(lambda: chain(lambda: None))
+    for _ in range(5):
+        for o in (*out, *bufs):
+            o.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(o, w) for o, w in zip(out, want))
+    npas.check_device_status(ws)
+
+
 def test_pack_then_convolve_in_one_graph():
     """The packers' two kernels and the convolution on what they write; the scan lets its successor start early."""
     lib = npas.load()
