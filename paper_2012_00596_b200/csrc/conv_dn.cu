@@ -89,8 +89,8 @@ conv_bp_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDnParams
     __syncthreads();
     tc_fence_after_sync();
     pdl_wait();                        // nothing above touches global memory
-    blob = behind_wait(blob); bias = behind_wait(bias); res = behind_wait(res);
-    const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob);
+    const int z = zero_behind_wait();
+    const uint32_t *hdr = reinterpret_cast<const uint32_t *>(blob) + z;
     const uint32_t tmem_base = bars->tmem_base;
     // Cold operands: the whole grid asks L2 for the operand image (one slice per CTA) and every CTA for the
     // input rows of its first item, so that DRAM latency is paid once, up front and in parallel, instead
@@ -118,7 +118,7 @@ conv_bp_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDnParams
     }
     // the producer starts at once; the other warps first stage the biases and the tap unions
     if (warp != 0) {
-        for (int i = tid - 32; i < p.K; i += kThreads - 32) bias_s[i] = bias ? __ldg(bias + i) : 0.f;
+        for (int i = tid - 32 + z; i < p.K; i += kThreads - 32) bias_s[i] = bias ? __ldg(bias + i) : 0.f;
         const uint32_t off_tapu = hdr[BP_OFF_TAPU];
         const uint32_t *tapu = reinterpret_cast<const uint32_t *>(blob + off_tapu);
         for (int i = tid - 32; i < (p.K / p.GI) * p.nCh; i += kThreads - 32) tapu_s[i] = off_tapu ? __ldg(tapu + i) : 0xFFFFFFFFu;
@@ -255,7 +255,7 @@ conv_bp_dn_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDnParams
                 }
                 if (!(mt ? val[1] : val[0])) return;
                 const int k0 = (gs * p.NG + g) * p.GI + c0;
-                const size_t o0 = (mt ? obase[1] : obase[0]) + k0;
+                const size_t o0 = (mt ? obase[1] : obase[0]) + (size_t)(k0 + z);
                 float v[16];
                 const float4 *b4 = reinterpret_cast<const float4 *>(bias_s + k0);
 #pragma unroll

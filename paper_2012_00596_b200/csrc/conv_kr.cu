@@ -323,8 +323,8 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         }
     }
     pdl_wait();
-    bias = behind_wait(bias); res = behind_wait(res);
-    for (int i = tid; i < p.GS * p.Mb; i += kThreads) bars->bias[i] = bias ? __ldg(bias + fb0 * p.Mb + i) : 0.f;
+    const int z = zero_behind_wait();
+    for (int i = tid + z; i < p.GS * p.Mb; i += kThreads) bars->bias[i] = bias ? __ldg(bias + fb0 * p.Mb + i) : 0.f;
     fence_proxy_async_smem();
     tc_fence_before_sync();
     __syncthreads();
@@ -547,7 +547,7 @@ conv_bp_kr_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             // fused epilogue: the warps that share a TMEM lane quarter split the filter columns
             const TileAt t = tile_at(p, tile);
             const bool valid = m < t.count;
-            const size_t o0 = ((size_t)t.first + m) * p.K + k0;
+            const size_t o0 = ((size_t)t.first + m) * p.K + (size_t)(k0 + z);
             const bool go = __all_sync(0xFFFFFFFFu, ok && mbar_wait(&bars->acc_full, it & 1, abort_flag, ws, 0x7700));    // (tcgen05.ld needs the whole warp)
             if (go) {
                 tc_fence_after_sync();

@@ -153,9 +153,9 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         __syncwarp();
     }
     pdl_wait();
-    bias = behind_wait(bias); res = behind_wait(res);
+    const int z = zero_behind_wait();
     if (warp > 2)
-        for (int i = tid - 96; i < p.NT; i += kThreads - 96) bias_s[i] = (bias && k0 + i < p.K) ? __ldg(bias + k0 + i) : 0.f;
+        for (int i = tid - 96 + z; i < p.NT; i += kThreads - 96) bias_s[i] = (bias && k0 + i < p.K) ? __ldg(bias + k0 + i) : 0.f;
 
     if (warp == 0) {
         // ---- slabs -----------------------------------------------------------------------------------------------
@@ -255,7 +255,7 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     for (int i = tid; i < p.rpr * oct; i += kThreads) {
         const int r = i / oct, c0 = (i - r * oct) * 8, m = rank * p.rpr + r, oy = m / p.Wp, ox = m - oy * p.Wp, yy = y0 + oy;
         if (m >= kRows || k0 + c0 >= p.K || oy >= p.TR || yy >= p.P || ox >= p.Q || ((yy | ox) & p.sh)) continue;
-        const size_t o0 = (((size_t)img * p.Po + (yy >> p.sh)) * p.Qo + (ox >> p.sh)) * p.K + k0 + c0;
+        const size_t o0 = (((size_t)img * p.Po + (yy >> p.sh)) * p.Qo + (ox >> p.sh)) * p.K + (size_t)(k0 + c0 + z);
         const uint8_t *src = smem + p.off_red + (size_t)r * p.red_pitch + (size_t)c0 * 4;
         float v[8];
 #pragma unroll

@@ -130,10 +130,12 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         }
     }
     pdl_wait();                        // nothing else above touches global memory
-    bias = behind_wait(bias); res = behind_wait(res);
+    const int z = zero_behind_wait();
     // the biases: staged by the epilogue warps, which meet again before the first use
     if (warp >= kFirstEpiWarp && warp < kResWarp) {
-        for (int i = tid - kFirstEpiWarp * 32; i < p.O; i += kEpiWarps * 32) bias_s[i] = bias ? __ldg(bias + i) : 0.f;
+        // (four at a time: 3136x512 -> 2048 9.99 us with single ones, 9.93 when they were still read ahead of the wait, 9.96 now)
+        for (int i = 4 * (tid - kFirstEpiWarp * 32) + z; i < p.O; i += 4 * kEpiWarps * 32)
+            *reinterpret_cast<float4 *>(bias_s + i) = bias ? __ldg(reinterpret_cast<const float4 *>(bias + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
         epi_sync();
     }
     const uint32_t tmem_base = bars->tmem_base;
@@ -323,7 +325,7 @@ linear_bb_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             const int row = mt * kRows + m;
             const bool valid = row < p.M;
             const int nch = width(nt) / 16;
-            const size_t o0 = (size_t)row * p.O + (size_t)nt * p.BN;
+            const size_t o0 = (size_t)row * p.O + (size_t)(nt * p.BN + z);
             const float *bs = bias_s + nt * p.BN;
             const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * p.BN;
 

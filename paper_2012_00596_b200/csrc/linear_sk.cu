@@ -88,10 +88,10 @@ linear_bb_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     const uint32_t tmem_base = bars->tmem_base;
     cluster_arrive();                  // this CTA is running: its shared memory may be written by the others
     pdl_wait();
-    bias = behind_wait(bias); res = behind_wait(res);
+    const int z = zero_behind_wait();
 
     if (warp >= 2)
-        for (int i = tid - 64; i < p.BN; i += kThreads - 64) bias_s[i] = (bias && i < cols) ? __ldg(bias + nt * p.BN + i) : 0.f;
+        for (int i = tid - 64 + z; i < p.BN; i += kThreads - 64) bias_s[i] = (bias && i < cols) ? __ldg(bias + nt * p.BN + i) : 0.f;
 
     if (warp == 0) {
         if (lane == 0) {
@@ -167,7 +167,7 @@ linear_bb_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     for (int i = tid; i < own * oct; i += kThreads) {
         const int r = i / oct, c0 = (i - r * oct) * 8;
         if (c0 >= cols) continue;
-        const size_t o0 = (size_t)(mt * kRows + rank * p.rpr + r) * p.O + (size_t)nt * p.BN + c0;
+        const size_t o0 = (size_t)(mt * kRows + rank * p.rpr + r) * p.O + (size_t)(nt * p.BN + c0 + z);
         const uint8_t *src = smem + p.off_red + (size_t)r * p.red_pitch + (size_t)c0 * 4;
         float v[8];
 #pragma unroll
