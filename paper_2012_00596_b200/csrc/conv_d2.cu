@@ -17,7 +17,8 @@
 //
 // The wide form (channels and filters in multiples of 16): the last slab of a position holds fewer than four chunks, the channels
 // past the end arriving as zeros that no MMA reads, and a CTA's half of the operand is several of the image's groups of 16, 32 or 64
-// filters, which one tensor copy lays next to one another (groups past the last one as zeros, their columns not stored).  Such
+// filters, which one tensor copy lays next to one another (a half that would go past the last group starts earlier; the columns it
+// shares with others are not stored).  Such
 // layers ran as the split form or on independent CTAs whose MMAs were as narrow as a group: 25x8x33x464 -> 480 73 -> 38 us,
 // 22x12x47x48 -> 432 33 -> 10.8, 17x64x21x320 -> 48 36 -> 12.5, 49x57x28x240 -> 96 strided 32 -> 21.
 //
@@ -39,6 +40,7 @@
 
 #include "common.cuh"
 #include "internal_api.h"
+#include "tail_start.h"
 #include "tc_pair.cuh"
 
 namespace npas {
@@ -256,8 +258,9 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         // 2048 bytes) and ONE box (128, 8, 1, rows of the stage) brings the stage's halves back to back (36
         // separate 1 KB copies per stage cost the issuing warp 2.5 k cycles, more than the stage's MMAs take).
         // One holding several groups (K off the multiples of 64, or 64 that fill no 128) has a map over (128 bytes, lines of
-        // a group's row, groups, rows of all (chunk, tap, octet)): ONE box puts the groups of every row next to one another,
-        // groups past the last one as zeros.
+        // a group's row, groups, rows of all (chunk, tap, octet)): ONE box puts the groups of every row next to one another.
+        // No box goes past the last group (tail_start.h; a blob that ended 256 bytes before unmapped memory ended in an illegal access):
+        // the last item's halves start earlier instead.
         const uint32_t copy_bytes = p.w_box_rows * 128u;      // 128 filters: one copy = one box of the weight map
         const bool runs = p.GH == 128 && !p.gathered;
         const int n_copies = runs ? (int)(p.w_bytes / copy_bytes) : 1;
@@ -282,7 +285,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 const uint32_t src = wsrc + (uint32_t)(chunk * 2 * p.RS) * (grow >> 7);     // rows of the image, in 128-byte map rows
                 if (p.gathered) {
                     if (lane == 0)
-                        tma_load_4d_pair(wdst, &tmap_w, w_full0 + s * 8u, 0, 0, fs * (p.NT / p.GI) + (int)rank * p.GG,
+                        tma_load_4d_pair(wdst, &tmap_w, w_full0 + s * 8u, 0, 0, tail_start((2 * fs + (int)rank) * p.GG, p.GG, p.K / p.GI),
                                          (int)(off_image / grow) + chunk * 2 * p.RS);
                 } else if (runs) {
                     for (int i = lane; i < n_copies; i += 32)
@@ -365,6 +368,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         const int il = p.IT > 1 ? m / p.img_pitch : 0, mr = m - il * p.img_pitch;    // image of the tile, position inside it
         const int oy = mr / p.Wp, ox = mr - oy * p.Wp;
         const int cpt = p.NT / 16;                          // chunks per position tile
+        const int groups = p.gathered ? p.K / p.GI : 0;
         const int sh = p.sh;                                // positions computed but not stored: divide by shifting
         const uint32_t acc_empty0 = map_to_cta(smem_u32(&bars->acc_empty[0]), 0u);   // the leader's
         uint32_t it = 0;
@@ -373,6 +377,9 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             const int ts = item / p.n_fsets, fs = item - ts * p.n_fsets;
             const uint32_t acc = it & (uint32_t)(p.nacc - 1), lap_acc = p.nacc == 4 ? it >> 2 : p.nacc == 2 ? it >> 1 : it;
             const int nch = p.MT * cpt;
+            // by how many filters each half of the columns starts early (by more than its width where it has none of its own)
+            const int g0 = 2 * fs * p.GG, g1 = g0 + p.GG;
+            const int early0 = p.gathered ? (g0 - tail_start(g0, p.GG, groups)) * p.GI : 0, early1 = p.gathered ? (g1 - tail_start(g1, p.GG, groups)) * p.GI : 0;
             const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * p.dcols;
 
             // where this thread's position of each tile goes (MT <= 2); with a stride the tile is computed
@@ -390,8 +397,9 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             auto finish = [&](const uint32_t (&r)[16], int j) {
                 const int mt = j >= cpt ? 1 : 0, c0 = (j - mt * cpt) * 16;
                 if (!(mt ? val[1] : val[0])) return;
-                const int k0 = fs * p.NT + c0;
-                if (k0 >= p.K) return;                      // the last item's filters past the end
+                const int early = c0 < p.GH ? early0 : early1;
+                if ((c0 < p.GH ? c0 : c0 - p.GH) < early) return;        // filters of another half
+                const int k0 = fs * p.NT + c0 - early;
                 const size_t o0 = (mt ? obase[1] : obase[0]) + k0;
                 float v[16];
                 const float4 *b4 = reinterpret_cast<const float4 *>(bias_s + k0);
@@ -598,7 +606,7 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             if (MT > 1 && p.n_tiles < 4) continue;
             ConvD2Params q = p;
             q.NT = NT; q.GH = NT / 2; q.MT = MT; q.n_fsets = (d.K + NT - 1) / NT;
-            q.gathered = gathered; q.GG = gathered ? q.GH / p.GI : 0;
+            q.gathered = gathered; q.GG = gathered ? q.GH / p.GI : 0;          // (NT < K + 2 GI: never more groups than there are)
             const long long items = (long long)((p.n_tiles + 2 * MT - 1) / (2 * MT)) * q.n_fsets;
             if (items > 0x7FFFFFFF) return false;
             q.n_items = (int)items;

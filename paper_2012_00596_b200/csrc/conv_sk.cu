@@ -18,6 +18,7 @@
 // What bounds it is the latency of the chain copy, MMAs, exchange, store: the weights are requested by a warp of their own, in
 // a chain of layers before the programmatic wait (`early`), the slabs right behind it.
 #include "common.cuh"
+#include "tail_start.h"
 #include "tc_pair.cuh"
 
 namespace npas {
@@ -81,7 +82,8 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int KS = p.KC * p.KT, rank = (int)cluster_ctarank(), work = blockIdx.x / KS;
-    const int tile = work / p.nFT, ft = work - tile * p.nFT, k0 = ft * p.NT;
+    // (the last tile of filters ends with the last one, tail_start.h, and leaves those it shares with the tile before to that one)
+    const int tile = work / p.nFT, ft = work - tile * p.nFT, k0 = tail_start(ft * p.NT, p.NT, p.K), shared = ft * p.NT - k0;
     const int img = tile / p.tiles_per_img, y0 = (tile - img * p.tiles_per_img) * p.TR;
     const int kc = rank / p.KT, kt = rank - kc * p.KT;
     const int blk_lo = kc * p.bpr, n_blk = max(0, min(p.nBlk - blk_lo, p.bpr));
@@ -155,7 +157,7 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     pdl_wait();
     const int z = zero_behind_wait();
     if (warp > 2)
-        for (int i = tid - 96 + z; i < p.NT; i += kThreads - 96) bias_s[i] = (bias && k0 + i < p.K) ? __ldg(bias + k0 + i) : 0.f;
+        for (int i = tid - 96 + z; i < p.NT; i += kThreads - 96) bias_s[i] = bias ? __ldg(bias + k0 + i) : 0.f;
 
     if (warp == 0) {
         // ---- slabs -----------------------------------------------------------------------------------------------
@@ -254,7 +256,7 @@ conv_bp_sk_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     const int oct = p.NT / 8;
     for (int i = tid; i < p.rpr * oct; i += kThreads) {
         const int r = i / oct, c0 = (i - r * oct) * 8, m = rank * p.rpr + r, oy = m / p.Wp, ox = m - oy * p.Wp, yy = y0 + oy;
-        if (m >= kRows || k0 + c0 >= p.K || oy >= p.TR || yy >= p.P || ox >= p.Q || ((yy | ox) & p.sh)) continue;
+        if (m >= kRows || c0 < shared || oy >= p.TR || yy >= p.P || ox >= p.Q || ((yy | ox) & p.sh)) continue;
         const size_t o0 = (((size_t)img * p.Po + (yy >> p.sh)) * p.Qo + (ox >> p.sh)) * p.K + (size_t)(k0 + c0 + z);
         const uint8_t *src = smem + p.off_red + (size_t)r * p.red_pitch + (size_t)c0 * 4;
         float v[8];
@@ -370,11 +372,12 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvSkParams &p, int 
     for (int nt = 16; nt <= 128; nt += 16) {
         if (want_nt && nt != want_nt) continue;
         if (nt < q.GI ? q.GI % nt != 0 : nt % q.GI != 0) continue;
-        if (!want_nt && nt > 16 && nt >= 2 * d.K) continue;
+        if (!want_nt && nt > d.K) continue;
+        const int tile = nt < d.K ? nt : d.K;                   // (a wider tile was asked for: all filters)
         for (int kc = 1; kc <= kMaxSplit && kc <= q.nBlk; ++kc)
             for (int kt = 1; kc * kt <= kMaxSplit && kt <= RS && kt <= 4; ++kt) {
                 if ((want_kc && kc != want_kc) || (want_kt && kt != want_kt)) continue;
-                q.NT = nt; q.nFT = (d.K + nt - 1) / nt; q.KC = kc; q.KT = kt;
+                q.NT = tile; q.nFT = (d.K + tile - 1) / tile; q.KC = kc; q.KT = kt;
                 q.bpr = (q.nBlk + kc - 1) / kc; q.tpr = (RS + kt - 1) / kt;
                 if ((kc - 1) * q.bpr >= q.nBlk || (kt - 1) * q.tpr >= RS) continue;     // a CTA without work
                 const int ks = kc * kt;
@@ -382,15 +385,15 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvSkParams &p, int 
                 if (ctas > (one_wave ? at_once(ks, sms) : 0x3FFFFFFF)) continue;
                 // the blob's tap unions (per image group and chunk) are read only where few enough blocks meet in a tile that a
                 // third of the taps must be missing: the two dependent reads cost 0.5 to 2 us where nothing else hides them
-                const int wide = nt > q.GI ? nt : q.GI, blocks = ((wide + bp.Mb - 1) / bp.Mb) * ((16 + bp.Nb - 1) / bp.Nb);
+                const int wide = tile > q.GI ? tile : q.GI, blocks = ((wide + bp.Mb - 1) / bp.Mb) * ((16 + bp.Nb - 1) / bp.Nb);
                 q.use_taps = bp.max_taps > 0 && blocks * bp.max_taps * 3 <= RS * 2;
-                q.lines = (nt < q.GI ? nt : q.GI) / 8;
+                q.lines = (tile < q.GI ? tile : q.GI) / 8;
                 q.rpr = (kRows + ks - 1) / ks;
-                q.w_chunk = 2u * q.tpr * nt * 16u;
+                q.w_chunk = 2u * q.tpr * tile * 16u;
                 q.stage_bytes = round_up((uint32_t)q.nph * q.act_stride + (uint32_t)(q.CB / 16) * q.w_chunk, 1024);
-                q.red_pitch = (uint32_t)nt * 4u + 16u;
+                q.red_pitch = (uint32_t)tile * 4u + 16u;
                 const uint32_t red = round_up((uint32_t)ks * q.rpr * q.red_pitch, 128);
-                const uint32_t fixed = red + round_up((uint32_t)nt * 4u, 128) + (uint32_t)sizeof(ConvSkBars) + 1024u + 128u;
+                const uint32_t fixed = red + round_up((uint32_t)tile * 4u, 128) + (uint32_t)sizeof(ConvSkBars) + 1024u + 128u;
                 if (fixed + q.stage_bytes > kSmemLimit) continue;
                 q.S = (int)((kSmemLimit - fixed) / q.stage_bytes);
                 if (q.S > q.bpr) q.S = q.bpr;
@@ -398,10 +401,10 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvSkParams &p, int 
                 if ((uint32_t)q.S * q.stage_bytes >= (1u << 18)) continue;               // descriptor addresses are 14 bits of 16 bytes
                 q.off_red = (uint32_t)q.S * q.stage_bytes;
                 q.off_bias = q.off_red + red;
-                q.off_bar = q.off_bias + round_up((uint32_t)nt * 4u, 128);
+                q.off_bar = q.off_bias + round_up((uint32_t)tile * 4u, 128);
                 q.smem_bytes = q.off_bar + (uint32_t)sizeof(ConvSkBars) + 1024u;
                 q.tmem_cols = 32;
-                while ((int)q.tmem_cols < nt) q.tmem_cols *= 2;
+                while ((int)q.tmem_cols < tile) q.tmem_cols *= 2;
                 const double cost = modelled(q, sms);
                 if (!found || cost < best) { best = cost; p = q; found = true; }
             }
@@ -490,7 +493,7 @@ int conv_sk_shapes(const npas_conv_desc &d, const npas_bp_desc &bp, int32_t *var
     const double best = modelled(p, sms);
     if (best > 1.5 * conv_dense_modelled(q, bp)) return 0;
     int n = 0;
-    for (int nt = 16; nt <= 128; nt += 16)
+    for (int nt = 16; nt <= 128 && nt <= d.K; nt += 16)
         for (int kc = 1; kc <= kMaxSplit; ++kc)
             for (int kt = 1; kc * kt <= kMaxSplit && kt <= 4; ++kt) {
                 q.variant = nt | (kc << 16) | (kt << 24);

@@ -1,6 +1,8 @@
 """Host-only checks of the kernel choice: the committed (case, path) table and the plan cache."""
 import ctypes
+import os
 import random
+import subprocess
 
 import pytest
 
@@ -115,6 +117,40 @@ def test_plan_of_the_pair_kernel_is_that_of_its_shape_alone(wide):
             planned += 1
             assert free == _pair_plan(*lay, 8, wide | free[0] | (free[1] << 16)), lay
     assert planned > (1500 if wide else 60)
+
+
+def test_tiles_of_filters_ask_for_nothing_past_the_last_and_store_every_filter_once(tmp_path):
+    """The last tiles of the wide pair kernel (two halves of whole filter groups) and of the split kernel, through the arithmetic that both
+    kernels use (csrc/tail_start.h, compiled here for the host): weights past the last filter are not asked for, which a tensor copy
+    would touch unmapped memory for, and what tiles share is stored by one of them."""
+    csrc = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2012_00596_b200", "csrc")
+    src, so = tmp_path / "tail.cpp", tmp_path / "tail.so"
+    src.write_text('#include "tail_start.h"\nextern "C" int start_of(int s, int w, int t) { return npas::tail_start(s, w, t); }\n')
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O1", "-std=c++17", "-fPIC", "-shared", "-I", csrc, "-o", str(so), str(src)])
+    start_of = ctypes.CDLL(str(so)).start_of
+    for K in range(16, 529, 16):
+        GI = 128
+        while K % GI:
+            GI //= 2
+        for NT in range(32, 257, 32):                              # the wide form's items
+            if GI >= 128 or NT % (2 * GI) or NT >= K + 2 * GI:
+                continue
+            GG, groups, stored = NT // 2 // GI, K // GI, []
+            for g0 in range(0, -(-K // NT) * 2 * GG, GG):
+                at = start_of(g0, GG, groups)
+                assert 0 <= at and at + GG <= groups, (K, NT, g0)
+                early = (g0 - at) * GI
+                stored += [g0 * GI + c - early for c in range(GG * GI) if c >= early]
+            assert stored == list(range(K)), (K, NT)
+        for NT in range(16, min(K, 128) + 1, 16):                  # the split form's tiles
+            if (GI % NT if NT < GI else NT % GI):
+                continue
+            stored = []
+            for k in range(0, K, NT):
+                at = start_of(k, NT, K)
+                assert 0 <= at and at + NT <= K and at % min(GI, NT) == 0, (K, NT, k)
+                stored += range(k, at + NT)
+            assert stored == list(range(K)), (K, NT)
 
 
 def test_plan_cache_round_trip_and_rejects_garbage():
