@@ -23,6 +23,7 @@ LINEARS = {"split": (64, 2048, 1024, 0, 0, 5), "single": (3136, 512, 512, 5, 0, 
 
 def _captured(f):
     s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
     with torch.cuda.stream(s):
         f()
     torch.cuda.synchronize()

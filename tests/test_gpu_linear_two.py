@@ -86,6 +86,7 @@ def test_network_with_layers_taken_together(N, H):
 
 def _graph_ms(f):
     s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
     with torch.cuda.stream(s):
         f()
     torch.cuda.synchronize()

@@ -34,6 +34,7 @@ def test_projections_beside_the_block(N, H):
     assert not bad
     x = xs[0].clone()
     s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
     with torch.cuda.stream(s):
         net.forward(x)
     torch.cuda.synchronize()

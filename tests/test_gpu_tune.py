@@ -85,6 +85,7 @@ def test_tuned_linear_plan_is_valid_and_not_slower():
 def _graph_us(f, reps=20):
     """Microseconds per call of a captured chain of calls (no host time in it), the best of several replays."""
     s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
     with torch.cuda.stream(s):
         f()
     torch.cuda.synchronize()
