@@ -12,32 +12,35 @@ pytestmark = pytest.mark.gpu
 WIDE = 1 << 24
 
 
-@pytest.mark.parametrize("kw", [
-    dict(N=2, H=14, W=14, C=16, K=16, Mb=16, Nb=8, keep=3),                       # a quarter of a channel block, half of an item's filters
-    dict(N=3, H=13, W=17, C=80, K=176, Mb=16, Nb=16, keep=4),                     # groups of 16, the last item lacks some
-    dict(N=2, H=20, W=11, C=112, K=96, Mb=32, Nb=16, keep=9),                     # groups of 32, three chunks in the last block
-    dict(N=1, H=30, W=30, C=272, K=272, Mb=16, Nb=16, keep=lambda fb, cb: (fb + cb) % 4),   # blocks without taps; 17 groups of 16
-    dict(N=2, H=9, W=30, C=128, K=320, Mb=16, Nb=8, keep=2),                      # groups of 64
-    dict(N=2, H=12, W=12, C=48, K=128, Mb=8, Nb=8, keep=5),                       # groups of 128 beside a partial channel block
-    dict(N=5, H=7, W=7, C=144, K=48, Mb=16, Nb=16, keep=3),                       # several images per tile
-    dict(N=3, H=15, W=13, C=32, K=32, Mb=16, Nb=16, keep=4, stride=2),            # by phases
-    dict(N=2, H=29, W=40, C=96, K=208, Mb=16, Nb=8, keep=9, stride=2),            # by phases, partial block, 13 groups of 16
-    dict(N=2, H=11, W=10, C=48, K=80, Mb=16, Nb=8, keep=1, R=1, S=1, pad=0),      # one tap
-    dict(N=1, H=9, W=12, C=80, K=48, Mb=16, Nb=8, keep=4, R=4, S=4, pad=1, stride=2),       # 16 taps, strided without phases
-    dict(N=40, H=28, W=28, C=80, K=112, Mb=16, Nb=16, keep=3),                    # more items than CTA pairs
+SHAPES = {"32x1": 32 | (1 << 16), "64x1": 64 | (1 << 16), "96x2": 96 | (2 << 16), "128x2": 128 | (2 << 16), "192x1": 192 | (1 << 16)}
+
+
+# takes: the shapes (filters per item x position tiles per CTA) that have to be taken; all others have to be refused
+@pytest.mark.parametrize("takes,kw", [
+    ("32x1", dict(N=2, H=14, W=14, C=16, K=16, Mb=16, Nb=8, keep=3)),             # a quarter of a channel block, half of an item's filters
+    ("32x1 64x1 96x2 128x2 192x1", dict(N=3, H=13, W=17, C=80, K=176, Mb=16, Nb=16, keep=4)),     # groups of 16, the last item lacks some
+    ("64x1 128x2", dict(N=2, H=20, W=11, C=112, K=96, Mb=32, Nb=16, keep=9)),     # groups of 32, three chunks in the last block
+    ("32x1 64x1 96x2 128x2 192x1", dict(N=1, H=30, W=30, C=272, K=272, Mb=16, Nb=16, keep=lambda fb, cb: (fb + cb) % 4)),   # blocks without taps; 17 groups of 16
+    ("64x1 128x2", dict(N=2, H=9, W=30, C=128, K=320, Mb=16, Nb=8, keep=2)),      # groups of 64
+    ("128x2", dict(N=2, H=12, W=12, C=48, K=128, Mb=8, Nb=8, keep=5)),            # groups of 128 beside a partial channel block
+    ("32x1 64x1", dict(N=5, H=7, W=7, C=144, K=48, Mb=16, Nb=16, keep=3)),        # several images per tile: too few tiles for two
+    ("64x1", dict(N=3, H=15, W=13, C=32, K=32, Mb=16, Nb=16, keep=4, stride=2)),  # by phases
+    ("32x1 64x1 192x1", dict(N=2, H=29, W=40, C=96, K=208, Mb=16, Nb=8, keep=9, stride=2)),       # by phases, partial block, 13 groups of 16
+    ("32x1 64x1", dict(N=2, H=11, W=10, C=48, K=80, Mb=16, Nb=8, keep=1, R=1, S=1, pad=0)),       # one tap
+    ("32x1 64x1", dict(N=1, H=9, W=12, C=80, K=48, Mb=16, Nb=8, keep=4, R=4, S=4, pad=1, stride=2)),      # 16 taps, strided without phases
+    ("32x1 64x1 96x2 128x2", dict(N=40, H=28, W=28, C=80, K=112, Mb=16, Nb=16, keep=3)),          # more items than CTA pairs
 ])
-@pytest.mark.parametrize("variant", [0, 32 | (1 << 16), 96 | (2 << 16), 192 | (1 << 16)])
-def test_wide_form_matches_oracle(kw, variant):
+@pytest.mark.parametrize("shape", [None, *SHAPES])
+def test_wide_form_matches_oracle(takes, kw, shape):
     c = inputs.conv_case(dtype="bf16", residual=True, seed=310, **kw)
-    if variant:
-        try:
-            y = run_case(c, path=7, variant=WIDE | variant)
-        except npas.NpasError as e:                                               # (not every shape divides, or fits)
-            assert e.code == 8
-            return
-    else:
-        y = run_case(c, path=7, variant=WIDE)
-        assert torch.equal(y, run_case(c, path=7, variant=WIDE))                  # run-to-run determinism
+    variant = WIDE | (SHAPES[shape] if shape else 0)
+    if shape and shape not in takes.split():
+        with pytest.raises(npas.NpasError) as e:
+            run_case(c, path=7, variant=variant)
+        assert e.value.code == 8
+        return
+    y = run_case(c, path=7, variant=variant)
+    assert torch.equal(y, run_case(c, path=7, variant=variant))                   # run-to-run determinism
     assert floored_rel_err(host(y), oracle_case(c)) < TOL_BF16
 
 
