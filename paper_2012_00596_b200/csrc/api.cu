@@ -146,7 +146,7 @@ static ConvChoice conv_choose(const npas_conv_desc &d, const npas_bp_desc &bp)
     return {d.path == 2 ? 0 : 1, false, false};
 }
 
-// (kept per thread like the plans: up to ten of them are compared)
+// (kept per thread like the plans: several of them are compared)
 static ConvChoice conv_choice(const npas_conv_desc &d, const npas_bp_desc &bp)
 {
     ConvChoice c{};

@@ -26,7 +26,7 @@
 // tiles of an image share one slab: 59 + 36 KB per item came in for 64x56x56x64 -> 64, 44 now (23.0 -> 22.5 us; 28x28x64 -> 128 13.6 -> 13.2).
 //
 // Roles per CTA (384 threads): warp 0 loads the slabs (ring of 64-channel stages), warp 2 loads this CTA's
-// half of the weight tiles through a 2-D tensor map laid over the blob (ring of 16- or 32-channel stages),
+// half of the weight tiles through a tensor map laid over the blob (ring of stages of 16, 32 or 64 channels),
 // warps 1 and 3 of the pair's leader (cluster rank 0) issue the MMAs, one warp per position tile and
 // accumulator, and, when they retire, signal the "empty" barriers and at the end of an item the
 // "accumulator full" barrier of BOTH CTAs (multicast commit).  Both CTAs' tensor copies complete on the
@@ -70,7 +70,7 @@ struct ConvD2Params {
     uint32_t tile16;                                          // from one position tile's slab to the next one's, 16-byte units
     int gathered, GG;                                         // a CTA's filters are GG whole groups of the image (else one group, or half of one)
     int RS, nCh, nBlk, GH, NT, MT, CPW, n_fsets, n_items, SA, SB, nacc, dcols;   // GH: filters per CTA, NT = 2 GH per item; CPW: chunks per weight stage
-    int GI;                                                   // filters per group of the blob's operand image (128, or 64 when 128 does not divide K)
+    int GI;                                                   // filters per group of the blob's operand image (the largest power of two up to 128 that divides K; wide form from 16 on, else 64)
     int relu, y_bf16, early;                                  // early: the blob may be read before the wait (Launch::blob_ready)
     uint32_t slab_bytes, act_stride, a_stage_bytes, w_bytes, off_w, off_tapu, off_bias, off_bar, smem_bytes, tmem_cols;
     uint32_t shift16[kMaxTapsD2];                             // operand start of every tap inside a tile's slabs, 16-byte units
@@ -620,8 +620,8 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
                 q.slab_bytes = (uint32_t)q.slab_rows * p.Wp * 128u;
                 q.act_stride = q.a_stage_bytes = round_up(reach + pitch > q.slab_bytes ? reach + pitch : q.slab_bytes, 1024);
             }
-            // a weight stage holds two chunks of a 64-filter half (32 KB at nine taps, as one chunk of a
-            // 128-filter half), one where the slabs leave no room for two such stages
+            // a weight stage holds one chunk of a half of more than 64 filters, two of one of 33 to 64 and four of a narrower one (up to
+            // 36 KB at nine taps), fewer where the slabs leave no room for two such stages
             // (whatever divides the chunks: a wait and a commit per chunk of nine MMAs made an odd number of chunks a third slower,
             // 37x8x16x368 -> 80 15.6 us on stages of one chunk and 10.5, 3x42x51x240 -> 96 11.7 and 8.7)
             q.CPW = q.GH > 64 ? 1 : q.GH > 32 ? 2 : 4;
