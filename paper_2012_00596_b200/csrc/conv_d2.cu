@@ -68,7 +68,7 @@ struct ConvD2Params {
     int IT, img_pitch;                                        // small maps: IT whole images per tile, img_pitch positions apart
     int NSL, resident;                                        // slabs per stage and phase; resident: all weight stages stay in shared memory
     uint32_t tile16;                                          // from one position tile's slab to the next one's, 16-byte units
-    int gathered, GG;                                         // a CTA's filters are GG whole groups of the image (else one group, or half of one)
+    int gathered, GG, groups;                                 // a CTA's filters are GG whole groups of the image (else one group, or half of one), which has `groups`
     int RS, nCh, nBlk, GH, NT, MT, CPW, n_fsets, n_items, SA, SB, nacc, dcols;   // GH: filters per CTA, NT = 2 GH per item; CPW: chunks per weight stage
     int GI;                                                   // filters per group of the blob's operand image (the largest power of two up to 128 that divides K; wide form from 16 on, else 64)
     int relu, y_bf16, early;                                  // early: the blob may be read before the wait (Launch::blob_ready)
@@ -122,6 +122,10 @@ __device__ __forceinline__ void tma_load_4d_pair(void *dst, const CUtensorMap *m
 // barrier among all warps but the two producers
 __device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 3, %0;" ::"n"(kThreads - 64) : "memory"); }
 
+// kGathered: a CTA's filters are several whole groups of the image.  kPart: the last channel block holds fewer than four chunks (its last
+// weight stage may start early).  Looked up per chunk and item by one kernel they cost the layers that need neither 2 to 3 %:
+// 32x14x14x256 -> 256 10.35 us, now 10.11; 64x7x7x512 -> 512 15.50 and 15.13; 30x6x61x128 -> 512 strided 8.32 and 8.06.
+template <bool kGathered, bool kPart>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w, const ConvD2Params p,
                   const uint8_t *__restrict__ blob, const float *__restrict__ bias,
@@ -178,8 +182,10 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     if (warp != 0 && warp != 2) {
         const int t = tid < 64 ? tid - 32 : tid - 64;         // 0 .. kThreads - 65 over warps 1, 3, 4, ...
         const uint32_t *tapu = reinterpret_cast<const uint32_t *>(blob + off_tapu);
-        const int ngrp = p.NT / p.GI, groups = p.K / p.GI;        // groups of the image per item
-        for (int i = t; i < p.n_fsets * p.nCh; i += kThreads - 64) {
+        const int ngrp = p.NT / p.GI, groups = p.groups;          // groups of the image per item
+        if (!kGathered && ngrp == 1)                              // (the usual case: no division on the way to the first MMA)
+            for (int i = t; i < p.n_fsets * p.nCh; i += kThreads - 64) tapu_s[i] = off_tapu ? __ldg(tapu + i) : 0xFFFFFFFFu;
+        else for (int i = t; i < p.n_fsets * p.nCh; i += kThreads - 64) {
             const int fs = i / p.nCh, ch = i - fs * p.nCh;
             uint32_t m = off_tapu ? 0u : 0xFFFFFFFFu;
             if (off_tapu)
@@ -262,7 +268,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         // No box goes past the last group (tail_start.h; a blob that ended 256 bytes before unmapped memory ended in an illegal access):
         // the last item's halves start earlier instead.
         const uint32_t copy_bytes = p.w_box_rows * 128u;      // 128 filters: one copy = one box of the weight map
-        const bool runs = p.GH == 128 && !p.gathered;
+        const bool runs = p.GH == 128 && !kGathered;
         const int n_copies = runs ? (int)(p.w_bytes / copy_bytes) : 1;
         const uint32_t grow = (uint32_t)p.GI * 16u;           // bytes of a (tap, octet) row of the image: GI filters x 8 channels
         const uint32_t w_full0 = map_to_cta(smem_u32(&bars->w_full[0]), 0u);      // the leader's barriers
@@ -283,9 +289,9 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 if (!ok) break;
                 uint8_t *wdst = smem + p.off_w + (size_t)s * p.w_bytes;
                 const uint32_t src = wsrc + (uint32_t)(chunk * 2 * p.RS) * (grow >> 7);     // rows of the image, in 128-byte map rows
-                if (p.gathered) {
+                if (kGathered) {
                     if (lane == 0)
-                        tma_load_4d_pair(wdst, &tmap_w, w_full0 + s * 8u, 0, 0, tail_start((2 * fs + (int)rank) * p.GG, p.GG, p.K / p.GI),
+                        tma_load_4d_pair(wdst, &tmap_w, w_full0 + s * 8u, 0, 0, tail_start((2 * fs + (int)rank) * p.GG, p.GG, p.groups),
                                          (int)(off_image / grow) + chunk * 2 * p.RS);
                 } else if (runs) {
                     for (int i = lane; i < n_copies; i += 32)
@@ -333,14 +339,14 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                         if (!pair_wait(&bars->a_full[sa], pha, abort_flag, peer_abort, ws, 0x7300)) { ok = false; break; }
                         uint32_t a16 = a_st;                    // 16 channels = 32 bytes inside the swizzled 128-byte row
                         // (the last block may hold fewer chunks: its slab's other channels are zeros that nothing reads)
-                        const int end = min(ch + 4, p.nCh);
+                        const int end = kPart ? min(ch + 4, p.nCh) : ch + 4;
                         while (ch < end) {
                             // (stages that stay are complete for good: the parity of their first and only phase)
                             if (!pair_wait(&bars->w_full[sb], p.resident ? 0u : phb, abort_flag, peer_abort, ws, 0x7320)) { ok = false; break; }
                             tc_fence_after_sync();
                             uint32_t b_lo = b_st;
-                            if (ch + p.CPW > p.nCh) b_lo += (uint32_t)(ch + p.CPW - p.nCh) * chunk16;
-                            for (int cc = 0; cc < p.CPW && ch < end; ++cc, ++ch, a16 += 2u, b_lo += chunk16) {
+                            if (kPart && ch + p.CPW > p.nCh) b_lo += (uint32_t)(ch + p.CPW - p.nCh) * chunk16;
+                            for (int cc = 0; cc < p.CPW && (!kPart || ch < end); ++cc, ++ch, a16 += 2u, b_lo += chunk16) {
                                 // a tap that no block of these (groups, chunk) keeps multiplies zeros: skipped, except
                                 // the very first MMA, which initialises the accumulator
                                 const uint32_t m = tu[ch] | (ch == 0 ? 1u : 0u);
@@ -368,7 +374,6 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         const int il = p.IT > 1 ? m / p.img_pitch : 0, mr = m - il * p.img_pitch;    // image of the tile, position inside it
         const int oy = mr / p.Wp, ox = mr - oy * p.Wp;
         const int cpt = p.NT / 16;                          // chunks per position tile
-        const int groups = p.gathered ? p.K / p.GI : 0;
         const int sh = p.sh;                                // positions computed but not stored: divide by shifting
         const uint32_t acc_empty0 = map_to_cta(smem_u32(&bars->acc_empty[0]), 0u);   // the leader's
         uint32_t it = 0;
@@ -379,7 +384,7 @@ conv_bp_d2_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             const int nch = p.MT * cpt;
             // by how many filters each half of the columns starts early (by more than its width where it has none of its own)
             const int g0 = 2 * fs * p.GG, g1 = g0 + p.GG;
-            const int early0 = p.gathered ? (g0 - tail_start(g0, p.GG, groups)) * p.GI : 0, early1 = p.gathered ? (g1 - tail_start(g1, p.GG, groups)) * p.GI : 0;
+            const int early0 = kGathered ? (g0 - tail_start(g0, p.GG, p.groups)) * p.GI : 0, early1 = kGathered ? (g1 - tail_start(g1, p.GG, p.groups)) * p.GI : 0;
             const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * p.dcols;
 
             // where this thread's position of each tile goes (MT <= 2); with a stride the tile is computed
@@ -606,7 +611,7 @@ bool plan(const npas_conv_desc &d, const npas_bp_desc &bp, ConvD2Params &p, int 
             if (MT > 1 && p.n_tiles < 4) continue;
             ConvD2Params q = p;
             q.NT = NT; q.GH = NT / 2; q.MT = MT; q.n_fsets = (d.K + NT - 1) / NT;
-            q.gathered = gathered; q.GG = gathered ? q.GH / p.GI : 0;          // (NT < K + 2 GI: never more groups than there are)
+            q.gathered = gathered; q.GG = gathered ? q.GH / p.GI : 0; q.groups = d.K / p.GI;      // (NT < K + 2 GI: never more groups than there are)
             const long long items = (long long)((p.n_tiles + 2 * MT - 1) / (2 * MT)) * q.n_fsets;
             if (items > 0x7FFFFFFF) return false;
             q.n_items = (int)items;
@@ -811,10 +816,13 @@ npas_status conv_d2_launch(const npas_conv_desc &d, const npas_bp_desc &bp, cons
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return NPAS_ERR_CUDA;
     }
-    if (allow_dynamic_smem(reinterpret_cast<const void *>(conv_bp_d2_kernel), (int)kSmemLimit) != NPAS_OK) return NPAS_ERR_CUDA;
+    const bool part = p.nCh % 4 != 0;                     // (stages of one, two or four chunks divide a whole block)
+    auto kernel = p.gathered ? (part ? conv_bp_d2_kernel<true, true> : conv_bp_d2_kernel<true, false>)
+                             : (part ? conv_bp_d2_kernel<false, true> : conv_bp_d2_kernel<false, false>);
+    if (allow_dynamic_smem(reinterpret_cast<const void *>(kernel), (int)kSmemLimit) != NPAS_OK) return NPAS_ERR_CUDA;
     const int n_pairs = p.n_items < pairs ? p.n_items : pairs;
     p.early = how.blob_ready;
-    const cudaError_t e = launch_pdl(how, conv_bp_d2_kernel, dim3(2 * n_pairs), dim3(kThreads), p.smem_bytes, st, tmap, tmap_w, p,
+    const cudaError_t e = launch_pdl(how, kernel, dim3(2 * n_pairs), dim3(kThreads), p.smem_bytes, st, tmap, tmap_w, p,
                                      static_cast<const uint8_t *>(blob), bias, res, y, ws);
     count_launch();
     return e == cudaSuccess ? launch_status() : NPAS_ERR_CUDA;
