@@ -13,7 +13,7 @@
 // Why matrix instructions: they run at the rate of the FMA instructions (64 FMAs per cycle and SM measured for both), but
 // an 8x8x4 tile takes 64 operand words where FMAs fed from shared memory need one or two 16-byte loads per four FMAs; with
 // FMAs the shared-memory path set the pace.  392x512 -> 512, 64x64 blocks keeping 32x32: 543 us with one row per thread
-// walking the lists, 28.6 with 2x4 register tiles, 16.3 with four groups of them; with matrix instructions 9.5, and 8.1 on 136
+// walking the lists, 28.6 with 2x4 register tiles, 16.3 with four groups of them; with matrix instructions 9.5, and 7.9 on 136
 // CTAs of 24 rows with the next block's loads on their way.
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -76,6 +76,10 @@ __device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b)
     asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
 }
 
+// Where the sum of row r of a block and row m of X lies in a group's accumulators: neighbours change places in every other eight rows, or a
+// half warp that reads sixteen rows of one m would meet every bank twice.
+__device__ __forceinline__ int acc_at(int r, int m) { return r * kAccPitch + (m ^ (r >> 3 & 1)); }
+
 struct LinSimtSmem { uint32_t groups, group_threads, phase_cols, off_grp, grp_bytes, bytes; };
 
 // Shared memory: the staged rows of X, then the accumulators of every group.
@@ -88,7 +92,7 @@ inline LinSimtSmem smem_plan(const npas_bb_desc &bb, int rows)
     s.grp_bytes = (uint32_t)bb.Bo * kAccPitch * 8u;
     s.group_threads = bb.Bo > 24 ? 128u : (uint32_t)(bb.Bo + 7) / 8 * 32u;
     s.groups = kMaxWarps * 32 / s.group_threads;
-    const uint32_t room = (232448u - 256u - s.off_grp) / s.grp_bytes;      // (beside the staged biases)
+    const uint32_t room = (232448u - 512u - s.off_grp) / s.grp_bytes;      // (beside the staged biases)
     if (s.groups > kMaxGroups) s.groups = kMaxGroups;
     if (s.groups > room) s.groups = room;
     if (s.groups > nBi) s.groups = nBi;
@@ -122,12 +126,13 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
 {
     constexpr int kRows = 8 * MT;
     extern __shared__ __align__(16) uint8_t sm[];
-    __shared__ float bias_s[64];
+    __shared__ double bias_s[64];
     const int t = threadIdx.x, nt = blockDim.x, gt = (int)S.group_threads, g = t / gt, tg = t - g * gt, lane = t & 31;
     float *xraw = reinterpret_cast<float *>(sm);                                               // [kRows][pitch]
     double *acc = reinterpret_cast<double *>(sm + S.off_grp + (size_t)g * S.grp_bytes);       // [Bo][kAccPitch]
 
-    const int bo = blockIdx.y, m0 = blockIdx.x * kRows, rows_here = min(kRows, d.M - m0), nBi = (int)L.nBi, G = (int)S.groups;
+    int bo = blockIdx.y, m0 = blockIdx.x * kRows;
+    const int rows_here = min(kRows, d.M - m0), nBi = (int)L.nBi, G = (int)S.groups;
     const bool x16 = sizeof(TX) == 4 && (d.I & 3) == 0 && (Bi & 3) == 0;
     const bool x2 = (d.I & 1) == 0 && (Bi & 1) == 0;
     const int per_phase = (int)S.phase_cols / Bi, k = lane & 3, q = lane >> 2, r_first = (tg >> 5) * 8;
@@ -136,7 +141,8 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
     if (g < G)                                                                                 // (the threads behind the groups help with X and Y)
         for (int e = tg; e < Bo * kAccPitch; e += gt) acc[e] = 0;
     tc::pdl_wait();
-    x = tc::behind_wait(x); blob = tc::behind_wait(blob); bias = tc::behind_wait(bias);
+    const int z = tc::zero_behind_wait();                              // (every address below follows from these two; opaque pointers: up to 3 % slower)
+    bo += z; m0 += z;
     const uint32_t *voff = reinterpret_cast<const uint32_t *>(blob + L.off_voff);
     const TX *vals = reinterpret_cast<const TX *>(blob + L.off_values);
 
@@ -177,7 +183,7 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
             else stage_row<true>(dst, src, width, x2, lane);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
-        if (t < Bo) bias_s[t] = bias ? __ldg(bias + bo * Bo + t) : 0.f;
+        if (t < Bo) bias_s[t] = bias ? (double)__ldg(bias + bo * Bo + t) : 0.;
         Part first = part(now, r_first, 0);
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
@@ -210,7 +216,7 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
                     for (int m = 0; m < MT; ++m) {
                         double2 *s = reinterpret_cast<double2 *>(acc + row * kAccPitch + m * 8 + 2 * k);
                         double2 v = *s;
-                        v.x += a[m][0]; v.y += a[m][1];
+                        v.x += row & 8 ? a[m][1] : a[m][0]; v.y += row & 8 ? a[m][0] : a[m][1];      // (acc_at)
                         *s = v;
                     }
                 }
@@ -219,37 +225,53 @@ linear_bb_simt_kernel(npas_linear_desc d, int Bo, int Bi, BbLayout L, LinSimtSme
         }
     }
     __syncthreads();
-    // the groups' sums in order, bias, residual, ReLU, one rounding.  A warp takes eight outputs of four rows at a time: whole
-    // 32-byte sectors of Y, and no two lanes of a half warp on one bank of the accumulators.
-    res = tc::behind_wait(res);
+    // The groups' sums in order, bias, residual, ReLU, one rounding.
     const double *acc0 = reinterpret_cast<const double *>(sm + S.off_grp);
     const size_t acc_step = S.grp_bytes / 8;
-    const int across = (Bo + 7) / 8, warps = nt >> 5, step_r = warps % across, step_m = warps / across;
-    int ru = (t >> 5) % across, mu = (t >> 5) / across;
-    for (const int m4 = (rows_here + 3) / 4; mu < m4;) {
-        // (four at a time: their loads do not wait for one another's stores)
-        int r[4], m[4];
-        float rv[4];
-        double v[4];
+    if (res) {
+        // A warp takes eight outputs of four rows at a time: whole 32-byte sectors.  Four of them, so that the residual's loads do
+        // not wait for one another's stores.
+        const int across = (Bo + 7) / 8, warps = nt >> 5, step_r = warps % across, step_m = warps / across;
+        int ru = (t >> 5) % across, mu = (t >> 5) / across;
+        for (const int m4 = (rows_here + 3) / 4; mu < m4;) {
+            int r[4], m[4];
+            float rv[4];
+            double v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            r[j] = ru * 8 + (lane & 7); m[j] = mu * 4 + (lane >> 3);
-            if (r[j] >= Bo || m[j] >= rows_here) m[j] = -1;
-            ru += step_r; mu += step_m;
-            if (ru >= across) { ru -= across; ++mu; }
-            rv[j] = res && m[j] >= 0 ? lin_load<true>(res + (size_t)(m0 + m[j]) * d.O + bo * Bo + r[j]) : 0.f;
-            v[j] = m[j] >= 0 ? acc0[r[j] * kAccPitch + m[j]] : 0.;
+            for (int j = 0; j < 4; ++j) {
+                r[j] = ru * 8 + (lane & 7); m[j] = mu * 4 + (lane >> 3);
+                if (r[j] >= Bo || m[j] >= rows_here) m[j] = -1;
+                ru += step_r; mu += step_m;
+                if (ru >= across) { ru -= across; ++mu; }
+                rv[j] = m[j] >= 0 ? lin_load<true>(res + (size_t)(m0 + m[j]) * d.O + bo * Bo + r[j]) : 0.f;
+                v[j] = m[j] >= 0 ? acc0[acc_at(r[j], m[j])] : 0.;
+            }
+            for (int i = 1; i < G; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] += m[j] >= 0 ? acc0[i * acc_step + acc_at(r[j], m[j])] : 0.;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (m[j] < 0) continue;
+                v[j] += bias_s[r[j]];
+                v[j] += (double)rv[j];
+                if (d.relu) v[j] = v[j] > 0 ? v[j] : 0;
+                lin_store(y + (size_t)(m0 + m[j]) * d.O + bo * Bo + r[j], (float)v[j]);
+            }
         }
-        for (int i = 1; i < G; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) v[j] += m[j] >= 0 ? acc0[i * acc_step + r[j] * kAccPitch + m[j]] : 0.;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (m[j] < 0) continue;
-            v[j] += (double)bias_s[r[j]];
-            v[j] += (double)rv[j];
-            if (d.relu) v[j] = v[j] > 0 ? v[j] : 0;
-            lin_store(y + (size_t)(m0 + m[j]) * d.O + bo * Bo + r[j], (float)v[j]);
+    } else {
+        // Consecutive threads along the row of Y.  (The form above without its loads: 1722x64 -> 512 7.5 us, here 5.7; 3136x64 -> 512 13.2 and
+        // 10.4; 392x512 -> 512 8.1 and 7.9.)
+        const int step_r = nt % Bo, step_m = nt / Bo;
+        int r = t % Bo;
+#pragma unroll 4
+        for (int m = t / Bo; m < rows_here;) {
+            double v = acc0[acc_at(r, m)];
+            for (int i = 1; i < G; ++i) v += acc0[i * acc_step + acc_at(r, m)];
+            v += bias_s[r];
+            if (d.relu) v = v > 0 ? v : 0;
+            lin_store(y + (size_t)(m0 + m) * d.O + bo * Bo + r, (float)v);
+            r += step_r; m += step_m;
+            if (r >= Bo) { r -= Bo; ++m; }
         }
     }
 }

@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
     (33, 640, 120, 40, 64, 33, 33), (16, 1088, 64, 64, 64, 16, 16), (300, 256, 512, 32, 32, 16, 32), (160, 512, 512, 16, 64, 8, 32),
     (200, 64, 1000, 8, 64, 4, 32), (700, 64, 512, 16, 64, 8, 16), (7, 36, 20, 4, 6, 2, 3), (65, 30, 33, 11, 10, 5, 0),
 ])
-@pytest.mark.parametrize("dtype,residual", [("f32", False), ("f32", True), ("bf16", True)])
+@pytest.mark.parametrize("dtype,residual", [("f32", False), ("f32", True), ("bf16", False), ("bf16", True)])
 def test_float64_gemm_at_the_edges(M, I, O, Bo, Bi, kr, kc, dtype, residual):
     c = inputs.linear_case(M=M, I=I, O=O, Bo=Bo, Bi=Bi, keep_rows=kr, keep_cols=kc, dtype=dtype, seed=1101)
     res = inputs.rng_for(1102).standard_normal((M, O), dtype=np.float32) if residual else None
