@@ -14,8 +14,8 @@
 // waits and conversions of 0.4 us, twice what its MMAs take), one warp for the residual, one for the stores.  Slots are taken in
 // the order of the slabs of Y1 and Y2 of a tile.  (Asking L2 for residual slabs ahead of their slots made it slower: 47 -> 60 us.)
 //
-// What bounds it: bytes (262 MB at least for 64 images of 56x56, 39 us at the copy rate; 47.5, the two launches 56.9), and for
-// few images the chain of both products.
+// What bounds it: for 64 images of 56x56 mostly bytes (262 MB at least, 40 us at the copy rate; 49.3 in calls by themselves, the two
+// launches 58.5), the rest being the chain of waits of a slab; for few images the chain of both products.
 #include "common.cuh"
 #include "tc_common.cuh"
 
@@ -399,7 +399,7 @@ bool encode_2d(CUtensorMap *map, const void *base, uint64_t inner, uint64_t oute
 }  // namespace
 
 // Two layers in one launch where both layers' weights stay in shared memory beside two X tiles and five slots, whatever the
-// rows (64 -> 256 -> 64, us, against the two launches: 784 rows 6.7 and 7.8, 12544 7.6 and 9.1, 200704 47.5 and 56.9).  With weights
+// rows (64 -> 256 -> 64, us, against the two launches: 784 rows 6.7 and 7.8, 12544 7.6 and 9.1, 200704 49.3 and 58.5).  With weights
 // that come through a ring, or too few slots for the residual's latency, it is the slower way (50176x128 -> 512 -> 128 44 and
 // 34, 50176x128 -> 256 -> 64 21.2 and 20.0): every CTA reads all weights again for each of its tiles.
 bool linear_two_preferred(const npas_linear_desc &a, const npas_linear_desc &b)
